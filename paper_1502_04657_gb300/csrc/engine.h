@@ -89,15 +89,15 @@ struct fmg_eig_handle {
   std::vector<void*> allocs;
   size_t bytes = 0;  // device bytes allocated
   bool dry = false;  // count the bytes of every allocation without allocating
-  int nh = 0, ntri = 0, nvert = 3, maxadj = 6;
+  int nh = 0, ntri = 0, nvert = 3;
   double tri_vol = 0.0;
   // per-instance arrays (sorted order): L1, M1, L1inv nh*nh; c, cstart nh + 1; scalars 1
   // L1 = A + W on level 1 (the small nonlinear solves), L1A the operator whose inverse is the
   // coarsest V-cycle solve (the same array unless the form is paper-literal)
   double *L1 = nullptr, *L1A = nullptr, *M1 = nullptr, *L1inv = nullptr;
-  int *tri = nullptr, *adj = nullptr;
-  int npat = 0;  // gather lists of the dense G(c) assembly (DenseProblem)
-  int *gent = nullptr, *gstart = nullptr, *gidx = nullptr;
+  int* tri = nullptr;
+  uint16_t* lists = nullptr;  // sparsity lists of the small dense solves (dense_lists.h)
+  fmg::DenseLists dims;
   double *lam = nullptr, *c = nullptr, *cstart = nullptr, *auu = nullptr, *buu = nullptr,
          *partials = nullptr, *partials2 = nullptr, *t3 = nullptr, *t3_partials = nullptr, *gAd = nullptr,
          *gMd = nullptr, *t1d = nullptr, *B1d = nullptr, *t0 = nullptr,

@@ -388,12 +388,11 @@ void build_coarse(fmg_eig_handle* h) {
   const int dim = h->prob.dim;
   const int nb = h->nb;
   const double H = h->prob.box_len / n1;
-  std::vector<int> tri, adj;
+  std::vector<int> tri;
   if (dim == 2) {
     h->nh = m * m;
     h->nvert = 3;
     h->ntri = 2 * n1 * n1;
-    h->maxadj = 6;
     h->tri_vol = H * H / 2.0;
     tri.resize(h->ntri * 3);
     auto id = [&](int i, int j) { return (i < 1 || j < 1 || i >= n1 || j >= n1) ? -1 : (i - 1) + (j - 1) * m; };
@@ -411,7 +410,6 @@ void build_coarse(fmg_eig_handle* h) {
     h->nh = m * m * m;
     h->nvert = 4;
     h->ntri = 6 * n1 * n1 * n1;
-    h->maxadj = 24;
     h->tri_vol = H * H * H / 6.0;
     tri.resize(h->ntri * 4);
     const int perm[6][3] = {{0, 1, 2}, {0, 2, 1}, {1, 0, 2}, {1, 2, 0}, {2, 0, 1}, {2, 1, 0}};
@@ -435,51 +433,17 @@ void build_coarse(fmg_eig_handle* h) {
           }
         }
   }
-  const int nv = h->nvert;
-  adj.assign(h->nh * h->maxadj, -1);
-  std::vector<int> fill(h->nh, 0);
-  for (int t = 0; t < h->ntri; ++t)
-    for (int v = 0; v < nv; ++v) {
-      const int a = tri[t * nv + v];
-      if (a >= 0) adj[a * h->maxadj + fill[a]++] = (t << 3) | v;
-    }
-  // gather lists of the dense solve's G(c) assembly: for each entry (a, b) with a simplex
-  // around a that has b as a vertex, the simplex-local indices in a's adjacency order
-  std::vector<int> gent, gstart{0}, gidx;
-  {
-    const int L = nv + 1;
-    for (int a = 0; a < h->nh; ++a)
-      for (int b = 0; b < h->nh; ++b) {
-        const size_t before = gidx.size();
-        for (int k = 0; k < h->maxadj; ++k) {
-          const int code = adj[a * h->maxadj + k];
-          if (code < 0) break;
-          const int t = code >> 3, la = code & 7;
-          for (int lb = 0; lb < nv; ++lb)
-            if (tri[t * nv + lb] == b) gidx.push_back(t * L * L + la * L + lb);
-        }
-        if (gidx.size() > before) {
-          gent.push_back(a * h->nh + b);
-          gstart.push_back((int)gidx.size());
-        }
-      }
-  }
-  h->npat = (int)gent.size();
+  // (a mesh beyond the lists' capacities is beyond dense_smem_bytes' limit too, and refused)
+  std::vector<uint16_t> lists(kDenseMaxLists);
+  if (!build_dense_lists(h->nh, h->ntri, h->nvert, tri.data(), lists.data(), &h->dims))
+    h->dims = DenseLists{};
+  const size_t nl = h->dims.npat ? h->dims.total(h->nh) : 1;
   h->tri = h->alloc<int>(tri.size());
-  h->adj = h->alloc<int>(adj.size());
-  h->gent = h->alloc<int>(gent.size());
-  h->gstart = h->alloc<int>(gstart.size());
-  h->gidx = h->alloc<int>(gidx.size());
+  h->lists = h->alloc<uint16_t>(nl);
   if (!h->dry) {
     cudaMemcpyAsync(h->tri, tri.data(), tri.size() * sizeof(int), cudaMemcpyHostToDevice,
                     h->stream);
-    cudaMemcpyAsync(h->adj, adj.data(), adj.size() * sizeof(int), cudaMemcpyHostToDevice,
-                    h->stream);
-    cudaMemcpyAsync(h->gent, gent.data(), gent.size() * sizeof(int), cudaMemcpyHostToDevice,
-                    h->stream);
-    cudaMemcpyAsync(h->gstart, gstart.data(), gstart.size() * sizeof(int),
-                    cudaMemcpyHostToDevice, h->stream);
-    cudaMemcpyAsync(h->gidx, gidx.data(), gidx.size() * sizeof(int), cudaMemcpyHostToDevice,
+    cudaMemcpyAsync(h->lists, lists.data(), nl * sizeof(uint16_t), cudaMemcpyHostToDevice,
                     h->stream);
   }
   const size_t nn = (size_t)h->nh * h->nh;
@@ -588,7 +552,7 @@ void enqueue_setup(fmg_eig_handle* h, cudaStream_t s, bool overlap = false) {
   }
   lv_dense_level1(h->L(1), h->L1, h->M1, s, true);
   if (h->literal()) lv_dense_level1(h->L(1), h->L1A, h->M1, s, false);
-  dense_spd_inverse(h->L1A, h->L1inv, h->nh, h->L(1).g.nb, s);
+  dense_spd_inverse(h->L1A, h->L1inv, h->nh, h->lists, h->dims, h->L(1).g.nb, s);
 }
 
 DenseProblem dense_base(fmg_eig_handle* h) {
@@ -597,14 +561,9 @@ DenseProblem dense_base(fmg_eig_handle* h) {
   d.ntri = h->ntri;
   d.nvert = h->nvert;
   d.tri = h->tri;
-  d.adj = h->adj;
-  d.maxadj = h->maxadj;
-  d.npat = h->npat;
-  d.gent = h->gent;
-  d.gstart = h->gstart;
-  d.gidx = h->gidx;
+  d.lists = h->lists;
+  d.dims = h->dims;
   d.quart_off = h->tri_vol * 2.0 * factorial(h->prob.dim) / factorial(h->prob.dim + 4);
-  d.tri_vol = h->tri_vol;
   d.L1 = h->L1;
   d.M1 = h->M1;
   d.nt3 = h->prob.dim == 2 ? 10 : 20;

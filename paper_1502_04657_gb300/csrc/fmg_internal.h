@@ -10,6 +10,7 @@
 #include <stdint.h>
 
 #include "../../include/fmg_eig.h"
+#include "dense_lists.h"
 
 namespace fmg {
 
@@ -303,7 +304,7 @@ void gather_level1_2d(const Grid& g1, const double* gA_pad, const double* gM_pad
                       double* t1, double* B1, cudaStream_t s, bool split = false);
 
 // ---- Dense small solves (dense.cu) -------------------------------------------------------
-// A batch of problems shares the geometry (tri, adj) and keeps the per-instance arrays
+// A batch of problems shares the geometry (tri, lists) and keeps the per-instance arrays
 // back to back: L1, M1, B1 nh*nh; gA, gM, t1 nh; t3 ntri*nt3; c_init, c_out nh + 1;
 // auu, buu, t0, lam_out, iters_out, status_out and params one each.
 struct DenseProblem {
@@ -313,17 +314,9 @@ struct DenseProblem {
   int nvert;           // vertices per simplex (3 in 2D, 4 in 3D)
   int nt3;             // entries of T3 per simplex (10 in 2D, 20 in 3D)
   const int* tri;      // ntri * nvert coarse interior indices, -1 on the boundary
-  const int* adj;      // nh * maxadj codes (simplex << 3 | local vertex), -1 terminated
-  int maxadj;
-  // Gather lists of the coarse block of G(c) (optional; nullptr: walk the adjacency): the
-  // npat structurally nonzero entries gent[q] = a nh + b, and for each the simplex-local
-  // indices gidx[gstart[q] .. gstart[q + 1]) = t (nvert + 1)^2 + la (nvert + 1) + lb of the
-  // simplices t around a (adjacency order, then vertex order) with vertex lb = b.
-  int npat;
-  const int* gent;
-  const int* gstart;
-  const int* gidx;
-  double tri_vol;      // |T|
+  // sparsity lists of the coarse block and of T3 (dense_lists.h), device memory
+  const uint16_t* lists;
+  DenseLists dims;
   double quart_off;    // |T| 2 d! / (d + 4)!, d = nvert - 1 (int_T w^2 mu_a mu_b / h_2)
   const double* L1;    // nh*nh, operator of level 1
   const double* M1;    // nh*nh, mass of level 1
@@ -353,8 +346,9 @@ constexpr size_t kDenseSmemLimit = 200 * 1024;  // dynamic shared memory of the 
 size_t dense_smem_bytes(int n, int ntri, int nvert, int aug);
 cudaError_t dense_prepare(size_t max_smem);  // opt in to large dynamic shared memory
 void dense_scf(const DenseProblem& p, int nb, cudaStream_t s);  // one CTA per problem
-// Linv = L^{-1} for SPD n x n matrices (LDL^T), one CTA per instance.
-void dense_spd_inverse(const double* L, double* Linv, int n, int nb, cudaStream_t s);
+// Linv = L^{-1} for the SPD n x n level-1 operators (nonzeros in `lists`), one CTA each.
+void dense_spd_inverse(const double* L, double* Linv, int n, const uint16_t* lists,
+                       const DenseLists& dims, int nb, cudaStream_t s);
 // y(padded level 1) = Linv * x(padded level 1) on the interior nodes (2D or 3D)
 void coarse_matvec(const Grid& g, const double* Linv, const double* x, double* y,
                    cudaStream_t s);

@@ -103,13 +103,12 @@ extern "C" int fmg_eig_coarse_solve_noalloc(const fmg_eig_problem* prob, double*
   int* status = reinterpret_cast<int*>(take(2));
   int* it = status + 1;
   int* tri = reinterpret_cast<int*>(take((size_t)ntri * 3 / 2 + 1));
-  int* adj = reinterpret_cast<int*>(take((size_t)nh * 6 / 2 + 1));
+  uint16_t* lists = reinterpret_cast<uint16_t*>(take(kDenseMaxLists / 4));
   if (off > kScratchDoubles) return FMG_EINVAL;
 
   // host-side tables on the stack (no heap use), copied into the fixed array
   int tri_h[2 * kMaxCoarseCells * kMaxCoarseCells * 3];
-  int adj_h[(kMaxCoarseCells - 1) * (kMaxCoarseCells - 1) * 6];
-  int fill[(kMaxCoarseCells - 1) * (kMaxCoarseCells - 1)];
+  uint16_t lists_h[kDenseMaxLists];
   auto id = [&](int i, int j) { return (i < 1 || j < 1 || i >= n1 || j >= n1) ? -1 : (i - 1) + (j - 1) * m; };
   for (int J = 0; J < n1; ++J)
     for (int I = 0; I < n1; ++I) {
@@ -121,13 +120,8 @@ extern "C" int fmg_eig_coarse_solve_noalloc(const fmg_eig_problem* prob, double*
         tri_h[(2 * cell + 1) * 3 + v] = t1[v];
       }
     }
-  for (int a = 0; a < nh; ++a) fill[a] = 0;
-  for (int e = 0; e < nh * 6; ++e) adj_h[e] = -1;
-  for (int t = 0; t < ntri; ++t)
-    for (int v = 0; v < 3; ++v) {
-      const int a = tri_h[t * 3 + v];
-      if (a >= 0) adj_h[a * 6 + fill[a]++] = (t << 3) | v;
-    }
+  DenseLists dims;
+  if (!build_dense_lists(nh, ntri, 3, tri_h, lists_h, &dims)) return FMG_EINVAL;
   PotentialParams pp{};
   pp.w0 = prob->w_const;
   pp.wx = prob->w_quad[0];
@@ -143,10 +137,9 @@ extern "C" int fmg_eig_coarse_solve_noalloc(const fmg_eig_problem* prob, double*
   d.ntri = ntri;
   d.nvert = 3;
   d.tri = tri;
-  d.adj = adj;
-  d.maxadj = 6;
-  d.tri_vol = g.h * g.h / 2.0;
-  d.quart_off = d.tri_vol / 180.0;  // |T| 2 d! / (d + 4)! with d = 2
+  d.lists = lists;
+  d.dims = dims;
+  d.quart_off = g.h * g.h / 360.0;  // |T| 2 d! / (d + 4)! with d = 2
   d.L1 = L1;
   d.M1 = M1;
   d.params = reinterpret_cast<const PotentialParams*>(params);
@@ -164,7 +157,8 @@ extern "C" int fmg_eig_coarse_solve_noalloc(const fmg_eig_problem* prob, double*
   if (cudaMemsetAsync(base, 0, off * sizeof(double), s) != cudaSuccess ||
       cudaMemsetAsync(status, 0xff, sizeof(int), s) != cudaSuccess ||
       cudaMemcpyAsync(tri, tri_h, sizeof(int) * ntri * 3, cudaMemcpyHostToDevice, s) != cudaSuccess ||
-      cudaMemcpyAsync(adj, adj_h, sizeof(int) * nh * 6, cudaMemcpyHostToDevice, s) != cudaSuccess ||
+      cudaMemcpyAsync(lists, lists_h, sizeof(uint16_t) * dims.total(nh), cudaMemcpyHostToDevice, s) !=
+          cudaSuccess ||
       cudaMemcpyAsync(params, &pp, sizeof(pp), cudaMemcpyHostToDevice, s) != cudaSuccess ||
       dense_prepare(dense_smem_bytes(nh, ntri, 3, 0)) != cudaSuccess) {
     cudaGetLastError();
