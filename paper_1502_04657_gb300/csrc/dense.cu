@@ -29,8 +29,9 @@
 //     h_3(w_1 .. w_nv, w_a) = .. [h_3 + w_a h_2 + w_a^2 h_1 + w_a^3], h_q the complete
 //     homogeneous symmetric polynomials of the vertex values, so each simplex forms h_1, h_2,
 //     h_3 once for its vertices.  K0, M and B1 are kept as their nonzeros.
-//   - c is not rescaled before an evaluation: every term is homogeneous in c, so the factor
-//     f = +-(c^T M c)^{-1/2} is applied to the sums.
+//   - c is rescaled only when c^T M c is off 1 by more than 1e-3 (the start, an inverse-power
+//     step), by a factor f applied to the sums: every term is homogeneous in c.  Otherwise the
+//     Newton system carries the constraint's defect, (M c)^T dc = -(c^T M c - 1) / 2.
 //   - The small scalar chains are Horner evaluations in c_u, one chain per lane.
 //   - The Jacobian A' (and K0 + zeta G) is assembled and inverted in single precision, whose
 //     pipes issue 64 times faster; what the ~1e-6 relative error of a step leaves is removed
@@ -43,6 +44,7 @@
 #include <stdint.h>
 
 #include "dense_lists.h"
+#include "dfloat.cuh"
 #include "fmg_internal.h"
 
 namespace fmg {
@@ -50,11 +52,15 @@ namespace {
 
 constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
-constexpr double kSwitch = 1e-2;  // relative residual below which Newton takes over
+// Relative residual below which Newton takes over (where its matrix is positive definite).  Over
+// coarse meshes of 3 to 9 (2D) and 3, 4 (3D) cells, zeta 1 to 5000 and traps 1 to 1000, 0.1
+// needed 3 to 22 steps where 1e-2 needed 3 to 47, never more, for the same ground state; 0.3
+// sometimes needed more (33 against 22).
+constexpr double kSwitch = 0.1;
 constexpr int kMaxChord = 2;      // steps with an inverse of an earlier iterate, per inverse
 constexpr int kMaxN = kDenseMaxNh + 1;
-constexpr int kSide = 16;         // the sweep's threads: kSide x kSide
-constexpr int kMaxTile = 6;       // at most kMaxTile x kMaxTile elements each (n <= 96)
+constexpr int kTile = 4;          // elements per side of a thread's tile in the FP32 sweep
+constexpr int kMaxSweep = 88;     // largest matrix the sweep takes: 22 x 23 / 2 tiles
 
 // Capacities of a CTA's shared arrays per dimension (vertices of a simplex), covering every
 // coarse mesh that dense_smem_bytes accepts (2D: 9 cells per side, 3D: 4).
@@ -62,7 +68,7 @@ template <int NV>
 struct Cap {
   static constexpr int nh = NV == 3 ? 64 : 27, pat = NV == 3 ? 386 : 223,
                        tri = NV == 3 ? 162 : 384, trip = NV == 3 ? 484 : 343,
-                       lists = NV == 3 ? 3872 : 3716;
+                       lists = NV == 3 ? 5488 : 5984;  // multiples of 8 (16-byte copies)
 };
 
 // One float matrix row: a multiple of 4 words that is 4 times an odd number, so that the 8
@@ -73,27 +79,35 @@ template <int NV>
 struct Smem {
   static constexpr int H = Cap<NV>::nh + 1, P = Cap<NV>::pat, T = Cap<NV>::tri;
   // nonzeros of the coarse blocks, sum_c w_c tau_abc per nonzero, and tau itself
+  alignas(16) uint16_t lists[Cap<NV>::lists];
   double K[P], M[P], B1[P], X[P], tau[Cap<NV>::trip];
   double h1[T], h2[T], h3[T];    // h_1, 2 h_2, 6 h_3 of each simplex's vertex values
   double w[H], w2[H], w3[H];     // c_H, its squares and doubled cubes; entry nh (boundary) is 0
   double Kc[H], Mc[H], Bc[H], Xc[H], S1[H], S2[H], S3[H], Q[H];
   double gA[H], gM[H], t1[H];
   double m64[H], r64[H];         // M c and the residual of the rescaled c
-  double dots[kWarps], red[2][kWarps];
-  double cu, f, zf3, lam, auu, buu, t0;
-  float h1f[T], h2f[T];
+  double cnt[H];                 // simplices around each coarse node
+  double dots[9];
+  double cu, f, g, lam, auu, buu, t0;
+  float h1f[T], h2f[T], wf[H];   // single precision, at the rescaled c (Jacobian)
   float r[kMaxN], m[kMaxN], y1[kMaxN], y2[kMaxN];
-  alignas(16) float piv[2][2][kSide * kMaxTile];  // the sweep's pivot rows, double-buffered
-  float rn;
-  uint16_t tri[T * NV], lists[Cap<NV>::lists];
+  alignas(16) float piv[2][kTile][kMaxSweep];  // the sweep's pivot rows, double-buffered
+  float red[2][kWarps];
+  int pivots_ok;
+  uint16_t tri[T * NV];
 };
 
 __device__ __forceinline__ double warp_sum(double v) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
 }
-__device__ __forceinline__ float warp_sum(float v) {
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+// Both sums by one butterfly: a's in the lower half of the warp, b's in the upper (five
+// additions instead of ten; order fixed).
+template <typename T>
+__device__ __forceinline__ T half_sums(T a, T b) {
+  const bool upper = threadIdx.x & 16;
+  T v = (upper ? b : a) + __shfl_xor_sync(0xffffffffu, upper ? a : b, 16);
+  for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
 }
 
@@ -107,6 +121,14 @@ __device__ __forceinline__ double recip(double d) {
   return y;
 }
 
+// The exponent of v, and 2^e as a float (clamped to its range)
+__device__ __forceinline__ int exponent_of(double v) {
+  return ((__double2hiint(v) >> 20) & 0x7ff) - 1023;
+}
+__device__ __forceinline__ float pow2f(int e) {
+  return __int_as_float(min(max(e + 127, 1), 254) << 23);
+}
+
 // Views of the staged lists (dense_lists.h)
 struct Lists {
   const uint16_t *row, *pair, *simptr, *sim, *x3ptr, *x3;
@@ -116,44 +138,53 @@ __device__ __forceinline__ Lists lists_of(const uint16_t* base, const DenseLists
                base + d.x3ptr(nh), base + d.x3(nh)};
 }
 
-// Sums at the iterate (w, cu): X, h_q per simplex; per row K0_HH w, M_HH w, B1 w, X w, the
+// Sums at the iterate c = (w, cu): X, h_q per simplex; per row (K0 c)_a, (M c)_a, B1 w, X w, the
 // sums S_q of h_q over the row's simplices and Q = 6 sum_T h_3(w.., w_a); and the dot
-// products with w: dots = [K0 w, Q, gA (level 1: sum w), gM, X w, B1 w, t1, M w].
+// products with w: dots = [K0 c, gA (level 1: sum w), M c, gM, X w, B1 w, t1, and Q over the
+// rows of warps 0 and 1].  zero: w = 0 (every augmented solve starts so).
 template <int NV>
-__device__ void sums(const DenseProblem& p, Smem<NV>& s) {
+__device__ __forceinline__ void sums(const DenseProblem& p, Smem<NV>& s, bool zero) {
   const int tid = threadIdx.x, nh = p.nh, npat = p.dims.npat;
   const Lists li = lists_of(s.lists, p.dims, nh);
   const int nx = p.aug ? npat : 0;
+  const int lg = nh <= 32 ? 5 : 6, kinds = p.aug ? 7 : 5;
   for (int e = tid; e < nx + p.ntri; e += kThreads) {
     if (e < nx) {
       double x = 0.0;
-      for (int k = li.x3ptr[e]; k < li.x3ptr[e + 1]; ++k) {
-        const int c = li.x3[k];
-        x = fma(s.w[c & 63], s.tau[c >> 6], x);
+      if (!zero) {
+        const int k1 = li.x3ptr[e + 1];
+#pragma unroll 2
+        for (int k = li.x3ptr[e]; k < k1; ++k) {
+          const int c = li.x3[k];
+          x = fma(s.w[c & 63], s.tau[c >> 6], x);
+        }
       }
       s.X[e] = x;
     } else {
       const int t = e - nx;
-      const uint16_t* v = s.tri + t * NV;
-      double p1 = s.w[v[0]] + s.w[v[1]], p2 = s.w2[v[0]] + s.w2[v[1]],
-             p3 = s.w3[v[0]] + s.w3[v[1]];
+      double p1 = 0.0, p2 = 0.0, p3 = 0.0;
+      if (!zero) {
+        const uint16_t* v = s.tri + t * NV;
+        p1 = s.w[v[0]] + s.w[v[1]];
+        p2 = s.w2[v[0]] + s.w2[v[1]];
+        p3 = s.w3[v[0]] + s.w3[v[1]];
 #pragma unroll
-      for (int q = 2; q < NV; ++q) {
-        p1 += s.w[v[q]];
-        p2 += s.w2[v[q]];
-        p3 += s.w3[v[q]];  // the doubled cubes: 2 p_3
+        for (int q = 2; q < NV; ++q) {
+          p1 += s.w[v[q]];
+          p2 += s.w2[v[q]];
+          p3 += s.w3[v[q]];  // the doubled cubes: 2 p_3
+        }
+        const double q1 = p1 * p1;
+        p3 = fma(p1, fma(3.0, p2, q1), p3);  // 6 h_3 = p_1^3 + 3 p_1 p_2 + 2 p_3
+        p2 = q1 + p2;                        // 2 h_2 = p_1^2 + p_2
       }
-      const double q1 = p1 * p1, h2 = q1 + p2;        // 2 h_2 = p_1^2 + p_2
       s.h1[t] = p1;
-      s.h2[t] = h2;
-      s.h3[t] = fma(p1, fma(3.0, p2, q1), p3);        // 6 h_3 = p_1^3 + 3 p_1 p_2 + 2 p_3
-      s.h1f[t] = (float)p1;
-      s.h2f[t] = (float)h2;
+      s.h2[t] = p2;
+      s.h3[t] = p3;
     }
   }
   __syncthreads();
   // seven row sums: one (sum, row) pair per thread
-  const int lg = nh <= 32 ? 5 : 6, kinds = p.aug ? 7 : 5;
   for (int q = tid; q < kinds << lg; q += kThreads) {
     const int kind = q >> lg, a = q & ((1 << lg) - 1);
     if (a >= nh) continue;
@@ -161,163 +192,188 @@ __device__ void sums(const DenseProblem& p, Smem<NV>& s) {
     double v = 0.0;
     if (kind >= 2 && kind < 5) {
       const double* h = kind == 2 ? s.h1 : kind == 3 ? s.h2 : s.h3;
-      for (int k = li.simptr[e0]; k < li.simptr[e0 + 1]; ++k) v += h[li.sim[k]];
+      const int k1 = zero ? 0 : li.simptr[e0 + 1];
+#pragma unroll 2
+      for (int k = li.simptr[e0]; k < k1; ++k) v += h[li.sim[k]];
       (kind == 2 ? s.S1 : kind == 3 ? s.S2 : s.S3)[a] = v;
     } else {
       const double* m = kind == 0 ? s.K : kind == 1 ? s.M : kind == 5 ? s.B1 : s.X;
-      for (int e = e0; e < li.row[a + 1]; ++e) v = fma(m[e], s.w[li.pair[e] & 255], v);
+      const int e1 = zero ? 0 : li.row[a + 1];
+      if (p.aug && kind < 2) v = s.cu * (kind == 0 ? s.gA : s.gM)[a];
+#pragma unroll 2
+      for (int e = e0; e < e1; ++e) v = fma(m[e], s.w[li.pair[e] & 255], v);
       (kind == 0 ? s.Kc : kind == 1 ? s.Mc : kind == 5 ? s.Bc : s.Xc)[a] = v;
     }
   }
   __syncthreads();
+  // dot products: Q's rows on warps 0 and 1, pairs of the others on warps 2, 3, 6, 7 (an even
+  // load on the SM's four FP64 units)
   const int warp = tid >> 5, lane = tid & 31;
-  const bool used = p.aug || warp < 3 || warp == 7;
-  double d = 0.0;
-  if (used) {
-    const double* y = warp == 0 ? s.Kc : warp == 2 ? s.gA : warp == 3 ? s.gM : warp == 4 ? s.Xc
-                    : warp == 5 ? s.Bc : warp == 6 ? s.t1 : s.Mc;
-    for (int a = lane; a < nh; a += 32) {
-      const double w = s.w[a];
-      double v;
-      if (warp == 1) {
-        const double cnt = (double)(li.simptr[li.row[a] + 1] - li.simptr[li.row[a]]);
-        // 6 sum_T [h_3 + w h_2 + w^2 h_1 + w^3] = S3 + w (3 S2 + 6 w (S1 + cnt w))
-        v = fma(w, fma(6.0 * w, fma(cnt, w, s.S1[a]), 3.0 * s.S2[a]), s.S3[a]);
-        s.Q[a] = v;
-      } else {
-        v = warp == 2 && !p.aug ? 1.0 : y[a];
-      }
-      d = fma(v, w, d);
+  if (warp < 2) {
+    const int a = tid;
+    double d = 0.0;
+    if (a < nh) {
+      // 6 sum_T [h_3 + w h_2 + w^2 h_1 + w^3] = S3 + 3 w (S2 + 2 w (S1 + cnt w))
+      const double w = s.w[a], w3 = 3.0 * w;
+      d = fma(w3, fma(w + w, fma(s.cnt[a], w, s.S1[a]), s.S2[a]), s.S3[a]);
+      s.Q[a] = d;
+      d *= w;
     }
     d = warp_sum(d);
+    if (lane == 0) s.dots[7 + warp] = d;
+  } else if ((warp & 2) && (warp < 4 || p.aug)) {
+    const int q = warp == 2 ? 0 : warp == 3 ? 2 : warp == 6 ? 4 : 6;
+    const double* y0 = q == 0 ? s.Kc : q == 2 ? s.Mc : q == 4 ? s.Xc : s.t1;
+    const double* y1 = q == 0 ? s.gA : q == 2 ? s.gM : s.Bc;
+    double d0 = 0.0, d1 = 0.0;
+    for (int a = lane; a < nh; a += 32) {
+      const double w = s.w[a];
+      d0 = fma(y0[a], w, d0);
+      if (!p.aug) d1 += w;
+      else if (q != 6) d1 = fma(y1[a], w, d1);
+    }
+    d0 = half_sums(d0, d1);
+    if ((lane & 15) == 0 && q + (lane >> 4) < 7) s.dots[q + (lane >> 4)] = d0;
   }
-  if (lane == 0) s.dots[warp] = d;
   __syncthreads();
 }
 
-// The residual at the iterate c = (w, cu), which it rescales to c^T M c = 1 with the sign of
-// the ground state: lambda, the relative residual s.rn, and in single precision the residual
-// r and M c.  Leaves s.f, the factor that was applied, for the sums that refer to the old c.
+// lambda and the residual r = (K0 + zeta G(c)) c - lambda M c at the iterate c = (w, cu), in
+// single precision with M c; returns the relative residual |r| / (|lambda| |M c|).  When
+// c^T M c is off 1 by more than 1e-3 (or c has the wrong sign) c is rescaled, by the factor
+// s.f that the sums at the old c still need; otherwise s.f = 1, and s.g = (c^T M c - 1) / 2 is
+// left to the Newton system (then lambda is off by a multiple of g, which r shows).
 template <int NV>
-__device__ void evaluate(const DenseProblem& p, Smem<NV>& s, double zeta) {
-  sums<NV>(p, s);
+__device__ __forceinline__ float evaluate(const DenseProblem& p, Smem<NV>& s, double zeta, bool zero) {
+  sums<NV>(p, s, zero);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, nh = p.nh, n = nh + p.aug;
   constexpr int kRowWarps = (kMaxN + 31) / 32;
   if (warp < kRowWarps) {
     // polynomials in c_u, one per lane: c^T K0 c, c^T M c, the load's u~ entry N_u, c^T N,
     // (K0 c)_u and (M c)_u
-    const double cu = p.aug ? s.cu : 0.0;
-    const double d2 = p.aug ? s.dots[2] : 0.0, d3 = s.dots[3], d4 = s.dots[4], d5 = s.dots[5],
-                 d6 = s.dots[6], qo = 0.5 * p.quart_off;
+    const double cu = p.aug ? s.cu : 0.0, qo = 0.5 * p.quart_off;
     double k0 = 0.0, k1 = 0.0, k2 = 0.0, k3 = 0.0, k4 = 0.0, m1 = 1.0, m2 = 1.0, m3 = 1.0;
-    switch (lane) {
-      case 0: k0 = s.dots[0]; k1 = d2; m1 = 2.0; k2 = s.auu; break;
-      case 1: k0 = s.dots[7]; k1 = d3; m1 = 2.0; k2 = s.buu; break;
-      case 2: k0 = d4; k1 = d5; m1 = 3.0; k2 = d6; m2 = 3.0; k3 = s.t0; break;
-      case 3: k0 = qo * s.dots[1]; k1 = d4; m1 = 4.0; k2 = d5; m2 = 6.0; k3 = d6; m3 = 4.0;
-              k4 = s.t0; break;
-      case 4: k0 = d2; k1 = s.auu; break;
-      case 5: k0 = d3; k1 = s.buu; break;
+    if (lane == 3) k0 = s.dots[7] + s.dots[8];
+    if (p.aug) {
+      const double d1 = s.dots[1], d3 = s.dots[3], d4 = s.dots[4], d5 = s.dots[5],
+                   d6 = s.dots[6];
+      switch (lane) {
+        case 0: k1 = d1; k2 = s.auu; break;
+        case 1: k1 = d3; k2 = s.buu; break;
+        case 2: k0 = d4; k1 = d5; m1 = 3.0; k2 = d6; m2 = 3.0; k3 = s.t0; break;
+        case 3: k1 = d4; m1 = 4.0; k2 = d5; m2 = 6.0; k3 = d6; m3 = 4.0; k4 = s.t0; break;
+        case 4: k0 = d1; k1 = s.auu; break;
+        case 5: k0 = d3; k1 = s.buu; break;
+      }
     }
+    k0 = lane == 0 ? s.dots[0] : lane == 1 ? s.dots[2] : lane == 3 ? qo * k0 : k0;
     const double v = fma(cu, fma(cu, fma(cu, fma(cu, k4, m3 * k3), m2 * k2), m1 * k1), k0);
     const double cKc = __shfl_sync(0xffffffffu, v, 0), cMc = __shfl_sync(0xffffffffu, v, 1),
                  Nu = __shfl_sync(0xffffffffu, v, 2), cN = __shfl_sync(0xffffffffu, v, 3),
                  Ku = __shfl_sync(0xffffffffu, v, 4), Mu = __shfl_sync(0xffffffffu, v, 5);
+    // tests on the high words: FP64 comparisons occupy the FP64 unit like any other operation
     const double dm = cMc - 1.0;
-    double f;
-    if (fabs(dm) <= 1e-3)  // (1 + dm)^{-1/2}, the next term below 3e-16
-      f = fma(dm, fma(dm, fma(dm, fma(dm, 0.2734375, -0.3125), 0.375), -0.5), 1.0);
-    else
-      f = 1.0 / sqrt(cMc);
-    if ((p.aug ? cu : s.dots[2]) < 0.0) f = -f;
-    const double f2 = f * f, zf2 = zeta * f2, zf3 = zf2 * f;
-    const double lam = f2 * fma(zf2, cN, cKc);
+    const bool rescale = (__double2hiint(dm) & 0x7fffffff) > 0x3f50624d ||  // |dm| > 1e-3
+                         __double2hiint(p.aug ? cu : s.dots[1]) < 0;
+    double f = 1.0, zf2 = zeta, g = 0.5 * dm, lam;
+    if (rescale) {
+      f = copysign(1.0 / sqrt(cMc), p.aug ? cu : s.dots[1]);
+      zf2 = zeta * (f * f);
+      g = 0.0;
+      lam = f * f * fma(zf2, cN, cKc);
+    } else {
+      lam = fma(zeta, cN, cKc);
+    }
     const int a = tid;
-    double rr = 0.0, mm = 0.0;
+    float rr = 0.0f, mm = 0.0f;
     if (a < n) {
-      double k, m, nl;
+      double k = Ku, m = Mu, nl = Nu;
       if (a < nh) {
         k = s.Kc[a];
         m = s.Mc[a];
         nl = qo * s.Q[a];
-        if (p.aug) {
-          k = fma(cu, s.gA[a], k);
-          m = fma(cu, s.gM[a], m);
-          nl = fma(cu, fma(3.0, s.Xc[a], cu * fma(3.0, s.Bc[a], cu * s.t1[a])), nl);
+        if (p.aug) nl = fma(cu, fma(3.0, s.Xc[a], cu * fma(3.0, s.Bc[a], cu * s.t1[a])), nl);
+        double w = s.w[a];
+        if (rescale) {
+          w *= f;
+          s.w[a] = w;
         }
-        s.w[a] *= f;
-      } else {
-        k = Ku;
-        m = Mu;
-        nl = Nu;
+        s.wf[a] = d2f_rn(w);
       }
-      m *= f;
-      const double r = fma(-lam, m, fma(zf3, nl, f * k));
+      double h = fma(zf2, nl, k);
+      if (rescale) {
+        m *= f;
+        h *= f;
+      }
+      const double r = fma(-lam, m, h);
       s.m64[a] = m;
       s.r64[a] = r;
-      s.m[a] = (float)m;
-      s.r[a] = (float)r;
-      rr = r * r;
-      mm = m * m;
+      const float rf = d2f_rn(r), mf = d2f_rn(m);
+      s.m[a] = mf;
+      s.r[a] = rf;
+      // norms in single precision, scaled by powers of two to the size of |M c| ~ sqrt(M_aa)
+      // and of lambda, so that their squares stay in range
+      const int em = exponent_of(s.M[0]) / 2, el = exponent_of(lam);
+      const float rs = rf * pow2f(-em - el), ms = mf * pow2f(-em);
+      rr = rs * rs;
+      mm = ms * ms;
     }
-    rr = warp_sum(rr);
-    mm = warp_sum(mm);
-    if (lane == 0) {
-      s.red[0][warp] = rr;
-      s.red[1][warp] = mm;
-    }
+    rr = half_sums(rr, mm);
+    if ((lane & 15) == 0) s.red[lane >> 4][warp] = rr;
     if (tid == 0) {
       s.f = f;
-      s.zf3 = zf3;
+      s.g = g;
       s.lam = lam;
+      s.wf[nh] = 0.0f;
     }
   }
   __syncthreads();
-  if (tid == 0) {
-    double rr = 0.0, mm = 0.0;
-    for (int q = 0; q < kRowWarps; ++q) {
-      rr += s.red[0][q];
-      mm += s.red[1][q];
-    }
-    const double den = s.lam * s.lam * mm;
-    s.red[0][0] = rr;
-    s.red[1][0] = den;
-    s.rn = sqrtf((float)(rr * recip(den)));
-    if (p.aug) s.cu *= s.f;
+  // cu belongs to the thread of its row from here on (others read it after a barrier)
+  if (p.aug && tid == nh) s.cu *= s.f;
+  float rr = 0.0f, mm = 0.0f;
+  for (int q = 0; q < kRowWarps; ++q) {
+    rr += s.red[0][q];
+    mm += s.red[1][q];
   }
-  __syncthreads();
+  const double lam = s.lam;  // its significand, in [1, 2)
+  const float l = __int_as_float((127 << 23) | (__double2hiint(lam) & 0xfffff) << 3);
+  return exponent_of(lam) < 1024 ? sqrtf(rr / mm) / l : __int_as_float(0x7fffffff);
 }
 
 // G(c)_ab of nonzero e = (a, b) at c = f (w_old, cu_old), from the sums of `sums` at the old
-// c and the rescaled w, in T (float: the Jacobian; double: the assembled system, and the
-// Jacobian of the fallback): sum_T int_T w_H^2 mu_a mu_b + 2 c_u X_ab + c_u^2 B1_ab, with
+// c, in T: sum_T int_T w_H^2 mu_a mu_b + 2 c_u X_ab + c_u^2 B1_ab, with
 //   int_T w^2 mu_a mu_b = |T| 2 d! / (d + 4)! h_2(w_1 .. w_nv, w_a, w_b)  (twice for a = b).
+// float (the Jacobian): the simplex sums h1f, h2f and wf are those of the rescaled c already.
+// double: the assembled system, and the Jacobian of the fallback.
 template <int NV, typename T>
 __device__ __forceinline__ T coarse_G(const DenseProblem& p, const Smem<NV>& s, const Lists& li,
                                       int e, T f, T cu) {
+  constexpr bool single = sizeof(T) == 4;
   const int a = li.pair[e] >> 8, b = li.pair[e] & 255;
   const int k0 = li.simptr[e], k1 = li.simptr[e + 1];
-  const T cnt = (T)(k1 - k0), wa = (T)s.w[a], wb = (T)s.w[b];
-  T g;
-  if (a == b) {
-    const T s1 = f * (T)s.S1[a], s2 = f * f * (T)s.S2[a];
-    g = (T)p.quart_off * (s2 + wa * ((T)4 * s1 + (T)6 * cnt * wa));
-  } else {
-    T s1 = 0, s2 = 0;
-    for (int k = k0; k < k1; ++k) {
-      const int t = li.sim[k];
-      if constexpr (sizeof(T) == 4) {
-        s1 += s.h1f[t];
-        s2 += s.h2f[t];
-      } else {
-        s1 += s.h1[t];
-        s2 += s.h2[t];
-      }
+  T s1 = 0, s2 = 0, wa, wb;
+  for (int k = k0; k < k1; ++k) {
+    const int t = li.sim[k];
+    if constexpr (single) {
+      s1 += s.h1f[t];
+      s2 += s.h2f[t];
+    } else {
+      s1 += s.h1[t];
+      s2 += s.h2[t];
     }
-    const T ws = wa + wb;
-    g = (T)(0.5 * p.quart_off) *
-        (f * f * s2 + (T)2 * (ws * f * s1 + cnt * (ws * ws - wa * wb)));
   }
+  if constexpr (single) {
+    wa = s.wf[a];
+    wb = s.wf[b];
+  } else {
+    wa = s.w[a];
+    wb = s.w[b];
+    s1 *= f;
+    s2 *= f * f;
+  }
+  const T ws = wa + wb, cnt = (T)(k1 - k0);
+  const T quart = (T)(a == b ? p.quart_off : 0.5 * p.quart_off);
+  T g = quart * (s2 + (T)2 * (ws * s1 + cnt * (ws * ws - wa * wb)));
   if (p.aug) g += cu * ((T)2 * f * (T)s.X[e] + cu * (T)s.B1[e]);
   return g;
 }
@@ -333,10 +389,24 @@ __device__ __forceinline__ T border_G(const Smem<NV>& s, int a, int nh, T f, T c
 // J += K0 - lam M + gz G at the current iterate, on the structural nonzeros (the others stay
 // zero), row stride ns
 template <int NV, typename T>
-__device__ void jacobian(const DenseProblem& p, const Smem<NV>& s, T* J, int ns, double lam,
-                         T gz) {
+__device__ __forceinline__ void jacobian(const DenseProblem& p, Smem<NV>& s, T* J, int ns, double lam, T gz) {
   const int nh = p.nh;
   const Lists li = lists_of(s.lists, p.dims, nh);
+  if constexpr (sizeof(T) == 4) {
+    for (int t = threadIdx.x; t < p.ntri; t += kThreads) {
+      const uint16_t* v = s.tri + t * NV;
+      float p1 = 0.0f, p2 = 0.0f;
+#pragma unroll
+      for (int q = 0; q < NV; ++q) {
+        const float w = s.wf[v[q]];
+        p1 += w;
+        p2 = fmaf(w, w, p2);
+      }
+      s.h1f[t] = p1;
+      s.h2f[t] = fmaf(p1, p1, p2);
+    }
+  }
+  __syncthreads();
   const T f = (T)s.f, cu = p.aug ? (T)s.cu : (T)0;
   for (int e = threadIdx.x; e < p.dims.npat; e += kThreads) {
     const int a = li.pair[e] >> 8, b = li.pair[e] & 255;
@@ -359,118 +429,138 @@ __device__ void jacobian(const DenseProblem& p, const Smem<NV>& s, T* J, int ns,
 // and after sweeping every index the matrix is -A^{-1}.  All four cases are one update
 // M_ij - F_i R_j once the pivot rows and columns of M are set to zero, with F_i = M_iP H
 // (pivot row: -H_i) and R_j = M_Pj (pivot column: -e_j), so no lane takes a branch of its own.
-// The indices go in pairs, one barrier per pair; 16 x 16 threads hold TS x TS elements each in
-// registers, and the owners of the next two pivot rows publish them to s.piv.  M stays
-// symmetric, so F is read from the pivot rows too.  A pair's chain (publish, barrier, read,
-// 2 x 2 inverse, update) is about 190 cycles: 50 x 50 takes 25 pairs.  Returns false at a
-// non-positive pivot (all threads read the same pivots, so all return together).
-template <int TS>
-__device__ __forceinline__ bool sweep_tiles(const float* J, float* Ainv, int ns, float tau,
-                                            const float* m, float (*piv)[2][kSide * kMaxTile],
-                                            int n) {
-  const int ti = threadIdx.x / kSide, tj = threadIdx.x % kSide, i0 = ti * TS, j0 = tj * TS;
-  float v[TS][TS];
+// The indices go in blocks of 4, one barrier per block, and M stays symmetric, so only its
+// upper triangle is kept: one 4 x 4 tile (ti <= tj) in the registers of each participating
+// thread (91 threads for n = 50, 28 for n = 28).  The owners of the next pivot rows publish
+// them to piv (double-buffered), tiles above the diagonal from their transposed columns.
+// A block takes about 940 cycles for n = 50 (its chain: publish, barrier, read, 4 x 4 inverse,
+// update; 3 cycles per instruction of the one warp on each partition), 12.2k cycles in all;
+// pairs of pivots with 2 x 2 inverses took 560 cycles a pair (14k), on full rows over all 256
+// threads 520 a pair, and 4 x 4 blocks of full rows with sequential pivots 28.8k in all.
+// Leaves whether every pivot was positive in *pivots_ok.
+__device__ __forceinline__ bool sweep_inverse(const float* J, float* Ainv, int ns, float tau,
+                                           const float* m, float (*piv)[kTile][kMaxSweep],
+                                           int n, int* pivots_ok) {
+  const int t = threadIdx.x, nt = (n + kTile - 1) / kTile, tiles = nt * (nt + 1) / 2;
+  const int team = (tiles + 31) & ~31;  // participating threads, whole warps
+  if (t < team) {
+    int tj = (int)((sqrtf(8.0f * t + 1.0f) - 1.0f) * 0.5f);
+    if ((tj + 1) * (tj + 2) / 2 <= t) ++tj;
+    if (tj * (tj + 1) / 2 > t) --tj;
+    int ti = t - tj * (tj + 1) / 2;
+    const bool own = t < tiles;
+    if (!own) ti = tj = nt - 1;  // idle lanes of the last warp: a copy that publishes nothing
+    const int i0 = ti * kTile, j0 = tj * kTile;
+    float v[4][4];
 #pragma unroll
-  for (int r = 0; r < TS; ++r)
+    for (int r = 0; r < 4; ++r)
 #pragma unroll
-    for (int c = 0; c < TS; ++c) {
-      const int i = i0 + r, j = j0 + c;
-      v[r][c] = i < n && j < n ? J[i * ns + j] : (i == j ? 1.0f : 0.0f);
-      if (tau != 0.0f && i < n && j < n) v[r][c] = fmaf(tau * m[i], m[j], v[r][c]);
-    }
-  if (ti == 0) {
-#pragma unroll
-    for (int r = 0; r < 2; ++r)
-#pragma unroll
-      for (int c = 0; c < TS; c += 2)
-        *reinterpret_cast<float2*>(&piv[0][r][j0 + c]) = make_float2(v[r][c], v[r][c + 1]);
-  }
-  __syncthreads();
-  int buf = 0;
-  for (int kt = 0; kt * TS < n; ++kt) {
-#pragma unroll
-    for (int q = 0; q < TS; q += 2) {
-      const int k = kt * TS + q;
-      if (k >= n) break;
-      const float* p0 = piv[buf][0];
-      const float* p1 = piv[buf][1];
-      const float a = p0[k], b = p0[k + 1], d = p1[k + 1];
-      const float det = fmaf(a, d, -b * b);
-      if (!(a > 0.0f) || !(det > 0.0f)) return false;
-      const float inv = __fdividef(1.0f, det);
-      const float h00 = d * inv, h01 = -b * inv, h11 = a * inv;
-      float f0[TS], f1[TS], r0[TS], r1[TS];
-#pragma unroll
-      for (int r = 0; r < TS; r += 2) {
-        const float2 x = *reinterpret_cast<const float2*>(&p0[i0 + r]);
-        const float2 y = *reinterpret_cast<const float2*>(&p1[i0 + r]);
-        f0[r] = fmaf(x.x, h00, y.x * h01);
-        f1[r] = fmaf(x.x, h01, y.x * h11);
-        f0[r + 1] = fmaf(x.y, h00, y.y * h01);
-        f1[r + 1] = fmaf(x.y, h01, y.y * h11);
-        const float2 z = *reinterpret_cast<const float2*>(&p0[j0 + r]);
-        const float2 w = *reinterpret_cast<const float2*>(&p1[j0 + r]);
-        r0[r] = z.x;
-        r0[r + 1] = z.y;
-        r1[r] = w.x;
-        r1[r + 1] = w.y;
-      }
-      const bool prow = ti == kt, pcol = tj == kt;
-      if (prow) {
-        f0[q] = -h00;
-        f1[q] = -h01;
-        f0[q + 1] = -h01;
-        f1[q + 1] = -h11;
-      }
-      if (pcol) {
-        r0[q] = -1.0f;
-        r1[q] = 0.0f;
-        r0[q + 1] = 0.0f;
-        r1[q + 1] = -1.0f;
-      }
-#pragma unroll
-      for (int r = 0; r < TS; ++r)
-#pragma unroll
-        for (int c = 0; c < TS; ++c) {
-          const bool zr = r == q || r == q + 1, zc = c == q || c == q + 1;
-          float x = v[r][c];
-          if (zr) x = prow ? 0.0f : x;
-          if (zc) x = pcol ? 0.0f : x;
-          v[r][c] = fmaf(-f0[r], r0[c], fmaf(-f1[r], r1[c], x));
+      for (int c = 0; c < 4; ++c) {
+        const int i = i0 + r, j = j0 + c;
+        float x = i == j ? 1.0f : 0.0f;
+        if (i < n && j < n) {
+          x = J[i * ns + j];
+          if (tau != 0.0f) x = fmaf(tau * m[i], m[j], x);
         }
-      // publish the next pair of pivot rows: of this tile row, or of the next one
-      if (q + 2 < TS ? prow : ti == kt + 1) {
-        constexpr int wrap = TS;
-        const int nr = (q + 2) % wrap;
-#pragma unroll
-        for (int r = 0; r < 2; ++r)
-#pragma unroll
-          for (int c = 0; c < TS; c += 2)
-            *reinterpret_cast<float2*>(&piv[buf ^ 1][r][j0 + c]) =
-                make_float2(v[nr + r][c], v[nr + r][c + 1]);
+        v[r][c] = x;
       }
-      buf ^= 1;
-      __syncthreads();
+    if (ti == 0 && own) {
+#pragma unroll
+      for (int r = 0; r < 4; ++r)
+        *reinterpret_cast<float4*>(&piv[0][r][j0]) = make_float4(v[r][0], v[r][1], v[r][2], v[r][3]);
     }
+    bool ok = true;
+    for (int kt = 0; kt < nt; ++kt) {
+      asm volatile("bar.sync 1, %0;" ::"r"(team) : "memory");
+      const float(*p)[kMaxSweep] = piv[kt & 1];
+      float h[4][4];  // H = (M_PP)^{-1} by its 2 x 2 blocks [A B; B^T D]
+      {
+        const float4 q0 = *reinterpret_cast<const float4*>(&p[0][kTile * kt]),
+                     q1 = *reinterpret_cast<const float4*>(&p[1][kTile * kt]),
+                     q2 = *reinterpret_cast<const float4*>(&p[2][kTile * kt]),
+                     q3 = *reinterpret_cast<const float4*>(&p[3][kTile * kt]);
+        const float da = fmaf(q0.x, q1.y, -q0.y * q0.y), ia = __fdividef(1.0f, da);
+        const float a00 = q1.y * ia, a01 = -q0.y * ia, a11 = q0.x * ia;
+        const float t00 = fmaf(a00, q0.z, a01 * q1.z), t01 = fmaf(a00, q0.w, a01 * q1.w),
+                    t10 = fmaf(a01, q0.z, a11 * q1.z), t11 = fmaf(a01, q0.w, a11 * q1.w);
+        const float s00 = fmaf(-q0.z, t00, fmaf(-q1.z, t10, q2.z)),
+                    s01 = fmaf(-q0.z, t01, fmaf(-q1.z, t11, q2.w)),
+                    s11 = fmaf(-q0.w, t01, fmaf(-q1.w, t11, q3.w));
+        const float ds = fmaf(s00, s11, -s01 * s01), is = __fdividef(1.0f, ds);
+        ok = q0.x > 0.0f && da > 0.0f && s00 > 0.0f && ds > 0.0f;
+        if (!ok) break;
+        h[2][2] = s11 * is;
+        h[2][3] = h[3][2] = -s01 * is;
+        h[3][3] = s00 * is;
+        const float u00 = fmaf(t00, h[2][2], t01 * h[2][3]), u01 = fmaf(t00, h[2][3], t01 * h[3][3]),
+                    u10 = fmaf(t10, h[2][2], t11 * h[2][3]), u11 = fmaf(t10, h[2][3], t11 * h[3][3]);
+        h[0][0] = fmaf(u00, t00, fmaf(u01, t01, a00));
+        h[0][1] = h[1][0] = fmaf(u00, t10, fmaf(u01, t11, a01));
+        h[1][1] = fmaf(u10, t10, fmaf(u11, t11, a11));
+        h[0][2] = h[2][0] = -u00;
+        h[0][3] = h[3][0] = -u01;
+        h[1][2] = h[2][1] = -u10;
+        h[1][3] = h[3][1] = -u11;
+      }
+      float f[4][4], y[4][4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const float4 x = *reinterpret_cast<const float4*>(&p[q][i0]);
+        const float4 z = *reinterpret_cast<const float4*>(&p[q][j0]);
+        const float xr[4] = {x.x, x.y, x.z, x.w};
+        y[q][0] = z.x; y[q][1] = z.y; y[q][2] = z.z; y[q][3] = z.w;
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+          for (int c = 0; c < 4; ++c) f[r][c] = q == 0 ? xr[r] * h[0][c] : fmaf(xr[r], h[q][c], f[r][c]);
+      }
+      if (ti == kt || tj == kt) {
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+          for (int c = 0; c < 4; ++c) {
+            v[r][c] = 0.0f;
+            if (ti == kt) f[r][c] = -h[r][c];
+            if (tj == kt) y[r][c] = r == c ? -1.0f : 0.0f;
+          }
+      }
+#pragma unroll
+      for (int r = 0; r < 4; ++r)
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+#pragma unroll
+          for (int q = 0; q < 4; ++q) v[r][c] = fmaf(-f[r][q], y[q][c], v[r][c]);
+      if (own && ti == kt + 1) {
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+          *reinterpret_cast<float4*>(&piv[(kt + 1) & 1][r][j0]) =
+              make_float4(v[r][0], v[r][1], v[r][2], v[r][3]);
+      } else if (own && tj == kt + 1) {
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+          *reinterpret_cast<float4*>(&piv[(kt + 1) & 1][c][i0]) =
+              make_float4(v[0][c], v[1][c], v[2][c], v[3][c]);
+      }
+    }
+    if (own && ok) {
+#pragma unroll
+      for (int r = 0; r < 4; ++r)
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+          if (i0 + r < n && j0 + c < n) {
+            Ainv[(i0 + r) * ns + j0 + c] = v[r][c];
+            if (ti != tj) Ainv[(j0 + c) * ns + i0 + r] = v[r][c];
+          }
+    }
+    if (t == 0) *pivots_ok = ok;  // every participating thread saw the same pivots
   }
-#pragma unroll
-  for (int r = 0; r < TS; ++r)
-#pragma unroll
-    for (int c = 0; c < TS; ++c)
-      if (i0 + r < n && j0 + c < n) Ainv[(i0 + r) * ns + j0 + c] = v[r][c];
   __syncthreads();
-  return true;
+  const bool ok = *pivots_ok != 0;
+  __syncthreads();  // pivots_ok may be written again
+  return ok;
 }
 
-__device__ __noinline__ bool sweep_inverse(const float* J, float* Ainv, int ns, float tau,
-                                           const float* m, float (*piv)[2][kSide * kMaxTile],
-                                           int n) {
-  if (n <= 2 * kSide) return sweep_tiles<2>(J, Ainv, ns, tau, m, piv, n);
-  if (n <= 4 * kSide) return sweep_tiles<4>(J, Ainv, ns, tau, m, piv, n);
-  return sweep_tiles<kMaxTile>(J, Ainv, ns, tau, m, piv, n);
-}
-
-// y = A^{-1} x for one or two vectors, Ainv = -A^{-1} in single precision: 4 threads per row
+// y = A^{-1} x for two vectors, Ainv = -A^{-1} in single precision: 4 threads per row
 __device__ __forceinline__ void apply_inverse(const float* Ainv, int ns, const float* x1,
                                               float* y1, const float* x2, float* y2, int n) {
   const int part = threadIdx.x & 3;
@@ -478,10 +568,11 @@ __device__ __forceinline__ void apply_inverse(const float* Ainv, int ns, const f
     const int row = row0 + (threadIdx.x >> 2);
     float a = 0.0f, b = 0.0f;
     if (row < n)
+#pragma unroll 4
       for (int j = part; j < n; j += 4) {
         const float v = Ainv[row * ns + j];
         a = fmaf(v, x1[j], a);
-        if (x2) b = fmaf(v, x2[j], b);
+        b = fmaf(v, x2[j], b);
       }
     a += __shfl_xor_sync(0xffffffffu, a, 1);
     a += __shfl_xor_sync(0xffffffffu, a, 2);
@@ -489,7 +580,7 @@ __device__ __forceinline__ void apply_inverse(const float* Ainv, int ns, const f
     b += __shfl_xor_sync(0xffffffffu, b, 2);
     if (part == 0 && row < n) {
       y1[row] = -a;
-      if (x2) y2[row] = -b;
+      y2[row] = -b;
     }
   }
   __syncthreads();
@@ -508,18 +599,20 @@ __device__ __forceinline__ void set_entry(const DenseProblem& p, Smem<NV>& s, in
   }
 }
 
-// c += dc = -y1 + dl y2 of the bordered Newton system; returns dl
+// c += dc = -y1 + dl y2 of the bordered Newton system with (M c)^T dc = -g; returns dl
 template <int NV>
-__device__ float newton_update(const DenseProblem& p, Smem<NV>& s) {
+__device__ __forceinline__ float newton_update(const DenseProblem& p, Smem<NV>& s) {
   const int n = p.nh + p.aug, lane = threadIdx.x & 31;
   float p1 = 0.0f, p2 = 0.0f;
   for (int a = lane; a < n; a += 32) {
     p1 = fmaf(s.m[a], s.y1[a], p1);
     p2 = fmaf(s.m[a], s.y2[a], p2);
   }
-  const float dl = warp_sum(p1) / warp_sum(p2);
+  const float v = half_sums(p1, p2), g = d2f_rn(s.g);
+  const float dl =
+      (__shfl_sync(0xffffffffu, v, 0) - g) / __shfl_sync(0xffffffffu, v, 16);
   for (int a = threadIdx.x; a < n; a += kThreads)
-    set_entry(p, s, a, (a < p.nh ? s.w[a] : s.cu) + (double)fmaf(dl, s.y2[a], -s.y1[a]));
+    set_entry(p, s, a, (a < p.nh ? s.w[a] : s.cu) + f2d_exact(fmaf(dl, s.y2[a], -s.y1[a])));
   __syncthreads();
   return dl;
 }
@@ -615,11 +708,14 @@ __device__ __noinline__ bool solve_fp64(const DenseProblem& p, Smem<NV>& s, doub
   return ok;
 }
 
+// (The steps of the iteration are inlined at one call site each: called functions would take
+// their shared arrays as generic pointers, whose loads are slower.)
 // One CTA of 256 threads per problem, a batch of problems one CTA each (two resident per SM:
 // at most 128 registers and half of the shared memory).  The iteration count is bounded by
 // max_iter (chord steps, at most kMaxChord per inverse, are not counted: they replace the
 // refinement of the Newton correction); hitting it sets status 1.
-template <int NV>
+// ASSEMBLE: only assemble K0, M and G(c_init) into K_out, M_out, G_out.
+template <int NV, bool ASSEMBLE>
 __global__ void __launch_bounds__(kThreads, 2) k_dense_scf(const __grid_constant__ DenseProblem p) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   Smem<NV>& s = *reinterpret_cast<Smem<NV>*>(smem_raw);
@@ -630,13 +726,15 @@ __global__ void __launch_bounds__(kThreads, 2) k_dense_scf(const __grid_constant
   const size_t ib = blockIdx.x;  // the instance, whose arrays lie at its slices
   const double *L1 = p.L1 + ib * nh * nh, *M1 = p.M1 + ib * nh * nh;
   const double zeta = p.params[ib].zeta;
-  for (int e = tid; e < p.dims.tripptr(nh); e += kThreads) s.lists[e] = p.lists[e];
+  {  // 16 bytes a load (the lists are padded to that on the device)
+    const uint4* from = reinterpret_cast<const uint4*>(p.lists);
+    uint4* to = reinterpret_cast<uint4*>(s.lists);
+    for (int e = tid; e < (p.dims.total(nh) + 7) / 8; e += kThreads) to[e] = from[e];
+  }
   for (int e = tid; e < p.ntri * NV; e += kThreads) {
     const int v = p.tri[e];
     s.tri[e] = (uint16_t)(v < 0 ? nh : v);
   }
-  for (int e = tid; e < 2 * n * ns; e += kThreads) J[e] = 0.0f;
-  if (tid < kWarps) s.dots[tid] = 0.0;
   if (tid <= nh) {
     double c = 0.0;
     if (p.c_init) c = tid < n ? p.c_init[ib * (nh + 1) + tid] : 0.0;
@@ -648,39 +746,51 @@ __global__ void __launch_bounds__(kThreads, 2) k_dense_scf(const __grid_constant
     s.w[tid] = c;
     s.w2[tid] = c * c;
     s.w3[tid] = 2.0 * (c * c * c);
-  }
-  if (p.aug) {
-    if (tid < nh) {
+    if (p.aug && tid < nh) {
       s.gA[tid] = p.gA[ib * nh + tid];
       s.gM[tid] = p.gM[ib * nh + tid];
       s.t1[tid] = p.t1[ib * nh + tid];
     }
-    const uint16_t* tp = p.lists + p.dims.tripptr(nh);
-    const uint16_t* ti = p.lists + p.dims.trip(nh);
-    const double* t3 = p.t3 + ib * p.ntri * p.nt3;
-    for (int q = tid; q < p.dims.nq; q += kThreads) {
-      double v = 0.0;
-      for (int k = tp[q]; k < tp[q + 1]; ++k) v += t3[ti[k]];
-      s.tau[q] = v;
-    }
   }
-  if (tid == 0) {
+  if (tid == kThreads - 1) {
     s.auu = p.aug ? p.auu[ib] : 0.0;
     s.buu = p.aug ? p.buu[ib] : 0.0;
     s.t0 = p.aug ? p.t0[ib] : 0.0;
   }
+  for (int e = tid; e < 2 * n * ns / 4; e += kThreads)
+    reinterpret_cast<float4*>(J)[e] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+  __syncthreads();
   {
-    const uint16_t* pr = p.lists + p.dims.pair(nh);
+    const Lists li = lists_of(s.lists, p.dims, nh);
     for (int e = tid; e < p.dims.npat; e += kThreads) {
-      const int k = (pr[e] >> 8) * nh + (pr[e] & 255);
+      const int k = (li.pair[e] >> 8) * nh + (li.pair[e] & 255);
       s.K[e] = L1[k];
       s.M[e] = M1[k];
       if (p.aug) s.B1[e] = p.B1[ib * nh * nh + k];
     }
+    if (tid < nh) s.cnt[tid] = (double)(li.simptr[li.row[tid] + 1] - li.simptr[li.row[tid]]);
+  }
+  if (p.aug) {
+    const uint16_t* tp = s.lists + p.dims.tripptr(nh);
+    const uint16_t* ti = s.lists + p.dims.trip(nh);
+    const double* t3 = p.t3 + ib * p.ntri * p.nt3;
+    for (int q = tid; q < p.dims.nq; q += kThreads) {
+      double v = 0.0;
+      const int k1 = tp[q + 1];
+      for (int k = tp[q]; k < k1; k += 6) {  // 6 loads in flight
+        double x[6];
+#pragma unroll
+        for (int j = 0; j < 6; ++j) x[j] = k + j < k1 ? t3[ti[k + j]] : 0.0;
+#pragma unroll
+        for (int j = 0; j < 6; ++j)
+          if (k + j < k1) v += x[j];
+      }
+      s.tau[q] = v;
+    }
   }
   __syncthreads();
-  if (p.K_out) {  // assemble-only mode: K0, M and G(c_init) as given
-    sums<NV>(p, s);
+  if constexpr (ASSEMBLE) {
+    sums<NV>(p, s, false);
     const Lists li = lists_of(s.lists, p.dims, nh);
     for (int e = tid; e < n * n; e += kThreads) p.K_out[e] = p.M_out[e] = p.G_out[e] = 0.0;
     __syncthreads();
@@ -703,62 +813,60 @@ __global__ void __launch_bounds__(kThreads, 2) k_dense_scf(const __grid_constant
   int it = 0, status = 1, chords = kMaxChord;  // kMaxChord: no inverse to step with
   float last = 0.0f;                           // the residual before the latest Newton step
   double dlam = 0.0;
+  bool zero = p.aug && !p.c_init;              // the start c = u~
+  bool newton = false;
+  bool failed = false;  // the Newton matrix of this iterate had a non-positive pivot
+  float rn = 0.0f;
   for (;;) {
-    evaluate<NV>(p, s, zeta);
-    const float rn = s.rn;
-    const bool converged = s.red[0][0] <= p.tol * p.tol * s.red[1][0];
-    // A step with the inverse of an earlier iterate cuts the residual by about twice what the
-    // latest step did (the Jacobian is off by the distance moved since, and by ~1e-6): it
-    // replaces a new inverse where that reaches the tolerance.  On convergence the same step,
-    // without another evaluation, takes c and lambda from the tolerance to rounding.
-    const bool chord = chords < kMaxChord && rn < 0.05f * last &&
-                       (converged || 4.0f * rn * rn <= last * (float)p.tol);
+    bool converged = false, chord = false;
+    if (!failed) {
+      rn = evaluate<NV>(p, s, zeta, zero);
+      zero = false;
+      converged = rn <= (float)p.tol;
+      // A step with the inverse of an earlier iterate cuts the residual by about twice what
+      // the latest step did (the Jacobian is off by the distance moved since, and by ~1e-6):
+      // it replaces a new inverse where that reaches the tolerance.  On convergence the same
+      // step, without another evaluation, takes c and lambda from the tolerance to rounding.
+      chord = chords < kMaxChord && rn < 0.05f * last &&
+              (converged || 4.0f * rn * rn <= last * (float)p.tol);
+      if (converged) status = 0;
+      if (!chord && (converged || it >= p.max_iter)) break;
+      if (!chord) newton = rn <= (float)kSwitch;
+    } else {
+      newton = false;
+    }
     if (chord) {
       ++chords;
-      apply_inverse(Pinv, ns, s.r, s.y1, s.m, s.y2, n);
+    } else {
+      // Newton: A' = K0 + 3 zeta G - lambda M + |lambda| (Mc)(Mc)^T; otherwise an
+      // inverse-power step c <- (K0 + zeta G)^{-1} M c
+      const double lam = newton ? s.lam : 0.0, gz = newton ? 3.0 * zeta : zeta;
+      jacobian<NV, float>(p, s, J, ns, lam, (float)gz);
+      const bool have = sweep_inverse(J, Pinv, ns, newton ? fabsf(d2f_rn(lam)) : 0.0f, s.m, s.piv,
+                                      n, &s.pivots_ok);
+      chords = have && newton ? 0 : kMaxChord;
+      if (!have && !solve_fp64<NV>(p, s, reinterpret_cast<double*>(J), J, ns, lam, gz,
+                                   newton ? fabs(lam) : 0.0, newton)) {
+        if (!newton) break;
+        failed = true;  // the same iterate again, by an inverse-power step
+        continue;
+      }
+      failed = false;
+      ++it;
+      chord = have;  // step with the inverse (the FP64 fallback has solved already)
+    }
+    if (chord) apply_inverse(Pinv, ns, newton ? s.r : s.m, s.y1, s.m, s.y2, n);
+    if (newton) {
       const float dl = newton_update(p, s);
       last = rn;
       if (converged) {
         dlam = (double)dl;
-        status = 0;
         break;
       }
-      continue;
-    }
-    if (converged) {
-      status = 0;
-      break;
-    }
-    if (it >= p.max_iter) break;
-    const double lam = s.lam;
-    bool newton = rn <= (float)kSwitch, have = false;
-    if (newton) {
-      const double tau = fabs(lam);
-      jacobian<NV, float>(p, s, J, ns, lam, (float)(3.0 * zeta));
-      have = sweep_inverse(J, Pinv, ns, (float)tau, s.m, s.piv, n);
-      if (have) {
-        apply_inverse(Pinv, ns, s.r, s.y1, s.m, s.y2, n);
-        chords = 0;
-        last = rn;
-      } else {
-        chords = kMaxChord;
-        newton = have = solve_fp64<NV>(p, s, reinterpret_cast<double*>(J), J, ns, lam,
-                                       3.0 * zeta, tau, true);
-      }
-      if (newton) newton_update(p, s);
-    }
-    if (!newton) {
-      // inverse-power step: c <- (K0 + zeta G)^{-1} M c
-      chords = kMaxChord;
-      jacobian<NV, float>(p, s, J, ns, 0.0, (float)zeta);
-      if (sweep_inverse(J, Pinv, ns, 0.0f, s.m, s.piv, n))
-        apply_inverse(Pinv, ns, s.m, s.y1, nullptr, nullptr, n);
-      else if (!solve_fp64<NV>(p, s, reinterpret_cast<double*>(J), J, ns, 0.0, zeta, 0.0, false))
-        break;
-      for (int a = tid; a < n; a += kThreads) set_entry(p, s, a, (double)s.y1[a]);
+    } else {
+      for (int a = tid; a < n; a += kThreads) set_entry(p, s, a, f2d_exact(s.y1[a]));
       __syncthreads();
     }
-    ++it;
   }
   for (int a = tid; a < n; a += kThreads) p.c_out[ib * (nh + 1) + a] = a < nh ? s.w[a] : s.cu;
   if (tid == 0) {
@@ -816,7 +924,8 @@ __global__ void __launch_bounds__(kThreads) k_spd_inverse(const double* __restri
                                                           const uint16_t* __restrict__ lists,
                                                           DenseLists dims) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ __align__(16) float piv[2][2][kSide * kMaxTile];
+  __shared__ __align__(16) float piv[2][kTile][kMaxSweep];
+  __shared__ int pivots_ok;
   L += blockIdx.x * (size_t)n * n;  // instance blockIdx.x
   Linv += blockIdx.x * (size_t)n * n;
   const int ns = row_stride(n), tid = threadIdx.x;
@@ -826,7 +935,7 @@ __global__ void __launch_bounds__(kThreads) k_spd_inverse(const double* __restri
   double* dinv = X + n * n;
   for (int e = tid; e < n * n; e += kThreads) R[(e / n) * ns + e % n] = (float)L[e];
   __syncthreads();
-  if (!sweep_inverse(R, Y, ns, 0.0f, nullptr, piv, n)) {
+  if (!sweep_inverse(R, Y, ns, 0.0f, nullptr, piv, n, &pivots_ok)) {
     const bool ok = inverse_fp64(L, reinterpret_cast<double*>(R), X, dinv, n);
     for (int e = tid; e < n * n; e += kThreads) Linv[e] = ok ? X[e] : nan("");
     return;
@@ -921,8 +1030,13 @@ size_t inverse_smem(int n) {
 
 void dense_scf(const DenseProblem& p, int nb, cudaStream_t s) {
   const size_t smem = scf_smem(p.nh + p.aug, p.nvert);
-  if (p.nvert == 3) k_dense_scf<3><<<nb, kThreads, smem, s>>>(p);
-  else k_dense_scf<4><<<nb, kThreads, smem, s>>>(p);
+  if (p.K_out) {
+    if (p.nvert == 3) k_dense_scf<3, true><<<nb, kThreads, smem, s>>>(p);
+    else k_dense_scf<4, true><<<nb, kThreads, smem, s>>>(p);
+  } else {
+    if (p.nvert == 3) k_dense_scf<3, false><<<nb, kThreads, smem, s>>>(p);
+    else k_dense_scf<4, false><<<nb, kThreads, smem, s>>>(p);
+  }
 }
 
 // The attributes are per function, shared by every handle in the process, so they are always
@@ -930,8 +1044,10 @@ void dense_scf(const DenseProblem& p, int nb, cudaStream_t s) {
 cudaError_t dense_prepare(size_t need) {
   if (need > kDenseSmemLimit) return cudaErrorInvalidValue;
   const struct { const void* f; size_t smem; } k[] = {
-      {(const void*)k_dense_scf<3>, scf_smem(Cap<3>::nh + 1, 3)},
-      {(const void*)k_dense_scf<4>, scf_smem(Cap<4>::nh + 1, 4)},
+      {(const void*)k_dense_scf<3, false>, scf_smem(Cap<3>::nh + 1, 3)},
+      {(const void*)k_dense_scf<4, false>, scf_smem(Cap<4>::nh + 1, 4)},
+      {(const void*)k_dense_scf<3, true>, scf_smem(Cap<3>::nh + 1, 3)},
+      {(const void*)k_dense_scf<4, true>, scf_smem(Cap<4>::nh + 1, 4)},
       {(const void*)k_spd_inverse, inverse_smem(kDenseMaxNh)}};
   for (const auto& q : k) {
     cudaError_t e = cudaFuncSetAttribute(q.f, cudaFuncAttributeMaxDynamicSharedMemorySize,

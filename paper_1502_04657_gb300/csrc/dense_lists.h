@@ -81,17 +81,21 @@ inline bool build_dense_lists(int nh, int ntri, int nv, const int* tri, uint16_t
       if (key[slot[s]] == k) return slot[s];
     }
   };
-  for (int t = 0; t < ntri; ++t) {
-    const int m = interior(t, lv);
-    for (int i = 0; i < m; ++i)
-      for (int j = i; j < m; ++j)
-        for (int k = j; k < m; ++k) {
-          const int q = find(tri[t * nv + lv[i]], tri[t * nv + lv[j]], tri[t * nv + lv[k]], true);
-          if (q < 0) return false;
-          ++count[q];
-          ++ntrip;
-        }
-  }
+  // numbered by their vertex count (1, 2, 3), so that the lists of neighbouring triples have
+  // about the same length
+  for (int verts = 1; verts <= 3; ++verts)
+    for (int t = 0; t < ntri; ++t) {
+      const int m = interior(t, lv);
+      for (int i = 0; i < m; ++i)
+        for (int j = i; j < m; ++j)
+          for (int k = j; k < m; ++k) {
+            if (1 + (i != j) + (j != k) != verts) continue;
+            const int q = find(tri[t * nv + lv[i]], tri[t * nv + lv[j]], tri[t * nv + lv[k]], true);
+            if (q < 0) return false;
+            ++count[q];
+            ++ntrip;
+          }
+    }
   // (a, b) entries of a triple with the remaining vertex c, by distinct ordered pairs
   auto pairs_of = [&](int q, auto&& f) {
     const int x = key[q] >> 16, y = key[q] >> 8 & 255, z = key[q] & 255;

@@ -437,7 +437,7 @@ void build_coarse(fmg_eig_handle* h) {
   std::vector<uint16_t> lists(kDenseMaxLists);
   if (!build_dense_lists(h->nh, h->ntri, h->nvert, tri.data(), lists.data(), &h->dims))
     h->dims = DenseLists{};
-  const size_t nl = h->dims.npat ? h->dims.total(h->nh) : 1;
+  const size_t nl = (h->dims.total(h->nh) + 7) / 8 * 8;  // the kernel copies 16 bytes at a time
   h->tri = h->alloc<int>(tri.size());
   h->lists = h->alloc<uint16_t>(nl);
   if (!h->dry) {
