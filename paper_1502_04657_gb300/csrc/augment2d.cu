@@ -42,11 +42,12 @@ __device__ __forceinline__ size_t at(int i, int j, int pitch) { return (size_t)j
 // NE: E, N).  s60, s180 = |K| / 60, / 180 (computed on the host: an FP64 division per node
 // would cost as much as a quarter of the kernel's arithmetic).
 // FP64 mode.
-__global__ void __launch_bounds__(32 * kStarWarps)
-    k_nload_density2d(int n, int pitch, size_t st, double s60, double s180,
-                      const double* __restrict__ u, double* __restrict__ nl,
-                      double* __restrict__ bC, double* __restrict__ bE,
-                      double* __restrict__ bN, double* __restrict__ bNE) {
+__device__ __noinline__ void nload_density2d_fp64(int n, int pitch, size_t st, double s60,
+                                                  double s180, const double* __restrict__ u,
+                                                  double* __restrict__ nl,
+                                                  double* __restrict__ bC, double* __restrict__ bE,
+                                                  double* __restrict__ bN,
+                                                  double* __restrict__ bNE) {
   using T = double;
   star2d_walk<T>(n, pitch, st, u, [&](size_t k, const Star2D<T>& p) {
     nl[k] = out_of(s60 * star_cubic(p));
@@ -54,6 +55,26 @@ __global__ void __launch_bounds__(32 * kStarWarps)
     put_entry(bE, k, s180 * fma(T(2), fma(p.H.s, p.H.s + (p.uNE + p.uS), p.H.F), p.qNE + p.qS));
     put_entry(bN, k, s180 * fma(T(2), fma(p.V.s, p.V.s + (p.uNE + p.uW), p.V.F), p.qNE + p.qW));
     put_entry(bNE, k, s180 * fma(T(2), fma(p.D.s, p.D.s + (p.uE + p.uN), p.D.F), p.qE + p.qN));
+  });
+}
+
+__global__ void __launch_bounds__(32 * kStarWarps, 4)
+    k_nload_density2d(int n, int pitch, size_t st, double s60, double s180,
+                      const double* __restrict__ u, double* __restrict__ nl,
+                      double* __restrict__ bC, double* __restrict__ bE,
+                      double* __restrict__ bN, double* __restrict__ bNE) {
+  const int e = star2d_exponent(n, pitch, st, u);
+  if (e == kFxNone) {
+    nload_density2d_fp64(n, pitch, st, s60, s180, u, nl, bC, bE, bN, bNE);
+    return;
+  }
+  const double a3 = fx_scale<kFx2>(s60, 3, e), a2 = fx_scale<kFx2>(s180, 2, e);
+  star2d_walk_fx<true>(n, pitch, st, u, e, [&](size_t k, const Star2DFx& p) {
+    nl[k] = to_double(star_cubic(p), a3);
+    bC[k] = to_double(madd<6>(p.u * madd<12>(p.u, p.M1), p.SF), a2);
+    bE[k] = to_double(madd<2>(fma(p.Hs, p.Hs + (p.uNE + p.uS), p.HF), p.qNE + p.qS), a2);
+    bN[k] = to_double(madd<2>(fma(p.Vs, p.Vs + (p.uNE + p.uW), p.VF), p.qNE + p.qW), a2);
+    bNE[k] = to_double(madd<2>(fma(p.Ds, p.Ds + (p.uE + p.uN), p.DF), p.qE + p.qN), a2);
   });
 }
 

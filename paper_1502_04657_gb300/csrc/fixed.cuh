@@ -1,0 +1,130 @@
+// 64-bit fixed-point arithmetic with a block exponent for the FP64 cubic-load kernels.
+//
+// On this part an FP64 operation issues at 2 lanes per clock and SM, a 64-bit integer addition
+// at 42 and a 32 x 32 -> 64 multiply-add at about 27 (measured).  The cubic-load and density
+// kernels sum products of at most three nodal values over a small neighbourhood, so a block
+// (3D) or a warp (2D) that covers a tile of nodes takes one exponent e for it, |u| < 2^e over
+// the tile, and computes in integers: a quantity of degree d in u is the integer
+//     I = value 2^(B_d - d e),  B_d = K - 3 d,
+// so every product is (I J) >> K, rounded, whatever the degrees, and a sum is an exact integer
+// addition.  Only products round, and u when it is read.  2D takes K = 61: u keeps 2^-59 of the
+// tile's maximum, squares 2^-56 and cubes 2^-53 of their maxima; 3D, whose sums of 24
+// tetrahedra need the headroom, K = 59.  The results are converted to FP64 and scaled once.
+//
+// The error is relative to the tile's maximum, FP64's to each node's own terms, so the tile has
+// to have one sign (no cancellation; the ground state's iterates do): a tile whose values of
+// the rarer sign exceed 2^-12 of the others, whose exponent lies outside +-kFxMaxExp
+// (infinities and NaN included), or of zeros, is computed in FP64 by the same walk (a called
+// function: inlined, its register pressure spilled the fixed-point path).  Measured
+// against 113-bit arithmetic on ground-state-like inputs (relative 2-norm, fixed point and
+// FP64): see nload2d / nload3d in grid2d.cu and grid3d.cu.
+#pragma once
+
+#include <stdint.h>
+
+#include "dfloat.cuh"
+
+namespace fmg {
+
+template <int K>
+struct fx {
+  static constexpr int B1 = K - 3;
+  long long v;
+  fx() = default;
+  __device__ constexpr explicit fx(int i) : v(i) {}  // raw (zero)
+  __device__ constexpr explicit fx(long long i) : v(i) {}
+};
+
+template <int K>
+__device__ __forceinline__ fx<K> operator+(fx<K> x, fx<K> y) {
+  return fx<K>(x.v + y.v);
+}
+// (x y) >> K to nearest: |x| < 2^(K - 1) (the callers put the smaller factor first), so x is
+// shifted to give the high word.  Both factors are split at a signed low half, which makes
+// every partial product a signed 32 x 32 one and bounds what the dropped low x low product
+// contributes by a quarter of a unit: three multiply-adds instead of four.
+template <int K>
+__device__ __forceinline__ fx<K> operator*(fx<K> x, fx<K> y) {
+  const long long a = x.v << (64 - K), b = y.v;
+  const int al = (int)a, bl = (int)b;
+  const int ah = (int)(a >> 32) + (int)((uint32_t)al >> 31);
+  const int bh = (int)(b >> 32) + (int)((uint32_t)bl >> 31);
+  const long long m = (long long)al * bh + ((long long)ah * bl + 0x80000000ll);
+  return fx<K>((long long)ah * bh + (m >> 32));
+}
+template <int K>
+__device__ __forceinline__ fx<K> fma(fx<K> x, fx<K> y, fx<K> z) {
+  return x * y + z;
+}
+template <int K>
+__device__ __forceinline__ fx<K> twice(fx<K> x) {
+  return fx<K>(x.v << 1);
+}
+// 2 u^3 from u and u^2
+__device__ __forceinline__ double twice_cube(double u, double u2) { return twice(u2 * u); }
+__device__ __forceinline__ dfloat twice_cube(dfloat u, dfloat u2) { return twice(u2 * u); }
+template <int K>
+__device__ __forceinline__ fx<K> twice_cube(fx<K> u, fx<K> u2) {
+  return twice(u) * u2;
+}
+
+// C x + y for a small integer C (one operation in FP64 and double-float)
+template <int C>
+__device__ __forceinline__ double madd(double x, double y) {
+  return fma((double)C, x, y);
+}
+template <int C>
+__device__ __forceinline__ dfloat madd(dfloat x, dfloat y) {
+  return fma(dfloat(C), x, y);
+}
+template <int C, int K>
+__device__ __forceinline__ fx<K> madd(fx<K> x, fx<K> y) {
+  return fx<K>(C * x.v + y.v);
+}
+
+__device__ __forceinline__ double fx_pow2(int e) {  // 2^e, -1022 <= e <= 1023
+  return __longlong_as_double((long long)(e + 1023) << 52);
+}
+// the factor of a result of degree d: s 2^(d e - B_d)
+template <int K>
+__device__ __forceinline__ double fx_scale(double s, int d, int e) {
+  return s * fx_pow2(d * e - (K - 3 * d));
+}
+template <int K>
+__device__ __forceinline__ double to_double(fx<K> x, double scale) {
+  return __ll2double_rn(x.v) * scale;
+}
+
+// u read in fixed point: scale = 2^(B1 - e)
+struct FxVec {
+  const double* __restrict__ u;
+  double scale;
+};
+template <typename T>
+__device__ __forceinline__ T get(const FxVec& u, size_t k) {
+  return T(__double2ll_rn(u.u[k] * u.scale));
+}
+
+constexpr int kFxMaxExp = 250;
+constexpr int kFxNone = -100000;  // no fixed-point exponent: compute the tile in FP64
+// The largest high words (without sign) of a tile's positive and negative values.
+struct FxTop {
+  int pos = 0, neg = 0;
+  __device__ __forceinline__ void add(double v) {
+    const int h = __double2hiint(v);
+    pos = max(pos, h);
+    neg = max(neg, h ^ (int)0x80000000);  // negative for h >= 0
+  }
+  __device__ __forceinline__ void warp_max() {
+    pos = __reduce_max_sync(0xffffffffu, pos);
+    neg = __reduce_max_sync(0xffffffffu, neg);
+  }
+  // e with |u| <= 2^e (1 - 2^-20) (the margin keeps the signed splits of products in range),
+  // or kFxNone
+  __device__ __forceinline__ int exponent() const {
+    const int e = ((max(pos, neg) + 1) >> 20) - 1022, minor = (min(pos, neg) >> 20) - 1022;
+    return e >= -kFxMaxExp && e <= kFxMaxExp && minor + 12 <= e ? e : kFxNone;
+  }
+};
+
+}  // namespace fmg

@@ -320,26 +320,54 @@ __global__ void k_rhs2d_node(int n, int pitch, size_t st, double h2_12, double h
   f[k] = fma(lam[ib], mu, -nscale * nl);
 }
 
-// The FP64 cubic-load kernels below walk columns (star2d.cuh): launch with star2d_grid /
-// star2d_block.
-__global__ void __launch_bounds__(32 * kStarWarps)
-    k_nload2d(int n, int pitch, size_t st, double scale, const double* __restrict__ u,
-              double* __restrict__ out) {
+// The FP64 cubic-load kernels below walk columns (star2d.cuh) in fixed point (fixed.cuh), the
+// warps whose tile that does not take in FP64: launch with star2d_grid / star2d_block.
+__device__ __noinline__ void nload2d_fp64(int n, int pitch, size_t st, double scale,
+                                          const double* __restrict__ u,
+                                          double* __restrict__ out) {
   star2d_walk<double>(n, pitch, st, u, [&](size_t k, const Star2D<double>& p) {
     out[k] = scale * star_cubic(p);
   });
 }
 
+__device__ __noinline__ void rhs2d_fp64(int n, int pitch, size_t st, double h2_24, double nscale,
+                                        double l, const double* __restrict__ u,
+                                        double* __restrict__ f) {
+  star2d_walk<double>(n, pitch, st, u, [&](size_t k, const Star2D<double>& p) {
+    const double mu = h2_24 * fma(12.0, p.u, p.M1);
+    f[k] = fma(l, mu, -nscale * star_cubic(p));
+  });
+}
+
+__global__ void __launch_bounds__(32 * kStarWarps, 4)
+    k_nload2d(int n, int pitch, size_t st, double scale, const double* __restrict__ u,
+              double* __restrict__ out) {
+  const int e = star2d_exponent(n, pitch, st, u);
+  if (e == kFxNone) {
+    nload2d_fp64(n, pitch, st, scale, u, out);
+    return;
+  }
+  const double s = fx_scale<kFx2>(scale, 3, e);
+  star2d_walk_fx<false>(n, pitch, st, u, e, [&](size_t k, const Star2DFx& p) {
+    out[k] = to_double(star_cubic(p), s);
+  });
+}
+
 // f = lambda M u - N(u); the mass stencil h^2/12 (6 u_p + neighbour sum) reuses the cubic
 // load's M1 (twice the neighbour sum): h^2/24 (12 u_p + M1)
-__global__ void __launch_bounds__(32 * kStarWarps)
+__global__ void __launch_bounds__(32 * kStarWarps, 4)
     k_rhs2d(int n, int pitch, size_t st, double h2_24, double h2_120,
             const double* __restrict__ lam, const PotentialParams* __restrict__ pp,
             const double* __restrict__ u, double* __restrict__ f) {
   const double nscale = pp[blockIdx.z].zeta * h2_120, l = lam[blockIdx.z];
-  star2d_walk<double>(n, pitch, st, u, [&](size_t k, const Star2D<double>& p) {
-    const double mu = h2_24 * fma(12.0, p.u, p.M1);
-    f[k] = fma(l, mu, -nscale * star_cubic(p));
+  const int e = star2d_exponent(n, pitch, st, u);
+  if (e == kFxNone) {
+    rhs2d_fp64(n, pitch, st, h2_24, nscale, l, u, f);
+    return;
+  }
+  const double s1 = l * fx_scale<kFx2>(h2_24, 1, e), s3 = fx_scale<kFx2>(nscale, 3, e);
+  star2d_walk_fx<false>(n, pitch, st, u, e, [&](size_t k, const Star2DFx& p) {
+    f[k] = fma(s1, __ll2double_rn(madd<12>(p.u, p.M1).v), -to_double(star_cubic(p), s3));
   });
 }
 

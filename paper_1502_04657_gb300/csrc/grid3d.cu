@@ -484,33 +484,35 @@ __device__ __forceinline__ T star3_cubic6(const Star3T<T>& p) {
   return fma(p.u, fma(p.u, fma(T(144), p.u, T(6) * p.S1), T(3) * p.S2), p.S3);
 }
 
-__global__ void __launch_bounds__(kS3X * kS3Y, 3)
-    k_nload3d(int n, int pitch, size_t st, double scale6, const double* __restrict__ u,
-              double* __restrict__ out) {
+// The same in fixed point.  In units of the tile's maximum S1 <= 96, S2 <= 480, S3 <= 2880 and
+// S1 + 24 u <= 120 (of 2^7 that fit), the degree-2 sums <= 1008 (of 2^10), the result <= 5040
+// (of 2^13).
+__device__ __forceinline__ fx<kFx3> star3_cubic6(const Star3T<fx<kFx3>>& p) {
+  const fx<kFx3> t = madd<2>(p.u * madd<24>(p.u, p.S1), p.S2);
+  return madd<3>(p.u * t, p.S3);
+}
+
+// the walks of the blocks that fixed point does not take
+__device__ __noinline__ void nload3d_fp64(int n, int pitch, size_t st, double scale6,
+                                          const double* __restrict__ u,
+                                          double* __restrict__ out) {
   star3_walk<false>(n, pitch, st, u, [&](size_t k, const Star3& p) {
     out[k] = scale6 * star3_cubic6(p);
   });
 }
 
-// f = lambda M u - zeta N(u); the mass stencil is h^3/120 (24 u_p + S1)
-__global__ void __launch_bounds__(kS3X * kS3Y, 3)
-    k_rhs3d(int n, int pitch, size_t st, double h3_120, double nscale6,
-            const double* __restrict__ lam, const PotentialParams* __restrict__ pp,
-            const double* __restrict__ u, double* __restrict__ f) {
-  const int ib = blockIdx.z / star3_zchunks(n);
-  const double l = lam[ib], zn = pp[ib].zeta * nscale6;
+__device__ __noinline__ void rhs3d_fp64(int n, int pitch, size_t st, double h3_120, double zn,
+                                        double l, const double* __restrict__ u,
+                                        double* __restrict__ f) {
   star3_walk<false>(n, pitch, st, u, [&](size_t k, const Star3& p) {
     f[k] = fma(l, h3_120 * fma(24.0, p.u, p.S1), -zn * star3_cubic6(p));
   });
 }
 
-// N(u~) and the density stencil, FP64: s140_6, s210_2, s420_2 = |K|/140/6, |K|/210/2,
-// |K|/420/2 against the sums of h1, 2 h2, 6 h3 (an edge lies in 6 tetrahedra along an axis
-// or the body diagonal, 4 along a face diagonal)
-__global__ void __launch_bounds__(kS3X * kS3Y, 2)
-    k_nload_density3d(int n, int pitch, size_t st, double s140_6, double s210_2,
-                      double s420_2, const double* __restrict__ u, double* __restrict__ nl,
-                      Density3D b) {
+__device__ __noinline__ void nload_density3d_fp64(int n, int pitch, size_t st, double s140_6,
+                                                  double s210_2, double s420_2,
+                                                  const double* __restrict__ u,
+                                                  double* __restrict__ nl, Density3D b) {
   star3_walk<true>(n, pitch, st, u, [&](size_t k, const Star3& p) {
     nl[k] = s140_6 * star3_cubic6(p);
     b.a[0][k] = s210_2 * fma(p.u, fma(144.0, p.u, 4.0 * p.S1), p.S2);
@@ -523,6 +525,68 @@ __global__ void __launch_bounds__(kS3X * kS3Y, 2)
       b.a[1 + d][k] = s420_2 * fma(two_ne, t, fma(fma(2.0, p.un[d], u2), p.E1[d], p.E2[d]));
     }
   });
+}
+
+__global__ void __launch_bounds__(kS3X * kS3Y, 3)
+    k_nload3d(int n, int pitch, size_t st, double scale6, const double* __restrict__ u,
+              double* __restrict__ out) {
+  const int e = star3_exponent(n, pitch, st, u);
+  if (e != kFxNone) {
+    const double s = fx_scale<kFx3>(scale6, 3, e);
+    star3_walk<false, fx<kFx3>>(
+        n, pitch, st, FxVec{u, fx_pow2(fx<kFx3>::B1 - e)},
+        [&](size_t k, const Star3T<fx<kFx3>>& p) { out[k] = to_double(star3_cubic6(p), s); });
+    return;
+  }
+  nload3d_fp64(n, pitch, st, scale6, u, out);
+}
+
+// f = lambda M u - zeta N(u); the mass stencil is h^3/120 (24 u_p + S1)
+__global__ void __launch_bounds__(kS3X * kS3Y, 3)
+    k_rhs3d(int n, int pitch, size_t st, double h3_120, double nscale6,
+            const double* __restrict__ lam, const PotentialParams* __restrict__ pp,
+            const double* __restrict__ u, double* __restrict__ f) {
+  const int ib = blockIdx.z / star3_zchunks(n);
+  const double l = lam[ib], zn = pp[ib].zeta * nscale6;
+  const int e = star3_exponent(n, pitch, st, u);
+  if (e != kFxNone) {
+    const double s1 = l * fx_scale<kFx3>(h3_120, 1, e), s3 = fx_scale<kFx3>(zn, 3, e);
+    star3_walk<false, fx<kFx3>>(n, pitch, st, FxVec{u, fx_pow2(fx<kFx3>::B1 - e)},
+                                [&](size_t k, const Star3T<fx<kFx3>>& p) {
+      f[k] = fma(s1, __ll2double_rn(madd<24>(p.u, p.S1).v), -to_double(star3_cubic6(p), s3));
+    });
+    return;
+  }
+  rhs3d_fp64(n, pitch, st, h3_120, zn, l, u, f);
+}
+
+// N(u~) and the density stencil, FP64: s140_6, s210_2, s420_2 = |K|/140/6, |K|/210/2,
+// |K|/420/2 against the sums of h1, 2 h2, 6 h3 (an edge lies in 6 tetrahedra along an axis
+// or the body diagonal, 4 along a face diagonal)
+__global__ void __launch_bounds__(kS3X * kS3Y, 3)
+    k_nload_density3d(int n, int pitch, size_t st, double s140_6, double s210_2,
+                      double s420_2, const double* __restrict__ u, double* __restrict__ nl,
+                      Density3D b) {
+  const int e = star3_exponent(n, pitch, st, u);
+  if (e != kFxNone) {
+    using T = fx<kFx3>;
+    const double a3 = fx_scale<kFx3>(s140_6, 3, e), a2 = fx_scale<kFx3>(s210_2, 2, e),
+                 c2 = fx_scale<kFx3>(s420_2, 2, e);
+    star3_walk<true, T>(n, pitch, st, FxVec{u, fx_pow2(T::B1 - e)},
+                        [&](size_t k, const Star3T<T>& p) {
+      nl[k] = to_double(star3_cubic6(p), a3);
+      b.a[0][k] = to_double(madd<4>(madd<36>(p.q, p.u * p.S1), p.S2), a2);
+      const T u2 = twice(p.u);
+#pragma unroll
+      for (int d = 0; d < 7; ++d) {
+        const T t = fma(p.u, p.un[d], p.q + p.qn[d]);  // u_p^2 + u_q^2 + u_p u_q
+        const T g = fma(madd<2>(p.un[d], u2), p.E1[d], p.E2[d]);
+        b.a[1 + d][k] = to_double((d >= 3 && d < 6) ? madd<8>(t, g) : madd<12>(t, g), c2);
+      }
+    });
+    return;
+  }
+  nload_density3d_fp64(n, pitch, st, s140_6, s210_2, s420_2, u, nl, b);
 }
 
 // The same two walks in double-float arithmetic from the split u (mixed-precision modes): the

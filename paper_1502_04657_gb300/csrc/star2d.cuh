@@ -19,10 +19,12 @@
 // end.  Every node's arithmetic is the same whichever lane and block computes it, so the
 // result does not depend on the launch shape.
 #pragma once
+#include "fixed.cuh"
 #include "fmg_internal.h"
-#include "dfloat.cuh"
 
 namespace fmg {
+
+constexpr int kFx2 = 61;  // fixed-point format of the walk (fixed.cuh)
 
 template <typename T>
 struct StarEdge {
@@ -89,6 +91,121 @@ constexpr unsigned kWalkMinBlocks = 2 * 152;
 inline bool star2d_walks(const Grid& lv) {
   const dim3 g = star2d_grid(lv.n, lv.nb);
   return lv.walk_all || (size_t)g.x * g.y * g.z >= kWalkMinBlocks;
+}
+
+// The fixed-point exponent of this warp's tile (its 32 columns, 16 rows and the row before and
+// after them), or kFxNone; uniform over the warp.  The walk reads the tile again from L1.
+__device__ __forceinline__ int star2d_exponent(int n, int pitch, size_t st, const double* u) {
+  const int i = kStarCols * blockIdx.x + threadIdx.x;
+  const int j0 = 1 + kStarRows * (blockIdx.y * blockDim.y + threadIdx.y);
+  const double* p = u + blockIdx.z * st + i;
+  FxTop m;
+#pragma unroll
+  for (int t = 0; t <= kStarRows + 2; ++t) {
+    const int r = j0 - 1 + t;
+    if (i <= n && r <= n) m.add(p[(size_t)r * pitch]);
+  }
+  m.warp_max();
+  return m.exponent();
+}
+
+// The walk in fixed point.  Sums of fixed-point values are exact, so the three opposite edges a
+// node takes from the row below it, the two of its own row and the one of the row above are
+// added up as the rows pass (start, acc), and neighbours' edges are exchanged as sums: 12
+// registers of state where eight carried edges take 48, and 9 exchanged words a row where the
+// FP64 walk exchanges 12.
+struct Star2DFx {
+  using T = fx<kFx2>;
+  T u, q, M1, SF, SE;                            // as Star2D
+  T Hs, HF, Vs, VF, Ds, DF;                      // own edges (density)
+  T uE, uN, uW, uS, uNE, qE, qN, qW, qS, qNE;    // neighbours (density)
+};
+
+// In units of the tile's maximum: 8u + M1 <= 20 and 12u + M1 <= 24 (of 2^5 that fit in 63
+// bits), the density sums <= 180 (of 2^8), the cubic load <= 120 (of 2^11).
+__device__ __forceinline__ fx<kFx2> star_cubic(const Star2DFx& p) {
+  return madd<3>(p.q * madd<8>(p.u, p.M1), fma(p.u, p.SF, p.SE));
+}
+
+template <int K>
+__device__ __forceinline__ fx<K> shfl_up1(fx<K> v) {
+  return fx<K>(__shfl_up_sync(0xffffffffu, v.v, 1));
+}
+template <int K>
+__device__ __forceinline__ fx<K> shfl_down1(fx<K> v) {
+  return fx<K>(__shfl_down_sync(0xffffffffu, v.v, 1));
+}
+// e: the warp's exponent (star2d_exponent).  Calls out(k, star) as star2d_walk does.
+template <bool DENSITY, typename Out>
+__device__ __forceinline__ void star2d_walk_fx(int n, int pitch, size_t st,
+                                               const double* __restrict__ u, int e, Out out) {
+  using T = fx<kFx2>;
+  const int lane = threadIdx.x;
+  const int i = kStarCols * blockIdx.x + lane;
+  const int j0 = 1 + kStarRows * (blockIdx.y * blockDim.y + threadIdx.y);
+  if (j0 >= n) return;  // uniform over the warp
+  const double scale = fx_pow2(T::B1 - e);
+  const double* col = u + blockIdx.z * st + i;
+  const bool produce = lane >= 1 && lane <= kStarCols && i <= n - 1;
+  auto ld = [&](int r) { return i <= n && r <= n ? col[(size_t)r * pitch] : 0.0; };
+  auto fix = [&](double v) { return T(__double2ll_rn(v * scale)); };
+  const T zero(0);
+  T u0 = fix(ld(j0 - 1)), q0 = u0 * u0;
+  T u0R = shfl_down1(u0), q0R = shfl_down1(q0);
+  double next = ld(j0);
+  T um1 = zero, qm1 = zero, um2 = zero, qm2 = zero;
+  T uRm1 = zero, qRm1 = zero, uLm1 = zero, qLm1 = zero;
+  T Hs = zero, HF = zero, Vs = zero, VF = zero, Ds = zero, DF = zero;  // own edges, row r - 1
+  T start[3] = {zero, zero, zero}, acc[3] = {zero, zero, zero};        // sums of (s, F, E3)
+#pragma unroll 2
+  for (int t = 0; t < kStarRows + 2; ++t) {
+    const int r = j0 - 1 + t;
+    const T u1 = fix(next);
+    next = ld(r + 2);
+    const T q1 = u1 * u1;
+    const T u1R = shfl_down1(u1), q1R = shfl_down1(q1);
+    T V[3], H[3], D[3];
+    auto edge = [&](T a, T qa, T b, T qb, T* o) {
+      const T s = a + b, qs = qa + qb;
+      o[0] = s;
+      o[1] = fma(s, s, qs);
+      o[2] = s * qs;
+    };
+    edge(u0, q0, u1, q1, V);
+    edge(u0, q0, u0R, q0R, H);
+    edge(u0, q0, u1R, q1R, D);
+    if (t >= 2 && produce && r - 1 <= n - 1) {
+      Star2DFx p;
+      p.u = um1;
+      p.q = qm1;
+      p.M1 = acc[0] + H[0];
+      p.SF = acc[1] + H[1];
+      p.SE = acc[2] + H[2];
+      if (DENSITY) {
+        p.Hs = Hs; p.HF = HF; p.Vs = Vs; p.VF = VF; p.Ds = Ds; p.DF = DF;
+        p.uE = uRm1; p.qE = qRm1;
+        p.uN = u0; p.qN = q0;
+        p.uW = uLm1; p.qW = qLm1;
+        p.uS = um2; p.qS = qm2;
+        p.uNE = u0R; p.qNE = q0R;
+      }
+      out(blockIdx.z * st + (size_t)(r - 1) * pitch + i, p);
+    }
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      acc[c] = start[c] + (shfl_up1(D[c]) + shfl_down1(V[c]));  // node r: its own row's edges
+      start[c] = D[c] + shfl_up1(V[c] + H[c]);                  // node r + 1: the row below
+    }
+    if (DENSITY) {
+      um2 = um1; qm2 = qm1;
+      uRm1 = u0R; qRm1 = q0R;
+      uLm1 = shfl_up1(u0); qLm1 = shfl_up1(q0);
+      Hs = H[0]; HF = H[1]; Vs = V[0]; VF = V[1]; Ds = D[0]; DF = D[1];
+    }
+    um1 = u0; qm1 = q0;
+    u0 = u1; q0 = q1;
+    u0R = u1R; q0R = q1R;
+  }
 }
 
 // Walks the rows of this thread's strip of instance blockIdx.z and calls out(k, star) for

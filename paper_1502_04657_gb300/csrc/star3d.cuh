@@ -1,6 +1,7 @@
 // Plane-walked star sums of the 3D cubic load and density stencil (device code of
-// grid3d.cu), in FP64 or, for the mixed-precision modes, in double-float arithmetic (T =
-// dfloat, u read from its split copy).
+// grid3d.cu): in 64-bit fixed point with an exponent per block (T = fx<kFx3>, fixed.cuh) for
+// the FP64 mode, in FP64 for the blocks that fixed point does not take, or, for the
+// mixed-precision modes, in double-float arithmetic (T = dfloat, u read from its split copy).
 //
 // On a tetrahedron K with vertex values a, b, c, d let h1, h2, h3 be the complete homogeneous
 // symmetric sums of degree 1, 2, 3 of the four values.  Exact integration of P1 functions
@@ -27,10 +28,12 @@
 // the node above it.  Every sum is taken in a fixed order, so the result does not depend on
 // the launch shape.
 #pragma once
-#include "dfloat.cuh"
+#include "fixed.cuh"
 #include "fmg_internal.h"
 
 namespace fmg {
+
+constexpr int kFx3 = 59;  // fixed-point format of the walk (fixed.cuh)
 
 constexpr int kS3X = 32, kS3Y = 8, kS3Z = 16;   // tile of columns (= threads), planes per block
 constexpr int kS3CX = kS3X + 1;                  // cube layer row (cubes x0 - 1 .. x0 + 31)
@@ -41,7 +44,8 @@ constexpr int kS3Vals = 21;  // per cube: 6 tetrahedra x (h1, 2 h2, 6 h3), then 
 // three plane slots of (u, u^2, u^3) and one cube layer (a double-float value takes the 8
 // bytes of a double)
 constexpr size_t kS3Smem = sizeof(double) * (9 * (size_t)kS3Nodes + (size_t)kS3Vals * kS3Cubes);
-static_assert(sizeof(dfloat) == sizeof(double), "double-float values share the FP64 layout");
+static_assert(sizeof(dfloat) == sizeof(double) && sizeof(fx<kFx3>) == sizeof(double),
+              "double-float and fixed-point values share the FP64 layout");
 
 // what a node hands to its epilogue: sums over its 24 tetrahedra of h1, 2 h2 and 6 h3, and for
 // each edge towards p + d (d = X, Y, Z, XY, XZ, YZ, XYZ) the sums of h1 and 2 h2 over the
@@ -70,6 +74,37 @@ constexpr unsigned kWalk3MinBlocks = 2 * 152;
 inline bool star3_walks(const Grid& lv) {
   const dim3 g = star3_grid(lv.n, lv.nb);
   return lv.walk_all || (size_t)g.x * g.y * g.z >= kWalk3MinBlocks;
+}
+
+// The fixed-point exponent of this block's tile (its 16 planes and the halo of the walk), or
+// kFxNone.  Reads the tile once; the walk reads it again from L2.
+__device__ __forceinline__ int star3_exponent(int n, int pitch, size_t st, const double* u) {
+  __shared__ int top[2];
+  const int tid = threadIdx.y * kS3X + threadIdx.x;
+  if (tid < 2) top[tid] = 0;
+  const int nzc = star3_zchunks(n);
+  const int ib = blockIdx.z / nzc;
+  const int z0 = 1 + (int)(blockIdx.z - ib * nzc) * kS3Z, z1 = min(z0 + kS3Z, n);
+  const int x0 = 1 + blockIdx.x * kS3X, y0 = 1 + blockIdx.y * kS3Y;
+  const long plane = (long)(n + 1) * pitch;
+  FxTop m;
+  for (int e = tid; e < kS3Nodes; e += kS3X * kS3Y) {
+    const int x = x0 - 1 + e % kS3NX, y = y0 - 1 + e / kS3NX;
+    if (x > n || y > n) continue;
+    const double* p = u + (size_t)ib * st + (long)y * pitch + x;
+#pragma unroll 6
+    for (int z = z0 - 1; z <= z1; ++z) m.add(p[z * plane]);
+  }
+  m.warp_max();
+  __syncthreads();
+  if ((tid & 31) == 0) {
+    atomicMax(&top[0], m.pos);
+    atomicMax(&top[1], m.neg);
+  }
+  __syncthreads();
+  m.pos = top[0];
+  m.neg = top[1];
+  return m.exponent();
 }
 
 // blockDim = (kS3X, kS3Y), kS3Smem bytes of dynamic shared memory; instance
@@ -102,7 +137,7 @@ __device__ __forceinline__ void star3_walk(int n, int pitch, size_t st, const U 
       const T v2 = v * v;
       su[sl + e] = v;
       sq[sl + e] = v2;
-      sc[sl + e] = twice(v2 * v);  // 2 u^3: 6 h3 takes 2 p3, and doubling is exact
+      sc[sl + e] = twice_cube(v, v2);  // 2 u^3: 6 h3 takes 2 p3, and doubling is exact
     }
   };
 
@@ -129,7 +164,7 @@ __device__ __forceinline__ void star3_walk(int n, int pitch, size_t st, const U 
         const T s2 = h1 * h1;
         h[t][0] = h1;
         h[t][1] = s2 + p2;                         // 2 h2
-        h[t][2] = fma(h1, fma(T(3), p2, s2), p3);  // 6 h3 (p3 from 2 u^3: 2 p3)
+        h[t][2] = fma(h1, madd<3>(p2, s2), p3);    // 6 h3 (p3 from 2 u^3: 2 p3)
       };
       tet(0, 0, XY);
       tet(1, 0, XZ);
