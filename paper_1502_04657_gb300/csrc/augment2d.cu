@@ -222,141 +222,149 @@ __global__ void k_coarsen_density2d(int nc, int pc, int pf, size_t stc, size_t s
 //   [14..17] edge B: sum u x^m  (T0: right s = r, x = tg;   T1: top t = r,  x = sg)
 //   [18..21] diagonal s = t: sum u sg^m
 //   [22..24] vertex values (T0: V00, V10, V11;  T1: V00, V11, V01)
+//
+// Interior: a thread takes a column s of the cell over kSumRows rows and adds its nodes to T0
+// (t < s) or T1 (t > s), 4 FP64 operations per node, so every column is the same length and
+// every node is read once; the rows are loaded eight at a time (a row at a time, with the
+// class of each node decided as it came, waited out a memory latency per row: 532 us on
+// 16.8M nodes, where the FP64 pipe needs 106).  Only the 32 rows around a warp's diagonal need
+// the comparison per lane.  Edges, diagonals and vertices (one block per cell) go apart.
 constexpr int kSums = 25;
-constexpr int kSumThreads = 256;
-constexpr int kSumRows = 1024;
+constexpr int kSumThreads = 128;
+constexpr int kSumRows = 128;
+constexpr int kInner = 20;  // interior sums of a cell: 10 of T0, 10 of T1
+constexpr int kLines = 24;  // sum u x^m, m < 4, of bottom, right, left, top, diagonal; vertices
 
-template <int T>
-__device__ void t3_sums_body(int pf, int n1, int r, const double* __restrict__ u,
-                             const double* __restrict__ pw, double* __restrict__ partials,
-                             int col_blocks) {
-  // instance blockIdx.z: u and partials arrive offset to it
-  __shared__ double sh[kSumThreads];
-  const int tri = blockIdx.y;
-  const int cell = tri >> 1;
-  const int I = cell % n1, J = cell / n1;
-  const int cb = blockIdx.x % col_blocks, rb = blockIdx.x / col_blocks;
-  const int s = cb * blockDim.x + threadIdx.x;
-  const int t0 = rb * kSumRows;
-  const int t1 = min(t0 + kSumRows, r + 1);
-  double c[4] = {0.0, 0.0, 0.0, 0.0};  // interior: sum_t u tg^l for this column
-  double ea = 0.0, eb = 0.0, ed = 0.0;  // per-column edge values (T0: bottom, -, diag)
-  double eb_t[4] = {0.0, 0.0, 0.0, 0.0};  // edge varying in t (T0 right / T1 left)
-  double vtx[3] = {0.0, 0.0, 0.0};
-  if (s <= r) {
-    const double* col = u + (size_t)(J * r) * pf + (size_t)(I * r + s);
-    // the rows of this column inside the triangle: T0 (lower) t <= s, T1 (upper) t >= s; the
-    // rows outside would add nothing.  The lanes of a warp read one row per step (coalesced),
-    // so T1 starts at the warp's first column, and its lanes skip the rows above their own.
-    const int ta = T == 0 ? t0 : max(t0, s - (int)(threadIdx.x & 31));
-    const int tb = T == 0 ? min(t1, s + 1) : t1;
-    for (int t = ta; t < tb; ++t) {
-      const double val = col[(size_t)t * pf];
-      const double* p = pw + 4 * t;  // tg^m, m = 0..3
-      if (T == 0) {
-        if (t == 0) {
-          if (s == 0) vtx[0] = val;
-          else if (s == r) vtx[1] = val;
-          else ea = val;
-        } else if (s == r) {
-          if (t == r) vtx[2] = val;
-          else {
+// c_m += sum_{ta <= t < tb} col[t pf] (t / r)^m
+__device__ __forceinline__ void column_sums(const double* __restrict__ col, int pf,
+                                            const double* __restrict__ pw, int ta, int tb,
+                                            double (&c)[4]) {
+  constexpr int kAhead = 8;
+  int t = ta;
+  for (; t + kAhead <= tb; t += kAhead) {
+    double v[kAhead];
 #pragma unroll
-            for (int m = 0; m < 4; ++m) eb_t[m] = fma(val, p[m], eb_t[m]);
-          }
-        } else if (t == s) {
-          ed = val;
-        } else if (t < s) {
+    for (int q = 0; q < kAhead; ++q) v[q] = col[(size_t)(t + q) * pf];
 #pragma unroll
-          for (int m = 0; m < 4; ++m) c[m] = fma(val, p[m], c[m]);
-        }
-      } else {
-        if (s == 0) {
-          if (t == 0) vtx[0] = val;
-          else if (t == r) vtx[2] = val;
-          else {
+    for (int q = 0; q < kAhead; ++q) {
+      const double* p = pw + 4 * (t + q);
+      c[0] += v[q];
 #pragma unroll
-            for (int m = 0; m < 4; ++m) eb_t[m] = fma(val, p[m], eb_t[m]);
-          }
-        } else if (t == r) {
-          if (s == r) vtx[1] = val;
-          else eb = val;
-        } else if (s == t) {
-          ed = val;
-        } else if (s < t) {
-#pragma unroll
-          for (int m = 0; m < 4; ++m) c[m] = fma(val, p[m], c[m]);
-        }
-      }
+      for (int m = 1; m < 4; ++m) c[m] = fma(v[q], p[m], c[m]);
     }
   }
-  double acc[kSums];
-  const double* ps = pw + 4 * (s <= r ? s : 0);  // sg^m
-  const double ok = s <= r ? 1.0 : 0.0;
-  // interior monomials in kMono order: (0,0),(1,0),(0,1),(2,0),(1,1),(0,2),(3,0),(2,1),(1,2),(0,3)
-  acc[0] = ok * c[0];
-  acc[1] = ok * ps[1] * c[0];
-  acc[2] = ok * c[1];
-  acc[3] = ok * ps[2] * c[0];
-  acc[4] = ok * ps[1] * c[1];
-  acc[5] = ok * c[2];
-  acc[6] = ok * ps[3] * c[0];
-  acc[7] = ok * ps[2] * c[1];
-  acc[8] = ok * ps[1] * c[2];
-  acc[9] = ok * c[3];
-  if (T == 0) {
+  for (; t < tb; ++t) {
+    const double v = col[(size_t)t * pf];
+    const double* p = pw + 4 * t;
+    c[0] += v;
 #pragma unroll
-    for (int m = 0; m < 4; ++m) {
-      acc[10 + m] = ok * ps[m] * ea;  // bottom, x = sg
-      acc[14 + m] = ok * eb_t[m];     // right, x = tg
-      acc[18 + m] = ok * ps[m] * ed;  // diagonal
-    }
-  } else {
-#pragma unroll
-    for (int m = 0; m < 4; ++m) {
-      acc[10 + m] = ok * eb_t[m];     // left, x = tg
-      acc[14 + m] = ok * ps[m] * eb;  // top, x = sg
-      acc[18 + m] = ok * ps[m] * ed;
-    }
+    for (int m = 1; m < 4; ++m) c[m] = fma(v, p[m], c[m]);
   }
-  acc[22] = ok * vtx[0];
-  acc[23] = ok * vtx[1];
-  acc[24] = ok * vtx[2];
-  block_sum_to<kSums>(acc, sh, partials + ((size_t)tri * gridDim.x + blockIdx.x) * kSums);
 }
 
 __global__ void __launch_bounds__(kSumThreads)
     k_t3_sums2d(int pf, int n1, int r, size_t st, size_t pst, const double* __restrict__ u,
-                const double* __restrict__ pw, double* __restrict__ partials, int col_blocks) {
-  u += blockIdx.z * st;
+                const double* __restrict__ pw, double* __restrict__ partials, int col_blocks,
+                int chunks) {
+  __shared__ double sh[kSumThreads];
+  const int cell = blockIdx.y, I = cell % n1, J = cell / n1;
+  u += blockIdx.z * st + (size_t)(J * r) * pf + (size_t)I * r;  // the cell's corner
   partials += blockIdx.z * pst;
-  if (blockIdx.y & 1)
-    t3_sums_body<1>(pf, n1, r, u, pw, partials, col_blocks);
-  else
-    t3_sums_body<0>(pf, n1, r, u, pw, partials, col_blocks);
+  double acc[kInner];
+  if ((int)blockIdx.x < chunks) {
+    const int cb = blockIdx.x % col_blocks, seg = blockIdx.x / col_blocks;
+    const int s = 1 + cb * blockDim.x + threadIdx.x;
+    const int ta = 1 + seg * kSumRows, tb = min(ta + kSumRows, r);
+    const int s0 = s - (int)(threadIdx.x & 31), s1 = min(s0 + 31, r - 1);  // the warp's columns
+    const double* col = u + min(s, r - 1);
+    double c0[4] = {0.0, 0.0, 0.0, 0.0}, c1[4] = {0.0, 0.0, 0.0, 0.0};
+    column_sums(col, pf, pw, ta, min(tb, s0), c0);
+    for (int t = max(ta, s0); t < min(tb, s1 + 1); ++t) {
+      const double v = col[(size_t)t * pf], v0 = t < s ? v : 0.0, v1 = t > s ? v : 0.0;
+      const double* p = pw + 4 * t;
+      c0[0] += v0;
+      c1[0] += v1;
+#pragma unroll
+      for (int m = 1; m < 4; ++m) {
+        c0[m] = fma(v0, p[m], c0[m]);
+        c1[m] = fma(v1, p[m], c1[m]);
+      }
+    }
+    column_sums(col, pf, pw, max(ta, s1 + 1), tb, c1);
+    const double* ps = pw + 4 * min(s, r - 1);  // sg^m
+    const double p1 = ps[1], p2 = ps[2], p3 = ps[3];
+    auto monomials = [&](const double (&c)[4], double* o) {
+      // kMono order: (0,0),(1,0),(0,1),(2,0),(1,1),(0,2),(3,0),(2,1),(1,2),(0,3)
+      const bool ok = s < r;
+      const double a0 = ok ? c[0] : 0.0, a1 = ok ? c[1] : 0.0, a2 = ok ? c[2] : 0.0,
+                   a3 = ok ? c[3] : 0.0;
+      o[0] = a0; o[1] = p1 * a0; o[2] = a1; o[3] = p2 * a0; o[4] = p1 * a1; o[5] = a2;
+      o[6] = p3 * a0; o[7] = p2 * a1; o[8] = p1 * a2; o[9] = a3;
+    };
+    monomials(c0, acc);
+    monomials(c1, acc + 10);
+    block_sum_to<kInner>(acc, sh, partials + ((size_t)cell * chunks + blockIdx.x) * kInner);
+    return;
+  }
+  double* out = partials + (size_t)n1 * n1 * chunks * kInner + (size_t)cell * kLines;
+#pragma unroll
+  for (int m = 0; m < kInner; ++m) acc[m] = 0.0;
+  for (int x = 1 + threadIdx.x; x < r; x += blockDim.x) {
+    const double v[5] = {u[x], u[(size_t)x * pf + r], u[(size_t)x * pf], u[(size_t)r * pf + x],
+                         u[(size_t)x * pf + x]};
+    const double* p = pw + 4 * x;
+#pragma unroll
+    for (int e = 0; e < 5; ++e) {
+      acc[4 * e] += v[e];
+#pragma unroll
+      for (int m = 1; m < 4; ++m) acc[4 * e + m] = fma(v[e], p[m], acc[4 * e + m]);
+    }
+  }
+  block_sum_to<kInner>(acc, sh, out);
+  if (threadIdx.x == 0) {
+    out[kInner] = u[0];
+    out[kInner + 1] = u[r];
+    out[kInner + 2] = u[(size_t)r * pf + r];
+    out[kInner + 3] = u[(size_t)r * pf];
+  }
 }
 
 // Finalise: T3^T_e = h^2 sum_m map[T][e][m] S_m, a fixed linear map of the 25 class sums per
 // triangle type, built on the host for the level's r (t3_map2d).
-__global__ void k_t3_finalize2d(int chunks, double h2, size_t pst, size_t tst,
+__global__ void k_t3_finalize2d(int cells, int chunks, double h2, size_t pst, size_t tst,
                                 const double* __restrict__ partials,
                                 const double* __restrict__ map, double* __restrict__ t3) {
   partials += blockIdx.y * pst;
   t3 += blockIdx.y * tst;
-  const int tri = blockIdx.x;
-  const int T = tri & 1;
+  const int tri = blockIdx.x, cell = tri >> 1, T = tri & 1;
   __shared__ double sums[kSums];
-  for (int m = threadIdx.x; m < kSums; m += blockDim.x) {
+  const int m = threadIdx.x;
+  if (m < 10) {
+    const double* p = partials + (size_t)cell * chunks * kInner + T * 10 + m;
     double s = 0.0;
-    for (int c = 0; c < chunks; ++c) s += partials[((size_t)tri * chunks + c) * kSums + m];
+#pragma unroll 8
+    for (int c = 0; c < chunks; ++c) s += p[(size_t)c * kInner];
     sums[m] = s;
+  } else if (m < kSums) {
+    const double* e = partials + (size_t)cells * chunks * kInner + (size_t)cell * kLines;
+    // edge A: bottom (T0) / left (T1); edge B: right / top; diagonal; vertices
+    const int q = m - 10;
+    int at;
+    if (q < 4) at = (T == 0 ? 0 : 8) + q;
+    else if (q < 8) at = (T == 0 ? 4 : 12) + q - 4;
+    else if (q < 12) at = 16 + q - 8;
+    else if (q == 12) at = kInner;
+    else if (q == 13) at = kInner + (T == 0 ? 1 : 2);
+    else at = kInner + (T == 0 ? 2 : 3);
+    sums[m] = e[at];
   }
   __syncthreads();
   const int e = threadIdx.x;
   if (e >= 10) return;
   const double* row = map + ((size_t)T * 10 + e) * kSums;
   double acc = 0.0;
-  for (int m = 0; m < kSums; ++m) acc = fma(row[m], sums[m], acc);
+#pragma unroll
+  for (int q = 0; q < kSums; ++q) acc = fma(row[q], sums[q], acc);
   t3[(size_t)tri * 10 + e] = h2 * acc;
 }
 
@@ -392,10 +400,10 @@ __global__ void k_gather_level1_2d(int n, int pitch, size_t st, const double* __
   put(-1, -1, b.NE, k - pitch - 1);
 }
 
-// a block takes blockDim.x columns (whole warps, up to kSumThreads) of kSumRows rows
-int t3_threads2d(int r) { return warps_for(r + 1, kSumThreads); }
-int t3_col_blocks(int r) { return (r + 1 + t3_threads2d(r) - 1) / t3_threads2d(r); }
-int t3_row_blocks(int r) { return (r + 1 + kSumRows - 1) / kSumRows; }
+// a block takes blockDim.x interior columns (whole warps, up to kSumThreads) of kSumRows rows
+int t3_threads2d(int r) { return warps_for(r - 1, kSumThreads); }
+int t3_col_blocks(int r) { return (r - 1 + t3_threads2d(r) - 1) / t3_threads2d(r); }
+int t3_chunks2d(int r) { return t3_col_blocks(r) * ((r - 1 + kSumRows - 1) / kSumRows); }
 
 dim3 grid_of(const Grid& g, int cx, int cy) {
   return dim3((cx + g.bx - 1) / g.bx, (cy + g.by - 1) / g.by, g.nb);
@@ -445,19 +453,17 @@ void gather_level1_2d(const Grid& g1, const double* gA_pad, const double* gM_pad
 }
 
 size_t t3_partials2d(const Grid& fine, int n1) {
-  const int r = fine.n / n1;
-  return (size_t)2 * n1 * n1 * t3_col_blocks(r) * t3_row_blocks(r) * kSums;
+  return (size_t)n1 * n1 * ((size_t)t3_chunks2d(fine.n / n1) * kInner + kLines);
 }
 
 void t3_moments2d(const Grid& fine, int n1, const double* u, const double* pw,
                   const double* map, double* partials, double* t3, cudaStream_t s) {
-  const int r = fine.n / n1;
-  const int cb = t3_col_blocks(r), rb = t3_row_blocks(r);
+  const int r = fine.n / n1, chunks = t3_chunks2d(r);
   const size_t pst = t3_partials2d(fine, n1);
-  k_t3_sums2d<<<dim3(cb * rb, 2 * n1 * n1, fine.nb), t3_threads2d(r), 0, s>>>(
-      fine.pitch, n1, r, fine.stride, pst, u, pw, partials, cb);
+  k_t3_sums2d<<<dim3(chunks + 1, n1 * n1, fine.nb), t3_threads2d(r), 0, s>>>(
+      fine.pitch, n1, r, fine.stride, pst, u, pw, partials, t3_col_blocks(r), chunks);
   k_t3_finalize2d<<<dim3(2 * n1 * n1, fine.nb), 32, 0, s>>>(
-      cb * rb, fine.h * fine.h, pst, (size_t)2 * n1 * n1 * 10, partials, map, t3);
+      n1 * n1, chunks, fine.h * fine.h, pst, (size_t)2 * n1 * n1 * 10, partials, map, t3);
 }
 
 // Host: moments m_ij = int_K lambda_v (ds)^i (dt)^j over each star triangle of a node (fine
@@ -493,7 +499,7 @@ void t3_class_moments2d(double out[2 * 7 * 10]) {
       star[t][m] = acc;
     }
   }
-  // classes: 0 interior, 1 edge A, 2 edge B, 3 diagonal, 4..6 vertices (see t3_sums_body);
+  // classes: 0 interior, 1 edge A, 2 edge B, 3 diagonal, 4..6 vertices (see the T3 class sums above);
   // star triangle t = pair (nb[t], nb[t+1]): 0 (E,NE) 1 (NE,N) 2 (N,W) 3 (W,SW) 4 (SW,S) 5 (S,E)
   const int sets[2][7][6] = {
       {{0, 1, 2, 3, 4, 5}, {0, 1, 2, -1}, {2, 3, 4, -1}, {4, 5, 0, -1}, {0, -1}, {2, -1}, {4, -1}},
@@ -533,7 +539,7 @@ void t3_map2d(int r, double out[2 * 10 * 25]) {
   const int mk[10] = {0, 1, 0, 2, 1, 0, 3, 2, 1, 0}, ml[10] = {0, 0, 1, 0, 1, 2, 0, 1, 2, 3};
   const double fall[4][4] = {{1, 0, 0, 0}, {1, 1, 0, 0}, {1, 2, 2, 0}, {1, 3, 6, 6}};
   const double fact[4] = {1, 1, 2, 6};
-  // index of S^class_{a,b} among the 25 sums (-1: identically zero); see t3_sums_body
+  // index of S^class_{a,b} among the 25 sums (-1: identically zero); see the T3 class sums above
   auto sum_index = [](int T, int cls, int a, int b) -> int {
     switch (cls) {
       case 0: { const int d = a + b; return d * (d + 1) / 2 + b; }

@@ -13,6 +13,7 @@
 // linear map of the 15 x 20 class monomial sums S^class_g = sum u~ (a,b,c)^g, |g| <= 3.
 #include <math.h>
 
+#include <algorithm>
 #include <map>
 #include <vector>
 
@@ -37,116 +38,138 @@ __device__ __forceinline__ void monomials(double a, double b, double c, double* 
   m[15] = a * m[9]; m[16] = m[7] * b; m[17] = m[7] * c; m[18] = b * m[9]; m[19] = m[9] * c;
 }
 
-// Interior class: a thread takes (x0, x2) lines of the coarse cell along x1 (kLinesPerThread of
-// them, strided by the grid; x0 fastest across the threads: coalesced loads), block (chunk of
-// lines, tet, instance), and adds their monomial sums before one block reduction (most of
-// a line's FP64 work had been that reduction, many lines being empty).  On a line, the nodes
-// strictly inside T_s are an interval of x1 (the chain order a > b > c of T_s bounds x1 by the
-// line's two other coordinates), and every monomial is (powers of the line's fixed chain
-// coordinates) x (a power of x1 / r): the thread sums u (x1/r)^e, e = 0..3, along its
-// interval with the powers from the level's table pw (4 FMAs per node, in two interleaved
-// sets of accumulators to halve the FP64 dependency chain) and then adds the 20 monomial
-// sums of its line.
-__constant__ int kMonoExpDev[20][3] = {{0, 0, 0}, {1, 0, 0}, {0, 1, 0}, {0, 0, 1}, {2, 0, 0},
+// Interior class: a thread takes (x0, x2) lines of the coarse cell along x1, x0 fastest across
+// the threads (coalesced loads), and adds their monomial sums before one block reduction.  x1
+// runs through three tetrahedra of the line, x1 < f2, f2 < x1 < f1 and x1 > f1 with f1 > f2 the
+// line's fixed coordinates, so one pass over a line serves all three, every node is read and
+// summed once, and the lanes of a warp read the same x1 (a pass per tetrahedron that started
+// each lane at its own x1 read uncoalesced and spent most of its FP64 slots on lanes outside
+// the tetrahedron: 464 us on 16.6M nodes).  Lines with x0 > x2 and x0 < x2 lie in different
+// tetrahedra and go to different blocks; their index runs over the pairs f1 > f2.  Every
+// monomial is (powers of f1 / r and f2 / r) x (a power of x1 / r): a thread sums u (x1/r)^e,
+// e = 0..3, with the powers from the level's table pw (4 FP64 operations per node) and then
+// adds the 3 x 20 monomial sums of its line.
+__device__ constexpr int kExpDev[20][3] = {{0, 0, 0}, {1, 0, 0}, {0, 1, 0}, {0, 0, 1}, {2, 0, 0},
                                        {1, 1, 0}, {1, 0, 1}, {0, 2, 0}, {0, 1, 1}, {0, 0, 2},
                                        {3, 0, 0}, {2, 1, 0}, {2, 0, 1}, {1, 2, 0}, {1, 1, 1},
                                        {1, 0, 2}, {0, 3, 0}, {0, 2, 1}, {0, 1, 2}, {0, 0, 3}};
-
-__device__ __forceinline__ int coord(int axis, int x0, int x1, int x2) {
-  return axis == 0 ? x0 : (axis == 1 ? x1 : x2);
-}
 
 __device__ __forceinline__ double pick4(double v0, double v1, double v2, double v3, int e) {
   return e == 0 ? v0 : (e == 1 ? v1 : (e == 2 ? v2 : v3));
 }
 
-__global__ void __launch_bounds__(kThreads)
+// tetrahedron (kPerm index) of a line's phase: [x0 < x2][x1 < f2, f2 < x1 < f1, x1 > f1]
+__constant__ int kPhaseTet[2][3] = {{1, 0, 2}, {4, 5, 3}};
+
+constexpr int kLineThreads = 128;
+constexpr int kLinesPerThread = 2;  // lines summed per thread before the block reduction
+
+__global__ void __launch_bounds__(kLineThreads)
     k_t3_interior3d(int pf, long planef, int n1, int r, size_t st, size_t pst,
                     const double* __restrict__ u, const double* __restrict__ pw,
                     double* __restrict__ partials) {
-  __shared__ double sh[kThreads];
+  __shared__ double sh[2][kLineThreads];
   u += blockIdx.z * st;  // instance blockIdx.z
   partials += blockIdx.z * pst;
-  const int tet = blockIdx.y;
-  const int cell = tet / 6, s = tet % 6;
+  const int cell = blockIdx.y >> 1, o = blockIdx.y & 1;  // o: x0 < x2
   const int I = cell % n1, J = (cell / n1) % n1, L = cell / (n1 * n1);
-  const int R = r + 1;
-  // chain position of axis 1 (the axis threads walk along)
-  const int pos1 = kPermDev[s][0] == 1 ? 0 : (kPermDev[s][1] == 1 ? 1 : 2);
-  double acc[kMono];
+  double acc[3][kMono];
 #pragma unroll
-  for (int m = 0; m < kMono; ++m) acc[m] = 0.0;
-  // a thread takes several lines (strided over the block's chunk of the grid) and sums their
-  // monomial sums before the one block reduction
-  for (int line = blockIdx.x * blockDim.x + threadIdx.x; line < R * R;
+  for (int p = 0; p < 3; ++p)
+#pragma unroll
+    for (int m = 0; m < kMono; ++m) acc[p][m] = 0.0;
+  const int lines = (r - 1) * (r - 2) / 2;
+  for (int line = blockIdx.x * blockDim.x + threadIdx.x; line < lines;
        line += gridDim.x * blockDim.x) {
-    const int x0 = line % R, x2 = line / R;
-    // the two fixed chain coordinates (positions q1 < q2, the ones other than pos1)
-    const int q1 = pos1 == 0 ? 1 : 0, q2 = pos1 == 2 ? 1 : 2;
-    const int f1 = coord(kPermDev[s][q1], x0, 0, x2), f2 = coord(kPermDev[s][q2], x0, 0, x2);
-    // interval of x1 (exclusive bounds) from r > a > b > c > 0
-    int lo = 0, hi = -1;
-    if (pos1 == 0) {  // x1 = a, fixed b = f1, c = f2
-      if (f1 > f2 && f2 > 0) { lo = f1; hi = r; }
-    } else if (pos1 == 1) {  // x1 = b, fixed a = f1, c = f2
-      if (f1 < r && f2 > 0) { lo = f2; hi = f1; }
-    } else {  // x1 = c, fixed a = f1, b = f2
-      if (f1 < r && f1 > f2) { lo = 0; hi = f2; }
-    }
-    if (lo + 1 < hi) {
-      const double* colp =
-          u + (size_t)(L * r + x2) * planef + (size_t)(J * r) * pf + (size_t)(I * r + x0);
-      double m[2][4] = {{0.0, 0.0, 0.0, 0.0}, {0.0, 0.0, 0.0, 0.0}};
-      int x1 = lo + 1;
-      for (; x1 + 1 < hi; x1 += 2) {
+    // line -> (g1, g2), 1 <= g2 < g1 <= r - 1, g2 fastest
+    int g1 = (int)((sqrtf(8.0f * line + 1.0f) + 1.0f) * 0.5f);  // g1 - 1
+    while (g1 * (g1 - 1) / 2 > line) --g1;
+    while ((g1 + 1) * g1 / 2 <= line) ++g1;
+    const int g2 = line - g1 * (g1 - 1) / 2 + 1;
+    ++g1;
+    // x0 < x2: x0 = g2, x2 = g1; x0 > x2: mirrored, so that x0 is fastest too
+    const int x0 = o ? g2 : r - g2, x2 = o ? g1 : r - g1;
+    const int f1 = max(x0, x2), f2 = min(x0, x2);
+    const double* col =
+        u + (size_t)(L * r + x2) * planef + (size_t)(J * r) * pf + (size_t)(I * r + x0);
+    double m[4] = {0.0, 0.0, 0.0, 0.0}, m0[4], m1[4];  // the running phase, phases 0 and 1
+    constexpr int kAhead = 8;
+    for (int x1 = 1; x1 < r; x1 += kAhead) {
+      double v[kAhead];
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const double val = colp[(size_t)(x1 + h) * pf];
-          const double* p = pw + 4 * (x1 + h);  // (x1/r)^e
-          m[h][0] += val;
-          m[h][1] = fma(val, p[1], m[h][1]);
-          m[h][2] = fma(val, p[2], m[h][2]);
-          m[h][3] = fma(val, p[3], m[h][3]);
+      for (int q = 0; q < kAhead; ++q) v[q] = x1 + q < r ? col[(size_t)(x1 + q) * pf] : 0.0;
+#pragma unroll
+      for (int q = 0; q < kAhead; ++q) {
+        const int x = x1 + q;
+        if (x < r) {
+          if (x == f2) {  // the diagonal planes belong to the boundary classes
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+              m0[e] = m[e];
+              m[e] = 0.0;
+            }
+          } else if (x == f1) {
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+              m1[e] = m[e];
+              m[e] = 0.0;
+            }
+          } else {
+            const double* p = pw + 4 * x;  // (x1/r)^e
+            m[0] += v[q];
+#pragma unroll
+            for (int e = 1; e < 4; ++e) m[e] = fma(v[q], p[e], m[e]);
+          }
         }
       }
-      if (x1 < hi) {
-        const double val = colp[(size_t)x1 * pf];
-        const double* p = pw + 4 * x1;
-        m[0][0] += val;
-        m[0][1] = fma(val, p[1], m[0][1]);
-        m[0][2] = fma(val, p[2], m[0][2]);
-        m[0][3] = fma(val, p[3], m[0][3]);
-      }
-      const double m0 = m[0][0] + m[1][0], m1 = m[0][1] + m[1][1], m2 = m[0][2] + m[1][2],
-                   m3 = m[0][3] + m[1][3];
-      const double* g1p = pw + 4 * f1;
-      const double* g2p = pw + 4 * f2;
+    }
+    double g[4][4];  // (f1/r)^i (f2/r)^j
+    {
+      const double *a = pw + 4 * f1, *b = pw + 4 * f2;
 #pragma unroll
-      for (int q = 0; q < kMono; ++q) {
-        const int e0 = kMonoExpDev[q][pos1], e1 = kMonoExpDev[q][q1], e2 = kMonoExpDev[q][q2];
-        acc[q] = fma(g1p[e1] * g2p[e2], pick4(m0, m1, m2, m3, e0), acc[q]);
-      }
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; i + j < 4; ++j) g[i][j] = i == 0 ? b[j] : (j == 0 ? a[i] : a[i] * b[j]);
+    }
+#pragma unroll
+    for (int q = 0; q < kMono; ++q) {
+      const int ea = kExpDev[q][0], eb = kExpDev[q][1], ec = kExpDev[q][2];
+      acc[0][q] = fma(g[ea][eb], m0[ec], acc[0][q]);  // (a, b, c) = (f1, f2, x1)
+      acc[1][q] = fma(g[ea][ec], m1[eb], acc[1][q]);  // (f1, x1, f2)
+      acc[2][q] = fma(g[eb][ec], m[ea], acc[2][q]);   // (x1, f1, f2)
     }
   }
-  block_sum_to<kMono>(acc, sh, partials + ((size_t)tet * gridDim.x + blockIdx.x) * kMono);
+  // block totals of the 60 sums, 30 at a time (as block_sum_to)
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    double w[30];
+#pragma unroll
+    for (int q = 0; q < 30; ++q) w[q] = acc[(30 * h + q) / kMono][(30 * h + q) % kMono];
+    sh[h][threadIdx.x] = warp_transpose_sum<30>(w);
+  }
+  __syncthreads();
+  for (int q = threadIdx.x; q < 60; q += blockDim.x) {
+    const int warps = blockDim.x >> 5, h = q / 30;
+    double t = 0.0;
+    for (int w = 0; w < warps; ++w) t += sh[h][w * 32 + q - 30 * h];
+    const int tet = 6 * cell + kPhaseTet[o][q / kMono];
+    partials[((size_t)tet * gridDim.x + blockIdx.x) * kMono + q % kMono] = t;
+  }
 }
 
 // Boundary classes: block (class - 1, tet, instance).
 //  * faces (F0..F3): two free chain coordinates p > q; a thread takes a row (fixed p) and
-//    walks q, summing u (q/r)^e, e = 0..3, then adds the row's 20 monomial sums (each
+//    walks q (a fixed stride per class), summing u (q/r)^e, e = 0..3, then adds the row's 20 monomial sums (each
 //    monomial is a power of p/r times a power of q/r on a face);
 //  * edges: one free coordinate, a thread per node; vertices: one node.
 // Chain coordinates (a, b, c) of each class as functions of the free ones p > q > 0 (r fine
 // cells per coarse cell): faces F0 (r, p, q), F1 (p, p, q), F2 (p, q, q), F3 (p, q, 0); edges
 // E01 (r, r, p), E02 (r, p, p), E03 (r, p, 0), E12 (p, p, p), E13 (p, p, 0), E23 (p, 0, 0);
 // vertices (0,0,0), (r,0,0), (r,r,0), (r,r,r).
-__device__ __forceinline__ double pw3(double v, int e) {
-  return e == 0 ? 1.0 : (e == 1 ? v : (e == 2 ? v * v : v * v * v));
-}
-
 __global__ void __launch_bounds__(kThreads)
     k_t3_boundary3d(int pf, long planef, int n1, int r, size_t st, size_t pst,
-                    const double* __restrict__ u, double* __restrict__ partials) {
+                    const double* __restrict__ u, const double* __restrict__ pw,
+                    double* __restrict__ partials) {
   __shared__ double sh[kThreads];
   u += blockIdx.z * st;  // instance blockIdx.z
   partials += blockIdx.z * pst;
@@ -154,40 +177,43 @@ __global__ void __launch_bounds__(kThreads)
   const int tet = blockIdx.y;
   const int cell = tet / 6, s = tet % 6;
   const int I = cell % n1, J = (cell / n1) % n1, L = cell / (n1 * n1);
-  const double inv_r = 1.0 / r;
   const double* base = u + (size_t)(L * r) * planef + (size_t)(J * r) * pf + (size_t)I * r;
-  auto node = [&](int a, int b, int c) {
-    int co[3];
-    co[kPermDev[s][0]] = a;
-    co[kPermDev[s][1]] = b;
-    co[kPermDev[s][2]] = c;
-    return base[(size_t)co[2] * planef + (size_t)co[1] * pf + co[0]];
+  // element strides of the chain coordinates (a, b, c)
+  auto stride = [&](int q) {
+    const int axis = kPermDev[s][q];
+    return axis == 0 ? 1l : (axis == 1 ? (long)pf : planef);
   };
+  const long sa = stride(0), sb = stride(1), sc = stride(2);
   double acc[kMono];
 #pragma unroll
   for (int m = 0; m < kMono; ++m) acc[m] = 0.0;
   if (cls <= 4) {
     // face rows: p = 2 .. r - 1 (F0..F2) with q in (0, p), F0 with p < r; F3: a = p, b = q
     for (int p = 2 + threadIdx.x; p < r; p += blockDim.x) {
+      // the row's first element and the stride of q, then u (q/r)^e over 0 < q < p, eight
+      // loads in flight
+      const double* row = base + (cls == 1 ? r * sa + p * sb : cls == 2 ? p * (sa + sb) : p * sa);
+      const long sq = cls <= 2 ? sc : cls == 3 ? sb + sc : sb;
       double m0 = 0.0, m1 = 0.0, m2 = 0.0, m3 = 0.0;
-      for (int q = 1; q < p; ++q) {
-        double v;
-        switch (cls) {
-          case 1: v = node(r, p, q); break;
-          case 2: v = node(p, p, q); break;
-          case 3: v = node(p, q, q); break;
-          default: v = node(p, q, 0); break;
-        }
-        const double t = q * inv_r, t2 = t * t;
-        m0 += v;
-        m1 = fma(v, t, m1);
-        m2 = fma(v, t2, m2);
-        m3 = fma(v, t2 * t, m3);
+      constexpr int kAhead = 8;
+      for (int q0 = 1; q0 < p; q0 += kAhead) {
+        double v[kAhead];
+#pragma unroll
+        for (int j = 0; j < kAhead; ++j) v[j] = q0 + j < p ? row[(q0 + j) * sq] : 0.0;
+#pragma unroll
+        for (int j = 0; j < kAhead; ++j)
+          if (q0 + j < p) {
+            const double* t = pw + 4 * (q0 + j);
+            m0 += v[j];
+            m1 = fma(v[j], t[1], m1);
+            m2 = fma(v[j], t[2], m2);
+            m3 = fma(v[j], t[3], m3);
+          }
       }
-      const double g = p * inv_r;
+      const double* g = pw + 4 * p;
 #pragma unroll
       for (int k = 0; k < kMono; ++k) {
-        const int ea = kMonoExpDev[k][0], eb = kMonoExpDev[k][1], ec = kMonoExpDev[k][2];
+        const int ea = kExpDev[k][0], eb = kExpDev[k][1], ec = kExpDev[k][2];
         int ep, eq;  // exponents of p / r and q / r of a^ea b^eb c^ec on the face
         bool zero = false;
         switch (cls) {
@@ -197,7 +223,7 @@ __global__ void __launch_bounds__(kThreads)
           default: ep = ea; eq = eb; zero = ec > 0; break;  // (p, q, 0)
         }
         if (!zero && ep <= 3 && eq <= 3)
-          acc[k] = fma(pw3(g, ep), pick4(m0, m1, m2, m3, eq), acc[k]);
+          acc[k] = fma(g[ep], pick4(m0, m1, m2, m3, eq), acc[k]);
       }
     }
   } else {
@@ -218,9 +244,9 @@ __global__ void __launch_bounds__(kThreads)
         case 13: abc[0] = r; abc[1] = r; abc[2] = 0; break;  // V2
         default: abc[0] = r; abc[1] = r; abc[2] = r; break;  // V3
       }
-      const double val = node(abc[0], abc[1], abc[2]);
+      const double val = base[abc[0] * sa + abc[1] * sb + abc[2] * sc];
       double m[kMono];
-      monomials(abc[0] * inv_r, abc[1] * inv_r, abc[2] * inv_r, m);
+      monomials(pw[4 * abc[0] + 1], pw[4 * abc[1] + 1], pw[4 * abc[2] + 1], m);
 #pragma unroll
       for (int k = 0; k < kMono; ++k) acc[k] = fma(val, m[k], acc[k]);
     }
@@ -245,23 +271,25 @@ __global__ void k_t3_finalize3d(int chunks, double h3, size_t pst, size_t tst,
   for (int e = threadIdx.x; e < (kClasses - 1) * kMono; e += blockDim.x)
     S[kMono + e] = pbd[(size_t)tet * (kClasses - 1) * kMono + e];
   __syncthreads();
-  const int e = threadIdx.x;
-  if (e >= 20) return;
+  // eight lanes per entry, each every eighth term (a lane per entry was one chain of 300)
+  const int e = threadIdx.x >> 3, part = threadIdx.x & 7;
   const double* row = map + (size_t)e * kClasses * kMono;
   double acc = 0.0;
-  for (int q = 0; q < kClasses * kMono; ++q) acc = fma(row[q], S[q], acc);
-  t3[(size_t)tet * 20 + e] = h3 * acc;
+#pragma unroll 4
+  for (int q = part; q < kClasses * kMono; q += 8) acc = fma(row[q], S[q], acc);
+  for (int o = 4; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+  if (part == 0) t3[(size_t)tet * 20 + e] = h3 * acc;
 }
 
-// Interior: a block takes interior_threads(r) lines (whole warps, up to kThreads) of the
-// (r + 1)^2 lines of a tetrahedron.  Boundary: the face rows and edge nodes of a class number
-// fewer than r, so a block of boundary_threads(r) covers them in one or a few passes.
-int interior_threads(int r) { return warps_for((long)(r + 1) * (r + 1), kThreads); }
-constexpr int kLinesPerThread = 8;  // lines summed per thread before the block reduction
+// Interior: a block takes kLinesPerThread lines per thread (whole warps, up to kLineThreads)
+// of the (r - 1)(r - 2) / 2 lines of a cell with x0 < x2 (or x0 > x2).  Boundary: the face rows
+// and edge nodes of a class number fewer than r, so a block of boundary_threads(r) covers them
+// in one or a few passes.
+int interior_threads(int r) { return warps_for((long)(r - 1) * (r - 2) / 2, kLineThreads); }
 int interior_chunks(int r) {
-  const long rows = (long)(r + 1) * (r + 1);
+  const long lines = (long)(r - 1) * (r - 2) / 2;
   const long per_block = (long)interior_threads(r) * kLinesPerThread;
-  return (int)((rows + per_block - 1) / per_block);
+  return std::max(1, (int)((lines + per_block - 1) / per_block));
 }
 int boundary_threads(int r) { return warps_for(r, kThreads); }
 
@@ -387,11 +415,11 @@ void t3_moments3d(const Grid& fine, int n1, const double* u, const double* pw,
   const size_t pst = t3_partials3d(fine, n1);  // per instance
   double* pin = partials;
   double* pbd = partials + (size_t)tets * chunks * kMono;
-  k_t3_interior3d<<<dim3(chunks, tets, fine.nb), interior_threads(r), 0, s>>>(
+  k_t3_interior3d<<<dim3(chunks, tets / 3, fine.nb), interior_threads(r), 0, s>>>(
       fine.pitch, planef, n1, r, fine.stride, pst, u, pw, pin);
   k_t3_boundary3d<<<dim3(kClasses - 1, tets, fine.nb), boundary_threads(r), 0, s>>>(
-      fine.pitch, planef, n1, r, fine.stride, pst, u, pbd);
-  k_t3_finalize3d<<<dim3(tets, fine.nb), 32, 0, s>>>(chunks, fine.h * fine.h * fine.h, pst,
+      fine.pitch, planef, n1, r, fine.stride, pst, u, pw, pbd);
+  k_t3_finalize3d<<<dim3(tets, fine.nb), 160, 0, s>>>(chunks, fine.h * fine.h * fine.h, pst,
                                                      (size_t)tets * 20, pin, pbd, map, t3);
 }
 

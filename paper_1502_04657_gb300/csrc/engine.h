@@ -98,6 +98,10 @@ struct fmg_eig_handle {
   int* tri = nullptr;
   uint16_t* lists = nullptr;  // sparsity lists of the small dense solves (dense_lists.h)
   fmg::DenseLists dims;
+  // The first npinned instances (the ones with the most levels) are 3D mixed-precision solves
+  // with single-precision V-cycles, whose small solves and third moments keep their rounding.
+  int npinned = 0;
+  fmg::PinnedTables pinned;
   double *lam = nullptr, *c = nullptr, *cstart = nullptr, *auu = nullptr, *buu = nullptr,
          *partials = nullptr, *partials2 = nullptr, *t3 = nullptr, *t3_partials = nullptr, *gAd = nullptr,
          *gMd = nullptr, *t1d = nullptr, *B1d = nullptr, *t0 = nullptr,

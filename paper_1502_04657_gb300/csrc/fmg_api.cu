@@ -142,9 +142,21 @@ void lv_coarsen_density(Level& fl, Level& cl, cudaStream_t s, bool split) {
   if (fl.g.dim == 2) coarsen_density2d(fl.g, cl.g, fl.b, cl.b, s, split);
   else coarsen_density3d(fl.g, cl.g, fl.b3, cl.b3, s, split);
 }
-void lv_t3(Level& l, int n1, const double* u, double* partials, double* t3, cudaStream_t s) {
-  if (l.g.dim == 2) t3_moments2d(l.g, n1, u, l.pw, l.t3map, partials, t3, s);
-  else t3_moments3d(l.g, n1, u, l.pw, l.t3map, partials, t3, s);
+// npinned: the leading instances that keep the pinned order of summation (3D)
+void lv_t3(Level& l, int n1, int npinned, const double* u, double* partials, double* t3,
+           cudaStream_t s) {
+  if (l.g.dim == 2) {
+    t3_moments2d(l.g, n1, u, l.pw, l.t3map, partials, t3, s);
+    return;
+  }
+  Grid g = l.g;
+  const int np = std::min(npinned, g.nb), rest = g.nb - np;
+  g.nb = np;
+  if (np) t3_moments3d_pinned(g, n1, u, l.pw, l.t3map, partials, t3, s);
+  g.nb = rest;
+  if (rest)
+    t3_moments3d(g, n1, u + np * g.stride, l.pw, l.t3map,
+                 partials + np * t3_partials3d_pinned(g, n1), t3 + (size_t)np * 120 * n1 * n1 * n1, s);
 }
 void lv_dense_level1(Level& l1, double* L, double* M, cudaStream_t s, bool full) {
   if (l1.g.dim == 2) dense_level1_2d(l1.g, full ? l1.cw : l1.c, L, M, s);
@@ -382,6 +394,45 @@ void build_levels(fmg_eig_handle* h) {
   }
 }
 
+// Adjacency and gather lists of the pinned small solves (PinnedTables).
+void build_pinned_tables(fmg_eig_handle* h, const std::vector<int>& tri) {
+  const int nv = h->nvert, nh = h->nh, maxadj = h->pinned.maxadj, L = nv + 1;
+  std::vector<int> adj((size_t)nh * maxadj, -1), fill(nh, 0), gent, gstart{0}, gidx;
+  for (int t = 0; t < h->ntri; ++t)
+    for (int v = 0; v < nv; ++v) {
+      const int a = tri[t * nv + v];
+      if (a >= 0) adj[a * maxadj + fill[a]++] = (t << 3) | v;
+    }
+  // for each entry (a, b) with a simplex around a that has b as a vertex, the simplex-local
+  // indices in a's adjacency order
+  for (int a = 0; a < nh; ++a)
+    for (int b = 0; b < nh; ++b) {
+      const size_t before = gidx.size();
+      for (int k = 0; k < maxadj; ++k) {
+        const int code = adj[a * maxadj + k];
+        if (code < 0) break;
+        const int t = code >> 3, la = code & 7;
+        for (int lb = 0; lb < nv; ++lb)
+          if (tri[t * nv + lb] == b) gidx.push_back(t * L * L + la * L + lb);
+      }
+      if (gidx.size() > before) {
+        gent.push_back(a * nh + b);
+        gstart.push_back((int)gidx.size());
+      }
+    }
+  auto upload = [&](const std::vector<int>& v) {
+    int* p = h->alloc<int>(v.size());
+    if (!h->dry)
+      cudaMemcpyAsync(p, v.data(), v.size() * sizeof(int), cudaMemcpyHostToDevice, h->stream);
+    return p;
+  };
+  h->pinned.npat = (int)gent.size();
+  h->pinned.adj = upload(adj);
+  h->pinned.gent = upload(gent);
+  h->pinned.gstart = upload(gstart);
+  h->pinned.gidx = upload(gidx);
+}
+
 void build_coarse(fmg_eig_handle* h) {
   const int n1 = h->prob.coarse_cells;
   const int m = n1 - 1;
@@ -433,6 +484,10 @@ void build_coarse(fmg_eig_handle* h) {
           }
         }
   }
+  // instances whose finest level runs single-precision V-cycles (3D)
+  for (int k = 1; dim == 3 && h->mixed() && k <= h->levels() && !h->npinned; ++k)
+    if (tma_sweep_applies(h->L(k).g)) h->npinned = h->cnt[k];
+  if (h->npinned) build_pinned_tables(h, tri);
   // (a mesh beyond the lists' capacities is beyond dense_smem_bytes' limit too, and refused)
   std::vector<uint16_t> lists(kDenseMaxLists);
   if (!build_dense_lists(h->nh, h->ntri, h->nvert, tri.data(), lists.data(), &h->dims))
@@ -465,7 +520,10 @@ void build_coarse(fmg_eig_handle* h) {
   size_t tp = 1;
   for (int k = 2; k <= h->levels(); ++k) {
     const Grid& g = h->L(k).g;
-    tp = std::max(tp, (dim == 2 ? t3_partials2d(g, n1) : t3_partials3d(g, n1)) * h->cnt[k]);
+    const int np = std::min(h->npinned, h->cnt[k]);
+    tp = std::max(tp, dim == 2 ? t3_partials2d(g, n1) * h->cnt[k]
+                               : t3_partials3d_pinned(g, n1) * np +
+                                     t3_partials3d(g, n1) * (h->cnt[k] - np));
   }
   h->t3_partials = h->alloc<double>(tp);
   h->gAd = h->alloc<double>((size_t)h->nh * nb);
@@ -552,7 +610,11 @@ void enqueue_setup(fmg_eig_handle* h, cudaStream_t s, bool overlap = false) {
   }
   lv_dense_level1(h->L(1), h->L1, h->M1, s, true);
   if (h->literal()) lv_dense_level1(h->L(1), h->L1A, h->M1, s, false);
-  dense_spd_inverse(h->L1A, h->L1inv, h->nh, h->lists, h->dims, h->L(1).g.nb, s);
+  const int np = h->npinned, rest = h->L(1).g.nb - np;  // all instances are active here
+  const size_t nn = (size_t)h->nh * h->nh;
+  if (np) dense_spd_inverse_pinned(h->L1A, h->L1inv, h->nh, np, s);
+  if (rest)
+    dense_spd_inverse(h->L1A + np * nn, h->L1inv + np * nn, h->nh, h->lists, h->dims, rest, s);
 }
 
 DenseProblem dense_base(fmg_eig_handle* h) {
@@ -575,6 +637,35 @@ DenseProblem dense_base(fmg_eig_handle* h) {
   return d;
 }
 
+// The small solves d of the first nb instances: the pinned ones in their form, the others by
+// dense.cu (their arrays start npinned instances further).
+void run_dense(fmg_eig_handle* h, const DenseProblem& d, int nb, cudaStream_t s) {
+  const int np = std::min(h->npinned, nb);
+  if (np) dense_scf_pinned(d, h->pinned, np, s);
+  if (nb == np) return;
+  const size_t nh = d.nh, nn = nh * nh;
+  DenseProblem e = d;
+  e.L1 += np * nn;
+  e.M1 += np * nn;
+  e.params += np;
+  e.c_out += np * (nh + 1);
+  e.lam_out += np;
+  e.iters_out += np;
+  e.status_out += np;
+  if (e.c_init) e.c_init += np * (nh + 1);
+  if (e.aug) {
+    e.gA += np * nh;
+    e.gM += np * nh;
+    e.t1 += np * nh;
+    e.B1 += np * nn;
+    e.t3 += (size_t)np * d.ntri * d.nt3;
+    e.auu += np;
+    e.buu += np;
+    e.t0 += np;
+  }
+  dense_scf(e, nb - np, s);
+}
+
 // Algorithm 3.2 step 1 into L(1).u and h->lam for the active instances
 void enqueue_coarse(fmg_eig_handle* h, cudaStream_t s) {
   Level& l1 = h->L(1);
@@ -584,7 +675,7 @@ void enqueue_coarse(fmg_eig_handle* h, cudaStream_t s) {
   d.c_init = h->cstart;
   d.iters_out = h->iters;
   d.status_out = h->status;
-  dense_scf(d, l1.g.nb, s);
+  run_dense(h, d, l1.g.nb, s);
   scatter_level1(l1.g, h->c, h->nh + 1, l1.u, s);
 }
 
@@ -832,7 +923,7 @@ void enqueue_augment(fmg_eig_handle* h, int k, const double* ut, cudaStream_t s)
   {
     const cudaStream_t b2 = h->side[1];
     prof_begin(h, kProfT3, k, b2);
-    lv_t3(l, h->prob.coarse_cells, ut, h->t3_partials, h->t3, b2);
+    lv_t3(l, h->prob.coarse_cells, h->npinned, ut, h->t3_partials, h->t3, b2);
     prof_end(h, kProfT3, k, b2);
   }
   // main branch: (A + W) u~, M u~, their dots and restriction chains.  The mixed modes form
@@ -888,7 +979,7 @@ void enqueue_correction(fmg_eig_handle* h, int k, cudaStream_t s) {
   d.iters_out = h->iters + (size_t)(k - 1) * h->nb;
   d.status_out = h->status + (size_t)(k - 1) * h->nb;
   prof_begin(h, kProfDense, k, s);
-  dense_scf(d, nb, s);
+  run_dense(h, d, nb, s);
   prof_end(h, kProfDense, k, s);
   // u = P_{k<-1} c_H + c_u u~
   scatter_level1(h->L(1).g, h->c, h->nh + 1, h->L(1).y, s);
@@ -1140,7 +1231,8 @@ int create_handle(const fmg_eig_problem* probs, int count, const CreateOptions& 
     delete h;
     return FMG_ENOTSUP;
   }
-  if (dense_prepare(h->dense_smem) != cudaSuccess) {
+  if (dense_prepare(h->dense_smem) != cudaSuccess ||
+      (h->npinned && dense_prepare_pinned() != cudaSuccess)) {
     cudaGetLastError();
     delete h;
     return FMG_ECUDA;

@@ -346,6 +346,21 @@ constexpr size_t kDenseSmemLimit = 200 * 1024;  // dynamic shared memory of the 
 size_t dense_smem_bytes(int n, int ntri, int nvert, int aug);
 cudaError_t dense_prepare(size_t max_smem);  // opt in to large dynamic shared memory
 void dense_scf(const DenseProblem& p, int nb, cudaStream_t s);  // one CTA per problem
+// The form of the small solves and of the third moments that 3D mixed-precision solves with
+// single-precision V-cycles keep, bit for bit (dense_pinned.cu, t3_pinned3d.cu).  Tables: the
+// adjacency codes (simplex << 3 | local vertex, -1 terminated) adj[nh * maxadj], and gather
+// lists of the coarse block of G(c): the npat structurally nonzero entries gent[q] = a nh + b,
+// and for each the simplex-local indices gidx[gstart[q] .. gstart[q + 1]).
+struct PinnedTables {
+  const int *adj = nullptr, *gent = nullptr, *gstart = nullptr, *gidx = nullptr;
+  int maxadj = 24, npat = 0;
+};
+cudaError_t dense_prepare_pinned();
+void dense_scf_pinned(const DenseProblem& p, const PinnedTables& pt, int nb, cudaStream_t s);
+void dense_spd_inverse_pinned(const double* L, double* Linv, int n, int nb, cudaStream_t s);
+size_t t3_partials3d_pinned(const Grid& fine, int n1);
+void t3_moments3d_pinned(const Grid& fine, int n1, const double* u, const double* pw,
+                         const double* map, double* partials, double* t3, cudaStream_t s);
 // Linv = L^{-1} for the SPD n x n level-1 operators (nonzeros in `lists`), one CTA each.
 void dense_spd_inverse(const double* L, double* Linv, int n, const uint16_t* lists,
                        const DenseLists& dims, int nb, cudaStream_t s);
