@@ -43,7 +43,12 @@ Level view(const Level& l, int first, int count) {
   adv(v.x); adv(v.xt); adv(v.f); adv(v.r); adv(v.u); adv(v.y); adv(v.z);
   adv(v.b.C); adv(v.b.E); adv(v.b.N); adv(v.b.NE);
   adv(v.x32); adv(v.xt32); adv(v.f32); adv(v.r32); adv(v.uhi); adv(v.ulo);
-  v.c.tab = v.c3.tab = v.cw.tab = v.cw3.tab = nullptr;  // per-instance tables are not sliced
+  v.c.tab = v.c3.tab = v.cw.tab = v.cw3.tab = nullptr;  // setup scratch is not sliced
+  for (Coef2D* c : {&v.c, &v.cw})
+    if (c->fxt) {
+      c->fxt += (size_t)first * 4 * (l.g.n + 1);
+      c->fxh += first;
+    }
   v.ct = CoefT{};
   v.g.nb = count;
   return v;
@@ -319,8 +324,16 @@ void build_levels(fmg_eig_handle* h) {
       l.b.E = h->alloc<double>(s);
       l.b.N = h->alloc<double>(s);
       l.b.NE = h->alloc<double>(s);
+      if (fxop2d_applies(l.g)) {
+        l.c.fxt = h->alloc<long long>(4 * (size_t)(l.g.n + 1) * l.cap);
+        l.c.fxh = h->alloc<FxHead2D>(l.cap);
+      }
       l.cw = l.c;
       if (h->literal()) {
+        if (fxop2d_applies(l.g)) {
+          l.cw.fxt = h->alloc<long long>(4 * (size_t)(l.g.n + 1) * l.cap);
+          l.cw.fxh = h->alloc<FxHead2D>(l.cap);
+        }
         l.cw.cC = h->alloc<double>(s);
         l.cw.cE = h->alloc<double>(s);
         l.cw.cN = h->alloc<double>(s);

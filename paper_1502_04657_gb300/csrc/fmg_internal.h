@@ -46,6 +46,13 @@ struct SplitVec {
   const float* lo;
 };
 
+// Fixed-point form of the 2D operator (fxop2d.cu), per instance: whether its formats hold the
+// potential, the shifts of the product sum and of the small terms, and their coefficients.
+struct PotentialParams;
+struct FxHead2D {
+  int ok, sa, sm, P, Q, R, S, pad;
+};
+
 // Stencil coefficients of L = A + W on one 2D level (see grid2d.cu for the closed forms).
 struct Coef2D {
   double* cC;    // diagonal
@@ -54,7 +61,24 @@ struct Coef2D {
   double* cNE;   // coupling (i,j)-(i+1,j+1)
   double* dinv;  // omega / cC
   double* tab;   // 8 * (n + 1) separable parts of the coefficients (setup scratch)
+  // levels of the fixed-point form only: 4 (n + 1) table entries and a header per instance
+  long long* fxt;
+  FxHead2D* fxh;
 };
+
+// Levels whose operator runs in fixed point (fxop2d.cu): from 512 cells per side on a sweep is
+// bound by the FP64 pipe (262k nodes: 3.3 us of it); below, by launch latency.  The choice
+// depends on n alone, so an instance of a batch takes the same form as alone.
+inline bool fxop2d_applies(const Grid& g) { return g.dim == 2 && g.n >= 512; }
+void fxop2d_tables(const Grid& g, const PotentialParams* p, const Coef2D& c, cudaStream_t s);
+void fxop2d_apply(const Grid& g, const Coef2D& c, const double* x, double* y, cudaStream_t s);
+void fxop2d_jacobi(const Grid& g, const Coef2D& c, const double* f, const double* x, double* xo,
+                   cudaStream_t s);
+void fxop2d_residual(const Grid& g, const Coef2D& c, const double* f, const double* x, double* r,
+                     cudaStream_t s);
+// the residual rounded to single precision (float, or bfloat16 behind the float pointer)
+void fxop2d_residual32(const Grid& g, const Coef2D& c, const double* f, const double* x, float* r,
+                       bool bf, cudaStream_t s);
 
 // Problem parameters that may change between solves of one handle.  They live in device
 // memory (uploaded at the start of every solve), so kernels take a device pointer to them.

@@ -1,0 +1,274 @@
+// The 2D level operator L = A + W on the large levels in 64-bit fixed point: damped Jacobi,
+// residual (FP64, or rounded to single precision for the mixed modes) and operator apply.
+//
+// The FP64 kernels (grid2d.cu) need 7 to 8 FP64 operations per node, 4 clocks of an SM's FP64
+// pipe (2 lanes per clock), and read the four stored coupling arrays.  Here a warp covers a
+// tile of 64 columns (62 produced, two per lane) x 8 rows (and one more on each side), takes
+// one exponent e for its x and f, and computes the stencil in integers in units of 2^(e - 58):
+//   - the stiffness 4x - E - W - N - S exactly (integer additions);
+//   - the potential's part from closed forms instead of stored couplings.  With node (i, j),
+//     the six neighbours and the P1 integrals at the head of grid2d.cu,
+//       W x = a (6x + sum of the six) + bx Dx + by Dy + small,
+//       a  = h^2 W(x_i, y_j) / 12,   bx = h^4 wx i / 12,   by = h^4 wy j / 12,
+//       Dx = (E - W) + (NE - SW),    Dy = (N - S) + (NE - SW),
+//       small = h^4 [ (wx + wy) x / 18 + (wx/40 + wy/180) (E + W) + (wx/180 + wy/40) (N + S)
+//                     + (wx + wy) (NE + SW) / 40 ],
+//     with a = ax[i] + ay[j], bx[i], by[j] from 1D tables, scaled by 2^(61 + sa) so that they
+//     fill the integers, and the small terms (h^2 below the others) from the high words.
+// Only the products, x and f round, at 2^-58 of the tile's maximum or below (FP64 rounds each
+// of its operations at 2^-53, and each stored coupling -1 + O(h^2) at 2^-53: a relative
+// perturbation of W by 2^-53 / h^2, 4e-9 at h = 1/4096, that this form does not have).
+// The update x + (omega / D) r is one FP64 operation as before.
+//
+// Tiles with infinities, NaN, all zeros or an exponent outside +-kFxMaxExp, and instances
+// whose potential is too large for the fixed formats (h^2 |W| > 12/64 or h^4 (|wx| + |wy|) >
+// 2^-28), run the FP64 expressions of grid2d.cu.
+#include <cuda_bf16.h>
+
+#include "dfloat.cuh"
+#include "fixed.cuh"
+#include "fmg_internal.h"
+
+namespace fmg {
+namespace {
+
+constexpr int kB = 58;         // x = I 2^(e - kB)
+constexpr int kRows = 8;       // rows a warp produces
+constexpr int kWarps = 4;      // warps of a block, stacked in y
+constexpr int kCols = 62;      // columns a warp produces
+
+// Tables ax, ay, bx, by (n + 1 entries each) and the header of each instance.
+__global__ void k_fxop2d_tables(int n, double h, const PotentialParams* __restrict__ pp,
+                                long long* __restrict__ tab, FxHead2D* __restrict__ head) {
+  const int x = blockIdx.x * blockDim.x + threadIdx.x;
+  if (x > n) return;
+  const PotentialParams p = pp[blockIdx.y];
+  tab += (size_t)blockIdx.y * 4 * (n + 1);
+  const double wl = p.operator_form == FMG_W_LEFT ? 1.0 : 0.0;
+  const double h2 = h * h, h4 = h2 * h2, L = n * h;
+  const double w0 = wl * p.w0, wx = wl * p.wx, wy = wl * p.wy;
+  const double amax = h2 / 12.0 * (fabs(w0) + (fabs(wx) + fabs(wy)) * L * L);
+  const double pmax = h4 * (fabs(wx) + fabs(wy));  // bounds the four small coefficients
+  // amax < 2^-sa, pmax < 2^-ss
+  const int sa = amax > 0.0 ? max(0, min(40, -(ilogb(amax) + 1))) : 40;
+  const int ss = pmax > 0.0 ? max(0, min(90, -(ilogb(pmax) + 1))) : 90;
+  const double s = ldexp(1.0, 61 + sa), d = x;
+  tab[x] = __double2ll_rn(s * (h2 * w0 / 12.0 + h4 * wx * d * d / 12.0));
+  tab[(n + 1) + x] = __double2ll_rn(s * (h4 * wy * d * d / 12.0));
+  tab[2 * (n + 1) + x] = __double2ll_rn(s * (h4 * wx * d / 12.0));
+  tab[3 * (n + 1) + x] = __double2ll_rn(s * (h4 * wy * d / 12.0));
+  if (x == 0) {
+    FxHead2D q;
+    q.ok = amax <= 1.0 / 64.0 && pmax <= 3.7252902984619141e-09 && ss - sa + 1 >= 0;
+    q.sa = sa - 3;       // shift of the products' sum
+    q.sm = min(63, ss - sa + 1);  // shift of the small terms to the products' units
+    const double t = ldexp(h4, 30 + ss);
+    q.P = (int)__double2ll_rn(t * (wx + wy) / 18.0);
+    q.Q = (int)__double2ll_rn(t * (wx / 40.0 + wy / 180.0));
+    q.R = (int)__double2ll_rn(t * (wx / 180.0 + wy / 40.0));
+    q.S = (int)__double2ll_rn(t * (wx + wy) / 40.0);
+    head[blockIdx.y] = q;
+  }
+}
+
+// high word of a 64 x 64 product (|a|, |b| < 2^62), within a unit and a half
+__device__ __forceinline__ long long mul_hi(long long a, long long b) {
+  const int al = (int)a, bl = (int)b;
+  const int ah = (int)(a >> 32) + (int)((uint32_t)al >> 31);
+  const int bh = (int)(b >> 32) + (int)((uint32_t)bl >> 31);
+  return (long long)ah * bh + (((long long)al * bh + (long long)ah * bl) >> 32);
+}
+
+// v 2^(kB - e) as an integer (truncated), |v| <= 2^e, on the integer pipes (a conversion
+// occupies the FP64 pipe like an FP64 operation)
+__device__ __forceinline__ long long to_fixed(double v, int shift) {  // shift = e + 1022 + 5
+  const int hi = __double2hiint(v);
+  const int ex = (hi >> 20) & 0x7ff;
+  const unsigned long long m =
+      ((unsigned long long)(((uint32_t)hi & 0xfffffu) | 0x100000u) << 32 |
+       (uint32_t)__double2loint(v)) << 10;
+  const int sh = min(shift - ex, 63);
+  const long long t = (long long)(m >> sh), sg = hi >> 31;
+  return (t ^ sg) - sg;
+}
+
+enum Mode { kJacobiMode, kResidualMode, kApplyMode };
+
+__device__ __forceinline__ void store(double* o, size_t k, double v) { o[k] = v; }
+__device__ __forceinline__ void store(float* o, size_t k, double v) { o[k] = d2f_rn(v); }
+__device__ __forceinline__ void store(__nv_bfloat16* o, size_t k, double v) {
+  o[k] = __float2bfloat16(d2f_rn(v));
+}
+
+// The tile in FP64, with the expressions of grid2d.cu / mixed.cu.
+template <int MODE, typename S>
+__device__ __noinline__ void tile_fp64(int n, int pitch, size_t base, int i0, int j0,
+                                       const Coef2D& c, const double* __restrict__ f,
+                                       const double* __restrict__ x, S* __restrict__ out) {
+  for (int j = j0; j < min(j0 + kRows, n); ++j)
+    for (int q = 0; q < 2; ++q) {
+      const int i = i0 + q, lane = threadIdx.x;
+      if (i < 1 || i > n - 1 || (lane == 0 && q == 0) || (lane == 31 && q == 1)) continue;
+      const size_t k = base + (size_t)j * pitch + i;
+      double r;
+      if (MODE == kApplyMode) {
+        r = c.cC[k] * x[k];
+        r = fma(c.cE[k], x[k + 1], r);
+        r = fma(c.cE[k - 1], x[k - 1], r);
+        r = fma(c.cN[k], x[k + pitch], r);
+        r = fma(c.cN[k - pitch], x[k - pitch], r);
+        r = fma(c.cNE[k], x[k + pitch + 1], r);
+        r = fma(c.cNE[k - pitch - 1], x[k - pitch - 1], r);
+      } else {
+        r = fma(-c.cC[k], x[k], f[k]);
+        r = fma(-c.cE[k], x[k + 1], r);
+        r = fma(-c.cE[k - 1], x[k - 1], r);
+        r = fma(-c.cN[k], x[k + pitch], r);
+        r = fma(-c.cN[k - pitch], x[k - pitch], r);
+        r = fma(-c.cNE[k], x[k + pitch + 1], r);
+        r = fma(-c.cNE[k - pitch - 1], x[k - pitch - 1], r);
+        if (MODE == kJacobiMode) r = fma(c.dinv[k], r, x[k]);
+      }
+      store(out, k, r);
+    }
+}
+
+template <int MODE, typename S>
+__global__ void __launch_bounds__(32 * kWarps, 4)
+    k_fxop2d(int n, int pitch, size_t st, const __grid_constant__ Coef2D c,
+             const double* __restrict__ f, const double* __restrict__ x, S* __restrict__ out) {
+  const int lane = threadIdx.x, ib = blockIdx.z;
+  const int i0 = kCols * blockIdx.x + 2 * lane;  // this lane's columns i0, i0 + 1
+  const int j0 = 1 + kRows * (blockIdx.y * kWarps + threadIdx.y);
+  if (j0 >= n) return;  // uniform over the warp
+  const size_t base = ib * st;
+  const bool in = i0 <= n;  // (i0 + 1 <= n + 1 < pitch then)
+  const double2 zero = make_double2(0.0, 0.0);
+  double2 xv[kRows + 2], fv[kRows];
+#pragma unroll
+  for (int t = 0; t < kRows + 2; ++t) {
+    const int r = j0 - 1 + t;
+    xv[t] = in && r <= n ? *reinterpret_cast<const double2*>(x + base + (size_t)r * pitch + i0) : zero;
+  }
+#pragma unroll
+  for (int t = 0; t < kRows; ++t) {
+    const int r = j0 + t;
+    fv[t] = MODE != kApplyMode && in && r < n
+                ? *reinterpret_cast<const double2*>(f + base + (size_t)r * pitch + i0) : zero;
+  }
+  const FxHead2D hd = c.fxh[ib];
+  // the tile's exponent: f counts an eighth (|f| <= 8 2^e fits beside the stencil of x)
+  int top = 0, topf = 0;
+#pragma unroll
+  for (int t = 0; t < kRows + 2; ++t)
+    top = max(top, max(__double2hiint(xv[t].x) & 0x7fffffff, __double2hiint(xv[t].y) & 0x7fffffff));
+  if (MODE != kApplyMode) {
+#pragma unroll
+    for (int t = 0; t < kRows; ++t)
+      topf = max(topf, max(__double2hiint(fv[t].x) & 0x7fffffff, __double2hiint(fv[t].y) & 0x7fffffff));
+    top = max(top, topf - (3 << 20));
+  }
+  top = __reduce_max_sync(0xffffffffu, top);
+  const int e = ((top + 1) >> 20) - 1022;
+  if (!hd.ok || e < -kFxMaxExp || e > kFxMaxExp) {
+    tile_fp64<MODE, S>(n, pitch, base, i0, j0, c, f, x, out);
+    return;
+  }
+  const int shift = e + 1022 + 5;
+  const double back = fx_pow2(e - kB);
+  const long long* tab = c.fxt + (size_t)ib * 4 * (n + 1);
+  const int ia = min(i0, n), ic = min(i0 + 1, n);
+  const long long axa = tab[ia], axb = tab[ic], bxa = tab[2 * (n + 1) + ia],
+                  bxb = tab[2 * (n + 1) + ic];
+  const long long half = 1ll << (hd.sa - 1);
+  // a row: this lane's pair (a, b), the left neighbour of a and the right one of b
+  struct Row {
+    long long l, a, b, r;
+  };
+  auto row = [&](const double2& v) {
+    Row q;
+    q.a = to_fixed(v.x, shift);
+    q.b = to_fixed(v.y, shift);
+    q.l = __shfl_up_sync(0xffffffffu, q.b, 1);
+    q.r = __shfl_down_sync(0xffffffffu, q.a, 1);
+    return q;
+  };
+  // one node: (A + W) x in units of 2^(e - kB)
+  auto node = [&](long long x0, long long xe, long long xw, long long xn, long long xs,
+                  long long xne, long long xsw, long long a, long long bx, long long by) {
+    const long long ew = xe + xw, ns = xn + xs, d = xne + xsw, g = xne - xsw;
+    const long long t = ew + ns;
+    const long long s6 = 6 * x0 + t + d;
+    long long sm = (long long)hd.P * (int)(x0 >> 32) + (long long)hd.Q * (int)(ew >> 32) +
+                   (long long)hd.R * (int)(ns >> 32) + (long long)hd.S * (int)(d >> 32);
+    long long w = mul_hi(a, s6) + mul_hi(bx, (xe - xw) + g) + mul_hi(by, (xn - xs) + g);
+    w += (sm >> hd.sm) + half;
+    return 4 * x0 - t + (w >> hd.sa);
+  };
+  Row s = row(xv[0]), m = row(xv[1]);
+#pragma unroll
+  for (int t = 0; t < kRows; ++t) {
+    const int j = j0 + t;
+    const Row p = row(xv[t + 2]);
+    if (j < n) {
+      const long long ay = tab[(n + 1) + j], by = tab[3 * (n + 1) + j];
+      long long ra = node(m.a, m.b, m.l, p.a, s.a, p.b, s.l, axa + ay, bxa, by);
+      long long rb = node(m.b, m.r, m.a, p.b, s.b, p.r, s.a, axb + ay, bxb, by);
+      if (MODE != kApplyMode) {
+        ra = to_fixed(fv[t].x, shift) - ra;
+        rb = to_fixed(fv[t].y, shift) - rb;
+      }
+      const size_t k = base + (size_t)j * pitch + i0;
+      const bool oka = lane > 0 && i0 <= n - 1, okb = lane < 31 && i0 + 1 <= n - 1;
+      double va = __ll2double_rn(ra), vb = __ll2double_rn(rb);
+      if (MODE == kJacobiMode) {
+        const double2 di = in ? *reinterpret_cast<const double2*>(c.dinv + k) : zero;
+        va = fma(di.x * back, va, xv[t + 1].x);
+        vb = fma(di.y * back, vb, xv[t + 1].y);
+      } else {
+        va *= back;
+        vb *= back;
+      }
+      if (sizeof(S) == 8 && oka && okb) {
+        *reinterpret_cast<double2*>(reinterpret_cast<double*>(out) + k) = make_double2(va, vb);
+      } else {
+        if (oka) store(out, k, va);
+        if (okb) store(out, k + 1, vb);
+      }
+    }
+    s = m;
+    m = p;
+  }
+}
+
+template <int MODE, typename S>
+void launch(const Grid& g, const Coef2D& c, const double* f, const double* x, S* out,
+            cudaStream_t s) {
+  const dim3 grid((g.n - 1 + kCols - 1) / kCols,
+                  (g.n - 1 + kRows * kWarps - 1) / (kRows * kWarps), g.nb);
+  k_fxop2d<MODE, S><<<grid, dim3(32, kWarps), 0, s>>>(g.n, g.pitch, g.stride, c, f, x, out);
+}
+
+}  // namespace
+
+void fxop2d_tables(const Grid& g, const PotentialParams* p, const Coef2D& c, cudaStream_t s) {
+  k_fxop2d_tables<<<dim3((g.n + 1 + 127) / 128, g.nb), 128, 0, s>>>(g.n, g.h, p, c.fxt, c.fxh);
+}
+void fxop2d_apply(const Grid& g, const Coef2D& c, const double* x, double* y, cudaStream_t s) {
+  launch<kApplyMode>(g, c, nullptr, x, y, s);
+}
+void fxop2d_jacobi(const Grid& g, const Coef2D& c, const double* f, const double* x, double* xo,
+                   cudaStream_t s) {
+  launch<kJacobiMode>(g, c, f, x, xo, s);
+}
+void fxop2d_residual(const Grid& g, const Coef2D& c, const double* f, const double* x, double* r,
+                     cudaStream_t s) {
+  launch<kResidualMode>(g, c, f, x, r, s);
+}
+void fxop2d_residual32(const Grid& g, const Coef2D& c, const double* f, const double* x, float* r,
+                       bool bf, cudaStream_t s) {
+  if (bf) launch<kResidualMode>(g, c, f, x, reinterpret_cast<__nv_bfloat16*>(r), s);
+  else launch<kResidualMode>(g, c, f, x, r, s);
+}
+
+}  // namespace fmg

@@ -452,9 +452,14 @@ void coef2d_setup(const Grid& g, const PotentialParams* p, const Coef2D& c, cuda
   k_coef1d<<<dim3((g.n + 1 + 127) / 128, g.nb), 128, 0, s>>>(g.n, g.h, p, c.tab);
   k_coef2d<<<grid_of(g, g.n + 1, g.n + 1), block_of(g), 0, s>>>(g.n, g.pitch, g.stride, c.tab,
                                                                  p, c);
+  if (c.fxt) fxop2d_tables(g, p, c, s);
 }
 
 void apply2d(const Grid& g, const Coef2D& c, const double* x, double* y, cudaStream_t s) {
+  if (c.fxt) {
+    fxop2d_apply(g, c, x, y, s);
+    return;
+  }
   k_apply2d<<<grid_of(g, g.n - 1, g.n - 1), block_of(g), 0, s>>>(g.n, g.pitch, g.stride, c, x,
                                                                   y);
 }
@@ -477,6 +482,10 @@ void mass2d_df(const Grid& g, SplitVec x, double* y, cudaStream_t s) {
 
 void jacobi2d(const Grid& g, const Coef2D& c, const double* f, const double* x, double* xo,
               bool x_is_zero, cudaStream_t s) {
+  if (c.fxt && !x_is_zero) {
+    fxop2d_jacobi(g, c, f, x, xo, s);
+    return;
+  }
   if (x_is_zero)
     k_jacobi2d_zero<<<grid_of(g, g.n - 1, g.n - 1), block_of(g), 0, s>>>(g.n, g.pitch, g.stride,
                                                                           c, f, xo);
@@ -493,6 +502,10 @@ void cheb2d(const Grid& g, const Coef2D& c, const double* f, const double* x, do
 
 void residual2d(const Grid& g, const Coef2D& c, const double* f, const double* x, double* r,
                 cudaStream_t s) {
+  if (c.fxt) {
+    fxop2d_residual(g, c, f, x, r, s);
+    return;
+  }
   k_residual2d<<<grid_of(g, g.n - 1, g.n - 1), block_of(g), 0, s>>>(g.n, g.pitch, g.stride, c,
                                                                      f, x, r);
 }

@@ -611,7 +611,9 @@ void add_f32(const float* e, double* x, size_t n, cudaStream_t s, bool bf) {
 
 void residual_mixed(const Grid& g, const Coef2D& c2, const Coef3D& c3, const double* f,
                     const double* x, float* r, cudaStream_t s, bool bf) {
-  if (g.dim == 2) {
+  if (g.dim == 2 && c2.fxt) {
+    fxop2d_residual32(g, c2, f, x, r, bf, s);
+  } else if (g.dim == 2) {
     if (bf)
       k_residual_mixed2d<bf16><<<grid2(g, g.n - 1, g.n - 1), blk(g), 0, s>>>(g.n, g.pitch, g.stride, c2, f, x, sp<bf16>(r));
     else

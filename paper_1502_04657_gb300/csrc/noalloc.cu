@@ -88,7 +88,7 @@ extern "C" int fmg_eig_coarse_solve_noalloc(const fmg_eig_problem* prob, double*
     off += (doubles + 31) / 32 * 32;  // keep every piece 256-byte aligned
     return p;
   };
-  Coef2D c;
+  Coef2D c{};
   c.cC = take(g.stride);
   c.cE = take(g.stride);
   c.cN = take(g.stride);
