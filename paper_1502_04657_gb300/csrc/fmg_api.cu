@@ -49,6 +49,11 @@ Level view(const Level& l, int first, int count) {
       c->fxt += (size_t)first * 4 * (l.g.n + 1);
       c->fxh += first;
     }
+  for (Coef3D* c : {&v.c3, &v.cw3})
+    if (c->fxt) {
+      c->fxt += (size_t)first * 6 * (l.g.n + 1);
+      c->fxh += first;
+    }
   v.ct = CoefT{};
   v.g.nb = count;
   return v;
@@ -346,8 +351,17 @@ void build_levels(fmg_eig_handle* h) {
       l.c3.dinv = h->alloc<double>(s);
       l.c3.tab = h->alloc<double>(15 * (size_t)(l.g.n + 1) * l.cap);
       for (int q = 0; q < 8; ++q) l.b3.a[q] = h->alloc<double>(s);
+      const bool fx3 = fxop3d_applies(l.g) && !h->mixed();
+      if (fx3) {
+        l.c3.fxt = h->alloc<long long>(6 * (size_t)(l.g.n + 1) * l.cap);
+        l.c3.fxh = h->alloc<FxHead3D>(l.cap);
+      }
       l.cw3 = l.c3;
       if (h->literal()) {
+        if (fx3) {
+          l.cw3.fxt = h->alloc<long long>(6 * (size_t)(l.g.n + 1) * l.cap);
+          l.cw3.fxh = h->alloc<FxHead3D>(l.cap);
+        }
         for (int q = 0; q < 8; ++q) l.cw3.a[q] = h->alloc<double>(s);
         l.cw3.dinv = h->alloc<double>(s);
         l.cw3.tab = h->alloc<double>(15 * (size_t)(l.g.n + 1) * l.cap);

@@ -50,7 +50,7 @@ struct SplitVec {
 // potential, the shifts of the product sum and of the small terms, and their coefficients.
 struct PotentialParams;
 struct FxHead2D {
-  int ok, sa, sm, P, Q, R, S, pad;
+  int ok, sa, sm, P, Q, R;
 };
 
 // Stencil coefficients of L = A + W on one 2D level (see grid2d.cu for the closed forms).
@@ -133,11 +133,28 @@ void start_vector(const Grid& g, double* c, int cstride, cudaStream_t s);
 // ---- 3D level kernels (grid3d.cu) -------------------------------------------------------
 // Couplings of L on the Kuhn mesh: a[0] diagonal, a[1 + d] the coupling of p with p + d for
 // d = X, Y, Z, XY, XZ, YZ, XYZ (the coupling with p - d is a[1 + d] at p - d).
+struct FxHead3D {  // as FxHead2D, for fxop3d.cu
+  int ok, sa, sm, P, A[3], F[3];
+};
 struct Coef3D {
   double* a[8];
   double* dinv;  // omega / diagonal
   double* tab;   // 15 * (n + 1) separable parts (setup scratch)
+  // FP64-mode levels of the fixed-point form only: 6 (n + 1) table entries and a header per
+  // instance
+  long long* fxt;
+  FxHead3D* fxh;
 };
+// Levels whose operator runs in fixed point (fxop3d.cu), FP64 mode only: the mixed modes'
+// single-precision V-cycles amplify the rounding of the FP64 steps around them (see
+// dense_pinned.cu).  Below 96 cells per side the plane walk has too few blocks.
+inline bool fxop3d_applies(const Grid& g) { return g.dim == 3 && g.n >= 96; }
+void fxop3d_tables(const Grid& g, const PotentialParams* p, const Coef3D& c, cudaStream_t s);
+void fxop3d_apply(const Grid& g, const Coef3D& c, const double* x, double* y, cudaStream_t s);
+void fxop3d_jacobi(const Grid& g, const Coef3D& c, const double* f, const double* x, double* xo,
+                   cudaStream_t s);
+void fxop3d_residual(const Grid& g, const Coef3D& c, const double* f, const double* x, double* r,
+                     cudaStream_t s);
 struct Density3D {
   double* a[8];  // same layout as Coef3D::a
 };

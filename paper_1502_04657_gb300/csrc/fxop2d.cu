@@ -3,26 +3,28 @@
 //
 // The FP64 kernels (grid2d.cu) need 7 to 8 FP64 operations per node, 4 clocks of an SM's FP64
 // pipe (2 lanes per clock), and read the four stored coupling arrays.  Here a warp covers a
-// tile of 64 columns (62 produced, two per lane) x 8 rows (and one more on each side), takes
+// tile of 64 columns (62 produced, two per lane) x 4 rows (and one more on each side), takes
 // one exponent e for its x and f, and computes the stencil in integers in units of 2^(e - 58):
 //   - the stiffness 4x - E - W - N - S exactly (integer additions);
 //   - the potential's part from closed forms instead of stored couplings.  With node (i, j),
 //     the six neighbours and the P1 integrals at the head of grid2d.cu,
 //       W x = a (6x + sum of the six) + bx Dx + by Dy + small,
-//       a  = h^2 W(x_i, y_j) / 12,   bx = h^4 wx i / 12,   by = h^4 wy j / 12,
+//       a  = h^2 W(x_i, y_j) / 12 + h^4 (wx + wy) / 40,   bx = h^4 wx i / 12,   by = h^4 wy j / 12,
 //       Dx = (E - W) + (NE - SW),    Dy = (N - S) + (NE - SW),
-//       small = h^4 [ (wx + wy) x / 18 + (wx/40 + wy/180) (E + W) + (wx/180 + wy/40) (N + S)
-//                     + (wx + wy) (NE + SW) / 40 ],
+//       small = -h^4 [ 17/180 (wx + wy) x + 7/360 wy (E + W) + 7/360 wx (N + S) ],
 //     with a = ax[i] + ay[j], bx[i], by[j] from 1D tables, scaled by 2^(61 + sa) so that they
 //     fill the integers, and the small terms (h^2 below the others) from the high words.
 // Only the products, x and f round, at 2^-58 of the tile's maximum or below (FP64 rounds each
 // of its operations at 2^-53, and each stored coupling -1 + O(h^2) at 2^-53: a relative
 // perturbation of W by 2^-53 / h^2, 4e-9 at h = 1/4096, that this form does not have).
-// The update x + (omega / D) r is one FP64 operation as before.
+// The update x + (omega / D) r is one FP64 operation as before.  What is left is the instruction
+// rate (about 200 integer instructions per node) and the latency between a tile's loads and its
+// arithmetic: 4 rows a warp and 5 blocks per SM took 156 us (Jacobi) and 127 us (residual) on
+// 16.8M nodes, 8 rows and 4 blocks 180 and 142; the FP64 form took 225 and 198.
 //
 // Tiles with infinities, NaN, all zeros or an exponent outside +-kFxMaxExp, and instances
 // whose potential is too large for the fixed formats (h^2 |W| > 12/64 or h^4 (|wx| + |wy|) >
-// 2^-28), run the FP64 expressions of grid2d.cu.
+// 2^-22), run the FP64 expressions of grid2d.cu.
 #include <cuda_bf16.h>
 
 #include "dfloat.cuh"
@@ -33,9 +35,10 @@ namespace fmg {
 namespace {
 
 constexpr int kB = 58;         // x = I 2^(e - kB)
-constexpr int kRows = 8;       // rows a warp produces
+constexpr int kRows = 4;       // rows a warp produces
 constexpr int kWarps = 4;      // warps of a block, stacked in y
 constexpr int kCols = 62;      // columns a warp produces
+constexpr int kBlocks = 5;     // resident blocks per SM
 
 // Tables ax, ay, bx, by (n + 1 entries each) and the header of each instance.
 __global__ void k_fxop2d_tables(int n, double h, const PotentialParams* __restrict__ pp,
@@ -47,26 +50,27 @@ __global__ void k_fxop2d_tables(int n, double h, const PotentialParams* __restri
   const double wl = p.operator_form == FMG_W_LEFT ? 1.0 : 0.0;
   const double h2 = h * h, h4 = h2 * h2, L = n * h;
   const double w0 = wl * p.w0, wx = wl * p.wx, wy = wl * p.wy;
-  const double amax = h2 / 12.0 * (fabs(w0) + (fabs(wx) + fabs(wy)) * L * L);
-  const double pmax = h4 * (fabs(wx) + fabs(wy));  // bounds the four small coefficients
+  const double amax = h2 / 12.0 * (fabs(w0) + (fabs(wx) + fabs(wy)) * (L * L + 0.3 * h2));
+  const double pmax = h4 * (fabs(wx) + fabs(wy));  // bounds the small coefficients
   // amax < 2^-sa, pmax < 2^-ss
   const int sa = amax > 0.0 ? max(0, min(40, -(ilogb(amax) + 1))) : 40;
   const int ss = pmax > 0.0 ? max(0, min(90, -(ilogb(pmax) + 1))) : 90;
   const double s = ldexp(1.0, 61 + sa), d = x;
-  tab[x] = __double2ll_rn(s * (h2 * w0 / 12.0 + h4 * wx * d * d / 12.0));
+  tab[x] = __double2ll_rn(s * (h2 * w0 / 12.0 + h4 * (wx + wy) / 40.0 + h4 * wx * d * d / 12.0));
   tab[(n + 1) + x] = __double2ll_rn(s * (h4 * wy * d * d / 12.0));
   tab[2 * (n + 1) + x] = __double2ll_rn(s * (h4 * wx * d / 12.0));
   tab[3 * (n + 1) + x] = __double2ll_rn(s * (h4 * wy * d / 12.0));
   if (x == 0) {
     FxHead2D q;
-    q.ok = amax <= 1.0 / 64.0 && pmax <= 3.7252902984619141e-09 && ss - sa + 1 >= 0;
+    // the small terms are 0.2 pmax of the maximum at most and lose 2^-26 of that: with pmax <=
+    // 2^-22 the loss is below 2^-50, what the FP64 form's roundings at 4x leave
+    q.ok = amax <= 1.0 / 64.0 && pmax <= 1.0 / 4194304.0 && ss - sa + 1 >= 0;
     q.sa = sa - 3;       // shift of the products' sum
     q.sm = min(63, ss - sa + 1);  // shift of the small terms to the products' units
     const double t = ldexp(h4, 30 + ss);
-    q.P = (int)__double2ll_rn(t * (wx + wy) / 18.0);
-    q.Q = (int)__double2ll_rn(t * (wx / 40.0 + wy / 180.0));
-    q.R = (int)__double2ll_rn(t * (wx / 180.0 + wy / 40.0));
-    q.S = (int)__double2ll_rn(t * (wx + wy) / 40.0);
+    q.P = (int)__double2ll_rn(t * (wx + wy) * (-17.0 / 180.0));
+    q.Q = (int)__double2ll_rn(t * wy * (-7.0 / 360.0));
+    q.R = (int)__double2ll_rn(t * wx * (-7.0 / 360.0));
     head[blockIdx.y] = q;
   }
 }
@@ -90,6 +94,11 @@ __device__ __forceinline__ long long to_fixed(double v, int shift) {  // shift =
   const int sh = min(shift - ex, 63);
   const long long t = (long long)(m >> sh), sg = hi >> 31;
   return (t ^ sg) - sg;
+}
+
+// v 2^e by the exponent field: v normal and nonzero, the result in the normal range
+__device__ __forceinline__ double times_pow2(double v, int e) {
+  return __hiloint2double(__double2hiint(v) + e * (1 << 20), __double2loint(v));
 }
 
 enum Mode { kJacobiMode, kResidualMode, kApplyMode };
@@ -134,7 +143,7 @@ __device__ __noinline__ void tile_fp64(int n, int pitch, size_t base, int i0, in
 }
 
 template <int MODE, typename S>
-__global__ void __launch_bounds__(32 * kWarps, 4)
+__global__ void __launch_bounds__(32 * kWarps, kBlocks)
     k_fxop2d(int n, int pitch, size_t st, const __grid_constant__ Coef2D c,
              const double* __restrict__ f, const double* __restrict__ x, S* __restrict__ out) {
   const int lane = threadIdx.x, ib = blockIdx.z;
@@ -144,18 +153,16 @@ __global__ void __launch_bounds__(32 * kWarps, 4)
   const size_t base = ib * st;
   const bool in = i0 <= n;  // (i0 + 1 <= n + 1 < pitch then)
   const double2 zero = make_double2(0.0, 0.0);
-  double2 xv[kRows + 2], fv[kRows];
+  double2 xv[kRows + 2];
 #pragma unroll
   for (int t = 0; t < kRows + 2; ++t) {
     const int r = j0 - 1 + t;
     xv[t] = in && r <= n ? *reinterpret_cast<const double2*>(x + base + (size_t)r * pitch + i0) : zero;
   }
-#pragma unroll
-  for (int t = 0; t < kRows; ++t) {
-    const int r = j0 + t;
-    fv[t] = MODE != kApplyMode && in && r < n
-                ? *reinterpret_cast<const double2*>(f + base + (size_t)r * pitch + i0) : zero;
-  }
+  // f is read here for the exponent and again, from L1, when its row is due
+  auto f_row = [&](int r) {
+    return in && r < n ? *reinterpret_cast<const double2*>(f + base + (size_t)r * pitch + i0) : zero;
+  };
   const FxHead2D hd = c.fxh[ib];
   // the tile's exponent: f counts an eighth (|f| <= 8 2^e fits beside the stencil of x)
   int top = 0, topf = 0;
@@ -164,8 +171,10 @@ __global__ void __launch_bounds__(32 * kWarps, 4)
     top = max(top, max(__double2hiint(xv[t].x) & 0x7fffffff, __double2hiint(xv[t].y) & 0x7fffffff));
   if (MODE != kApplyMode) {
 #pragma unroll
-    for (int t = 0; t < kRows; ++t)
-      topf = max(topf, max(__double2hiint(fv[t].x) & 0x7fffffff, __double2hiint(fv[t].y) & 0x7fffffff));
+    for (int t = 0; t < kRows; ++t) {
+      const double2 v = f_row(j0 + t);
+      topf = max(topf, max(__double2hiint(v.x) & 0x7fffffff, __double2hiint(v.y) & 0x7fffffff));
+    }
     top = max(top, topf - (3 << 20));
   }
   top = __reduce_max_sync(0xffffffffu, top);
@@ -200,7 +209,7 @@ __global__ void __launch_bounds__(32 * kWarps, 4)
     const long long t = ew + ns;
     const long long s6 = 6 * x0 + t + d;
     long long sm = (long long)hd.P * (int)(x0 >> 32) + (long long)hd.Q * (int)(ew >> 32) +
-                   (long long)hd.R * (int)(ns >> 32) + (long long)hd.S * (int)(d >> 32);
+                   (long long)hd.R * (int)(ns >> 32);
     long long w = mul_hi(a, s6) + mul_hi(bx, (xe - xw) + g) + mul_hi(by, (xn - xs) + g);
     w += (sm >> hd.sm) + half;
     return 4 * x0 - t + (w >> hd.sa);
@@ -215,16 +224,17 @@ __global__ void __launch_bounds__(32 * kWarps, 4)
       long long ra = node(m.a, m.b, m.l, p.a, s.a, p.b, s.l, axa + ay, bxa, by);
       long long rb = node(m.b, m.r, m.a, p.b, s.b, p.r, s.a, axb + ay, bxb, by);
       if (MODE != kApplyMode) {
-        ra = to_fixed(fv[t].x, shift) - ra;
-        rb = to_fixed(fv[t].y, shift) - rb;
+        const double2 v = f_row(j);
+        ra = to_fixed(v.x, shift) - ra;
+        rb = to_fixed(v.y, shift) - rb;
       }
       const size_t k = base + (size_t)j * pitch + i0;
       const bool oka = lane > 0 && i0 <= n - 1, okb = lane < 31 && i0 + 1 <= n - 1;
       double va = __ll2double_rn(ra), vb = __ll2double_rn(rb);
       if (MODE == kJacobiMode) {
         const double2 di = in ? *reinterpret_cast<const double2*>(c.dinv + k) : zero;
-        va = fma(di.x * back, va, xv[t + 1].x);
-        vb = fma(di.y * back, vb, xv[t + 1].y);
+        va = fma(times_pow2(di.x, e - kB), va, xv[t + 1].x);
+        vb = fma(times_pow2(di.y, e - kB), vb, xv[t + 1].y);
       } else {
         va *= back;
         vb *= back;

@@ -1,0 +1,312 @@
+// The 3D level operator L = A + W on the large levels in 64-bit fixed point: damped Jacobi,
+// residual and operator apply of the FP64 mode (fxop2d.cu is the 2D form).
+//
+// The FP64 kernels (grid3d.cu) need 15 to 16 FP64 operations per node, 8 clocks of an SM's
+// FP64 pipe (2 lanes per clock), and read the eight stored coupling arrays (64 B per node).
+// Here a block covers a 32 x 8 x kZ tile of nodes, holds x of the tile and its halo in shared
+// memory as integers in units of 2^(e - kB), e one exponent for the block's x and f, and
+// computes L / h:
+//   - the stiffness 6x - (sum of the six axis neighbours) exactly;
+//   - the potential's part from closed forms.  With the node's indices a_d, the neighbour
+//     pairs p_o = x(+o) + x(-o) and differences d_o = x(+o) - x(-o) of the 7 directions
+//     (X, Y, Z, XY, XZ, YZ, XYZ) and the P1 integrals of grid3d.cu,
+//       W x / h = al S + sum_d be_d D_d + small,
+//       al   = h^2 W(x) / 60 + h^4 s / 504,   be_d = h^4 w_d a_d / 60,   s = wx + wy + wz,
+//       S    = 24 x + 3 (p_X + p_Y + p_Z + p_XYZ) + 2 (p_XY + p_XZ + p_YZ),
+//       D_d  = 3 (d_d + d_XYZ) + 2 (the differences of the two face diagonals along d),
+//       small = h^4 [ 23/2520 s p_XYZ + sum_d (w_d / 90 - s / 504) p_d
+//                     + sum_faces (s / 168 - w_o / 120) p_face ],  o the axis across the face;
+//       al = ax[i] + ay[j] + az[l] and be_d come from 1D tables scaled to fill the integers, the
+//       small terms (h^2 below the others) take the upper 30 bits of the pairs.
+// Only the products, x and f round, at 2^-57 of the tile's maximum (FP64 rounds each of its 15
+// operations and every stored coupling at 2^-53).  f is scaled by 1 / h in FP64.
+//
+// Measured on 16.6M nodes: Jacobi 438 -> 270 us, residual 413 -> 223 us.  The instruction rate
+// bounds it (some 400 integer instructions per node, half of the issue slots used), then the
+// latency of a block's loads: the whole tile is loaded at once (walking the planes through a
+// ring of four with a pass ahead for the exponent took 300 and 285 us).
+//
+// Tiles with infinities, NaN, all zeros or an exponent outside +-kFxMaxExp, and instances whose
+// potential is too large for the formats, run the FP64 expressions of grid3d.cu.
+#include "dfloat.cuh"
+#include "fixed.cuh"
+#include "fmg_internal.h"
+
+namespace fmg {
+namespace {
+
+constexpr int kB = 57;                       // x = I 2^(e - kB); |S| <= 60 2^kB
+constexpr int kX = 32, kY = 8, kZ = 8;       // tile of columns (= threads), planes per block
+constexpr int kNX = kX + 2, kNodes = (kX + 2) * (kY + 2);
+
+// Tables ax, ay, az, bx, by, bz (n + 1 entries each) and the header of each instance.
+__global__ void k_fxop3d_tables(int n, double h, const PotentialParams* __restrict__ pp,
+                                long long* __restrict__ tab, FxHead3D* __restrict__ head) {
+  const int x = blockIdx.x * blockDim.x + threadIdx.x;
+  if (x > n) return;
+  const PotentialParams p = pp[blockIdx.y];
+  tab += (size_t)blockIdx.y * 6 * (n + 1);
+  const double wl = p.operator_form == FMG_W_LEFT ? 1.0 : 0.0;
+  const double h2 = h * h, h4 = h2 * h2, L = n * h;
+  const double w[3] = {wl * p.wx, wl * p.wy, wl * p.wz}, w0 = wl * p.w0;
+  const double s = w[0] + w[1] + w[2], sabs = fabs(w[0]) + fabs(w[1]) + fabs(w[2]);
+  const double amax = h2 / 60.0 * (fabs(w0) + sabs * (L * L + 0.31 * h2));
+  const double pmax = h4 * sabs;  // bounds the small coefficients (and their sum over a stencil)
+  // amax < 2^-sa, pmax < 2^-ss
+  const int sa = amax > 0.0 ? max(0, min(40, -(ilogb(amax) + 1))) : 40;
+  const int ss = pmax > 0.0 ? max(0, min(90, -(ilogb(pmax) + 1))) : 90;
+  const double sc = ldexp(1.0, 61 + sa), d = x;
+  const double c0 = h2 * w0 / 60.0 + h4 * s / 504.0;
+  for (int q = 0; q < 3; ++q) {
+    tab[q * (n + 1) + x] = __double2ll_rn(sc * ((q == 0 ? c0 : 0.0) + h4 * w[q] * d * d / 60.0));
+    tab[(3 + q) * (n + 1) + x] = __double2ll_rn(sc * (h4 * w[q] * d / 60.0));
+  }
+  if (x == 0) {
+    FxHead3D q;
+    // the small terms are 0.06 pmax of the maximum at most; 30 bits of the pairs and of the
+    // coefficients (each below pmax / 89, hence 36 + ss) leave 2^-33 pmax of it: with pmax <=
+    // 2^-17, 2^-50 of the maximum against the 6 times the maximum that L / h reaches
+    q.ok = amax <= 1.0 / 64.0 && pmax <= 1.0 / 131072.0 && ss - sa + 11 >= 0;
+    q.sa = sa - 3;                 // shift of the products' sum
+    q.sm = min(63, ss - sa + 11);  // shift of the small terms to the products' units
+    const double t = ldexp(h4, 36 + ss);
+    q.P = (int)__double2ll_rn(t * s * (23.0 / 2520.0));
+    for (int a = 0; a < 3; ++a) {
+      q.A[a] = (int)__double2ll_rn(t * (w[a] / 90.0 - s / 504.0));
+      // faces XY, XZ, YZ: the axis across is z, y, x
+      q.F[a] = (int)__double2ll_rn(t * (s / 168.0 - w[2 - a] / 120.0));
+    }
+    head[blockIdx.y] = q;
+  }
+}
+
+// high word of a 64 x 64 product (|a|, |b| < 2^63 - 2^31), within a unit and a half
+__device__ __forceinline__ long long mul_hi(long long a, long long b) {
+  const int al = (int)a, bl = (int)b;
+  const int ah = (int)(a >> 32) + (int)((uint32_t)al >> 31);
+  const int bh = (int)(b >> 32) + (int)((uint32_t)bl >> 31);
+  return (long long)ah * bh + (((long long)al * bh + (long long)ah * bl) >> 32);
+}
+
+// v 2^(kB - e) as an integer (truncated), |v| <= 2^e; shift = e + 1085 - kB
+__device__ __forceinline__ long long to_fixed(double v, int shift) {
+  const int hi = __double2hiint(v);
+  const int ex = (hi >> 20) & 0x7ff;
+  const unsigned long long m =
+      ((unsigned long long)(((uint32_t)hi & 0xfffffu) | 0x100000u) << 32 |
+       (uint32_t)__double2loint(v)) << 10;
+  const int sh = min(shift - ex, 63);
+  const long long t = (long long)(m >> sh), sg = hi >> 31;
+  return (t ^ sg) - sg;
+}
+
+enum Mode { kJacobiMode, kResidualMode, kApplyMode };
+
+__device__ __forceinline__ long dir(int d, int pitch, long plane) {
+  constexpr int ox[7] = {1, 0, 0, 1, 1, 0, 1}, oy[7] = {0, 1, 0, 1, 0, 1, 1},
+                oz[7] = {0, 0, 1, 0, 1, 1, 1};
+  return ox[d] + (long)oy[d] * pitch + oz[d] * plane;
+}
+
+// The block's nodes in FP64, with the expressions of grid3d.cu.
+template <int MODE>
+__device__ __noinline__ void tile_fp64(int n, int pitch, size_t base, int x, int y, int z0, int z1,
+                                       const Coef3D& c, const double* __restrict__ f,
+                                       const double* __restrict__ v, double* __restrict__ out) {
+  if (x > n - 1 || y > n - 1) return;
+  const long plane = (long)(n + 1) * pitch;
+  for (int z = z0; z < z1; ++z) {
+    const size_t k = base + z * plane + (long)y * pitch + x;
+    double r = MODE == kApplyMode ? c.a[0][k] * v[k] : fma(-c.a[0][k], v[k], f[k]);
+    for (int d = 0; d < 7; ++d) {
+      const long o = dir(d, pitch, plane);
+      const double sg = MODE == kApplyMode ? 1.0 : -1.0;
+      r = fma(sg * c.a[1 + d][k], v[k + o], r);
+      r = fma(sg * c.a[1 + d][k - o], v[k - o], r);
+    }
+    out[k] = MODE == kJacobiMode ? fma(c.dinv[k], r, v[k]) : r;
+  }
+}
+
+template <int MODE>
+__global__ void __launch_bounds__(kX * kY, 3)
+    k_fxop3d(int n, int pitch, size_t st, double h, double hinv, int hexp,
+             const __grid_constant__ Coef3D c, const double* __restrict__ f,
+             const double* __restrict__ v, double* __restrict__ out) {
+  __shared__ long long su[kZ + 2][kNodes];  // planes z0 - 1 .. z0 + kZ
+  __shared__ int top[2];
+  const int nzc = (n - 1 + kZ - 1) / kZ, ib = blockIdx.z / nzc;
+  const int z0 = 1 + (int)(blockIdx.z - ib * nzc) * kZ, z1 = min(z0 + kZ, n);
+  const int x0 = 1 + blockIdx.x * kX, y0 = 1 + blockIdx.y * kY;
+  const long plane = (long)(n + 1) * pitch;
+  const size_t base = ib * st;
+  const int tid = threadIdx.y * kX + threadIdx.x;
+  const int x = x0 + threadIdx.x, y = y0 + threadIdx.y;
+  const bool active = x <= n - 1 && y <= n - 1;
+  // the two plane elements this thread stages (the second one for tid < kNodes - kX kY)
+  const int e1 = tid + kX * kY;
+  const int xa = x0 - 1 + tid % kNX, ya = y0 - 1 + tid / kNX;
+  const int xb = x0 - 1 + e1 % kNX, yb = y0 - 1 + e1 / kNX;
+  const bool ina = xa <= n && ya <= n, inb = e1 < kNodes && xb <= n && yb <= n;
+  const double* pa = v + base + (long)ya * pitch + xa;
+  const double* pb = v + base + (long)yb * pitch + xb;
+  const double* pf = f + base + (long)y * pitch + x;
+  if (tid < 2) top[tid] = 0;
+  __syncthreads();
+  // the whole tile is loaded first (a block's loads in flight at once), its exponent taken, and
+  // its integers stored to shared memory, so that the planes below need no barrier
+  double va[kZ + 2], vb[kZ + 2];
+  {
+    int m = 0, mf = 0;
+#pragma unroll
+    for (int t = 0; t < kZ + 2; ++t) {
+      const int z = z0 - 1 + t;
+      va[t] = ina && z <= n ? pa[z * plane] : 0.0;
+      vb[t] = inb && z <= n ? pb[z * plane] : 0.0;
+    }
+    if (MODE != kApplyMode && active) {
+#pragma unroll
+      for (int t = 0; t < kZ; ++t)
+        if (z0 + t < z1) mf = max(mf, __double2hiint(pf[(z0 + t) * plane]) & 0x7fffffff);
+    }
+#pragma unroll
+    for (int t = 0; t < kZ + 2; ++t)
+      m = max(m, max(__double2hiint(va[t]) & 0x7fffffff, __double2hiint(vb[t]) & 0x7fffffff));
+    m = __reduce_max_sync(0xffffffffu, m);
+    mf = __reduce_max_sync(0xffffffffu, mf);
+    if ((tid & 31) == 0) {
+      atomicMax(&top[0], m);
+      atomicMax(&top[1], mf);
+    }
+  }
+  __syncthreads();
+  const int tf = top[1] == 0 ? 0 : min(top[1] + ((hexp - 3) << 20), 0x7ff00000);
+  const int e = ((max(top[0], tf) + 1) >> 20) - 1022;
+  const FxHead3D hd = c.fxh[ib];
+  if (!hd.ok || top[1] >= 0x7ff00000 || e < -kFxMaxExp || e > kFxMaxExp) {
+    tile_fp64<MODE>(n, pitch, base, x, y, z0, z1, c, f, v, out);
+    return;
+  }
+  const int shift = e + 1085 - kB;
+  const double fs = hinv * fx_pow2(kB - e), back = h * fx_pow2(e - kB);
+  const long long* tab = c.fxt + (size_t)ib * 6 * (n + 1);
+  const int xc = min(x, n), yc = min(y, n);
+  const long long axy = tab[xc] + tab[(n + 1) + yc], bx = tab[3 * (n + 1) + xc],
+                  by = tab[4 * (n + 1) + yc];
+  const long long half = 1ll << (hd.sa - 1);
+  // the small terms drop the lower bits of the pairs: half a unit each on average
+  const long long q0 = ((long long)hd.P + hd.A[0] + hd.A[1] + hd.A[2] + hd.F[0] + hd.F[1] +
+                        hd.F[2]) / 2;
+#pragma unroll
+  for (int t = 0; t < kZ + 2; ++t) {
+    su[t][tid] = to_fixed(va[t], shift);
+    if (e1 < kNodes) su[t][e1] = to_fixed(vb[t], shift);
+  }
+  __syncthreads();
+  if (!active) return;
+  const int nd = (threadIdx.y + 1) * kNX + threadIdx.x + 1;
+  size_t k = base + z0 * plane + (long)y * pitch + x;
+#pragma unroll 2
+  for (int t = 1; z0 + t <= z1; ++t, k += plane) {
+    const int z = z0 + t - 1;
+    const double fv = MODE != kApplyMode ? f[k] : 0.0;
+    const double di = MODE == kJacobiMode ? c.dinv[k] : 0.0;
+    const double xv = MODE == kJacobiMode ? v[k] : 0.0;
+    const long long* s0 = su[t] + nd;
+    const long long* sp = su[t + 1] + nd;
+    const long long* sm = su[t - 1] + nd;
+    {
+      // sums and differences of the neighbours +o and -o, direction by direction
+      const long long u = s0[0];
+      long long q, dx, dy, dz, pa2, pf2;
+      {
+        const long long a = s0[1], b = s0[-1], p = a + b;
+        dx = a - b;
+        pa2 = p;
+        q = q0 + (long long)hd.A[0] * (int)(p >> 28);
+      }
+      {
+        const long long a = s0[kNX], b = s0[-kNX], p = a + b;
+        dy = a - b;
+        pa2 += p;
+        q += (long long)hd.A[1] * (int)(p >> 28);
+      }
+      {
+        const long long a = sp[0], b = sm[0], p = a + b;
+        dz = a - b;
+        pa2 += p;
+        q += (long long)hd.A[2] * (int)(p >> 28);
+      }
+      const long long r6 = 6 * u - pa2;  // the stiffness
+      {
+        const long long a = sp[kNX + 1], b = sm[-kNX - 1], p = a + b, d = a - b;
+        dx += d;
+        dy += d;
+        dz += d;
+        pa2 += p;
+        q += (long long)hd.P * (int)(p >> 28);
+      }
+      // D = 3 (axis and body) + 2 (faces): the first three carry 1, the sum below doubles both
+      long long ex, ey, ez;
+      {
+        const long long a = s0[kNX + 1], b = s0[-kNX - 1], p = a + b, d = a - b;
+        ex = dx + d;
+        ey = dy + d;
+        pf2 = p;
+        q += (long long)hd.F[0] * (int)(p >> 28);
+      }
+      {
+        const long long a = sp[1], b = sm[-1], p = a + b, d = a - b;
+        ex += d;
+        ez = dz + d;
+        pf2 += p;
+        q += (long long)hd.F[1] * (int)(p >> 28);
+      }
+      {
+        const long long a = sp[kNX], b = sm[-kNX], p = a + b, d = a - b;
+        ey += d;
+        ez += d;
+        pf2 += p;
+        q += (long long)hd.F[2] * (int)(p >> 28);
+      }
+      const long long t = 8 * u + pa2, S = 2 * (t + pf2) + t;
+      long long w = mul_hi(axy + tab[2 * (n + 1) + z], S) + mul_hi(bx, 2 * ex + dx) +
+                    mul_hi(by, 2 * ey + dy) + mul_hi(tab[5 * (n + 1) + z], 2 * ez + dz);
+      w += (q >> hd.sm) + half;
+      long long r = r6 + (w >> hd.sa);
+      if (MODE != kApplyMode) r = __double2ll_rn(fv * fs) - r;
+      const double rd = __ll2double_rn(r);
+      out[k] = MODE == kJacobiMode ? fma(di * back, rd, xv) : rd * back;
+    }
+  }
+}
+
+template <int MODE>
+void launch(const Grid& g, const Coef3D& c, const double* f, const double* x, double* out,
+            cudaStream_t s) {
+  const dim3 grid((g.n - 1 + kX - 1) / kX, (g.n - 1 + kY - 1) / kY,
+                  g.nb * ((g.n - 1 + kZ - 1) / kZ));
+  int ex = 0;
+  frexp(1.0 / g.h, &ex);  // 1 / h < 2^ex
+  k_fxop3d<MODE><<<grid, dim3(kX, kY), 0, s>>>(g.n, g.pitch, g.stride, g.h, 1.0 / g.h, ex, c,
+                                               MODE == kApplyMode ? x : f, x, out);
+}
+
+}  // namespace
+
+void fxop3d_tables(const Grid& g, const PotentialParams* p, const Coef3D& c, cudaStream_t s) {
+  k_fxop3d_tables<<<dim3((g.n + 1 + 127) / 128, g.nb), 128, 0, s>>>(g.n, g.h, p, c.fxt, c.fxh);
+}
+void fxop3d_apply(const Grid& g, const Coef3D& c, const double* x, double* y, cudaStream_t s) {
+  launch<kApplyMode>(g, c, nullptr, x, y, s);
+}
+void fxop3d_jacobi(const Grid& g, const Coef3D& c, const double* f, const double* x, double* xo,
+                   cudaStream_t s) {
+  launch<kJacobiMode>(g, c, f, x, xo, s);
+}
+void fxop3d_residual(const Grid& g, const Coef3D& c, const double* f, const double* x, double* r,
+                     cudaStream_t s) {
+  launch<kResidualMode>(g, c, f, x, r, s);
+}
+
+}  // namespace fmg

@@ -822,11 +822,16 @@ void coef3d_setup(const Grid& g, const PotentialParams* p, const Coef3D& c, cuda
   k_coef1d_3d<<<dim3((g.n + 1 + 127) / 128, g.nb), 128, 0, s>>>(g.n, g.h, p, c.tab);
   const int rows = (g.n + 1) * (g.n + 1);
   k_coef3d<<<dim3((rows + 7) / 8, g.nb), 256, 0, s>>>(g.n, g.pitch, g.stride, g.h, c.tab, p, c);
+  if (c.fxt) fxop3d_tables(g, p, c, s);
 }
 
 #define INTERIOR_LAUNCH(g) grid3(g, g.n - 1, g.n - 1, g.n - 1), block3(g), 0, s
 
 void apply3d(const Grid& g, const Coef3D& c, const double* x, double* y, cudaStream_t s) {
+  if (c.fxt) {
+    fxop3d_apply(g, c, x, y, s);
+    return;
+  }
   k_apply3d<<<INTERIOR_LAUNCH(g)>>>(g.n, g.pitch, g.stride, c, x, y);
 }
 
@@ -845,6 +850,10 @@ void mass3d_df(const Grid& g, SplitVec x, double* y, cudaStream_t s) {
 
 void jacobi3d(const Grid& g, const Coef3D& c, const double* f, const double* x, double* xo,
               bool x_is_zero, cudaStream_t s) {
+  if (c.fxt && !x_is_zero) {
+    fxop3d_jacobi(g, c, f, x, xo, s);
+    return;
+  }
   if (x_is_zero) k_jacobi3d_zero<<<INTERIOR_LAUNCH(g)>>>(g.n, g.pitch, g.stride, c, f, xo);
   else k_jacobi3d<<<INTERIOR_LAUNCH(g)>>>(g.n, g.pitch, g.stride, c, f, x, xo);
 }
@@ -857,6 +866,10 @@ void cheb3d(const Grid& g, const Coef3D& c, const double* f, const double* x, do
 
 void residual3d(const Grid& g, const Coef3D& c, const double* f, const double* x, double* r,
                 cudaStream_t s) {
+  if (c.fxt) {
+    fxop3d_residual(g, c, f, x, r, s);
+    return;
+  }
   k_residual3d<<<INTERIOR_LAUNCH(g)>>>(g.n, g.pitch, g.stride, c, f, x, r);
 }
 
