@@ -431,17 +431,12 @@ void nload_density2d_df(const Grid& g, SplitVec u, double* nl, const Density2D& 
       dfloat(g.h * g.h / 360.0), u, nl, b.C, b.E, b.N, b.NE);
 }
 
-void coarsen_density2d(const Grid& fine, const Grid& coarse, const Density2D& bf,
-                       const Density2D& bc, cudaStream_t s, bool split) {
+void coarsen_density2d_df(const Grid& fine, const Grid& coarse, const Density2D& bf,
+                          const Density2D& bc, cudaStream_t s) {
   const dim3 grid = grid_of(fine, coarse.n - 1, coarse.n - 1), block(fine.bx, fine.by);
-  if (split)
-    k_coarsen_density2d<dfloat><<<grid, block, 0, s>>>(
-        coarse.n, coarse.pitch, fine.pitch, coarse.stride, fine.stride, bf.C, bf.E, bf.N,
-        bf.NE, bc.C, bc.E, bc.N, bc.NE);
-  else
-    k_coarsen_density2d<double><<<grid, block, 0, s>>>(
-        coarse.n, coarse.pitch, fine.pitch, coarse.stride, fine.stride, bf.C, bf.E, bf.N,
-        bf.NE, bc.C, bc.E, bc.N, bc.NE);
+  k_coarsen_density2d<dfloat><<<grid, block, 0, s>>>(
+      coarse.n, coarse.pitch, fine.pitch, coarse.stride, fine.stride, bf.C, bf.E, bf.N, bf.NE,
+      bc.C, bc.E, bc.N, bc.NE);
 }
 
 void gather_level1_2d(const Grid& g1, const double* gA_pad, const double* gM_pad,

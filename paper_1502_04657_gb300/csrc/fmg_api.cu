@@ -149,8 +149,8 @@ void lv_nload_density_df(Level& l, SplitVec v, double* nl, cudaStream_t s) {
 }
 // split: the density stencils hold double-float splits (mixed modes, from the _df kernels)
 void lv_coarsen_density(Level& fl, Level& cl, cudaStream_t s, bool split) {
-  if (fl.g.dim == 2) coarsen_density2d(fl.g, cl.g, fl.b, cl.b, s, split);
-  else coarsen_density3d(fl.g, cl.g, fl.b3, cl.b3, s, split);
+  if (fl.g.dim == 2) (split ? coarsen_density2d_df : coarsen_density2d)(fl.g, cl.g, fl.b, cl.b, s);
+  else (split ? coarsen_density3d_df : coarsen_density3d)(fl.g, cl.g, fl.b3, cl.b3, s);
 }
 // npinned: the leading instances that keep the pinned order of summation (3D)
 void lv_t3(Level& l, int n1, int npinned, const double* u, double* partials, double* t3,

@@ -191,7 +191,9 @@ void rhs3d_df(const Grid& g, const double* lam, const PotentialParams* p_dev, Sp
 void nload_density3d_df(const Grid& g, SplitVec u, double* nl, const Density3D& b,
                         cudaStream_t s);
 void coarsen_density3d(const Grid& fine, const Grid& coarse, const Density3D& bf,
-                       const Density3D& bc, cudaStream_t s, bool split = false);
+                       const Density3D& bc, cudaStream_t s);
+void coarsen_density3d_df(const Grid& fine, const Grid& coarse, const Density3D& bf,
+                          const Density3D& bc, cudaStream_t s);
 void dense_level1_3d(const Grid& g, const Coef3D& c, double* L, double* M, cudaStream_t s);
 void density_dense3d(const Grid& g, const Density3D& b, double* B, cudaStream_t s,
                      bool split = false);
@@ -325,10 +327,12 @@ void nload_density2d(const Grid& g, const double* u, double* nl, const Density2D
                      cudaStream_t s);
 void nload_density2d_df(const Grid& g, SplitVec u, double* nl, const Density2D& b,
                         cudaStream_t s);
-// Galerkin coarsening of the density stencil: bc = P^T bf P.
-// split: the entries are stored as double-float splits (mixed modes; see nload_density*_df)
+// Galerkin coarsening of the density stencil: bc = P^T bf P (coarsen_fx.cu; _df: the entries
+// are stored as double-float splits, see nload_density*_df).
 void coarsen_density2d(const Grid& fine, const Grid& coarse, const Density2D& bf,
-                       const Density2D& bc, cudaStream_t s, bool split = false);
+                       const Density2D& bc, cudaStream_t s);
+void coarsen_density2d_df(const Grid& fine, const Grid& coarse, const Density2D& bf,
+                          const Density2D& bc, cudaStream_t s);
 // T3^T_abc = int_T u mu_a mu_b mu_c per coarse triangle (10 per triangle, a <= b <= c,
 // lexicographic), from per-class monomial sums.  pw: (x/r)^m table of the level, map: the
 // level's 2 x 10 x 25 map (t3_map2d), partials: t3_partials2d(fine, n1) doubles.

@@ -12,7 +12,6 @@
 // (Y, Z, XZ, YZ by permuting the axes; the coupling to p - d is the one of p - d to p).  The
 // mass stencil is h^3 (2/5 at C, 1/20 along axes and the body diagonal, 1/30 along face
 // diagonals).  As in 2D, the 8 coupling arrays and omega/D are materialised once per solve.
-#include <type_traits>
 
 #include "fmg_internal.h"
 #include "dfloat.cuh"
@@ -668,8 +667,9 @@ __global__ void __launch_bounds__(256, MINB)
   for (int d = 0; d < 7; ++d) put_entry(b.a[1 + d], k, s420 * e[1 + d]);
 }
 
-// Galerkin coarsening of the 15-point density stencil: Bc(a, b) = sum P_va P_wb B(v, w) over
-// the 15-node fine supports of the coarse hats (weights 1 at 2a, 1/2 at 2a +- d).
+// Galerkin coarsening of the 15-point density stencil in double-float arithmetic (mixed modes,
+// entries stored split: put_entry; coarsen_fx.cu is the FP64 one): Bc(a, b) = sum P_va P_wb
+// B(v, w) over the 15-node fine supports of the coarse hats (weights 1 at 2a, 1/2 at 2a +- d).
 __device__ __forceinline__ int nb_of(int dx, int dy, int dz) {
   // index of the neighbour (dx,dy,dz) in {0: self, 1 + 2d: +d, 2 + 2d: -d}, -1 if not one
   if (dx == 0 && dy == 0 && dz == 0) return 0;
@@ -680,28 +680,26 @@ __device__ __forceinline__ int nb_of(int dx, int dy, int dz) {
   return -1;
 }
 
-template <typename V>
-__device__ __forceinline__ V fine_entry3(const Density3D& f, size_t kv, int code, int pitch,
+__device__ __forceinline__ dfloat fine_entry3(const Density3D& f, size_t kv, int code, int pitch,
                                          long plane) {
-  if (code == 0) return get_entry<V>(f.a[0], kv);
+  if (code == 0) return get_entry<dfloat>(f.a[0], kv);
   const int d = (code - 1) >> 1;
-  if (((code - 1) & 1) == 0) return get_entry<V>(f.a[1 + d], kv);
-  return get_entry<V>(f.a[1 + d], kv - dir_off(d, pitch, plane));
+  if (((code - 1) & 1) == 0) return get_entry<dfloat>(f.a[1 + d], kv);
+  return get_entry<dfloat>(f.a[1 + d], kv - dir_off(d, pitch, plane));
 }
 
-template <typename V, int T>
-__device__ __forceinline__ V coarse_entry3(const Density3D& f, size_t kf, int pf, long planef) {
+template <int T>
+__device__ __forceinline__ dfloat coarse_entry3(const Density3D& f, size_t kf, int pf, long planef) {
   // target offset in coarse units: T = 0 self, 1 + d for +d
   const int tx = T == 0 ? 0 : kDir[T - 1][0], ty = T == 0 ? 0 : kDir[T - 1][1],
             tz = T == 0 ? 0 : kDir[T - 1][2];
-  // FP64: one FMA per pair.  Double-float: the entries (int u~^2 phi phi) are non-negative, so
-  // they are summed per weight class (1, 1/2, 1/4) with double-float additions, three
-  // independent chains, and scaled exactly once at the end.  The diagonal entry (T = 0) pairs
-  // the support with itself, and (p, q), (q, p) read the same fine entry, so it takes each
-  // unordered pair once with twice its weight (an exact doubling).
+  // The entries (int u~^2 phi phi) are non-negative, so they are summed per weight class (1,
+  // 1/2, 1/4) with double-float additions, three independent chains, and scaled exactly once at
+  // the end.  The diagonal entry (T = 0) pairs the support with itself, and (p, q), (q, p) read
+  // the same fine entry, so it takes each unordered pair once with twice its weight (an exact
+  // doubling).
   constexpr bool kDiag = T == 0;
-  V acc = 0;
-  V part[3] = {V(0), V(0), V(0)};
+  dfloat part[3] = {dfloat(0), dfloat(0), dfloat(0)};
 #pragma unroll
   for (int p = 0; p < 15; ++p) {
     const int px = p == 0 ? 0 : ((p - 1) & 1 ? -kDir[(p - 1) >> 1][0] : kDir[(p - 1) >> 1][0]);
@@ -716,26 +714,16 @@ __device__ __forceinline__ V coarse_entry3(const Density3D& f, size_t kf, int pf
       if (code >= 0) {
         const size_t kv = kf + px + (long)py * pf + (long)pz * planef;
         const bool twice_w = kDiag && q != p;
-        if constexpr (std::is_same<V, dfloat>::value) {
-          const dfloat e = fine_entry3<V>(f, kv, code, pf, planef);
-          part[(p != 0) + (q != 0)] += twice_w ? twice(e) : e;
-        } else {
-          const V w((twice_w ? 2.0 : 1.0) * (p == 0 ? 1.0 : 0.5) * (q == 0 ? 1.0 : 0.5));
-          acc = fma(w, fine_entry3<V>(f, kv, code, pf, planef), acc);
-        }
+        const dfloat e = fine_entry3(f, kv, code, pf, planef);
+        part[(p != 0) + (q != 0)] += twice_w ? twice(e) : e;
       }
     }
   }
-  if constexpr (std::is_same<V, dfloat>::value) {
-    const dfloat h1(part[1].hi * 0.5f, part[1].lo * 0.5f);
-    const dfloat h2(part[2].hi * 0.25f, part[2].lo * 0.25f);
-    acc = part[0] + (h1 + h2);
-  }
-  return acc;
+  const dfloat h1(part[1].hi * 0.5f, part[1].lo * 0.5f);
+  const dfloat h2(part[2].hi * 0.25f, part[2].lo * 0.25f);
+  return part[0] + (h1 + h2);
 }
 
-// V = double (FP64 mode) or dfloat (mixed modes: entries stored split, see put_entry)
-template <typename V>
 __global__ void k_coarsen_density3d(int nc, int pc, int pf, size_t stc, size_t stf,
                                     Density3D f, Density3D c) {
   const int I = 1 + blockIdx.x * blockDim.x + threadIdx.x;
@@ -746,16 +734,16 @@ __global__ void k_coarsen_density3d(int nc, int pc, int pf, size_t stc, size_t s
   const long planef = (long)(2 * nc + 1) * pf;
   const size_t kf = ib * stf + (size_t)(2 * L) * planef + (size_t)(2 * J) * pf + 2 * I;
   const size_t kc = ib * stc + ((size_t)L * (nc + 1) + J) * pc + I;
-  put_entry(c.a[0], kc, coarse_entry3<V, 0>(f, kf, pf, planef));
+  put_entry(c.a[0], kc, coarse_entry3<0>(f, kf, pf, planef));
   // couplings to coarse neighbours outside the interior are never read: skip them
-  if (I + 1 < nc) put_entry(c.a[1], kc, coarse_entry3<V, 1>(f, kf, pf, planef));
-  if (J + 1 < nc) put_entry(c.a[2], kc, coarse_entry3<V, 2>(f, kf, pf, planef));
-  if (L + 1 < nc) put_entry(c.a[3], kc, coarse_entry3<V, 3>(f, kf, pf, planef));
-  if (I + 1 < nc && J + 1 < nc) put_entry(c.a[4], kc, coarse_entry3<V, 4>(f, kf, pf, planef));
-  if (I + 1 < nc && L + 1 < nc) put_entry(c.a[5], kc, coarse_entry3<V, 5>(f, kf, pf, planef));
-  if (J + 1 < nc && L + 1 < nc) put_entry(c.a[6], kc, coarse_entry3<V, 6>(f, kf, pf, planef));
+  if (I + 1 < nc) put_entry(c.a[1], kc, coarse_entry3<1>(f, kf, pf, planef));
+  if (J + 1 < nc) put_entry(c.a[2], kc, coarse_entry3<2>(f, kf, pf, planef));
+  if (L + 1 < nc) put_entry(c.a[3], kc, coarse_entry3<3>(f, kf, pf, planef));
+  if (I + 1 < nc && J + 1 < nc) put_entry(c.a[4], kc, coarse_entry3<4>(f, kf, pf, planef));
+  if (I + 1 < nc && L + 1 < nc) put_entry(c.a[5], kc, coarse_entry3<5>(f, kf, pf, planef));
+  if (J + 1 < nc && L + 1 < nc) put_entry(c.a[6], kc, coarse_entry3<6>(f, kf, pf, planef));
   if (I + 1 < nc && J + 1 < nc && L + 1 < nc)
-    put_entry(c.a[7], kc, coarse_entry3<V, 7>(f, kf, pf, planef));
+    put_entry(c.a[7], kc, coarse_entry3<7>(f, kf, pf, planef));
 }
 
 // dense level-1 matrices from a 15-point stencil given per node as (C, +d couplings)
@@ -980,15 +968,11 @@ void rhs3d_df(const Grid& g, const double* lam, const PotentialParams* p, SplitV
                                      lam, p, u, f);
 }
 
-void coarsen_density3d(const Grid& fine, const Grid& coarse, const Density3D& bf,
-                       const Density3D& bc, cudaStream_t s, bool split) {
-  const dim3 grid = grid3(fine, coarse.n - 1, coarse.n - 1, coarse.n - 1);
-  if (split)
-    k_coarsen_density3d<dfloat><<<grid, block3(fine), 0, s>>>(
-        coarse.n, coarse.pitch, fine.pitch, coarse.stride, fine.stride, bf, bc);
-  else
-    k_coarsen_density3d<double><<<grid, block3(fine), 0, s>>>(
-        coarse.n, coarse.pitch, fine.pitch, coarse.stride, fine.stride, bf, bc);
+void coarsen_density3d_df(const Grid& fine, const Grid& coarse, const Density3D& bf,
+                          const Density3D& bc, cudaStream_t s) {
+  k_coarsen_density3d<<<grid3(fine, coarse.n - 1, coarse.n - 1, coarse.n - 1), block3(fine), 0,
+                        s>>>(coarse.n, coarse.pitch, fine.pitch, coarse.stride, fine.stride, bf,
+                             bc);
 }
 
 void dense_level1_3d(const Grid& g, const Coef3D& c, double* L, double* M, cudaStream_t s) {
