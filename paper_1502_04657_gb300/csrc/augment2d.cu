@@ -16,8 +16,6 @@
 // with m_ij the moments of phi_v over the fine triangles of v's star that lie in T.  Those
 // depend only on v's class (interior of T, one of T's three edges, one of its vertices), so
 // T3 follows from monomial sums of u~ per class: 4 FP64 FMAs per interior node.
-#include <type_traits>
-
 #include "fmg_internal.h"
 #include "reduce_dev.cuh"
 #include "dfloat.cuh"
@@ -41,7 +39,7 @@ __device__ __forceinline__ size_t at(int i, int j, int pitch) { return (size_t)j
 // for the edge p-q shared by the triangles closed by r1 and r2 (E: NE, S; N: NE, W;
 // NE: E, N).  s60, s180 = |K| / 60, / 180 (computed on the host: an FP64 division per node
 // would cost as much as a quarter of the kernel's arithmetic).
-// FP64 mode.
+template <int R>
 __device__ __noinline__ void nload_density2d_fp64(int n, int pitch, size_t st, double s60,
                                                   double s180, const double* __restrict__ u,
                                                   double* __restrict__ nl,
@@ -49,27 +47,28 @@ __device__ __noinline__ void nload_density2d_fp64(int n, int pitch, size_t st, d
                                                   double* __restrict__ bN,
                                                   double* __restrict__ bNE) {
   using T = double;
-  star2d_walk<T>(n, pitch, st, u, [&](size_t k, const Star2D<T>& p) {
-    nl[k] = out_of(s60 * star_cubic(p));
-    put_entry(bC, k, s180 * fma(p.u, fma(T(72), p.u, T(6) * p.M1), p.SF));
-    put_entry(bE, k, s180 * fma(T(2), fma(p.H.s, p.H.s + (p.uNE + p.uS), p.H.F), p.qNE + p.qS));
-    put_entry(bN, k, s180 * fma(T(2), fma(p.V.s, p.V.s + (p.uNE + p.uW), p.V.F), p.qNE + p.qW));
-    put_entry(bNE, k, s180 * fma(T(2), fma(p.D.s, p.D.s + (p.uE + p.uN), p.D.F), p.qE + p.qN));
+  star2d_walk<T, R>(n, pitch, st, u, [&](size_t k, const Star2D<T>& p) {
+    nl[k] = s60 * star_cubic(p);
+    bC[k] = s180 * fma(p.u, fma(T(72), p.u, T(6) * p.M1), p.SF);
+    bE[k] = s180 * fma(T(2), fma(p.H.s, p.H.s + (p.uNE + p.uS), p.H.F), p.qNE + p.qS);
+    bN[k] = s180 * fma(T(2), fma(p.V.s, p.V.s + (p.uNE + p.uW), p.V.F), p.qNE + p.qW);
+    bNE[k] = s180 * fma(T(2), fma(p.D.s, p.D.s + (p.uE + p.uN), p.D.F), p.qE + p.qN);
   });
 }
 
+template <int R>
 __global__ void __launch_bounds__(32 * kStarWarps, 4)
     k_nload_density2d(int n, int pitch, size_t st, double s60, double s180,
                       const double* __restrict__ u, double* __restrict__ nl,
                       double* __restrict__ bC, double* __restrict__ bE,
                       double* __restrict__ bN, double* __restrict__ bNE) {
-  const int e = star2d_exponent(n, pitch, st, u);
+  const int e = star2d_exponent<R>(n, pitch, st, u);
   if (e == kFxNone) {
-    nload_density2d_fp64(n, pitch, st, s60, s180, u, nl, bC, bE, bN, bNE);
+    nload_density2d_fp64<R>(n, pitch, st, s60, s180, u, nl, bC, bE, bN, bNE);
     return;
   }
   const double a3 = fx_scale<kFx2>(s60, 3, e), a2 = fx_scale<kFx2>(s180, 2, e);
-  star2d_walk_fx<true>(n, pitch, st, u, e, [&](size_t k, const Star2DFx& p) {
+  star2d_walk_fx<true, R>(n, pitch, st, u, e, [&](size_t k, const Star2DFx& p) {
     nl[k] = to_double(star_cubic(p), a3);
     bC[k] = to_double(madd<6>(p.u * madd<12>(p.u, p.M1), p.SF), a2);
     bE[k] = to_double(madd<2>(fma(p.Hs, p.Hs + (p.uNE + p.uS), p.HF), p.qNE + p.qS), a2);
@@ -78,13 +77,11 @@ __global__ void __launch_bounds__(32 * kStarWarps, 4)
   });
 }
 
-// The same quantities node by node: the cubic load through the pair sums
-// m_k = n_k + n_{k+1} (nload_at in grid2d.cu) and the density stencil from the two triangle
-// formulas above.  T, U: FP64 (double, const double*) for launches too small to fill the GPU
-// as column walks, or double-float from the split u (dfloat, SplitVec) in the mixed modes,
-// whose entries stay split for the coarsening chain.  s60, s90, s180 = |K| / 60, / 90, / 180.
-template <typename T, typename U>
-__global__ void k_nload_density2d_node(int n, int pitch, size_t st, T s60, T s90, T s180, U u,
+// The same quantities node by node in FP64, for levels below n = 64: the cubic load through the
+// pair sums m_k = n_k + n_{k+1} (nload_at in grid2d.cu) and the density stencil from the two
+// triangle formulas above.  s60, s90, s180 = |K| / 60, / 90, / 180.
+__global__ void k_nload_density2d_node(int n, int pitch, size_t st, double s60, double s90,
+                                       double s180, const double* __restrict__ u,
                                        double* __restrict__ nl, double* __restrict__ bC,
                                        double* __restrict__ bE, double* __restrict__ bN,
                                        double* __restrict__ bNE) {
@@ -92,126 +89,41 @@ __global__ void k_nload_density2d_node(int n, int pitch, size_t st, T s60, T s90
   const int j = 1 + blockIdx.y * blockDim.y + threadIdx.y;
   if (i >= n || j >= n) return;
   const size_t k = blockIdx.z * st + at(i, j, pitch);
-  const T up = get<T>(u, k);
-  const T nE = get<T>(u, k + 1), nNE = get<T>(u, k + pitch + 1), nN = get<T>(u, k + pitch);
-  const T nW = get<T>(u, k - 1), nSW = get<T>(u, k - pitch - 1), nS = get<T>(u, k - pitch);
+  const double up = u[k];
+  const double nE = u[k + 1], nNE = u[k + pitch + 1], nN = u[k + pitch];
+  const double nW = u[k - 1], nSW = u[k - pitch - 1], nS = u[k - pitch];
   // the cubic load through the pair sums m_k = n_k + n_{k+1} (see nload_at in grid2d.cu)
-  const T m0 = nE + nNE, m1 = nNE + nN, m2 = nN + nW, m3 = nW + nSW, m4 = nSW + nS,
+  const double m0 = nE + nNE, m1 = nNE + nN, m2 = nN + nW, m3 = nW + nSW, m4 = nSW + nS,
           m5 = nS + nE;
-  const T qE = nE * nE, qNE = nNE * nNE, qN = nN * nN, qW = nW * nW, qSW = nSW * nSW,
+  const double qE = nE * nE, qNE = nNE * nNE, qN = nN * nN, qW = nW * nW, qSW = nSW * nSW,
           qS = nS * nS;
-  const T M1 = ((m0 + m1) + (m2 + m3)) + (m4 + m5);  // 2 S1
-  T M2 = m0 * m0;
+  const double M1 = ((m0 + m1) + (m2 + m3)) + (m4 + m5);  // 2 S1
+  double M2 = m0 * m0;
   M2 = fma(m1, m1, M2);
   M2 = fma(m2, m2, M2);
   M2 = fma(m3, m3, M2);
   M2 = fma(m4, m4, M2);
   M2 = fma(m5, m5, M2);
-  const T s2 = ((qE + qNE) + (qN + qW)) + (qSW + qS);
-  T M3 = m0 * (qE + qNE);
+  const double s2 = ((qE + qNE) + (qN + qW)) + (qSW + qS);
+  double M3 = m0 * (qE + qNE);
   M3 = fma(m1, qNE + qN, M3);
   M3 = fma(m2, qN + qW, M3);
   M3 = fma(m3, qW + qSW, M3);
   M3 = fma(m4, qSW + qS, M3);
   M3 = fma(m5, qS + qE, M3);
-  const T u2 = up * up;
-  const T s2p = fma(T(0.5), M2, s2);  // 2 S2 + P
-  nl[k] = out_of(s60 * (fma(T(2) * up, s2p, u2 * fma(T(24), up, T(3) * M1)) + M3));
+  const double u2 = up * up;
+  const double s2p = fma(0.5, M2, s2);  // 2 S2 + P
+  nl[k] = s60 * (fma(2.0 * up, s2p, u2 * fma(24.0, up, 3.0 * M1)) + M3);
   // density stencil, diagonal: sum over the six triangles
-  put_entry(bC, k, s90 * fma(T(36), u2, fma(T(3) * up, M1, s2p)));
+  bC[k] = s90 * fma(36.0, u2, fma(3.0 * up, M1, s2p));
   // edge p-q shared by the triangles closed by r1 and r2
-  const T u26 = T(6) * u2;
-  put_entry(bE, k, s180 * fma(T(6), qE,
-                              u26 + fma(T(8) * up, nE, fma(T(2) * (up + nE), nNE + nS, qNE + qS))));
-  put_entry(bN, k, s180 * fma(T(6), qN,
-                              u26 + fma(T(8) * up, nN, fma(T(2) * (up + nN), nNE + nW, qNE + qW))));
-  put_entry(bNE, k, s180 * fma(T(6), qNE,
-                               u26 + fma(T(8) * up, nNE, fma(T(2) * (up + nNE), nE + nN, qE + qN))));
-}
-
-// Galerkin coarsening of a 7-point stencil: Bc(a,b) = sum_{v,w} P_va P_wb B(v,w).  The
-// fine support of coarse hat a is 2a plus the offsets below with weights 1 and 1/2.
-__device__ constexpr int kSX[7] = {0, 1, -1, 0, 0, 1, -1};
-__device__ constexpr int kSY[7] = {0, 0, 0, 1, -1, 1, -1};
-
-template <typename T>
-__device__ __forceinline__ T fine_entry(const double* bC, const double* bE, const double* bN,
-                                        const double* bNE, size_t kv, int dx, int dy,
-                                        int pitch) {
-  if (dx == 0 && dy == 0) return get_entry<T>(bC, kv);
-  if (dx == 1 && dy == 0) return get_entry<T>(bE, kv);
-  if (dx == -1 && dy == 0) return get_entry<T>(bE, kv - 1);
-  if (dx == 0 && dy == 1) return get_entry<T>(bN, kv);
-  if (dx == 0 && dy == -1) return get_entry<T>(bN, kv - pitch);
-  if (dx == 1 && dy == 1) return get_entry<T>(bNE, kv);
-  return get_entry<T>(bNE, kv - pitch - 1);  // dx == dy == -1
-}
-
-__host__ __device__ constexpr bool in_stencil(int dx, int dy) {
-  return (dx == 0 && dy == 0) || (dx == 1 && dy == 0) || (dx == -1 && dy == 0) ||
-         (dx == 0 && dy == 1) || (dx == 0 && dy == -1) || (dx == 1 && dy == 1) ||
-         (dx == -1 && dy == -1);
-}
-
-// FP64: one FMA per pair.  Double-float: the entries (int u~^2 phi phi) are non-negative, so
-// they are summed per weight class (1, 1/2, 1/4) with double-float additions, three
-// independent chains, and scaled exactly once at the end.  The diagonal entry (TX = TY = 0)
-// pairs both supports with themselves, and (p, q), (q, p) read the same fine entry, so it
-// takes each unordered pair once with twice its weight (an exact doubling).
-template <typename T, int TX, int TY>
-__device__ __forceinline__ T coarse_entry(const double* bC, const double* bE, const double* bN,
-                                          const double* bNE, size_t kf, int pf) {
-  constexpr bool kDiag = TX == 0 && TY == 0;
-  T acc = 0;
-  T part[3] = {T(0), T(0), T(0)};
-#pragma unroll
-  for (int p = 0; p < 7; ++p) {
-#pragma unroll
-    for (int q = kDiag ? p : 0; q < 7; ++q) {
-      const int dx = 2 * TX + kSX[q] - kSX[p];
-      const int dy = 2 * TY + kSY[q] - kSY[p];
-      if (in_stencil(dx, dy)) {
-        const size_t kv = kf + (long)kSY[p] * pf + kSX[p];
-        const bool twice_w = kDiag && q != p;
-        if constexpr (std::is_same<T, dfloat>::value) {
-          const dfloat e = fine_entry<T>(bC, bE, bN, bNE, kv, dx, dy, pf);
-          part[(p != 0) + (q != 0)] += twice_w ? twice(e) : e;
-        } else {
-          const T w((twice_w ? 2.0 : 1.0) * (p == 0 ? 1.0 : 0.5) * (q == 0 ? 1.0 : 0.5));
-          acc = fma(w, fine_entry<T>(bC, bE, bN, bNE, kv, dx, dy, pf), acc);
-        }
-      }
-    }
-  }
-  if constexpr (std::is_same<T, dfloat>::value) {
-    const dfloat h1(part[1].hi * 0.5f, part[1].lo * 0.5f);
-    const dfloat h2(part[2].hi * 0.25f, part[2].lo * 0.25f);
-    acc = part[0] + (h1 + h2);
-  }
-  return acc;
-}
-
-// T = double (FP64 mode) or dfloat (mixed modes: entries stored split, see put_entry)
-template <typename T>
-__global__ void k_coarsen_density2d(int nc, int pc, int pf, size_t stc, size_t stf,
-                                    const double* __restrict__ fC,
-                                    const double* __restrict__ fE,
-                                    const double* __restrict__ fN,
-                                    const double* __restrict__ fNE, double* __restrict__ cC,
-                                    double* __restrict__ cE, double* __restrict__ cN,
-                                    double* __restrict__ cNE) {
-  const int I = 1 + blockIdx.x * blockDim.x + threadIdx.x;
-  const int J = 1 + blockIdx.y * blockDim.y + threadIdx.y;
-  if (I >= nc || J >= nc) return;
-  const size_t kf = blockIdx.z * stf + at(2 * I, 2 * J, pf);
-  const size_t kc = blockIdx.z * stc + at(I, J, pc);
-  put_entry(cC, kc, coarse_entry<T, 0, 0>(fC, fE, fN, fNE, kf, pf));
-  // couplings to coarse neighbours outside the interior are never read; skip them so no
-  // fine entry beyond the interior is touched
-  if (I + 1 < nc) put_entry(cE, kc, coarse_entry<T, 1, 0>(fC, fE, fN, fNE, kf, pf));
-  if (J + 1 < nc) put_entry(cN, kc, coarse_entry<T, 0, 1>(fC, fE, fN, fNE, kf, pf));
-  if (I + 1 < nc && J + 1 < nc)
-    put_entry(cNE, kc, coarse_entry<T, 1, 1>(fC, fE, fN, fNE, kf, pf));
+  const double u26 = 6.0 * u2;
+  bE[k] = s180 * fma(6.0, qE,
+                     u26 + fma(8.0 * up, nE, fma(2.0 * (up + nE), nNE + nS, qNE + qS)));
+  bN[k] = s180 * fma(6.0, qN,
+                     u26 + fma(8.0 * up, nN, fma(2.0 * (up + nN), nNE + nW, qNE + qW)));
+  bNE[k] = s180 * fma(6.0, qNE,
+                      u26 + fma(8.0 * up, nNE, fma(2.0 * (up + nNE), nE + nN, qE + qN)));
 }
 
 // ---- T3 class sums -----------------------------------------------------------------------
@@ -370,7 +282,7 @@ __global__ void k_t3_finalize2d(int cells, int chunks, double h2, size_t pst, si
 
 __global__ void k_gather_level1_2d(int n, int pitch, size_t st, const double* __restrict__ gA_pad,
                                    const double* __restrict__ gM_pad,
-                                   const double* __restrict__ t1_pad, Density2D b, int split,
+                                   const double* __restrict__ t1_pad, Density2D b,
                                    double* __restrict__ gA, double* __restrict__ gM,
                                    double* __restrict__ t1, double* __restrict__ B1) {
   const int m = n - 1;
@@ -385,12 +297,11 @@ __global__ void k_gather_level1_2d(int n, int pitch, size_t st, const double* __
   t1[q] = t1_pad[k];
   double* row = B1 + blockIdx.y * nh * nh + (size_t)p * nh;
   for (int q = 0; q < m * m; ++q) row[q] = 0.0;
-  const bool sp = split != 0;  // entries stored as double-float splits (mixed modes)
-  row[p] = entry_fp64(b.C, k, sp);
+  row[p] = b.C[k];
   auto put = [&](int di, int dj, const double* a, size_t ka) {
     const int ii = i + di, jj = j + dj;
     if (ii < 1 || jj < 1 || ii >= n || jj >= n) return;
-    row[(ii - 1) + (jj - 1) * m] = entry_fp64(a, ka, sp);
+    row[(ii - 1) + (jj - 1) * m] = a[ka];
   };
   put(1, 0, b.E, k);
   put(-1, 0, b.E, k - 1);
@@ -413,38 +324,25 @@ dim3 grid_of(const Grid& g, int cx, int cy) {
 
 void nload_density2d(const Grid& g, const double* u, double* nl, const Density2D& b,
                      cudaStream_t s) {
-  if (!star2d_walks(g)) {
-    k_nload_density2d_node<double, const double*>
-        <<<grid_of(g, g.n - 1, g.n - 1), dim3(g.bx, g.by), 0, s>>>(
-            g.n, g.pitch, g.stride, g.h * g.h / 120.0, g.h * g.h / 180.0, g.h * g.h / 360.0, u,
-            nl, b.C, b.E, b.N, b.NE);
+  if (!star2d_rows(g)) {
+    k_nload_density2d_node<<<grid_of(g, g.n - 1, g.n - 1), dim3(g.bx, g.by), 0, s>>>(
+        g.n, g.pitch, g.stride, g.h * g.h / 120.0, g.h * g.h / 180.0, g.h * g.h / 360.0, u, nl,
+        b.C, b.E, b.N, b.NE);
     return;
   }
-  k_nload_density2d<<<star2d_grid(g.n, g.nb), star2d_block(), 0, s>>>(
-      g.n, g.pitch, g.stride, g.h * g.h / 120.0, g.h * g.h / 360.0, u, nl, b.C, b.E, b.N, b.NE);
-}
-
-void nload_density2d_df(const Grid& g, SplitVec u, double* nl, const Density2D& b,
-                        cudaStream_t s) {
-  k_nload_density2d_node<dfloat, SplitVec><<<grid_of(g, g.n - 1, g.n - 1), dim3(g.bx, g.by), 0, s>>>(
-      g.n, g.pitch, g.stride, dfloat(g.h * g.h / 120.0), dfloat(g.h * g.h / 180.0),
-      dfloat(g.h * g.h / 360.0), u, nl, b.C, b.E, b.N, b.NE);
-}
-
-void coarsen_density2d_df(const Grid& fine, const Grid& coarse, const Density2D& bf,
-                          const Density2D& bc, cudaStream_t s) {
-  const dim3 grid = grid_of(fine, coarse.n - 1, coarse.n - 1), block(fine.bx, fine.by);
-  k_coarsen_density2d<dfloat><<<grid, block, 0, s>>>(
-      coarse.n, coarse.pitch, fine.pitch, coarse.stride, fine.stride, bf.C, bf.E, bf.N, bf.NE,
-      bc.C, bc.E, bc.N, bc.NE);
+  star2d_dispatch(g, [&](auto r) {
+    k_nload_density2d<r><<<star2d_grid(g.n, g.nb, r), star2d_block(), 0, s>>>(
+        g.n, g.pitch, g.stride, g.h * g.h / 120.0, g.h * g.h / 360.0, u, nl, b.C, b.E, b.N,
+        b.NE);
+  });
 }
 
 void gather_level1_2d(const Grid& g1, const double* gA_pad, const double* gM_pad,
                       const double* t1_pad, const Density2D& b1, double* gA, double* gM,
-                      double* t1, double* B1, cudaStream_t s, bool split) {
+                      double* t1, double* B1, cudaStream_t s) {
   const int m = g1.n - 1;
   k_gather_level1_2d<<<dim3((m * m + 63) / 64, g1.nb), 64, 0, s>>>(
-      g1.n, g1.pitch, g1.stride, gA_pad, gM_pad, t1_pad, b1, split ? 1 : 0, gA, gM, t1, B1);
+      g1.n, g1.pitch, g1.stride, gA_pad, gM_pad, t1_pad, b1, gA, gM, t1, B1);
 }
 
 size_t t3_partials2d(const Grid& fine, int n1) {

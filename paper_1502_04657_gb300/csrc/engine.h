@@ -30,7 +30,7 @@ struct Level {
   // mixed precision: FP32 coefficient tables and single-precision V-cycle vectors
   CoefT ct{};
   float *x32 = nullptr, *xt32 = nullptr, *f32 = nullptr, *r32 = nullptr;
-  // mixed precision: double-float split (hi + lo) of the vector the nonlinear kernels read
+  // 3D mixed precision: double-float split (hi + lo) of the vector the nonlinear kernels read
   float *uhi = nullptr, *ulo = nullptr;
   // mixed precision, large 2D levels: tensor maps of the two x buffers (tile + halo box) and
   // of f32 (tile box) for the TMA-fed sweeps; tm_base[q] is the buffer tm_x[q] describes
@@ -120,6 +120,8 @@ struct fmg_eig_handle {
   bool literal() const { return prob.operator_form == FMG_PAPER_LITERAL; }
   bool mixed() const { return prob.precision != FMG_FP64; }
   bool bf16() const { return prob.precision == FMG_MIXED_BF16; }
+  // the nonlinear kernels compute in double-float arithmetic (3D mixed modes)
+  bool dfloat_loads() const { return mixed() && prob.dim == 3; }
   // profiling: event pairs around the first finest-level launch of each profiled step
   cudaEvent_t prof[fmg::kProfCount][2] = {};
   bool prof_armed[fmg::kProfCount] = {};

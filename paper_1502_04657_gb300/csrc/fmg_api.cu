@@ -87,8 +87,7 @@ void lv_mass(Level& l, const double* x, double* y, cudaStream_t s) {
   else mass3d(l.g, x, y, s);
 }
 void lv_mass_df(Level& l, SplitVec x, double* y, cudaStream_t s) {
-  if (l.g.dim == 2) mass2d_df(l.g, x, y, s);
-  else mass3d_df(l.g, x, y, s);
+  mass3d_df(l.g, x, y, s);
 }
 void lv_jacobi(Level& l, const double* f, const double* x, double* xo, bool zero, cudaStream_t s) {
   if (l.g.dim == 2) jacobi2d(l.g, l.c, f, x, xo, zero, s);
@@ -131,7 +130,7 @@ void lv_nload_density(Level& l, const double* u, double* nl, cudaStream_t s) {
   if (l.g.dim == 2) nload_density2d(l.g, u, nl, l.b, s);
   else nload_density3d(l.g, u, nl, l.b3, s);
 }
-// Mixed-precision modes: the nonlinear kernels compute in double-float arithmetic from the
+// 3D mixed-precision modes: the nonlinear kernels compute in double-float arithmetic from the
 // split of u into l.uhi + l.ulo (written here, on the same stream, just before).
 SplitVec lv_split(Level& l, const double* u, cudaStream_t s) {
   split_df(u, l.uhi, l.ulo, l.g.stride * l.g.nb, s);
@@ -140,16 +139,14 @@ SplitVec lv_split(Level& l, const double* u, cudaStream_t s) {
 void lv_rhs_df(Level& l, const double* lam, const PotentialParams* p, const double* u, double* f,
                cudaStream_t s) {
   const SplitVec v = lv_split(l, u, s);
-  if (l.g.dim == 2) rhs2d_df(l.g, lam, p, v, f, s);
-  else rhs3d_df(l.g, lam, p, v, f, s);
+  rhs3d_df(l.g, lam, p, v, f, s);
 }
 void lv_nload_density_df(Level& l, SplitVec v, double* nl, cudaStream_t s) {
-  if (l.g.dim == 2) nload_density2d_df(l.g, v, nl, l.b, s);
-  else nload_density3d_df(l.g, v, nl, l.b3, s);
+  nload_density3d_df(l.g, v, nl, l.b3, s);
 }
-// split: the density stencils hold double-float splits (mixed modes, from the _df kernels)
+// split: the density stencils hold double-float splits (3D mixed modes, from the _df kernels)
 void lv_coarsen_density(Level& fl, Level& cl, cudaStream_t s, bool split) {
-  if (fl.g.dim == 2) (split ? coarsen_density2d_df : coarsen_density2d)(fl.g, cl.g, fl.b, cl.b, s);
+  if (fl.g.dim == 2) coarsen_density2d(fl.g, cl.g, fl.b, cl.b, s);
   else (split ? coarsen_density3d_df : coarsen_density3d)(fl.g, cl.g, fl.b3, cl.b3, s);
 }
 // npinned: the leading instances that keep the pinned order of summation (3D)
@@ -179,7 +176,7 @@ void lv_start(Level& l1, double* c, int cstride, cudaStream_t s) {
 void lv_gather_level1(Level& l1, double* gA, double* gM, double* t1, double* B1, cudaStream_t s,
                       bool split) {
   if (l1.g.dim == 2) {
-    gather_level1_2d(l1.g, l1.y, l1.z, l1.r, l1.b, gA, gM, t1, B1, s, split);
+    gather_level1_2d(l1.g, l1.y, l1.z, l1.r, l1.b, gA, gM, t1, B1, s);
   } else {
     gather_vec3d(l1.g, l1.y, l1.z, l1.r, gA, gM, t1, s);
     density_dense3d(l1.g, l1.b3, B1, s, split);
@@ -379,8 +376,10 @@ void build_levels(fmg_eig_handle* h) {
       l.xt32 = single();
       l.f32 = single();
       l.r32 = single();
-      l.uhi = h->alloc<float>(s);
-      l.ulo = h->alloc<float>(s);
+      if (h->dfloat_loads()) {
+        l.uhi = h->alloc<float>(s);
+        l.ulo = h->alloc<float>(s);
+      }
       if (!h->dry && tma_sweep_applies(l.g) && !(h->prob.flags & FMG_FLAG_NO_TMA)) {
         const bool bf = h->bf16();
         l.tma = encode_level_map(l.g, l.cap, l.x32, bf, true, &l.tm_x[0]) &&
@@ -928,22 +927,23 @@ void enqueue_augment(fmg_eig_handle* h, int k, const double* ut, cudaStream_t s)
   Level& l = h->L(k);
   const int nb = l.g.nb;
   const size_t st = l.g.stride;
-  // mixed modes: the double-float split of u~, read by N(u~) / B(u~) and by the mass apply
-  const SplitVec us = h->mixed() ? lv_split(l, ut, s) : SplitVec{};
+  // 3D mixed modes: the double-float split of u~, read by N(u~) / B(u~) and by the mass apply
+  const bool df = h->dfloat_loads();
+  const SplitVec us = df ? lv_split(l, ut, s) : SplitVec{};
   fork_sides(h, s, 0, 2);
   // branch 1 (side 0): N(u~) and B(u~), T0, and the restriction / coarsening chains of both.
-  // They run on the integer (FP64 mode) or FP32 pipes (mixed modes), beside the FP64 T3 sums
+  // They run on the integer or FP32 pipes (3D mixed modes), beside the FP64 T3 sums
   // and applies of the other branches.
   {
     const cudaStream_t b1 = h->side[0];
     prof_begin(h, kProfMoments, k, b1);
-    if (h->mixed()) lv_nload_density_df(l, us, l.r, b1);
+    if (df) lv_nload_density_df(l, us, l.r, b1);
     else lv_nload_density(l, ut, l.r, b1);
     prof_end(h, kProfMoments, k, b1);
     dot(ut, l.r, st, h->partials2, h->t0, b1, nb, st);
     for (int j = k; j >= 2; --j) {
       lv_restrict(h->L(j), h->L(j - 1), h->L(j).r, h->L(j - 1).r, b1);
-      lv_coarsen_density(h->L(j), h->L(j - 1), b1, h->mixed());
+      lv_coarsen_density(h->L(j), h->L(j - 1), b1, df);
     }
   }
   // branch 2 (side 1): T3 per coarse simplex
@@ -953,11 +953,11 @@ void enqueue_augment(fmg_eig_handle* h, int k, const double* ut, cudaStream_t s)
     lv_t3(l, h->prob.coarse_cells, h->npinned, ut, h->t3_partials, h->t3, b2);
     prof_end(h, kProfT3, k, b2);
   }
-  // main branch: (A + W) u~, M u~, their dots and restriction chains.  The mixed modes form
+  // main branch: (A + W) u~, M u~, their dots and restriction chains.  The 3D mixed modes form
   // M u~ in double-float on the FP32 pipes (positive weights: ~2^-47 of the result); the
   // operator apply stays FP64 (its stencil cancels to O(h^2) of its terms).
   lv_apply_full(l, ut, l.y, s);
-  if (h->mixed()) lv_mass_df(l, us, l.z, s);
+  if (df) lv_mass_df(l, us, l.z, s);
   else lv_mass(l, ut, l.z, s);
   dot(ut, l.y, st, h->partials, h->auu, s, nb, st);
   dot(ut, l.z, st, h->partials, h->buu, s, nb, st);
@@ -965,7 +965,7 @@ void enqueue_augment(fmg_eig_handle* h, int k, const double* ut, cudaStream_t s)
     lv_restrict(h->L(j), h->L(j - 1), h->L(j).y, h->L(j - 1).y, s, h->L(j).z, h->L(j - 1).z);
   join_sides(h, s, 0, 2);
   Level& l1 = h->L(1);
-  lv_gather_level1(l1, h->gAd, h->gMd, h->t1d, h->B1d, s, h->mixed());
+  lv_gather_level1(l1, h->gAd, h->gMd, h->t1d, h->B1d, s, df);
 }
 
 DenseProblem dense_augmented(fmg_eig_handle* h) {
@@ -991,7 +991,7 @@ void enqueue_correction(fmg_eig_handle* h, int k, cudaStream_t s) {
   prof_begin(h, kProfRhs, k, s);
   if (h->mixed() && (h->prob.flags & FMG_FLAG_FP32_RHS))
     lv_rhs_f32(l, h->lam, h->dparams, l.u, l.f, s);
-  else if (h->mixed())
+  else if (h->dfloat_loads())
     lv_rhs_df(l, h->lam, h->dparams, l.u, l.f, s);
   else lv_rhs(l, h->lam, h->dparams, l.u, l.f, s);
   if (h->literal()) lv_sub_wmass(l, l.u, l.f, s);
@@ -1086,7 +1086,7 @@ void time_mix(fmg_eig_handle* h, Level& l, int k, cudaStream_t s) {
     else
       lv_jacobi(l, l.f, l.x, l.xt, false, s);
   }
-  if (h->mixed()) {
+  if (h->dfloat_loads()) {
     lv_nload_density_df(l, lv_split(l, l.u, s), l.r, s);
     lv_rhs_df(l, h->lam, h->dparams, l.u, l.f, s);
   } else {

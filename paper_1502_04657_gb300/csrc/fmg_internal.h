@@ -95,7 +95,6 @@ void coef2d_setup(const Grid& g, const PotentialParams* p_dev, const Coef2D& c, 
 void apply2d(const Grid& g, const Coef2D& c, const double* x, double* y, cudaStream_t s);
 void mass2d(const Grid& g, const double* x, double* y, cudaStream_t s);
 // the same from the double-float split of x (mixed-precision modes)
-void mass2d_df(const Grid& g, SplitVec x, double* y, cudaStream_t s);
 // f -= W u, W u = (A + W) u - A u from the coefficient sets cw (A + W) and ca (A)
 void sub_wmass2d(const Grid& g, const Coef2D& cw, const Coef2D& ca, const double* u, double* f,
                  cudaStream_t s);
@@ -122,8 +121,6 @@ void rhs2d(const Grid& g, const double* lam, const PotentialParams* p_dev, const
 void rhs2d_f32(const Grid& g, const double* lam, const PotentialParams* p_dev, const double* u,
                double* f, cudaStream_t s);
 // the same right-hand side in double-float arithmetic from the split u (mixed-precision modes)
-void rhs2d_df(const Grid& g, const double* lam, const PotentialParams* p_dev, SplitVec u,
-              double* f, cudaStream_t s);
 // Dense level-1 matrices L_1 and M_1 (n1-1)^2 square, row-major, interior numbering (one
 // pair per instance, back to back).
 void dense_level1_2d(const Grid& g, const Coef2D& c, double* L, double* M, cudaStream_t s);
@@ -325,14 +322,9 @@ struct Density2D {
 // nl = N(u) (int u^3 phi_p) and the density stencil of u on level g, in one pass.
 void nload_density2d(const Grid& g, const double* u, double* nl, const Density2D& b,
                      cudaStream_t s);
-void nload_density2d_df(const Grid& g, SplitVec u, double* nl, const Density2D& b,
-                        cudaStream_t s);
-// Galerkin coarsening of the density stencil: bc = P^T bf P (coarsen_fx.cu; _df: the entries
-// are stored as double-float splits, see nload_density*_df).
+// Galerkin coarsening of the density stencil: bc = P^T bf P (coarsen_fx.cu).
 void coarsen_density2d(const Grid& fine, const Grid& coarse, const Density2D& bf,
                        const Density2D& bc, cudaStream_t s);
-void coarsen_density2d_df(const Grid& fine, const Grid& coarse, const Density2D& bf,
-                          const Density2D& bc, cudaStream_t s);
 // T3^T_abc = int_T u mu_a mu_b mu_c per coarse triangle (10 per triangle, a <= b <= c,
 // lexicographic), from per-class monomial sums.  pw: (x/r)^m table of the level, map: the
 // level's 2 x 10 x 25 map (t3_map2d), partials: t3_partials2d(fine, n1) doubles.
@@ -346,7 +338,7 @@ void t3_power_table(int r, double* out);  // 4 * (r + 1) doubles
 // level-1 vectors and the level-1 density stencil (per instance, back to back)
 void gather_level1_2d(const Grid& g1, const double* gA_pad, const double* gM_pad,
                       const double* t1_pad, const Density2D& b1, double* gA, double* gM,
-                      double* t1, double* B1, cudaStream_t s, bool split = false);
+                      double* t1, double* B1, cudaStream_t s);
 
 // ---- Dense small solves (dense.cu) -------------------------------------------------------
 // A batch of problems shares the geometry (tri, lists) and keeps the per-instance arrays

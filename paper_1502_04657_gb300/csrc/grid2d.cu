@@ -136,18 +136,6 @@ __global__ void k_mass2d(int n, int pitch, size_t st, double h2_12, const double
   y[k] = h2_12 * fma(6.0, x[k], s);
 }
 
-// The same mass apply in double-float arithmetic from the split of x (mixed-precision modes'
-// augmented pass): every weight is positive, so the sloppy double-float sums keep ~2^-47 of
-// the result; FP64 output.
-__global__ void k_mass2d_df(int n, int pitch, size_t st, dfloat h2_12, SplitVec x,
-                            double* __restrict__ y) {
-  INTERIOR_2D
-  auto X = [&](size_t q) { return get<dfloat>(x, q); };
-  const dfloat s = ((X(k + 1) + X(k - 1)) + (X(k + pitch) + X(k - pitch))) +
-                   (X(k + pitch + 1) + X(k - pitch - 1));
-  y[k] = to_double(h2_12 * fma(dfloat(6), X(k), s));
-}
-
 __global__ void k_jacobi2d(int n, int pitch, size_t st, Coef2D c, const double* __restrict__ f,
                            const double* __restrict__ x, double* __restrict__ xo) {
   INTERIOR_2D
@@ -268,11 +256,9 @@ __global__ void k_prolong2d(int nc, int pf, int pc, size_t st, size_t stc,
 // Through the pair sums m_k = n_k + n_{k+1} and squares q_k = n_k^2 (2 S1 = M1 = sum m_k,
 // 2 (2 S2 + P) = M2 + 2 S2 with M2 = sum m_k^2, 2 S3 + Q = M3 = sum m_k (q_k + q_{k+1})):
 //   |K|/60 [u^2 (24u + 3 M1) + u (M2 + 2 S2) + M3].
-// This per-node form serves the double-float and single-precision right-hand sides (T =
-// dfloat with u read as a SplitVec, or float) and the FP64 kernels of small launches; large
-// FP64 launches evaluate the same sums per mesh edge (star2d.cuh), which saves FP64
-// instructions but, in double-float arithmetic, loses more to the longer dependency chains
-// and lane shuffles than it saves.
+// This per-node form serves the single-precision right-hand side (T = float) and the FP64
+// kernels of the smallest levels; the others evaluate the same sums per mesh edge in fixed
+// point (star2d.cuh).
 // M1 (twice the neighbour sum) is returned through m1_out when given: the mass stencil of
 // the right-hand side needs the same sum.
 template <typename T, typename U = const double*>
@@ -302,7 +288,7 @@ __device__ __forceinline__ T nload_at(const U& u, size_t k, int pitch, T* m1_out
   return v + M3;
 }
 
-// FP64 node by node, for launches too small to fill the GPU as column walks
+// FP64 node by node, for levels below n = 64
 __global__ void k_nload2d_node(int n, int pitch, size_t st, double scale,
                                const double* __restrict__ u, double* __restrict__ out) {
   INTERIOR_2D
@@ -322,68 +308,57 @@ __global__ void k_rhs2d_node(int n, int pitch, size_t st, double h2_12, double h
 
 // The FP64 cubic-load kernels below walk columns (star2d.cuh) in fixed point (fixed.cuh), the
 // warps whose tile that does not take in FP64: launch with star2d_grid / star2d_block.
+template <int R>
 __device__ __noinline__ void nload2d_fp64(int n, int pitch, size_t st, double scale,
                                           const double* __restrict__ u,
                                           double* __restrict__ out) {
-  star2d_walk<double>(n, pitch, st, u, [&](size_t k, const Star2D<double>& p) {
+  star2d_walk<double, R>(n, pitch, st, u, [&](size_t k, const Star2D<double>& p) {
     out[k] = scale * star_cubic(p);
   });
 }
 
+template <int R>
 __device__ __noinline__ void rhs2d_fp64(int n, int pitch, size_t st, double h2_24, double nscale,
                                         double l, const double* __restrict__ u,
                                         double* __restrict__ f) {
-  star2d_walk<double>(n, pitch, st, u, [&](size_t k, const Star2D<double>& p) {
+  star2d_walk<double, R>(n, pitch, st, u, [&](size_t k, const Star2D<double>& p) {
     const double mu = h2_24 * fma(12.0, p.u, p.M1);
     f[k] = fma(l, mu, -nscale * star_cubic(p));
   });
 }
 
+template <int R>
 __global__ void __launch_bounds__(32 * kStarWarps, 4)
     k_nload2d(int n, int pitch, size_t st, double scale, const double* __restrict__ u,
               double* __restrict__ out) {
-  const int e = star2d_exponent(n, pitch, st, u);
+  const int e = star2d_exponent<R>(n, pitch, st, u);
   if (e == kFxNone) {
-    nload2d_fp64(n, pitch, st, scale, u, out);
+    nload2d_fp64<R>(n, pitch, st, scale, u, out);
     return;
   }
   const double s = fx_scale<kFx2>(scale, 3, e);
-  star2d_walk_fx<false>(n, pitch, st, u, e, [&](size_t k, const Star2DFx& p) {
+  star2d_walk_fx<false, R>(n, pitch, st, u, e, [&](size_t k, const Star2DFx& p) {
     out[k] = to_double(star_cubic(p), s);
   });
 }
 
 // f = lambda M u - N(u); the mass stencil h^2/12 (6 u_p + neighbour sum) reuses the cubic
 // load's M1 (twice the neighbour sum): h^2/24 (12 u_p + M1)
+template <int R>
 __global__ void __launch_bounds__(32 * kStarWarps, 4)
     k_rhs2d(int n, int pitch, size_t st, double h2_24, double h2_120,
             const double* __restrict__ lam, const PotentialParams* __restrict__ pp,
             const double* __restrict__ u, double* __restrict__ f) {
   const double nscale = pp[blockIdx.z].zeta * h2_120, l = lam[blockIdx.z];
-  const int e = star2d_exponent(n, pitch, st, u);
+  const int e = star2d_exponent<R>(n, pitch, st, u);
   if (e == kFxNone) {
-    rhs2d_fp64(n, pitch, st, h2_24, nscale, l, u, f);
+    rhs2d_fp64<R>(n, pitch, st, h2_24, nscale, l, u, f);
     return;
   }
   const double s1 = l * fx_scale<kFx2>(h2_24, 1, e), s3 = fx_scale<kFx2>(nscale, 3, e);
-  star2d_walk_fx<false>(n, pitch, st, u, e, [&](size_t k, const Star2DFx& p) {
+  star2d_walk_fx<false, R>(n, pitch, st, u, e, [&](size_t k, const Star2DFx& p) {
     f[k] = fma(s1, __ll2double_rn(madd<12>(p.u, p.M1).v), -to_double(star_cubic(p), s3));
   });
-}
-
-// The same right-hand side in double-float arithmetic from the split u (mixed-precision
-// modes): ~2^-47 relative rounding per operation on the FP32 pipes; the FP64 result combines
-// the two FP64-converted parts.
-// The scales h^2/12 and h^2/120 arrive as double-float constants, so each node spends only
-// the two FP64 conversions and the final combination on the FP64 pipe.
-__global__ void k_rhs2d_df(int n, int pitch, size_t st, dfloat h2_12, dfloat h2_120,
-                           const double* __restrict__ lam, const PotentialParams* __restrict__ pp,
-                           SplitVec u, double* __restrict__ f) {
-  INTERIOR_2D
-  dfloat m1;  // twice the sum of the six neighbours
-  const double nl = to_double(h2_120 * nload_at<dfloat>(u, k, pitch, &m1));
-  const double mu = to_double(h2_12 * fma(dfloat(6), get<dfloat>(u, k), dfloat(0.5) * m1));
-  f[k] = fma(lam[ib], mu, -pp[ib].zeta * nl);
 }
 
 // FP32 auxiliary right-hand side of the mixed-precision iteration (same closed forms in
@@ -475,11 +450,6 @@ void mass2d(const Grid& g, const double* x, double* y, cudaStream_t s) {
                                                                  g.h * g.h / 12.0, x, y);
 }
 
-void mass2d_df(const Grid& g, SplitVec x, double* y, cudaStream_t s) {
-  k_mass2d_df<<<grid_of(g, g.n - 1, g.n - 1), block_of(g), 0, s>>>(
-      g.n, g.pitch, g.stride, dfloat(g.h * g.h / 12.0), x, y);
-}
-
 void jacobi2d(const Grid& g, const Coef2D& c, const double* f, const double* x, double* xo,
               bool x_is_zero, cudaStream_t s) {
   if (c.fxt && !x_is_zero) {
@@ -530,36 +500,34 @@ void prolong2d(const Grid& fine, const Grid& coarse, const double* ec, double* x
 }
 
 void nload2d(const Grid& g, const double* u, double* out, cudaStream_t s) {
-  if (!star2d_walks(g)) {
+  if (!star2d_rows(g)) {
     k_nload2d_node<<<grid_of(g, g.n - 1, g.n - 1), block_of(g), 0, s>>>(
         g.n, g.pitch, g.stride, g.h * g.h / 120.0, u, out);
     return;
   }
-  k_nload2d<<<star2d_grid(g.n, g.nb), star2d_block(), 0, s>>>(g.n, g.pitch, g.stride,
-                                                               g.h * g.h / 120.0, u, out);
+  star2d_dispatch(g, [&](auto r) {
+    k_nload2d<r><<<star2d_grid(g.n, g.nb, r), star2d_block(), 0, s>>>(g.n, g.pitch, g.stride,
+                                                                      g.h * g.h / 120.0, u, out);
+  });
 }
 
 void rhs2d(const Grid& g, const double* lam, const PotentialParams* p, const double* u,
            double* f, cudaStream_t s) {
-  if (!star2d_walks(g)) {
+  if (!star2d_rows(g)) {
     k_rhs2d_node<<<grid_of(g, g.n - 1, g.n - 1), block_of(g), 0, s>>>(
         g.n, g.pitch, g.stride, g.h * g.h / 12.0, g.h * g.h / 120.0, lam, p, u, f);
     return;
   }
-  k_rhs2d<<<star2d_grid(g.n, g.nb), star2d_block(), 0, s>>>(
-      g.n, g.pitch, g.stride, g.h * g.h / 24.0, g.h * g.h / 120.0, lam, p, u, f);
+  star2d_dispatch(g, [&](auto r) {
+    k_rhs2d<r><<<star2d_grid(g.n, g.nb, r), star2d_block(), 0, s>>>(
+        g.n, g.pitch, g.stride, g.h * g.h / 24.0, g.h * g.h / 120.0, lam, p, u, f);
+  });
 }
 
 void rhs2d_f32(const Grid& g, const double* lam, const PotentialParams* p, const double* u,
                double* f, cudaStream_t s) {
   k_rhs2d_f32<<<grid_of(g, g.n - 1, g.n - 1), block_of(g), 0, s>>>(
       g.n, g.pitch, g.stride, (float)(g.h * g.h / 12.0), (float)(g.h * g.h / 120.0), lam, p, u, f);
-}
-
-void rhs2d_df(const Grid& g, const double* lam, const PotentialParams* p, SplitVec u, double* f,
-              cudaStream_t s) {
-  k_rhs2d_df<<<grid_of(g, g.n - 1, g.n - 1), block_of(g), 0, s>>>(
-      g.n, g.pitch, g.stride, dfloat(g.h * g.h / 12.0), dfloat(g.h * g.h / 120.0), lam, p, u, f);
 }
 
 void dense_level1_2d(const Grid& g, const Coef2D& c, double* L, double* M, cudaStream_t s) {

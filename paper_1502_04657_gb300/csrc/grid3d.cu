@@ -471,10 +471,7 @@ __global__ void k_rhs3d_node(int n, int pitch, size_t st, double h3, double nsca
   f[k] = fma(lam[ib], mu, -(pp[ib].zeta * nscale) * nl);
 }
 
-// Three blocks per SM (74 KB of shared memory each, registers capped at 80) for the walks
-// that fit without spills; the FP64 density walk keeps two (at three it spills and measured
-// slower: 7.98 against 7.93 ms on the finest 3D level, where the right-hand side went from
-// 5.28 to 5.19 ms and the double-float walks from 2.28 / 1.46 to 2.22 / 1.26 ms).
+// Three blocks per SM (74 KB of shared memory each, registers capped at 80) for all the walks.
 // FP64 kernels from the plane walk (star3d.cuh): 6 x the star sum of
 // h3 + u_p h2 + u_p^2 h1 + u_p^3 is S3 + 3 u_p S2 + 6 u_p^2 S1 + 144 u_p^3 in its sums of
 // h1, 2 h2, 6 h3; launch with star3_grid / star3_block and kS3Smem bytes.
@@ -492,27 +489,30 @@ __device__ __forceinline__ fx<kFx3> star3_cubic6(const Star3T<fx<kFx3>>& p) {
 }
 
 // the walks of the blocks that fixed point does not take
+template <int P>
 __device__ __noinline__ void nload3d_fp64(int n, int pitch, size_t st, double scale6,
                                           const double* __restrict__ u,
                                           double* __restrict__ out) {
-  star3_walk<false>(n, pitch, st, u, [&](size_t k, const Star3& p) {
+  star3_walk<false, P>(n, pitch, st, u, [&](size_t k, const Star3& p) {
     out[k] = scale6 * star3_cubic6(p);
   });
 }
 
+template <int P>
 __device__ __noinline__ void rhs3d_fp64(int n, int pitch, size_t st, double h3_120, double zn,
                                         double l, const double* __restrict__ u,
                                         double* __restrict__ f) {
-  star3_walk<false>(n, pitch, st, u, [&](size_t k, const Star3& p) {
+  star3_walk<false, P>(n, pitch, st, u, [&](size_t k, const Star3& p) {
     f[k] = fma(l, h3_120 * fma(24.0, p.u, p.S1), -zn * star3_cubic6(p));
   });
 }
 
+template <int P>
 __device__ __noinline__ void nload_density3d_fp64(int n, int pitch, size_t st, double s140_6,
                                                   double s210_2, double s420_2,
                                                   const double* __restrict__ u,
                                                   double* __restrict__ nl, Density3D b) {
-  star3_walk<true>(n, pitch, st, u, [&](size_t k, const Star3& p) {
+  star3_walk<true, P>(n, pitch, st, u, [&](size_t k, const Star3& p) {
     nl[k] = s140_6 * star3_cubic6(p);
     b.a[0][k] = s210_2 * fma(p.u, fma(144.0, p.u, 4.0 * p.S1), p.S2);
     const double u2 = twice(p.u);
@@ -526,52 +526,55 @@ __device__ __noinline__ void nload_density3d_fp64(int n, int pitch, size_t st, d
   });
 }
 
+template <int P>
 __global__ void __launch_bounds__(kS3X * kS3Y, 3)
     k_nload3d(int n, int pitch, size_t st, double scale6, const double* __restrict__ u,
               double* __restrict__ out) {
-  const int e = star3_exponent(n, pitch, st, u);
+  const int e = star3_exponent<P>(n, pitch, st, u);
   if (e != kFxNone) {
     const double s = fx_scale<kFx3>(scale6, 3, e);
-    star3_walk<false, fx<kFx3>>(
+    star3_walk<false, P, fx<kFx3>>(
         n, pitch, st, FxVec{u, fx_pow2(fx<kFx3>::B1 - e)},
         [&](size_t k, const Star3T<fx<kFx3>>& p) { out[k] = to_double(star3_cubic6(p), s); });
     return;
   }
-  nload3d_fp64(n, pitch, st, scale6, u, out);
+  nload3d_fp64<P>(n, pitch, st, scale6, u, out);
 }
 
 // f = lambda M u - zeta N(u); the mass stencil is h^3/120 (24 u_p + S1)
+template <int P>
 __global__ void __launch_bounds__(kS3X * kS3Y, 3)
     k_rhs3d(int n, int pitch, size_t st, double h3_120, double nscale6,
             const double* __restrict__ lam, const PotentialParams* __restrict__ pp,
             const double* __restrict__ u, double* __restrict__ f) {
-  const int ib = blockIdx.z / star3_zchunks(n);
+  const int ib = blockIdx.z / star3_zchunks(n, P);
   const double l = lam[ib], zn = pp[ib].zeta * nscale6;
-  const int e = star3_exponent(n, pitch, st, u);
+  const int e = star3_exponent<P>(n, pitch, st, u);
   if (e != kFxNone) {
     const double s1 = l * fx_scale<kFx3>(h3_120, 1, e), s3 = fx_scale<kFx3>(zn, 3, e);
-    star3_walk<false, fx<kFx3>>(n, pitch, st, FxVec{u, fx_pow2(fx<kFx3>::B1 - e)},
+    star3_walk<false, P, fx<kFx3>>(n, pitch, st, FxVec{u, fx_pow2(fx<kFx3>::B1 - e)},
                                 [&](size_t k, const Star3T<fx<kFx3>>& p) {
       f[k] = fma(s1, __ll2double_rn(madd<24>(p.u, p.S1).v), -to_double(star3_cubic6(p), s3));
     });
     return;
   }
-  rhs3d_fp64(n, pitch, st, h3_120, zn, l, u, f);
+  rhs3d_fp64<P>(n, pitch, st, h3_120, zn, l, u, f);
 }
 
 // N(u~) and the density stencil, FP64: s140_6, s210_2, s420_2 = |K|/140/6, |K|/210/2,
 // |K|/420/2 against the sums of h1, 2 h2, 6 h3 (an edge lies in 6 tetrahedra along an axis
 // or the body diagonal, 4 along a face diagonal)
+template <int P>
 __global__ void __launch_bounds__(kS3X * kS3Y, 3)
     k_nload_density3d(int n, int pitch, size_t st, double s140_6, double s210_2,
                       double s420_2, const double* __restrict__ u, double* __restrict__ nl,
                       Density3D b) {
-  const int e = star3_exponent(n, pitch, st, u);
+  const int e = star3_exponent<P>(n, pitch, st, u);
   if (e != kFxNone) {
     using T = fx<kFx3>;
     const double a3 = fx_scale<kFx3>(s140_6, 3, e), a2 = fx_scale<kFx3>(s210_2, 2, e),
                  c2 = fx_scale<kFx3>(s420_2, 2, e);
-    star3_walk<true, T>(n, pitch, st, FxVec{u, fx_pow2(T::B1 - e)},
+    star3_walk<true, P, T>(n, pitch, st, FxVec{u, fx_pow2(T::B1 - e)},
                         [&](size_t k, const Star3T<T>& p) {
       nl[k] = to_double(star3_cubic6(p), a3);
       b.a[0][k] = to_double(madd<4>(madd<36>(p.q, p.u * p.S1), p.S2), a2);
@@ -585,7 +588,7 @@ __global__ void __launch_bounds__(kS3X * kS3Y, 3)
     });
     return;
   }
-  nload_density3d_fp64(n, pitch, st, s140_6, s210_2, s420_2, u, nl, b);
+  nload_density3d_fp64<P>(n, pitch, st, s140_6, s210_2, s420_2, u, nl, b);
 }
 
 // The same two walks in double-float arithmetic from the split u (mixed-precision modes): the
@@ -595,7 +598,7 @@ __global__ void __launch_bounds__(kS3X * kS3Y, 3)
 __global__ void __launch_bounds__(kS3X * kS3Y, 3)
     k_nload_density3d_df(int n, int pitch, size_t st, dfloat s140_6, dfloat s210_2,
                          dfloat s420_2, SplitVec u, double* __restrict__ nl, Density3D b) {
-  star3_walk<true, dfloat>(n, pitch, st, u, [&](size_t k, const Star3T<dfloat>& p) {
+  star3_walk<true, kS3Z, dfloat>(n, pitch, st, u, [&](size_t k, const Star3T<dfloat>& p) {
     nl[k] = out_of(s140_6 * star3_cubic6(p));
     put_entry(b.a[0], k, s210_2 * fma(p.u, fma(dfloat(144), p.u, dfloat(4) * p.S1), p.S2));
     const dfloat u2 = twice(p.u);
@@ -615,7 +618,7 @@ __global__ void __launch_bounds__(kS3X * kS3Y, 3)
                 double* __restrict__ f) {
   const int ib = blockIdx.z / star3_zchunks(n);
   const double l = lam[ib], zeta = pp[ib].zeta;
-  star3_walk<false, dfloat>(n, pitch, st, u, [&](size_t k, const Star3T<dfloat>& p) {
+  star3_walk<false, kS3Z, dfloat>(n, pitch, st, u, [&](size_t k, const Star3T<dfloat>& p) {
     const double mu = to_double(h3_120 * fma(dfloat(24), p.u, p.S1));
     f[k] = fma(l, mu, -zeta * to_double(nscale6 * star3_cubic6(p)));
   });
@@ -893,28 +896,32 @@ static cudaError_t star3_prepare(K* kernel) {
 
 void nload3d(const Grid& g, const double* u, double* out, cudaStream_t s) {
   const double vol = g.h * g.h * g.h / 6.0;
-  if (!star3_walks(g)) {
+  if (!star3_planes(g)) {
     k_nload3d_node<<<INTERIOR_LAUNCH(g)>>>(g.n, g.pitch, g.stride, vol / 140.0, u, out);
     return;
   }
-  static const cudaError_t attr = star3_prepare(k_nload3d);
-  (void)attr;
-  k_nload3d<<<star3_grid(g.n, g.nb), star3_block(), kS3Smem, s>>>(g.n, g.pitch, g.stride,
-                                                                  vol / 140.0 / 6.0, u, out);
+  star3_dispatch(g, [&](auto p) {
+    static const cudaError_t attr = star3_prepare(k_nload3d<p>);
+    (void)attr;
+    k_nload3d<p><<<star3_grid(g.n, g.nb, p), star3_block(), kS3Smem, s>>>(
+        g.n, g.pitch, g.stride, vol / 140.0 / 6.0, u, out);
+  });
 }
 
 void rhs3d(const Grid& g, const double* lam, const PotentialParams* p, const double* u,
            double* f, cudaStream_t s) {
   const double h3 = g.h * g.h * g.h;
-  if (!star3_walks(g)) {
+  if (!star3_planes(g)) {
     k_rhs3d_node<<<INTERIOR_LAUNCH(g)>>>(g.n, g.pitch, g.stride, h3, h3 / 6.0 / 140.0, lam, p,
                                          u, f);
     return;
   }
-  static const cudaError_t attr = star3_prepare(k_rhs3d);
-  (void)attr;
-  k_rhs3d<<<star3_grid(g.n, g.nb), star3_block(), kS3Smem, s>>>(
-      g.n, g.pitch, g.stride, h3 / 120.0, h3 / 6.0 / 140.0 / 6.0, lam, p, u, f);
+  star3_dispatch(g, [&](auto planes) {
+    static const cudaError_t attr = star3_prepare(k_rhs3d<planes>);
+    (void)attr;
+    k_rhs3d<planes><<<star3_grid(g.n, g.nb, planes), star3_block(), kS3Smem, s>>>(
+        g.n, g.pitch, g.stride, h3 / 120.0, h3 / 6.0 / 140.0 / 6.0, lam, p, u, f);
+  });
 }
 
 void rhs3d_f32(const Grid& g, const double* lam, const PotentialParams* p, const double* u,
@@ -927,15 +934,17 @@ void rhs3d_f32(const Grid& g, const double* lam, const PotentialParams* p, const
 void nload_density3d(const Grid& g, const double* u, double* nl, const Density3D& b,
                      cudaStream_t s) {
   const double vol = g.h * g.h * g.h / 6.0;
-  if (!star3_walks(g)) {
+  if (!star3_planes(g)) {
     k_nload_density3d_node<double, const double*, 1><<<INTERIOR_LAUNCH(g)>>>(
         g.n, g.pitch, g.stride, vol / 140.0, vol / 210.0, vol / 420.0, u, nl, b);
     return;
   }
-  static const cudaError_t attr = star3_prepare(k_nload_density3d);
-  (void)attr;
-  k_nload_density3d<<<star3_grid(g.n, g.nb), star3_block(), kS3Smem, s>>>(
-      g.n, g.pitch, g.stride, vol / 140.0 / 6.0, vol / 210.0 / 2.0, vol / 420.0 / 2.0, u, nl, b);
+  star3_dispatch(g, [&](auto p) {
+    static const cudaError_t attr = star3_prepare(k_nload_density3d<p>);
+    (void)attr;
+    k_nload_density3d<p><<<star3_grid(g.n, g.nb, p), star3_block(), kS3Smem, s>>>(
+        g.n, g.pitch, g.stride, vol / 140.0 / 6.0, vol / 210.0 / 2.0, vol / 420.0 / 2.0, u, nl, b);
+  });
 }
 
 void nload_density3d_df(const Grid& g, SplitVec u, double* nl, const Density3D& b,

@@ -19,6 +19,8 @@
 // end.  Every node's arithmetic is the same whichever lane and block computes it, so the
 // result does not depend on the launch shape.
 #pragma once
+#include <type_traits>
+
 #include "fixed.cuh"
 #include "fmg_internal.h"
 
@@ -72,36 +74,46 @@ __device__ __forceinline__ T star_cubic(const Star2D<T>& p) {
   return fma(T(3), p.q * fma(T(8), p.u, p.M1), fma(p.u, p.SF, p.SE));
 }
 
-constexpr int kStarRows = 16;   // rows one thread walks
 constexpr int kStarWarps = 4;   // warps of a block, stacked in y
 constexpr int kStarCols = 30;   // producing columns of a warp
 
-inline dim3 star2d_grid(int n, int nb) {
+inline dim3 star2d_grid(int n, int nb, int rows) {
   return dim3((n - 1 + kStarCols - 1) / kStarCols,
-              (n - 1 + kStarRows * kStarWarps - 1) / (kStarRows * kStarWarps), nb);
+              (n - 1 + rows * kStarWarps - 1) / (rows * kStarWarps), nb);
 }
 inline dim3 star2d_block() { return dim3(32, kStarWarps); }
 
-// A walk is a chain of dependent row steps, and a block's FP64 work lands on one SM, so a
-// level with few blocks is latency-bound (about 33 us for any n <= 512 on one GB300, against
-// 8 us node by node at n = 128).  The walk is taken when it gives at least two blocks per SM
-// (single 2D instances from n = 1024 on); smaller launches run node by node.
-// (FMG_FLAG_STAR_WALKS takes it everywhere.)
-constexpr unsigned kWalkMinBlocks = 2 * 152;
-inline bool star2d_walks(const Grid& lv) {
-  const dim3 g = star2d_grid(lv.n, lv.nb);
-  return lv.walk_all || (size_t)g.x * g.y * g.z >= kWalkMinBlocks;
+// Rows one thread walks on a level (the kernels' template argument), or 0: node by node in FP64.
+// A walk is a chain of dependent row steps (about 0.8 us each), so small levels take short
+// walks, which are more and shorter chains but compute more rows twice (R + 2 for R).  The
+// density kernel on one instance took, in us, node by node 8.2, 14.4 and 47 at n = 128, 256 and
+// 512, 16 in 16-row walks at each, and 6.1, 6.5 (R = 4) and 12.7 (R = 8) at n = 112, 224 and
+// 448; filled with instances, 8 rows cost 8% more per node than 16.
+// The rule depends on n alone, so an instance gives the same bits alone and in a batch.
+// (FMG_FLAG_STAR_WALKS walks below n = 64 as well.)
+inline int star2d_rows(const Grid& lv) {
+  return lv.n >= 1024 ? 16 : lv.n >= 256 ? 8 : lv.n >= 64 || lv.walk_all ? 4 : 0;
+}
+// f(std::integral_constant<int, rows>) for the level's rows
+template <typename F>
+void star2d_dispatch(const Grid& lv, F f) {
+  switch (star2d_rows(lv)) {
+    case 16: f(std::integral_constant<int, 16>()); break;
+    case 8: f(std::integral_constant<int, 8>()); break;
+    default: f(std::integral_constant<int, 4>());
+  }
 }
 
-// The fixed-point exponent of this warp's tile (its 32 columns, 16 rows and the row before and
+// The fixed-point exponent of this warp's tile (its 32 columns, R rows and the row before and
 // after them), or kFxNone; uniform over the warp.  The walk reads the tile again from L1.
+template <int R>
 __device__ __forceinline__ int star2d_exponent(int n, int pitch, size_t st, const double* u) {
   const int i = kStarCols * blockIdx.x + threadIdx.x;
-  const int j0 = 1 + kStarRows * (blockIdx.y * blockDim.y + threadIdx.y);
+  const int j0 = 1 + R * (blockIdx.y * blockDim.y + threadIdx.y);
   const double* p = u + blockIdx.z * st + i;
   FxTop m;
 #pragma unroll
-  for (int t = 0; t <= kStarRows + 2; ++t) {
+  for (int t = 0; t <= R + 2; ++t) {
     const int r = j0 - 1 + t;
     if (i <= n && r <= n) m.add(p[(size_t)r * pitch]);
   }
@@ -136,13 +148,13 @@ __device__ __forceinline__ fx<K> shfl_down1(fx<K> v) {
   return fx<K>(__shfl_down_sync(0xffffffffu, v.v, 1));
 }
 // e: the warp's exponent (star2d_exponent).  Calls out(k, star) as star2d_walk does.
-template <bool DENSITY, typename Out>
+template <bool DENSITY, int R, typename Out>
 __device__ __forceinline__ void star2d_walk_fx(int n, int pitch, size_t st,
                                                const double* __restrict__ u, int e, Out out) {
   using T = fx<kFx2>;
   const int lane = threadIdx.x;
   const int i = kStarCols * blockIdx.x + lane;
-  const int j0 = 1 + kStarRows * (blockIdx.y * blockDim.y + threadIdx.y);
+  const int j0 = 1 + R * (blockIdx.y * blockDim.y + threadIdx.y);
   if (j0 >= n) return;  // uniform over the warp
   const double scale = fx_pow2(T::B1 - e);
   const double* col = u + blockIdx.z * st + i;
@@ -158,7 +170,7 @@ __device__ __forceinline__ void star2d_walk_fx(int n, int pitch, size_t st,
   T Hs = zero, HF = zero, Vs = zero, VF = zero, Ds = zero, DF = zero;  // own edges, row r - 1
   T start[3] = {zero, zero, zero}, acc[3] = {zero, zero, zero};        // sums of (s, F, E3)
 #pragma unroll 2
-  for (int t = 0; t < kStarRows + 2; ++t) {
+  for (int t = 0; t < R + 2; ++t) {
     const int r = j0 - 1 + t;
     const T u1 = fix(next);
     next = ld(r + 2);
@@ -211,11 +223,11 @@ __device__ __forceinline__ void star2d_walk_fx(int n, int pitch, size_t st,
 // Walks the rows of this thread's strip of instance blockIdx.z and calls out(k, star) for
 // every interior node it produces (k = the node's index in the batched arrays).  u is read
 // through get<T>: FP64 or the split double-float copy.  blockDim = (32, kStarWarps).
-template <typename T, typename U, typename Out>
+template <typename T, int R, typename U, typename Out>
 __device__ __forceinline__ void star2d_walk(int n, int pitch, size_t st, const U& u, Out out) {
   const int lane = threadIdx.x;
   const int i = kStarCols * blockIdx.x + lane;  // lane 0 = first produced column - 1
-  const int j0 = 1 + kStarRows * (blockIdx.y * blockDim.y + threadIdx.y);
+  const int j0 = 1 + R * (blockIdx.y * blockDim.y + threadIdx.y);
   if (j0 >= n) return;  // uniform over the warp
   const size_t base = blockIdx.z * st;
   const bool produce = lane >= 1 && lane <= kStarCols && i <= n - 1;
@@ -231,7 +243,7 @@ __device__ __forceinline__ void star2d_walk(int n, int pitch, size_t st, const U
   T uRm1 = T(0), qRm1 = T(0), uLm1 = T(0), qLm1 = T(0);
   StarEdge<T> Dm1{}, Dm2{}, VLm1{}, VLm2{}, HLm1{}, HLm2{}, DLm1{}, VRm1{}, Hm1{}, Vm1{};
 #pragma unroll
-  for (int t = 0; t < kStarRows + 2; ++t) {
+  for (int t = 0; t < R + 2; ++t) {
     const int r = j0 - 1 + t;
     const T u1 = ld(r + 1);
     const T q1 = u1 * u1;

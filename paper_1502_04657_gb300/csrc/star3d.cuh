@@ -28,6 +28,8 @@
 // the node above it.  Every sum is taken in a fixed order, so the result does not depend on
 // the launch shape.
 #pragma once
+#include <type_traits>
+
 #include "fixed.cuh"
 #include "fmg_internal.h"
 
@@ -35,7 +37,8 @@ namespace fmg {
 
 constexpr int kFx3 = 59;  // fixed-point format of the walk (fixed.cuh)
 
-constexpr int kS3X = 32, kS3Y = 8, kS3Z = 16;   // tile of columns (= threads), planes per block
+constexpr int kS3X = 32, kS3Y = 8;               // tile of columns (= threads)
+constexpr int kS3Z = 16;                         // planes per block of a double-float walk
 constexpr int kS3CX = kS3X + 1;                  // cube layer row (cubes x0 - 1 .. x0 + 31)
 constexpr int kS3Cubes = (kS3X + 1) * (kS3Y + 1);
 constexpr int kS3NX = kS3X + 2;                  // node plane row (nodes x0 - 1 .. x0 + 32)
@@ -59,16 +62,18 @@ struct Star3T {
 };
 using Star3 = Star3T<double>;
 
-__host__ __device__ inline int star3_zchunks(int n) { return (n - 1 + kS3Z - 1) / kS3Z; }
-inline dim3 star3_grid(int n, int nb) {
-  return dim3((n - 1 + kS3X - 1) / kS3X, (n - 1 + kS3Y - 1) / kS3Y, nb * star3_zchunks(n));
+__host__ __device__ inline int star3_zchunks(int n, int planes = kS3Z) {
+  return (n - 1 + planes - 1) / planes;
+}
+inline dim3 star3_grid(int n, int nb, int planes = kS3Z) {
+  return dim3((n - 1 + kS3X - 1) / kS3X, (n - 1 + kS3Y - 1) / kS3Y, nb * star3_zchunks(n, planes));
 }
 inline dim3 star3_block() { return dim3(kS3X, kS3Y); }
 
-// A block's 16 planes are dependent steps on one SM, so a level with few blocks is
-// latency-bound (about 0.23 ms for any n <= 64 on one GB300, against 0.025 ms node by node at
-// n = 32).  The walk is taken when it gives at least two blocks per SM (single 3D instances
-// from n = 128 on); smaller launches run node by node.
+// A block's planes are dependent steps on one SM, so a level with few blocks is
+// latency-bound (the double-float walk: about 0.23 ms for any n <= 64, against 0.025 ms node by
+// node at n = 32).  The double-float walk is taken when it gives at least two blocks per SM
+// (single 3D instances from n = 128 on); smaller launches run node by node.
 // (FMG_FLAG_STAR_WALKS takes it everywhere.)
 constexpr unsigned kWalk3MinBlocks = 2 * 152;
 inline bool star3_walks(const Grid& lv) {
@@ -76,15 +81,32 @@ inline bool star3_walks(const Grid& lv) {
   return lv.walk_all || (size_t)g.x * g.y * g.z >= kWalk3MinBlocks;
 }
 
-// The fixed-point exponent of this block's tile (its 16 planes and the halo of the walk), or
+// Planes per block of the fixed-point walk on a level (the kernels' template argument), or 0:
+// node by node in FP64.  A plane step takes about 4.5 us, so small levels take short walks, which
+// compute more planes twice (P + 1 cube layers for P).  The density kernel took 213 us node by
+// node, 78 in 16-plane walks and 33 in 4-plane ones at n = 64, and 33, 78 and 24 at n = 32 (the
+// right-hand side 132, 51, 22 and 22, 51, 17).
+// The rule depends on n alone, so an instance gives the same bits alone and in a batch.
+inline int star3_planes(const Grid& lv) {
+  return lv.n >= 128 ? 16 : lv.n >= 32 || lv.walk_all ? 4 : 0;
+}
+// f(std::integral_constant<int, planes>) for the level's planes
+template <typename F>
+void star3_dispatch(const Grid& lv, F f) {
+  if (star3_planes(lv) == 16) f(std::integral_constant<int, 16>());
+  else f(std::integral_constant<int, 4>());
+}
+
+// The fixed-point exponent of this block's tile (its P planes and the halo of the walk), or
 // kFxNone.  Reads the tile once; the walk reads it again from L2.
+template <int P>
 __device__ __forceinline__ int star3_exponent(int n, int pitch, size_t st, const double* u) {
   __shared__ int top[2];
   const int tid = threadIdx.y * kS3X + threadIdx.x;
   if (tid < 2) top[tid] = 0;
-  const int nzc = star3_zchunks(n);
+  const int nzc = star3_zchunks(n, P);
   const int ib = blockIdx.z / nzc;
-  const int z0 = 1 + (int)(blockIdx.z - ib * nzc) * kS3Z, z1 = min(z0 + kS3Z, n);
+  const int z0 = 1 + (int)(blockIdx.z - ib * nzc) * P, z1 = min(z0 + P, n);
   const int x0 = 1 + blockIdx.x * kS3X, y0 = 1 + blockIdx.y * kS3Y;
   const long plane = (long)(n + 1) * pitch;
   FxTop m;
@@ -108,20 +130,20 @@ __device__ __forceinline__ int star3_exponent(int n, int pitch, size_t st, const
 }
 
 // blockDim = (kS3X, kS3Y), kS3Smem bytes of dynamic shared memory; instance
-// blockIdx.z / star3_zchunks(n).  out(k, star) for every interior node the block produces.
+// blockIdx.z / star3_zchunks(n, P).  out(k, star) for every interior node the block produces.
 // T: the arithmetic (double, or dfloat with u a SplitVec); the FP64 instantiation evaluates
 // exactly the expressions it did before it was templated.
-template <bool EDGES, typename T = double, typename U = const double*, typename Out>
+template <bool EDGES, int P, typename T = double, typename U = const double*, typename Out>
 __device__ __forceinline__ void star3_walk(int n, int pitch, size_t st, const U u, Out out) {
   extern __shared__ double s3sm[];
   T* const su = reinterpret_cast<T*>(s3sm);  // [3][kS3Nodes]
   T* const sq = su + 3 * kS3Nodes;           // u^2
   T* const sc = sq + 3 * kS3Nodes;           // 2 u^3
   T* const cube = sc + 3 * kS3Nodes;         // [kS3Vals][kS3Cubes]
-  const int nzc = star3_zchunks(n);
+  const int nzc = star3_zchunks(n, P);
   const int ib = blockIdx.z / nzc;
-  const int z0 = 1 + (int)(blockIdx.z - ib * nzc) * kS3Z;
-  const int z1 = min(z0 + kS3Z, n);
+  const int z0 = 1 + (int)(blockIdx.z - ib * nzc) * P;
+  const int z1 = min(z0 + P, n);
   const int x0 = 1 + blockIdx.x * kS3X, y0 = 1 + blockIdx.y * kS3Y;
   const long plane = (long)(n + 1) * pitch;
   const size_t base = (size_t)ib * st;
