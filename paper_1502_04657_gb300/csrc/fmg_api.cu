@@ -77,6 +77,11 @@ void lv_apply_full(Level& l, const double* x, double* y, cudaStream_t s) {
   if (l.g.dim == 2) apply2d(l.g, l.cw, x, y, s);
   else apply3d(l.g, l.cw3, x, y, s);
 }
+// the same and z = M x
+void lv_apply_mass_full(Level& l, const double* x, double* y, double* z, cudaStream_t s) {
+  if (l.g.dim == 2) apply_mass2d(l.g, l.cw, x, y, z, s);
+  else apply_mass3d(l.g, l.cw3, x, y, z, s);
+}
 // f -= W u (paper-literal form: W moves to the right-hand side)
 void lv_sub_wmass(Level& l, const double* u, double* f, cudaStream_t s) {
   if (l.g.dim == 2) sub_wmass2d(l.g, l.cw, l.c, u, f, s);
@@ -538,7 +543,7 @@ void build_coarse(fmg_eig_handle* h) {
   h->auu = h->alloc<double>(nb);
   h->buu = h->alloc<double>(nb);
   h->scal = h->alloc<double>(3 * (size_t)nb + 8);
-  h->partials = h->alloc<double>((size_t)kReduceBlocks * nb);
+  h->partials = h->alloc<double>((size_t)2 * kReduceBlocks * nb);
   if (h->prob.smoother == FMG_SMOOTH_CG) h->cg = h->alloc<double>(3 * (size_t)nb);
   h->partials2 = h->alloc<double>((size_t)kReduceBlocks * nb);
   const int nt3 = dim == 2 ? 10 : 20;
@@ -956,11 +961,13 @@ void enqueue_augment(fmg_eig_handle* h, int k, const double* ut, cudaStream_t s)
   // main branch: (A + W) u~, M u~, their dots and restriction chains.  The 3D mixed modes form
   // M u~ in double-float on the FP32 pipes (positive weights: ~2^-47 of the result); the
   // operator apply stays FP64 (its stencil cancels to O(h^2) of its terms).
-  lv_apply_full(l, ut, l.y, s);
-  if (df) lv_mass_df(l, us, l.z, s);
-  else lv_mass(l, ut, l.z, s);
-  dot(ut, l.y, st, h->partials, h->auu, s, nb, st);
-  dot(ut, l.z, st, h->partials, h->buu, s, nb, st);
+  if (df) {
+    lv_apply_full(l, ut, l.y, s);
+    lv_mass_df(l, us, l.z, s);
+  } else {
+    lv_apply_mass_full(l, ut, l.y, l.z, s);
+  }
+  dot2(ut, l.y, l.z, st, h->partials, h->auu, h->buu, s, nb, st);
   for (int j = k; j >= 2; --j)  // both chains in one launch per level
     lv_restrict(h->L(j), h->L(j - 1), h->L(j).y, h->L(j - 1).y, s, h->L(j).z, h->L(j - 1).z);
   join_sides(h, s, 0, 2);
@@ -1055,11 +1062,9 @@ void enqueue_checks(fmg_eig_handle* h, cudaStream_t s) {
     if (count <= 0) continue;
     Level v = view(h->L(k), first, count);
     const size_t st = v.g.stride;
-    lv_apply_full(v, v.u, v.y, s);
-    lv_mass(v, v.u, v.z, s);
+    lv_apply_mass_full(v, v.u, v.y, v.z, s);
     lv_nload(v, v.u, v.r, s);
-    dot(v.u, v.y, st, h->partials, sa + first, s, count, st);
-    dot(v.u, v.z, st, h->partials, sb + first, s, count, st);
+    dot2(v.u, v.y, v.z, st, h->partials, sa + first, sb + first, s, count, st);
     dot(v.u, v.r, st, h->partials, sn + first, s, count, st);
   }
 }

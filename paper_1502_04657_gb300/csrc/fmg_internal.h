@@ -72,6 +72,8 @@ struct Coef2D {
 inline bool fxop2d_applies(const Grid& g) { return g.dim == 2 && g.n >= 512; }
 void fxop2d_tables(const Grid& g, const PotentialParams* p, const Coef2D& c, cudaStream_t s);
 void fxop2d_apply(const Grid& g, const Coef2D& c, const double* x, double* y, cudaStream_t s);
+void fxop2d_apply_mass(const Grid& g, const Coef2D& c, const double* x, double* y, double* mx,
+                       cudaStream_t s);
 void fxop2d_jacobi(const Grid& g, const Coef2D& c, const double* f, const double* x, double* xo,
                    cudaStream_t s);
 void fxop2d_residual(const Grid& g, const Coef2D& c, const double* f, const double* x, double* r,
@@ -94,6 +96,9 @@ struct PotentialParams {
 void coef2d_setup(const Grid& g, const PotentialParams* p_dev, const Coef2D& c, cudaStream_t s);
 void apply2d(const Grid& g, const Coef2D& c, const double* x, double* y, cudaStream_t s);
 void mass2d(const Grid& g, const double* x, double* y, cudaStream_t s);
+// y = L x, z = M x
+void apply_mass2d(const Grid& g, const Coef2D& c, const double* x, double* y, double* z,
+                  cudaStream_t s);
 // the same from the double-float split of x (mixed-precision modes)
 // f -= W u, W u = (A + W) u - A u from the coefficient sets cw (A + W) and ca (A)
 void sub_wmass2d(const Grid& g, const Coef2D& cw, const Coef2D& ca, const double* u, double* f,
@@ -148,6 +153,8 @@ struct Coef3D {
 inline bool fxop3d_applies(const Grid& g) { return g.dim == 3 && g.n >= 96; }
 void fxop3d_tables(const Grid& g, const PotentialParams* p, const Coef3D& c, cudaStream_t s);
 void fxop3d_apply(const Grid& g, const Coef3D& c, const double* x, double* y, cudaStream_t s);
+void fxop3d_apply_mass(const Grid& g, const Coef3D& c, const double* x, double* y, double* mx,
+                       cudaStream_t s);
 void fxop3d_jacobi(const Grid& g, const Coef3D& c, const double* f, const double* x, double* xo,
                    cudaStream_t s);
 void fxop3d_residual(const Grid& g, const Coef3D& c, const double* f, const double* x, double* r,
@@ -161,6 +168,9 @@ struct Stencil15 {
 void coef3d_setup(const Grid& g, const PotentialParams* p_dev, const Coef3D& c, cudaStream_t s);
 void apply3d(const Grid& g, const Coef3D& c, const double* x, double* y, cudaStream_t s);
 void mass3d(const Grid& g, const double* x, double* y, cudaStream_t s);
+// y = L x, z = M x
+void apply_mass3d(const Grid& g, const Coef3D& c, const double* x, double* y, double* z,
+                  cudaStream_t s);
 void mass3d_df(const Grid& g, SplitVec x, double* y, cudaStream_t s);
 void sub_wmass3d(const Grid& g, const Coef3D& cw, const Coef3D& ca, const double* u, double* f,
                  cudaStream_t s);
@@ -293,6 +303,9 @@ void vcycle32_up(const Grid& g, const CoefT& ct, const Grid& gc, const float* f,
 constexpr int kReduceBlocks = 1024;
 void dot(const double* a, const double* b, size_t n, double* partials, double* out,
          cudaStream_t s, int nb = 1, size_t vst = 0);
+// out = a . b and out2 = a . c in one pass (each as dot sums it); partials: 2 kReduceBlocks nb
+void dot2(const double* a, const double* b, const double* c, size_t n, double* partials,
+          double* out, double* out2, cudaStream_t s, int nb, size_t vst);
 // Conjugate gradient smoother steps over nb instances of `stride` elements (n = nb stride):
 // x += a p, r -= a q with a = rr[b] / pq[b]; then p = r + (rr_new[b] / rr_old[b]) p
 void cg_update(size_t n, size_t stride, const double* rr, const double* pq, const double* p,

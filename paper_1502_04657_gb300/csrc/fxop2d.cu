@@ -17,6 +17,8 @@
 // Only the products, x and f round, at 2^-58 of the tile's maximum or below (FP64 rounds each
 // of its operations at 2^-53, and each stored coupling -1 + O(h^2) at 2^-53: a relative
 // perturbation of W by 2^-53 / h^2, 4e-9 at h = 1/4096, that this form does not have).
+// The operator apply of the augmented pass also stores M x = h^2/12 (6x + sum of the six), whose
+// sum is at hand: the two applies took 117 and 227 us on 16.8M nodes, together 152 us.
 // The update x + (omega / D) r is one FP64 operation as before.  What is left is the instruction
 // rate (about 200 integer instructions per node) and the latency between a tile's loads and its
 // arithmetic: 4 rows a warp and 5 blocks per SM took 156 us (Jacobi) and 127 us (residual) on
@@ -101,7 +103,8 @@ __device__ __forceinline__ double times_pow2(double v, int e) {
   return __hiloint2double(__double2hiint(v) + e * (1 << 20), __double2loint(v));
 }
 
-enum Mode { kJacobiMode, kResidualMode, kApplyMode };
+enum Mode { kJacobiMode, kResidualMode, kApplyMode, kApplyMassMode };
+constexpr bool applies(int mode) { return mode == kApplyMode || mode == kApplyMassMode; }
 
 __device__ __forceinline__ void store(double* o, size_t k, double v) { o[k] = v; }
 __device__ __forceinline__ void store(float* o, size_t k, double v) { o[k] = d2f_rn(v); }
@@ -113,14 +116,15 @@ __device__ __forceinline__ void store(__nv_bfloat16* o, size_t k, double v) {
 template <int MODE, typename S>
 __device__ __noinline__ void tile_fp64(int n, int pitch, size_t base, int i0, int j0,
                                        const Coef2D& c, const double* __restrict__ f,
-                                       const double* __restrict__ x, S* __restrict__ out) {
+                                       const double* __restrict__ x, S* __restrict__ out,
+                                       double mscale, double* __restrict__ mx) {
   for (int j = j0; j < min(j0 + kRows, n); ++j)
     for (int q = 0; q < 2; ++q) {
       const int i = i0 + q, lane = threadIdx.x;
       if (i < 1 || i > n - 1 || (lane == 0 && q == 0) || (lane == 31 && q == 1)) continue;
       const size_t k = base + (size_t)j * pitch + i;
       double r;
-      if (MODE == kApplyMode) {
+      if (applies(MODE)) {
         r = c.cC[k] * x[k];
         r = fma(c.cE[k], x[k + 1], r);
         r = fma(c.cE[k - 1], x[k - 1], r);
@@ -139,13 +143,17 @@ __device__ __noinline__ void tile_fp64(int n, int pitch, size_t base, int i0, in
         if (MODE == kJacobiMode) r = fma(c.dinv[k], r, x[k]);
       }
       store(out, k, r);
+      if (MODE == kApplyMassMode)
+        mx[k] = mscale * fma(6.0, x[k], ((x[k + 1] + x[k - 1]) + (x[k + pitch] + x[k - pitch])) +
+                                            (x[k + pitch + 1] + x[k - pitch - 1]));
     }
 }
 
 template <int MODE, typename S>
 __global__ void __launch_bounds__(32 * kWarps, kBlocks)
     k_fxop2d(int n, int pitch, size_t st, const __grid_constant__ Coef2D c,
-             const double* __restrict__ f, const double* __restrict__ x, S* __restrict__ out) {
+             const double* __restrict__ f, const double* __restrict__ x, S* __restrict__ out,
+             double mscale, double* __restrict__ mx) {
   const int lane = threadIdx.x, ib = blockIdx.z;
   const int i0 = kCols * blockIdx.x + 2 * lane;  // this lane's columns i0, i0 + 1
   const int j0 = 1 + kRows * (blockIdx.y * kWarps + threadIdx.y);
@@ -169,7 +177,7 @@ __global__ void __launch_bounds__(32 * kWarps, kBlocks)
 #pragma unroll
   for (int t = 0; t < kRows + 2; ++t)
     top = max(top, max(__double2hiint(xv[t].x) & 0x7fffffff, __double2hiint(xv[t].y) & 0x7fffffff));
-  if (MODE != kApplyMode) {
+  if (!applies(MODE)) {
 #pragma unroll
     for (int t = 0; t < kRows; ++t) {
       const double2 v = f_row(j0 + t);
@@ -180,11 +188,11 @@ __global__ void __launch_bounds__(32 * kWarps, kBlocks)
   top = __reduce_max_sync(0xffffffffu, top);
   const int e = ((top + 1) >> 20) - 1022;
   if (!hd.ok || e < -kFxMaxExp || e > kFxMaxExp) {
-    tile_fp64<MODE, S>(n, pitch, base, i0, j0, c, f, x, out);
+    tile_fp64<MODE, S>(n, pitch, base, i0, j0, c, f, x, out, mscale, mx);
     return;
   }
   const int shift = e + 1022 + 5;
-  const double back = fx_pow2(e - kB);
+  const double back = fx_pow2(e - kB), mback = mscale * back;
   const long long* tab = c.fxt + (size_t)ib * 4 * (n + 1);
   const int ia = min(i0, n), ic = min(i0 + 1, n);
   const long long axa = tab[ia], axb = tab[ic], bxa = tab[2 * (n + 1) + ia],
@@ -204,10 +212,11 @@ __global__ void __launch_bounds__(32 * kWarps, kBlocks)
   };
   // one node: (A + W) x in units of 2^(e - kB)
   auto node = [&](long long x0, long long xe, long long xw, long long xn, long long xs,
-                  long long xne, long long xsw, long long a, long long bx, long long by) {
+                  long long xne, long long xsw, long long a, long long bx, long long by,
+                  long long& s6) {
     const long long ew = xe + xw, ns = xn + xs, d = xne + xsw, g = xne - xsw;
     const long long t = ew + ns;
-    const long long s6 = 6 * x0 + t + d;
+    s6 = 6 * x0 + t + d;
     long long sm = (long long)hd.P * (int)(x0 >> 32) + (long long)hd.Q * (int)(ew >> 32) +
                    (long long)hd.R * (int)(ns >> 32);
     long long w = mul_hi(a, s6) + mul_hi(bx, (xe - xw) + g) + mul_hi(by, (xn - xs) + g);
@@ -221,9 +230,10 @@ __global__ void __launch_bounds__(32 * kWarps, kBlocks)
     const Row p = row(xv[t + 2]);
     if (j < n) {
       const long long ay = tab[(n + 1) + j], by = tab[3 * (n + 1) + j];
-      long long ra = node(m.a, m.b, m.l, p.a, s.a, p.b, s.l, axa + ay, bxa, by);
-      long long rb = node(m.b, m.r, m.a, p.b, s.b, p.r, s.a, axb + ay, bxb, by);
-      if (MODE != kApplyMode) {
+      long long ma, mb;  // 12 / h^2 of the mass apply
+      long long ra = node(m.a, m.b, m.l, p.a, s.a, p.b, s.l, axa + ay, bxa, by, ma);
+      long long rb = node(m.b, m.r, m.a, p.b, s.b, p.r, s.a, axb + ay, bxb, by, mb);
+      if (!applies(MODE)) {
         const double2 v = f_row(j);
         ra = to_fixed(v.x, shift) - ra;
         rb = to_fixed(v.y, shift) - rb;
@@ -245,6 +255,15 @@ __global__ void __launch_bounds__(32 * kWarps, kBlocks)
         if (oka) store(out, k, va);
         if (okb) store(out, k + 1, vb);
       }
+      if (MODE == kApplyMassMode) {
+        const double za = __ll2double_rn(ma) * mback, zb = __ll2double_rn(mb) * mback;
+        if (oka && okb) {
+          *reinterpret_cast<double2*>(mx + k) = make_double2(za, zb);
+        } else {
+          if (oka) mx[k] = za;
+          if (okb) mx[k + 1] = zb;
+        }
+      }
     }
     s = m;
     m = p;
@@ -253,10 +272,11 @@ __global__ void __launch_bounds__(32 * kWarps, kBlocks)
 
 template <int MODE, typename S>
 void launch(const Grid& g, const Coef2D& c, const double* f, const double* x, S* out,
-            cudaStream_t s) {
+            cudaStream_t s, double* mx = nullptr) {
   const dim3 grid((g.n - 1 + kCols - 1) / kCols,
                   (g.n - 1 + kRows * kWarps - 1) / (kRows * kWarps), g.nb);
-  k_fxop2d<MODE, S><<<grid, dim3(32, kWarps), 0, s>>>(g.n, g.pitch, g.stride, c, f, x, out);
+  k_fxop2d<MODE, S><<<grid, dim3(32, kWarps), 0, s>>>(g.n, g.pitch, g.stride, c, f, x, out,
+                                                     g.h * g.h / 12.0, mx);
 }
 
 }  // namespace
@@ -266,6 +286,10 @@ void fxop2d_tables(const Grid& g, const PotentialParams* p, const Coef2D& c, cud
 }
 void fxop2d_apply(const Grid& g, const Coef2D& c, const double* x, double* y, cudaStream_t s) {
   launch<kApplyMode>(g, c, nullptr, x, y, s);
+}
+void fxop2d_apply_mass(const Grid& g, const Coef2D& c, const double* x, double* y, double* mx,
+                       cudaStream_t s) {
+  launch<kApplyMassMode>(g, c, nullptr, x, y, s, mx);
 }
 void fxop2d_jacobi(const Grid& g, const Coef2D& c, const double* f, const double* x, double* xo,
                    cudaStream_t s) {

@@ -136,6 +136,18 @@ __global__ void k_mass2d(int n, int pitch, size_t st, double h2_12, const double
   y[k] = h2_12 * fma(6.0, x[k], s);
 }
 
+// y = L x and z = M x for the levels below the fixed-point operator's: one launch (small levels)
+// and one pass over x instead of two
+__global__ void k_apply_mass2d(int n, int pitch, size_t st, double h2_12, Coef2D c,
+                               const double* __restrict__ x, double* __restrict__ y,
+                               double* __restrict__ z) {
+  INTERIOR_2D
+  y[k] = lop(c, x, k, pitch);
+  const double s = ((x[k + 1] + x[k - 1]) + (x[k + pitch] + x[k - pitch])) +
+                   (x[k + pitch + 1] + x[k - pitch - 1]);
+  z[k] = h2_12 * fma(6.0, x[k], s);
+}
+
 __global__ void k_jacobi2d(int n, int pitch, size_t st, Coef2D c, const double* __restrict__ f,
                            const double* __restrict__ x, double* __restrict__ xo) {
   INTERIOR_2D
@@ -437,6 +449,16 @@ void apply2d(const Grid& g, const Coef2D& c, const double* x, double* y, cudaStr
   }
   k_apply2d<<<grid_of(g, g.n - 1, g.n - 1), block_of(g), 0, s>>>(g.n, g.pitch, g.stride, c, x,
                                                                   y);
+}
+
+void apply_mass2d(const Grid& g, const Coef2D& c, const double* x, double* y, double* z,
+                  cudaStream_t s) {
+  if (c.fxt) {
+    fxop2d_apply_mass(g, c, x, y, z, s);
+    return;
+  }
+  k_apply_mass2d<<<grid_of(g, g.n - 1, g.n - 1), block_of(g), 0, s>>>(
+      g.n, g.pitch, g.stride, g.h * g.h / 12.0, c, x, y, z);
 }
 
 void sub_wmass2d(const Grid& g, const Coef2D& cw, const Coef2D& ca, const double* u, double* f,

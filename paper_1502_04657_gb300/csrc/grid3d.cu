@@ -209,6 +209,16 @@ __global__ void k_mass3d(int n, int pitch, size_t st, double h3, const double* _
   y[k] = h3 * mass_at(x, k, pitch, plane);
 }
 
+// y = L x and z = M x for the levels below the fixed-point operator's: one launch (small levels)
+// and one pass over x instead of two
+__global__ void k_apply_mass3d(int n, int pitch, size_t st, double h3, Coef3D c,
+                               const double* __restrict__ x, double* __restrict__ y,
+                               double* __restrict__ z) {
+  INTERIOR_3D
+  y[k] = lop3(c, x, k, pitch, plane);
+  z[k] = h3 * mass_at(x, k, pitch, plane);
+}
+
 // The same in double-float arithmetic from the split of x (mixed-precision modes' augmented
 // pass; positive weights, so ~2^-47 of the result); FP64 output.
 __global__ void k_mass3d_df(int n, int pitch, size_t st, dfloat h3, SplitVec x,
@@ -824,6 +834,15 @@ void apply3d(const Grid& g, const Coef3D& c, const double* x, double* y, cudaStr
     return;
   }
   k_apply3d<<<INTERIOR_LAUNCH(g)>>>(g.n, g.pitch, g.stride, c, x, y);
+}
+
+void apply_mass3d(const Grid& g, const Coef3D& c, const double* x, double* y, double* z,
+                  cudaStream_t s) {
+  if (c.fxt) {
+    fxop3d_apply_mass(g, c, x, y, z, s);
+    return;
+  }
+  k_apply_mass3d<<<INTERIOR_LAUNCH(g)>>>(g.n, g.pitch, g.stride, g.h * g.h * g.h, c, x, y, z);
 }
 
 void sub_wmass3d(const Grid& g, const Coef3D& cw, const Coef3D& ca, const double* u, double* f,

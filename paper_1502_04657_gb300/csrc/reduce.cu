@@ -59,29 +59,86 @@ __global__ void k_dot_partial(const double* __restrict__ a, const double* __rest
   if (threadIdx.x == 0) partials[blockIdx.x] = t;
 }
 
-__global__ void k_sum_final(const double* __restrict__ partials, int m, double* out) {
+// a . b into partials, a . c into the second half (gridDim.y instances on): each in the order
+// of k_dot_partial, with a read once
+__global__ void k_dot2_partial(const double* __restrict__ a, const double* __restrict__ b,
+                               const double* __restrict__ c, size_t n, size_t vst, size_t chunk,
+                               double* __restrict__ partials) {
+  __shared__ double sh[2][kThreads / 32];
+  a += blockIdx.y * vst;
+  b += blockIdx.y * vst;
+  c += blockIdx.y * vst;
+  const size_t beg = blockIdx.x * chunk;
+  const size_t end = beg >= n ? beg : (beg + chunk < n ? beg + chunk : n);
+  const size_t pend = beg + ((end - beg) & ~(size_t)1);
+  double s[2][4] = {};
+  auto pair = [&](size_t i, int q) {
+    const double2 x = *reinterpret_cast<const double2*>(a + i);
+    const double2 y = *reinterpret_cast<const double2*>(b + i);
+    const double2 z = *reinterpret_cast<const double2*>(c + i);
+    s[0][q] = fma(x.x, y.x, s[0][q]);
+    s[0][q + 1] = fma(x.y, y.y, s[0][q + 1]);
+    s[1][q] = fma(x.x, z.x, s[1][q]);
+    s[1][q + 1] = fma(x.y, z.y, s[1][q + 1]);
+  };
+  size_t i = beg + 2 * threadIdx.x;
+  for (; i + 2 * kThreads < pend; i += 4 * kThreads) {
+    pair(i, 0);
+    pair(i + 2 * kThreads, 2);
+  }
+  if (i < pend) pair(i, 0);
+  if (threadIdx.x == 0 && pend < end) {
+    s[0][0] = fma(a[pend], b[pend], s[0][0]);
+    s[1][0] = fma(a[pend], c[pend], s[1][0]);
+  }
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {
+    const double t = block_sum_warps((s[q][0] + s[q][1]) + (s[q][2] + s[q][3]), sh[q]);
+    if (threadIdx.x == 0)
+      partials[((size_t)q * gridDim.y + blockIdx.y) * kReduceBlocks + blockIdx.x] = t;
+  }
+}
+
+// instance blockIdx.x of the dot blockIdx.y
+__global__ void k_sum_final(const double* __restrict__ partials, int m, double* out,
+                            double* out2) {
   __shared__ double sh[kThreads / 32];
-  partials += (size_t)blockIdx.x * kReduceBlocks;  // instance blockIdx.x
-  out += blockIdx.x;
+  partials += ((size_t)blockIdx.y * gridDim.x + blockIdx.x) * kReduceBlocks;
+  out = (blockIdx.y ? out2 : out) + blockIdx.x;
   double s = 0.0;
   for (int i = threadIdx.x; i < m; i += kThreads) s += partials[i];
   const double t = block_sum_warps(s, sh);
   if (threadIdx.x == 0) out[0] = t;
 }
 
-}  // namespace
-
-void dot(const double* a, const double* b, size_t n, double* partials, double* out,
-         cudaStream_t s, int nb, size_t vst) {
+// the split of a dot product of n elements
+unsigned dot_blocks(size_t n, size_t& chunk) {
   // at least 8192 elements (32 per thread) per block, at most kReduceBlocks blocks: the
   // split depends on n only, so an instance sums in the same order alone and in a batch
   size_t blocks = (n + 8191) / 8192;
   if (blocks > (size_t)kReduceBlocks) blocks = kReduceBlocks;
   if (blocks < 1) blocks = 1;
-  size_t chunk = (n + blocks - 1) / blocks;
+  chunk = (n + blocks - 1) / blocks;
   chunk += chunk & 1;  // even: every block's pairs start 16-byte aligned
-  k_dot_partial<<<dim3((unsigned)blocks, nb), kThreads, 0, s>>>(a, b, n, vst, chunk, partials);
-  k_sum_final<<<nb, kThreads, 0, s>>>(partials, (int)blocks, out);
+  return (unsigned)blocks;
+}
+
+}  // namespace
+
+void dot(const double* a, const double* b, size_t n, double* partials, double* out,
+         cudaStream_t s, int nb, size_t vst) {
+  size_t chunk;
+  const unsigned blocks = dot_blocks(n, chunk);
+  k_dot_partial<<<dim3(blocks, nb), kThreads, 0, s>>>(a, b, n, vst, chunk, partials);
+  k_sum_final<<<nb, kThreads, 0, s>>>(partials, (int)blocks, out, nullptr);
+}
+
+void dot2(const double* a, const double* b, const double* c, size_t n, double* partials,
+          double* out, double* out2, cudaStream_t s, int nb, size_t vst) {
+  size_t chunk;
+  const unsigned blocks = dot_blocks(n, chunk);
+  k_dot2_partial<<<dim3(blocks, nb), kThreads, 0, s>>>(a, b, c, n, vst, chunk, partials);
+  k_sum_final<<<dim3(nb, 2), kThreads, 0, s>>>(partials, (int)blocks, out, out2);
 }
 
 namespace {
