@@ -106,7 +106,8 @@ struct fmg_eig_handle {
          *partials = nullptr, *partials2 = nullptr, *t3 = nullptr, *t3_partials = nullptr, *gAd = nullptr,
          *gMd = nullptr, *t1d = nullptr, *B1d = nullptr, *t0 = nullptr,
          *lam_levels = nullptr, *scal = nullptr, *kscratch = nullptr, *uout = nullptr;
-  double* cg = nullptr;  // conjugate gradient smoother: r.r (2 slots) and p.L p per instance
+  double* cg = nullptr;  // conjugate gradient smoother: r.r (2 slots) per instance
+  double* cg_parts = nullptr;  // and its partial sums
   int *iters = nullptr, *status = nullptr;  // [level][instance]
   int* wait_fail = nullptr;  // [instance]: 1 when a bounded device wait gave up in the solve
   int* inv_order = nullptr;                 // sorted index of the caller's instance i

@@ -544,7 +544,10 @@ void build_coarse(fmg_eig_handle* h) {
   h->buu = h->alloc<double>(nb);
   h->scal = h->alloc<double>(3 * (size_t)nb + 8);
   h->partials = h->alloc<double>((size_t)2 * kReduceBlocks * nb);
-  if (h->prob.smoother == FMG_SMOOTH_CG) h->cg = h->alloc<double>(3 * (size_t)nb);
+  if (h->prob.smoother == FMG_SMOOTH_CG) {
+    h->cg = h->alloc<double>(2 * (size_t)nb);
+    h->cg_parts = h->alloc<double>((size_t)kReduceBlocks * nb);
+  }
   h->partials2 = h->alloc<double>((size_t)kReduceBlocks * nb);
   const int nt3 = dim == 2 ? 10 : 20;
   h->t3 = h->alloc<double>((size_t)h->ntri * nt3 * nb);
@@ -739,7 +742,7 @@ void cheb_coefficients(int nu, std::vector<double>& alpha, std::vector<double>& 
 void enqueue_smooth(fmg_eig_handle* h, Level& l, int j, int nu, bool& zero, cudaStream_t s) {
   if (h->prob.smoother == FMG_SMOOTH_CG) {
     // nu CG steps on L x = f from x (Section 4): r in l.r, direction p in l.z, q = L p in l.y;
-    // per-instance scalars r.r (two slots, old / new) and p.q in h->cg
+    // per-instance scalars r.r (two slots, old / new) in h->cg
     if (nu <= 0) return;
     const size_t st = l.g.stride, n = st * l.g.nb;
     if (zero) {
@@ -749,17 +752,19 @@ void enqueue_smooth(fmg_eig_handle* h, Level& l, int j, int nu, bool& zero, cuda
       lv_residual(l, l.f, l.x, l.r, s);
     }
     zero = false;
-    cudaMemcpyAsync(l.z, l.r, n * sizeof(double), cudaMemcpyDeviceToDevice, s);
+    // partial sums of p.q in partials; of r.r in partials2 (the initial ones) and then in turn
     double* rr = h->cg;
     double* rr_new = h->cg + h->nb;
-    double* pq = h->cg + 2 * h->nb;
-    dot(l.r, l.r, st, h->partials, rr, s, l.g.nb, st);
+    double* parts = h->partials2;
+    double* spare = h->cg_parts;
+    cg_start(st, l.g.nb, l.r, l.z, parts, s);
     for (int it = 0; it < nu; ++it) {
       lv_apply(l, l.z, l.y, s);
-      dot(l.z, l.y, st, h->partials, pq, s, l.g.nb, st);
-      cg_update(n, st, rr, pq, l.z, l.y, l.x, l.r, s);
-      dot(l.r, l.r, st, h->partials, rr_new, s, l.g.nb, st);
-      cg_direction(n, st, rr_new, rr, l.r, l.z, s);
+      cg_dot(st, l.g.nb, l.z, l.y, h->partials, s);
+      cg_update(st, l.g.nb, rr, it == 0 ? parts : nullptr, h->partials, l.z, l.y, l.x, l.r, spare,
+                s);
+      if (it + 1 == nu) break;  // the next direction is not needed
+      cg_direction(st, l.g.nb, rr, spare, rr_new, l.r, l.z, s);
       std::swap(rr, rr_new);
     }
     return;
@@ -934,6 +939,7 @@ void enqueue_augment(fmg_eig_handle* h, int k, const double* ut, cudaStream_t s)
   const size_t st = l.g.stride;
   // 3D mixed modes: the double-float split of u~, read by N(u~) / B(u~) and by the mass apply
   const bool df = h->dfloat_loads();
+  const size_t per = df ? kDotPinned : kDotElements;
   const SplitVec us = df ? lv_split(l, ut, s) : SplitVec{};
   fork_sides(h, s, 0, 2);
   // branch 1 (side 0): N(u~) and B(u~), T0, and the restriction / coarsening chains of both.
@@ -945,7 +951,7 @@ void enqueue_augment(fmg_eig_handle* h, int k, const double* ut, cudaStream_t s)
     if (df) lv_nload_density_df(l, us, l.r, b1);
     else lv_nload_density(l, ut, l.r, b1);
     prof_end(h, kProfMoments, k, b1);
-    dot(ut, l.r, st, h->partials2, h->t0, b1, nb, st);
+    dot(ut, l.r, st, h->partials2, h->t0, b1, nb, st, per);
     for (int j = k; j >= 2; --j) {
       lv_restrict(h->L(j), h->L(j - 1), h->L(j).r, h->L(j - 1).r, b1);
       lv_coarsen_density(h->L(j), h->L(j - 1), b1, df);
@@ -967,7 +973,7 @@ void enqueue_augment(fmg_eig_handle* h, int k, const double* ut, cudaStream_t s)
   } else {
     lv_apply_mass_full(l, ut, l.y, l.z, s);
   }
-  dot2(ut, l.y, l.z, st, h->partials, h->auu, h->buu, s, nb, st);
+  dot2(ut, l.y, l.z, st, h->partials, h->auu, h->buu, s, nb, st, per);
   for (int j = k; j >= 2; --j)  // both chains in one launch per level
     lv_restrict(h->L(j), h->L(j - 1), h->L(j).y, h->L(j - 1).y, s, h->L(j).z, h->L(j - 1).z);
   join_sides(h, s, 0, 2);
@@ -1054,6 +1060,7 @@ void enqueue_outputs(fmg_eig_handle* h, cudaStream_t s) {
 
 // b(u,u), a(u,u) + (Wu,u) and int u^4 of every instance's final u into h->scal (3 x nb).
 void enqueue_checks(fmg_eig_handle* h, cudaStream_t s) {
+  const size_t per = h->dfloat_loads() ? kDotPinned : kDotElements;
   double* sa = h->scal;
   double* sb = h->scal + h->nb;
   double* sn = h->scal + 2 * h->nb;
@@ -1064,8 +1071,8 @@ void enqueue_checks(fmg_eig_handle* h, cudaStream_t s) {
     const size_t st = v.g.stride;
     lv_apply_mass_full(v, v.u, v.y, v.z, s);
     lv_nload(v, v.u, v.r, s);
-    dot2(v.u, v.y, v.z, st, h->partials, sa + first, sb + first, s, count, st);
-    dot(v.u, v.r, st, h->partials, sn + first, s, count, st);
+    dot2(v.u, v.y, v.z, st, h->partials, sa + first, sb + first, s, count, st, per);
+    dot(v.u, v.r, st, h->partials, sn + first, s, count, st, per);
   }
 }
 

@@ -301,16 +301,29 @@ void vcycle32_up(const Grid& g, const CoefT& ct, const Grid& gc, const float* f,
 // deterministic two-stage tree whose order depends on n only.  `partials` holds
 // nb * kReduceBlocks doubles.
 constexpr int kReduceBlocks = 1024;
+// Elements per block, at least: 2048, 8 per thread (a reduction over a small level is bound by a
+// thread's chain of loads and sums; 8192 took 15.7 us for both dots of a 1.1M-node level, 2048
+// takes 12.8 for a 0.83M-node one).  The 3D mixed modes keep 8192, whose order of summation their
+// amplified rounding shows.
+constexpr size_t kDotElements = 2048, kDotPinned = 8192;
 void dot(const double* a, const double* b, size_t n, double* partials, double* out,
-         cudaStream_t s, int nb = 1, size_t vst = 0);
+         cudaStream_t s, int nb, size_t vst, size_t per_block);
 // out = a . b and out2 = a . c in one pass (each as dot sums it); partials: 2 kReduceBlocks nb
 void dot2(const double* a, const double* b, const double* c, size_t n, double* partials,
-          double* out, double* out2, cudaStream_t s, int nb, size_t vst);
-// Conjugate gradient smoother steps over nb instances of `stride` elements (n = nb stride):
-// x += a p, r -= a q with a = rr[b] / pq[b]; then p = r + (rr_new[b] / rr_old[b]) p
-void cg_update(size_t n, size_t stride, const double* rr, const double* pq, const double* p,
-               const double* q, double* x, double* r, cudaStream_t s);
-void cg_direction(size_t n, size_t stride, const double* rr_new, const double* rr_old,
+          double* out, double* out2, cudaStream_t s, int nb, size_t vst, size_t per_block);
+// Conjugate gradient smoother over nb instances of n elements (one level's stride; even),
+// kReduceBlocks partial sums per instance and dot product:
+//   start      p = r, rr_parts = parts of r.r
+//   dot        pq_parts = parts of p.q
+//   update     a = rr / pq, x += a p, r -= a q, parts = parts of the new r.r; rr[b] is read, or
+//              (rr_parts given) summed from rr_parts and written
+//   direction  rr_new[b] = sum of parts, p = r + (rr_new / rr_old) p
+void cg_start(size_t n, int nb, const double* r, double* p, double* rr_parts, cudaStream_t s);
+void cg_dot(size_t n, int nb, const double* p, const double* q, double* pq_parts, cudaStream_t s);
+void cg_update(size_t n, int nb, double* rr, const double* rr_parts, const double* pq_parts,
+               const double* p, const double* q, double* x, double* r, double* parts,
+               cudaStream_t s);
+void cg_direction(size_t n, int nb, const double* rr_old, const double* parts, double* rr_new,
                   const double* r, double* p, cudaStream_t s);
 
 // ---- Interior <-> padded packing (pack.cu) ----------------------------------------------
