@@ -77,12 +77,13 @@ extern "C" {
  * expression, so the results are bit-identical; the flag exists for comparison and for
  * drivers where tensor maps cannot be encoded (the library also falls back by itself).     */
 #define FMG_FLAG_NO_TMA 4
-/* flags: evaluate the FP64 cubic load, auxiliary right-hand side and density stencil as
- * column (2D) or plane (3D) walks on every level.  The walks form each mesh edge's (2D) or
+/* flags: evaluate the cubic load, auxiliary right-hand side and density stencil as column
+ * (2D) or plane (3D) walks on every level.  The walks form each mesh edge's (2D) or
  * tetrahedron's (3D) share of the exact integrals of Section 2 once, for all the nodes that
- * need it; by default they are taken only where the launch gives them at least two blocks
- * per SM, and smaller launches run node by node.  Both evaluate the same closed forms, so
- * results agree to rounding; the flag exists for comparison and testing.                   */
+ * need it; by default levels below 64 (2D) or 32 (3D) cells per side run node by node, and in
+ * the 3D mixed modes every launch that gives a walk less than two blocks per SM.  Both
+ * evaluate the same closed forms, so results agree to rounding; the flag exists for
+ * comparison and testing.                                                                   */
 #define FMG_FLAG_STAR_WALKS 8
 /* flags (test hook, no counterpart in the paper): every bounded device wait of the solve's
  * TMA-fed sweeps (FMG_MIXED_FP32 / FMG_MIXED_BF16 levels with at least 512 (2D) or 128 (3D)
@@ -94,9 +95,10 @@ extern "C" {
 #define FMG_FLAG_EXPIRE_WAITS 32
 /* flags: run the fused levels of V-cycles as separate kernels, one per sweep and transfer:
  * the 2D FP64 levels of at most 32 cells per side (damped Jacobi; otherwise one kernel per
- * V-cycle with one CTA per instance) and the single-precision levels below the TMA-fed ones
+ * V-cycle with one CTA per instance), the FP64 levels above them that launch latency bounds (up
+ * to 256 cells in 2D, 32 in 3D; otherwise one kernel per leg) and the single-precision levels below the TMA-fed ones
  * of at most 256 cells (2D) or 32 cells (3D) per side (mixed modes; otherwise two kernels per
- * level on 32 x 32 or 8 x 8 x 8 tiles).  Both evaluate the same expressions in the same
+ * level on 32 x 32 or 8 x 8 x 8 tiles).  All evaluate the same expressions in the same
  * order, so the results are bit-identical; the flag exists for comparison and testing.      */
 #define FMG_FLAG_SEPARATE_VCYCLE 16
 

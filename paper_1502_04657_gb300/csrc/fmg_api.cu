@@ -824,23 +824,37 @@ void enqueue_vcycle(fmg_eig_handle* h, int j, bool x_zero, cudaStream_t s) {
   }
   if (enqueue_vcycle_fused(h, j, x_zero, s)) return;
   const fmg_eig_problem& p = h->prob;
+  Level& lc = h->L(j - 1);
+  // one kernel per leg on the launch-bound levels (but the finest level's first V-cycle, whose
+  // steps are profiled)
+  const bool legs = p.smoother == FMG_SMOOTH_JACOBI && !(p.flags & FMG_FLAG_SEPARATE_VCYCLE) &&
+                    !(j == h->levels() && h->prof_armed[kProfProlong]);
   bool zero = x_zero;
   prof_begin(h, kProfVcycle, j, s);
-  enqueue_smooth(h, l, j, p.nu_pre, zero, s);
-  if (zero) cudaMemsetAsync(l.x, 0, l.g.stride * l.g.nb * sizeof(double), s);
-  Level& lc = h->L(j - 1);
-  prof_begin(h, kProfResidual, j, s);
-  lv_residual(l, l.f, l.x, l.r, s);
-  prof_end(h, kProfResidual, j, s);
-  prof_begin(h, kProfRestrict, j, s);
-  lv_restrict(l, lc, l.r, lc.f, s);
-  prof_end(h, kProfRestrict, j, s);
+  if (legs && vcycle_leg_applies(l.g, p.nu_pre, true)) {
+    vcycle_down(l.g, l.c, l.c3, lc.g, l.f, l.x, l.xt, lc.f, p.nu_pre, zero, s);
+    std::swap(l.x, l.xt);
+  } else {
+    enqueue_smooth(h, l, j, p.nu_pre, zero, s);
+    if (zero) cudaMemsetAsync(l.x, 0, l.g.stride * l.g.nb * sizeof(double), s);
+    prof_begin(h, kProfResidual, j, s);
+    lv_residual(l, l.f, l.x, l.r, s);
+    prof_end(h, kProfResidual, j, s);
+    prof_begin(h, kProfRestrict, j, s);
+    lv_restrict(l, lc, l.r, lc.f, s);
+    prof_end(h, kProfRestrict, j, s);
+  }
   enqueue_vcycle(h, j - 1, true, s);
-  prof_begin(h, kProfProlong, j, s);
-  lv_prolong(l, lc, lc.x, l.x, true, nullptr, nullptr, 0, s);
-  prof_end(h, kProfProlong, j, s);
-  bool post_zero = false;
-  enqueue_smooth(h, l, j, p.nu_post, post_zero, s);
+  if (legs && vcycle_leg_applies(l.g, p.nu_post, false)) {
+    vcycle_up(l.g, l.c, l.c3, lc.g, l.f, lc.x, l.x, l.xt, p.nu_post, s);
+    std::swap(l.x, l.xt);
+  } else {
+    prof_begin(h, kProfProlong, j, s);
+    lv_prolong(l, lc, lc.x, l.x, true, nullptr, nullptr, 0, s);
+    prof_end(h, kProfProlong, j, s);
+    bool post_zero = false;
+    enqueue_smooth(h, l, j, p.nu_post, post_zero, s);
+  }
   prof_end(h, kProfVcycle, j, s);
 }
 

@@ -296,6 +296,26 @@ void vcycle32_up(const Grid& g, const CoefT& ct, const Grid& gc, const float* f,
                  const float* x, float* xo, const float* ec, int nu_post, cudaStream_t s,
                  bool bf = false);
 
+// ---- FP64 V-cycle legs of the middle levels (vcycle_legs.cu) -----------------------------
+// Launch-bound levels, by cells per side and by the instances' nodes together: 2D both legs to
+// 256 cells, 65,536 nodes (solve at h = 1/256 1.13 -> 1.01 ms, h = 1/896 1.92 -> 1.72 ms); 3D up
+// to 32 cells, 32,768 nodes (launches of 16 us -> 11), down to 24 cells, 13,824 nodes (18 -> 8;
+// at 32 cells its 512 blocks take 27 us where the four kernels take 19).  Results are
+// bit-identical to the separate kernels', so the choice may depend on nb.
+inline bool vcycle_leg_applies(const Grid& g, int nu, bool down) {
+  const size_t n = g.n, m = g.nb * n * n;
+  if (g.dim == 2) return nu <= 3 && n <= 256 && m <= 256 * 256;
+  const size_t most = down ? 24 : 32;
+  return nu <= 2 && n <= most && m * n <= most * most * most;
+}
+// xo = nu sweeps on L x = f from x (not read if zero), fc = P^T (f - L xo)
+void vcycle_down(const Grid& g, const Coef2D& c2, const Coef3D& c3, const Grid& gc,
+                 const double* f, const double* x, double* xo, double* fc, int nu, bool zero,
+                 cudaStream_t s);
+// xo = nu sweeps from x + P ec
+void vcycle_up(const Grid& g, const Coef2D& c2, const Coef3D& c3, const Grid& gc, const double* f,
+               const double* ec, const double* x, double* xo, int nu, cudaStream_t s);
+
 // ---- Reductions (reduce.cu) -------------------------------------------------------------
 // out[b] = sum_i a[b vst + i] * b[b vst + i] over n entries for instances b < nb;
 // deterministic two-stage tree whose order depends on n only.  `partials` holds
