@@ -152,14 +152,12 @@ namespace {
 // where one per operation and sum took 7 and 4: a solve on 3D h = 1/64 went from 2.86 to 2.25 ms.
 // Block blockIdx.x takes elements [beg, end) of an even chunk, 2048 (8 per thread) or more.
 
-// the sum of m partial sums, for every thread of the block
-__device__ double sum_partials(const double* __restrict__ partials, int m, double* sh) {
+// the sum of m partial sums, for thread 0
+__device__ __forceinline__ double sum_partials(const double* __restrict__ partials, int m,
+                                               double* sh) {
   double s = 0.0;
   for (int i = threadIdx.x; i < m; i += kThreads) s += partials[i];
-  const double t = block_sum_warps(s, sh);
-  if (threadIdx.x == 0) sh[kThreads / 32] = t;
-  __syncthreads();
-  return sh[kThreads / 32];
+  return block_sum_warps(s, sh);
 }
 
 // f(i) for this thread's pairs of elements (i, i + 1), in a fixed order (n is even)
@@ -172,7 +170,7 @@ __device__ __forceinline__ void for_chunk(size_t n, size_t chunk, F f) {
 __global__ void __launch_bounds__(kThreads)
     k_cg_start(size_t n, size_t chunk, const double* __restrict__ r, double* __restrict__ p,
                double* __restrict__ partials) {
-  __shared__ double sh[kThreads / 32 + 1];
+  __shared__ double sh[kThreads / 32];
   const size_t b = blockIdx.y * n;
   double s0 = 0.0, s1 = 0.0;
   for_chunk(n, chunk, [&](size_t i) {
@@ -188,7 +186,7 @@ __global__ void __launch_bounds__(kThreads)
 __global__ void __launch_bounds__(kThreads)
     k_cg_dot(size_t n, size_t chunk, const double* __restrict__ p, const double* __restrict__ q,
              double* __restrict__ partials) {
-  __shared__ double sh[kThreads / 32 + 1];
+  __shared__ double sh[kThreads / 32];
   const size_t b = blockIdx.y * n;
   double s0 = 0.0, s1 = 0.0;
   for_chunk(n, chunk, [&](size_t i) {
@@ -209,18 +207,17 @@ __global__ void __launch_bounds__(kThreads)
                 const double* __restrict__ rr_parts, const double* __restrict__ pq_parts,
                 const double* __restrict__ p, const double* __restrict__ q,
                 double* __restrict__ x, double* __restrict__ r, double* __restrict__ partials) {
-  __shared__ double sh[kThreads / 32 + 1];
+  __shared__ double sh[2][kThreads / 32], step;
   const size_t b = blockIdx.y * n, pb = (size_t)blockIdx.y * kReduceBlocks;
-  const double pq = sum_partials(pq_parts + pb, gridDim.x, sh);
-  double rr_old;
-  if (rr_parts) {
-    __syncthreads();  // sh is written again
-    rr_old = sum_partials(rr_parts + pb, gridDim.x, sh);
-    if (blockIdx.x == 0 && threadIdx.x == 0) rr[blockIdx.y] = rr_old;
-  } else {
-    rr_old = rr[blockIdx.y];
+  const double pq = sum_partials(pq_parts + pb, gridDim.x, sh[0]);
+  const double sum = rr_parts ? sum_partials(rr_parts + pb, gridDim.x, sh[1]) : 0.0;
+  if (threadIdx.x == 0) {
+    const double rr_old = rr_parts ? sum : rr[blockIdx.y];
+    if (rr_parts && blockIdx.x == 0) rr[blockIdx.y] = rr_old;
+    step = pq > 0.0 ? rr_old / pq : 0.0;
   }
-  const double a = pq > 0.0 ? rr_old / pq : 0.0;
+  __syncthreads();
+  const double a = step;
   double s0 = 0.0, s1 = 0.0;
   for_chunk(n, chunk, [&](size_t i) {
     const double2 pv = *reinterpret_cast<const double2*>(p + b + i);
@@ -235,8 +232,7 @@ __global__ void __launch_bounds__(kThreads)
     s0 = fma(rv.x, rv.x, s0);
     s1 = fma(rv.y, rv.y, s1);
   });
-  __syncthreads();  // sh is written again
-  const double t = block_sum_warps(s0 + s1, sh);
+  const double t = block_sum_warps(s0 + s1, sh[0]);
   if (threadIdx.x == 0) partials[pb + blockIdx.x] = t;
 }
 
@@ -245,11 +241,15 @@ __global__ void __launch_bounds__(kThreads)
     k_cg_direction(size_t n, size_t chunk, const double* __restrict__ rr_old,
                    const double* __restrict__ parts, double* __restrict__ rr_new,
                    const double* __restrict__ r, double* __restrict__ p) {
-  __shared__ double sh[kThreads / 32 + 1];
+  __shared__ double sh[kThreads / 32], ratio;
   const double rn = sum_partials(parts + (size_t)blockIdx.y * kReduceBlocks, gridDim.x, sh);
-  const double ro = rr_old[blockIdx.y];
-  if (blockIdx.x == 0 && threadIdx.x == 0) rr_new[blockIdx.y] = rn;
-  const double c = ro > 0.0 ? rn / ro : 0.0;
+  if (threadIdx.x == 0) {
+    const double ro = rr_old[blockIdx.y];
+    if (blockIdx.x == 0) rr_new[blockIdx.y] = rn;
+    ratio = ro > 0.0 ? rn / ro : 0.0;
+  }
+  __syncthreads();
+  const double c = ratio;
   const size_t b = blockIdx.y * n;
   for_chunk(n, chunk, [&](size_t i) {
     const double2 rv = *reinterpret_cast<const double2*>(r + b + i);
