@@ -15,7 +15,7 @@
 // expansion of q about node v is exact, so int_T phi_v q = sum_{i+j<=3} d^{ij}q(v)/(i!j!) m_ij
 // with m_ij the moments of phi_v over the fine triangles of v's star that lie in T.  Those
 // depend only on v's class (interior of T, one of T's three edges, one of its vertices), so
-// T3 follows from monomial sums of u~ per class: 4 FP64 FMAs per interior node.
+// T3 follows from monomial sums of u~ per class: 4 FP64 operations per interior node.
 #include "fmg_internal.h"
 #include "reduce_dev.cuh"
 #include "dfloat.cuh"

@@ -12,9 +12,10 @@
 // h^2/12 (6 at C, 1 at the six neighbours).  (Derived once by symbolic integration over the
 // six triangles of a node's star.)
 //
-// FP64 on this part issues at ~1/64 of the FP32 rate, so the kernels trade bandwidth for
+// FP64 on this part issues at ~1/64 of the FP32 rate, so the kernels here trade bandwidth for
 // FP64 instructions: the four coupling arrays and omega/D are materialised once per solve
-// (40 B/node extra traffic) and every sweep then costs 9 FP64 instructions per node.
+// (40 B/node extra traffic) and a sweep costs 8 FP64 instructions per node.  The levels from 512
+// cells per side on take the operator in fixed point instead, without the couplings (fxop2d.cu).
 #include "fmg_internal.h"
 #include "dfloat.cuh"
 #include "star2d.cuh"

@@ -11,7 +11,8 @@
 //   XYZ:       w0 h^3 /20  + h^5 [wx (63i^2+63i+19)/1260 + wy (..j..) + wz (..l..)]
 // (Y, Z, XZ, YZ by permuting the axes; the coupling to p - d is the one of p - d to p).  The
 // mass stencil is h^3 (2/5 at C, 1/20 along axes and the body diagonal, 1/30 along face
-// diagonals).  As in 2D, the 8 coupling arrays and omega/D are materialised once per solve.
+// diagonals).  As in 2D, the 8 coupling arrays and omega/D are materialised once per solve, but
+// for the FP64-mode levels whose operator runs in fixed point (fxop3d.cu).
 
 #include "fmg_internal.h"
 #include "dfloat.cuh"

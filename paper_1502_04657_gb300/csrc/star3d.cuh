@@ -103,7 +103,9 @@ template <int P>
 __device__ __forceinline__ int star3_exponent(int n, int pitch, size_t st, const double* u) {
   __shared__ int top[2];
   const int tid = threadIdx.y * kS3X + threadIdx.x;
+  __shared__ unsigned low;
   if (tid < 2) top[tid] = 0;
+  if (tid == 0) low = 0xffffffffu;
   const int nzc = star3_zchunks(n, P);
   const int ib = blockIdx.z / nzc;
   const int z0 = 1 + (int)(blockIdx.z - ib * nzc) * P, z1 = min(z0 + P, n);
@@ -122,10 +124,12 @@ __device__ __forceinline__ int star3_exponent(int n, int pitch, size_t st, const
   if ((tid & 31) == 0) {
     atomicMax(&top[0], m.pos);
     atomicMax(&top[1], m.neg);
+    atomicMin(&low, m.low);
   }
   __syncthreads();
   m.pos = top[0];
   m.neg = top[1];
+  m.low = low;
   return m.exponent();
 }
 
