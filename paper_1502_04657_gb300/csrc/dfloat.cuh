@@ -106,6 +106,17 @@ __device__ __forceinline__ float d2f_rn(double v) {
   return __uint_as_float(r | ((uint32_t)(b >> 32) & 0x80000000u));
 }
 
+// w / c to an ulp in four FP64 operations (the division takes several times that): the
+// single-precision reciprocal y of c leaves e = 1 - c y below 2^-22, and w / c = w y (1 + e +
+// e^2) to 2^-66.  c outside the single-precision range (or not a number) is divided.
+__device__ __forceinline__ double ratio(double w, double c) {
+  const uint32_t ex = ((uint32_t)__double2hiint(c) >> 20) & 0x7ffu;
+  if (ex < 923u || ex > 1123u) return w / c;  // |c| below 2^-100 or above 2^100
+  const double y = f2d_exact(__frcp_rn(d2f_rn(c)));
+  const double e = fma(-c, y, 1.0), wy = w * y;
+  return fma(wy, fma(e, e, e), wy);
+}
+
 // The nonlinear kernels read u either as FP64 or as its split copy (SplitVec: hi and lo
 // arrays written by split_df) and compute in T.
 template <typename T>

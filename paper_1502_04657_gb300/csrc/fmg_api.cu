@@ -43,7 +43,10 @@ Level view(const Level& l, int first, int count) {
   adv(v.x); adv(v.xt); adv(v.f); adv(v.r); adv(v.u); adv(v.y); adv(v.z);
   adv(v.b.C); adv(v.b.E); adv(v.b.N); adv(v.b.NE);
   adv(v.x32); adv(v.xt32); adv(v.f32); adv(v.r32); adv(v.uhi); adv(v.ulo);
-  v.c.tab = v.c3.tab = v.cw.tab = v.cw3.tab = nullptr;  // setup scratch is not sliced
+  for (Coef2D* c : {&v.c, &v.cw})
+    if (c->tab) c->tab += (size_t)first * 8 * (l.g.n + 1);
+  for (Coef3D* c : {&v.c3, &v.cw3})
+    if (c->tab) c->tab += (size_t)first * 15 * (l.g.n + 1);
   for (Coef2D* c : {&v.c, &v.cw})
     if (c->fxt) {
       c->fxt += (size_t)first * 4 * (l.g.n + 1);
@@ -320,24 +323,30 @@ void build_levels(fmg_eig_handle* h) {
     l.g.nb = l.cap;
     l.g.walk_all = (p.flags & FMG_FLAG_STAR_WALKS) != 0;
     const size_t s = l.g.stride * l.cap;
+    // the fixed-point form (fx) reads no couplings; Chebyshev steps and W u of the literal form do
+    const bool fx = dim == 2 ? fxop2d_applies(l.g) : fxop3d_applies(l.g) && !h->mixed();
+    const bool stored = !fx || p.smoother == FMG_SMOOTH_CHEBYSHEV || h->literal();
+    const bool dinv = stored || !h->mixed();
     if (dim == 2) {
-      l.c.cC = h->alloc<double>(s);
-      l.c.cE = h->alloc<double>(s);
-      l.c.cN = h->alloc<double>(s);
-      l.c.cNE = h->alloc<double>(s);
-      l.c.dinv = h->alloc<double>(s);
+      if (stored) {
+        l.c.cC = h->alloc<double>(s);
+        l.c.cE = h->alloc<double>(s);
+        l.c.cN = h->alloc<double>(s);
+        l.c.cNE = h->alloc<double>(s);
+      }
+      if (dinv) l.c.dinv = h->alloc<double>(s);
       l.c.tab = h->alloc<double>(8 * (size_t)(l.g.n + 1) * l.cap);
       l.b.C = h->alloc<double>(s);
       l.b.E = h->alloc<double>(s);
       l.b.N = h->alloc<double>(s);
       l.b.NE = h->alloc<double>(s);
-      if (fxop2d_applies(l.g)) {
+      if (fx) {
         l.c.fxt = h->alloc<long long>(4 * (size_t)(l.g.n + 1) * l.cap);
         l.c.fxh = h->alloc<FxHead2D>(l.cap);
       }
       l.cw = l.c;
       if (h->literal()) {
-        if (fxop2d_applies(l.g)) {
+        if (fx) {
           l.cw.fxt = h->alloc<long long>(4 * (size_t)(l.g.n + 1) * l.cap);
           l.cw.fxh = h->alloc<FxHead2D>(l.cap);
         }
@@ -349,18 +358,18 @@ void build_levels(fmg_eig_handle* h) {
         l.cw.tab = h->alloc<double>(8 * (size_t)(l.g.n + 1) * l.cap);
       }
     } else {
-      for (int q = 0; q < 8; ++q) l.c3.a[q] = h->alloc<double>(s);
-      l.c3.dinv = h->alloc<double>(s);
+      if (stored)
+        for (int q = 0; q < 8; ++q) l.c3.a[q] = h->alloc<double>(s);
+      if (dinv) l.c3.dinv = h->alloc<double>(s);
       l.c3.tab = h->alloc<double>(15 * (size_t)(l.g.n + 1) * l.cap);
       for (int q = 0; q < 8; ++q) l.b3.a[q] = h->alloc<double>(s);
-      const bool fx3 = fxop3d_applies(l.g) && !h->mixed();
-      if (fx3) {
+      if (fx) {
         l.c3.fxt = h->alloc<long long>(6 * (size_t)(l.g.n + 1) * l.cap);
         l.c3.fxh = h->alloc<FxHead3D>(l.cap);
       }
       l.cw3 = l.c3;
       if (h->literal()) {
-        if (fx3) {
+        if (fx) {
           l.cw3.fxt = h->alloc<long long>(6 * (size_t)(l.g.n + 1) * l.cap);
           l.cw3.fxh = h->alloc<FxHead3D>(l.cap);
         }

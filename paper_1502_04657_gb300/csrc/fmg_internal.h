@@ -51,16 +51,20 @@ struct SplitVec {
 struct PotentialParams;
 struct FxHead2D {
   int ok, sa, sm, P, Q, R;
+  double omega;
 };
 
-// Stencil coefficients of L = A + W on one 2D level (see grid2d.cu for the closed forms).
+// Stencil coefficients of L = A + W on one 2D level (see grid2d.cu for the closed forms).  The
+// levels of the fixed-point form keep the couplings only for the Chebyshev smoother and the
+// paper-literal form, and the mixed modes' no omega / cC either (null: their sweeps are single
+// precision; a Jacobi sweep of the component call forms it from tab).
 struct Coef2D {
   double* cC;    // diagonal
   double* cE;    // coupling (i,j)-(i+1,j)
   double* cN;    // coupling (i,j)-(i,j+1)
   double* cNE;   // coupling (i,j)-(i+1,j+1)
   double* dinv;  // omega / cC
-  double* tab;   // 8 * (n + 1) separable parts of the coefficients (setup scratch)
+  double* tab;   // 8 * (n + 1) separable parts of the coefficients per instance
   // levels of the fixed-point form only: 4 (n + 1) table entries and a header per instance
   long long* fxt;
   FxHead2D* fxh;
@@ -135,13 +139,15 @@ void start_vector(const Grid& g, double* c, int cstride, cudaStream_t s);
 // ---- 3D level kernels (grid3d.cu) -------------------------------------------------------
 // Couplings of L on the Kuhn mesh: a[0] diagonal, a[1 + d] the coupling of p with p + d for
 // d = X, Y, Z, XY, XZ, YZ, XYZ (the coupling with p - d is a[1 + d] at p - d).
+// The levels of the fixed-point form keep a as Coef2D says.
 struct FxHead3D {  // as FxHead2D, for fxop3d.cu
   int ok, sa, sm, P, A[3], F[3];
+  double K[8];  // constant parts of the couplings (the others are in tab)
 };
 struct Coef3D {
   double* a[8];
   double* dinv;  // omega / diagonal
-  double* tab;   // 15 * (n + 1) separable parts (setup scratch)
+  double* tab;   // 15 * (n + 1) separable parts per instance
   // FP64-mode levels of the fixed-point form only: 6 (n + 1) table entries and a header per
   // instance
   long long* fxt;

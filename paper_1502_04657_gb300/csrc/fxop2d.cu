@@ -73,6 +73,7 @@ __global__ void k_fxop2d_tables(int n, double h, const PotentialParams* __restri
     q.P = (int)__double2ll_rn(t * (wx + wy) * (-17.0 / 180.0));
     q.Q = (int)__double2ll_rn(t * wy * (-7.0 / 360.0));
     q.R = (int)__double2ll_rn(t * wx * (-7.0 / 360.0));
+    q.omega = p.omega;
     head[blockIdx.y] = q;
   }
 }
@@ -103,7 +104,9 @@ __device__ __forceinline__ double times_pow2(double v, int e) {
   return __hiloint2double(__double2hiint(v) + e * (1 << 20), __double2loint(v));
 }
 
-enum Mode { kJacobiMode, kResidualMode, kApplyMode, kApplyMassMode };
+// kJacobiTabMode: Jacobi with omega / D from the tables (levels that don't store it)
+enum Mode { kJacobiMode, kJacobiTabMode, kResidualMode, kApplyMode, kApplyMassMode };
+constexpr bool jacobi(int mode) { return mode == kJacobiMode || mode == kJacobiTabMode; }
 constexpr bool applies(int mode) { return mode == kApplyMode || mode == kApplyMassMode; }
 
 __device__ __forceinline__ void store(double* o, size_t k, double v) { o[k] = v; }
@@ -112,12 +115,19 @@ __device__ __forceinline__ void store(__nv_bfloat16* o, size_t k, double v) {
   o[k] = __float2bfloat16(d2f_rn(v));
 }
 
-// The tile in FP64, with the expressions of grid2d.cu / mixed.cu.
+// The tile in FP64, with the expressions of grid2d.cu / mixed.cu (the couplings, which these
+// levels don't store, from the same tables).
 template <int MODE, typename S>
-__device__ __noinline__ void tile_fp64(int n, int pitch, size_t base, int i0, int j0,
+__device__ __noinline__ void tile_fp64(int n, int pitch, size_t base, int ib, int i0, int j0,
                                        const Coef2D& c, const double* __restrict__ f,
                                        const double* __restrict__ x, S* __restrict__ out,
                                        double mscale, double* __restrict__ mx) {
+  const int s = n + 1;
+  const double* t = c.tab + (size_t)ib * 8 * s;
+  auto cC = [&](int i, int j) { return t[i] + t[4 * s + j]; };
+  auto cE = [&](int i, int j) { return t[s + i] + t[5 * s + j]; };
+  auto cN = [&](int i, int j) { return t[2 * s + i] + t[6 * s + j]; };
+  auto cNE = [&](int i, int j) { return t[3 * s + i] + t[7 * s + j]; };
   for (int j = j0; j < min(j0 + kRows, n); ++j)
     for (int q = 0; q < 2; ++q) {
       const int i = i0 + q, lane = threadIdx.x;
@@ -125,22 +135,25 @@ __device__ __noinline__ void tile_fp64(int n, int pitch, size_t base, int i0, in
       const size_t k = base + (size_t)j * pitch + i;
       double r;
       if (applies(MODE)) {
-        r = c.cC[k] * x[k];
-        r = fma(c.cE[k], x[k + 1], r);
-        r = fma(c.cE[k - 1], x[k - 1], r);
-        r = fma(c.cN[k], x[k + pitch], r);
-        r = fma(c.cN[k - pitch], x[k - pitch], r);
-        r = fma(c.cNE[k], x[k + pitch + 1], r);
-        r = fma(c.cNE[k - pitch - 1], x[k - pitch - 1], r);
+        r = cC(i, j) * x[k];
+        r = fma(cE(i, j), x[k + 1], r);
+        r = fma(cE(i - 1, j), x[k - 1], r);
+        r = fma(cN(i, j), x[k + pitch], r);
+        r = fma(cN(i, j - 1), x[k - pitch], r);
+        r = fma(cNE(i, j), x[k + pitch + 1], r);
+        r = fma(cNE(i - 1, j - 1), x[k - pitch - 1], r);
       } else {
-        r = fma(-c.cC[k], x[k], f[k]);
-        r = fma(-c.cE[k], x[k + 1], r);
-        r = fma(-c.cE[k - 1], x[k - 1], r);
-        r = fma(-c.cN[k], x[k + pitch], r);
-        r = fma(-c.cN[k - pitch], x[k - pitch], r);
-        r = fma(-c.cNE[k], x[k + pitch + 1], r);
-        r = fma(-c.cNE[k - pitch - 1], x[k - pitch - 1], r);
-        if (MODE == kJacobiMode) r = fma(c.dinv[k], r, x[k]);
+        r = fma(-cC(i, j), x[k], f[k]);
+        r = fma(-cE(i, j), x[k + 1], r);
+        r = fma(-cE(i - 1, j), x[k - 1], r);
+        r = fma(-cN(i, j), x[k + pitch], r);
+        r = fma(-cN(i, j - 1), x[k - pitch], r);
+        r = fma(-cNE(i, j), x[k + pitch + 1], r);
+        r = fma(-cNE(i - 1, j - 1), x[k - pitch - 1], r);
+        if (jacobi(MODE)) {
+          const double di = MODE == kJacobiMode ? c.dinv[k] : ratio(c.fxh[ib].omega, cC(i, j));
+          r = fma(di, r, x[k]);
+        }
       }
       store(out, k, r);
       if (MODE == kApplyMassMode)
@@ -188,7 +201,7 @@ __global__ void __launch_bounds__(32 * kWarps, kBlocks)
   top = __reduce_max_sync(0xffffffffu, top);
   const int e = ((top + 1) >> 20) - 1022;
   if (!hd.ok || e < -kFxMaxExp || e > kFxMaxExp) {
-    tile_fp64<MODE, S>(n, pitch, base, i0, j0, c, f, x, out, mscale, mx);
+    tile_fp64<MODE, S>(n, pitch, base, ib, i0, j0, c, f, x, out, mscale, mx);
     return;
   }
   const int shift = e + 1022 + 5;
@@ -241,8 +254,15 @@ __global__ void __launch_bounds__(32 * kWarps, kBlocks)
       const size_t k = base + (size_t)j * pitch + i0;
       const bool oka = lane > 0 && i0 <= n - 1, okb = lane < 31 && i0 + 1 <= n - 1;
       double va = __ll2double_rn(ra), vb = __ll2double_rn(rb);
-      if (MODE == kJacobiMode) {
-        const double2 di = in ? *reinterpret_cast<const double2*>(c.dinv + k) : zero;
+      if (jacobi(MODE)) {
+        double2 di;
+        if (MODE == kJacobiMode) {
+          di = in ? *reinterpret_cast<const double2*>(c.dinv + k) : zero;
+        } else {
+          const double* t8 = c.tab + (size_t)ib * 8 * (n + 1);
+          const double y = t8[4 * (n + 1) + j];
+          di = make_double2(ratio(hd.omega, t8[ia] + y), ratio(hd.omega, t8[ic] + y));
+        }
         va = fma(times_pow2(di.x, e - kB), va, xv[t + 1].x);
         vb = fma(times_pow2(di.y, e - kB), vb, xv[t + 1].y);
       } else {
@@ -293,7 +313,8 @@ void fxop2d_apply_mass(const Grid& g, const Coef2D& c, const double* x, double* 
 }
 void fxop2d_jacobi(const Grid& g, const Coef2D& c, const double* f, const double* x, double* xo,
                    cudaStream_t s) {
-  launch<kJacobiMode>(g, c, f, x, xo, s);
+  if (c.dinv) launch<kJacobiMode>(g, c, f, x, xo, s);
+  else launch<kJacobiTabMode>(g, c, f, x, xo, s);
 }
 void fxop2d_residual(const Grid& g, const Coef2D& c, const double* f, const double* x, double* r,
                      cudaStream_t s) {

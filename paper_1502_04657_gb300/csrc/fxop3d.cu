@@ -79,6 +79,11 @@ __global__ void k_fxop3d_tables(int n, double h, const PotentialParams* __restri
       // faces XY, XZ, YZ: the axis across is z, y, x
       q.F[a] = (int)__double2ll_rn(t * (s / 168.0 - w[2 - a] / 120.0));
     }
+    // the constant parts of the couplings, as k_coef3d forms them
+    const double w3 = wl * (h * h * h) * p.w0;
+    const double axis = -h + w3 * (1.0 / 20.0), face = w3 * (1.0 / 30.0);
+    const double K[8] = {6.0 * h + w3 * 0.4, axis, axis, axis, face, face, face, w3 * (1.0 / 20.0)};
+    for (int a = 0; a < 8; ++a) q.K[a] = K[a];
     head[blockIdx.y] = q;
   }
 }
@@ -112,23 +117,37 @@ __device__ __forceinline__ long dir(int d, int pitch, long plane) {
   return ox[d] + (long)oy[d] * pitch + oz[d] * plane;
 }
 
-// The block's nodes in FP64, with the expressions of grid3d.cu.
+// The block's nodes in FP64, with the expressions of grid3d.cu (the couplings, which these levels
+// don't store, from k_coef3d's tables and constants).
 template <int MODE>
-__device__ __noinline__ void tile_fp64(int n, int pitch, size_t base, int x, int y, int z0, int z1,
+__device__ __noinline__ void tile_fp64(int n, int pitch, size_t base, int ib, int x, int y, int z0,
+                                       int z1,
                                        const Coef3D& c, const double* __restrict__ f,
                                        const double* __restrict__ v, double* __restrict__ out,
                                        double mscale, double* __restrict__ mv) {
   if (x > n - 1 || y > n - 1) return;
   const long plane = (long)(n + 1) * pitch;
+  constexpr int kQ[8][3] = {{0, 0, 0}, {1, 2, 2}, {2, 1, 2}, {2, 2, 1},
+                            {3, 3, 4}, {3, 4, 3}, {4, 3, 3}, {1, 1, 1}};
+  const int s = n + 1;
+  const double* T = c.tab + (size_t)ib * 15 * s;
+  // coupling q of the node (x, y, z) - b d(q - 1)
+  auto a = [&](int q, int z, int b) {
+    const int ox = b && (q == 1 || q == 4 || q == 5 || q == 7),
+              oy = b && (q == 2 || q == 4 || q == 6 || q == 7),
+              oz = b && (q == 3 || q == 5 || q == 6 || q == 7);
+    return ((c.fxh[ib].K[q] + T[(5 + kQ[q][1]) * s + y - oy]) + T[(10 + kQ[q][2]) * s + z - oz]) +
+           T[kQ[q][0] * s + x - ox];
+  };
   for (int z = z0; z < z1; ++z) {
     const size_t k = base + z * plane + (long)y * pitch + x;
-    double r = applies(MODE) ? c.a[0][k] * v[k] : fma(-c.a[0][k], v[k], f[k]);
+    double r = applies(MODE) ? a(0, z, 0) * v[k] : fma(-a(0, z, 0), v[k], f[k]);
     double m = 24.0 * v[k];
     for (int d = 0; d < 7; ++d) {
       const long o = dir(d, pitch, plane);
       const double sg = applies(MODE) ? 1.0 : -1.0;
-      r = fma(sg * c.a[1 + d][k], v[k + o], r);
-      r = fma(sg * c.a[1 + d][k - o], v[k - o], r);
+      r = fma(sg * a(1 + d, z, 0), v[k + o], r);
+      r = fma(sg * a(1 + d, z, 1), v[k - o], r);
       if (MODE == kApplyMassMode) m = fma(d >= 3 && d < 6 ? 2.0 : 3.0, v[k + o] + v[k - o], m);
     }
     if (MODE == kApplyMassMode) mv[k] = mscale * m;
@@ -193,7 +212,7 @@ __global__ void __launch_bounds__(kX * kY, 3)
   const int e = ((max(top[0], tf) + 1) >> 20) - 1022;
   const FxHead3D hd = c.fxh[ib];
   if (!hd.ok || top[1] >= 0x7ff00000 || e < -kFxMaxExp || e > kFxMaxExp) {
-    tile_fp64<MODE>(n, pitch, base, x, y, z0, z1, c, f, v, out, mscale, mv);
+    tile_fp64<MODE>(n, pitch, base, ib, x, y, z0, z1, c, f, v, out, mscale, mv);
     return;
   }
   const int shift = e + 1085 - kB;

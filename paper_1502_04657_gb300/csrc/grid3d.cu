@@ -87,6 +87,9 @@ __device__ __forceinline__ double recip(double c) {
 // formed its constants and sums itself.  Couplings: C (tables 0, 0, 0), the axis
 // directions d (table 1 along d, 2 across), the face diagonals opposite axis e (table 3 on
 // the two axes of the face, 4 on e) and the body diagonal (table 1 on every axis).
+// STORED = false, for the levels that keep no couplings (the fixed-point operator's): omega / C
+// alone, five FP64 operations and one store per node.  16.6M nodes: 557 -> 280 us.
+template <bool STORED>
 __global__ void k_coef3d(int n, int pitch, size_t st, double h, const double* __restrict__ tab,
                          const PotentialParams* __restrict__ pp, Coef3D c) {
   const int lane = threadIdx.x & 31;
@@ -104,21 +107,22 @@ __global__ void k_coef3d(int n, int pitch, size_t st, double h, const double* __
                             {3, 3, 4}, {3, 4, 3}, {4, 3, 3}, {1, 1, 1}};
   const double axis = -h + w3 * (1.0 / 20.0), face = w3 * (1.0 / 30.0);
   const double K[8] = {6.0 * h + w3 * 0.4, axis, axis, axis, face, face, face, w3 * (1.0 / 20.0)};
-  double R[8];
+  constexpr int kCount = STORED ? 8 : 1;
+  double R[kCount];
 #pragma unroll
-  for (int q = 0; q < 8; ++q)
+  for (int q = 0; q < kCount; ++q)
     R[q] = (K[q] + T[(5 + kQ[q][1]) * s + j]) + T[(10 + kQ[q][2]) * s + l];
   const size_t base = ib * st + ((size_t)l * s + j) * pitch;
   for (int i = lane; i <= n; i += 32) {
     const size_t k = base + i;
     double cc = 0.0;
 #pragma unroll
-    for (int q = 0; q < 8; ++q) {
+    for (int q = 0; q < kCount; ++q) {
       const double v = R[q] + T[kQ[q][0] * s + i];
-      c.a[q][k] = v;
+      if (STORED) c.a[q][k] = v;
       if (q == 0) cc = v;
     }
-    c.dinv[k] = p.omega * recip(cc);
+    c.dinv[k] = STORED ? p.omega * recip(cc) : ratio(p.omega, cc);
   }
 }
 
@@ -823,7 +827,9 @@ dim3 block3(const Grid& g) { return dim3(g.bx, g.by); }
 void coef3d_setup(const Grid& g, const PotentialParams* p, const Coef3D& c, cudaStream_t s) {
   k_coef1d_3d<<<dim3((g.n + 1 + 127) / 128, g.nb), 128, 0, s>>>(g.n, g.h, p, c.tab);
   const int rows = (g.n + 1) * (g.n + 1);
-  k_coef3d<<<dim3((rows + 7) / 8, g.nb), 256, 0, s>>>(g.n, g.pitch, g.stride, g.h, c.tab, p, c);
+  const dim3 grid((rows + 7) / 8, g.nb);
+  if (c.a[0]) k_coef3d<true><<<grid, 256, 0, s>>>(g.n, g.pitch, g.stride, g.h, c.tab, p, c);
+  else if (c.dinv) k_coef3d<false><<<grid, 256, 0, s>>>(g.n, g.pitch, g.stride, g.h, c.tab, p, c);
   if (c.fxt) fxop3d_tables(g, p, c, s);
 }
 

@@ -33,12 +33,14 @@ def _empty(p, k):
     return torch.empty(p.size(k), dtype=torch.float64, device="cuda")
 
 
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
 @pytest.mark.parametrize("w_const,scale", [(0.3, 1.0), (0.3, 1e-90), (0.3, 1e-120), (2e8, 1.0)],
                          ids=["", "small", "out_of_range", "large_potential"])
-def test_operator_2d(w_const, scale):
+def test_operator_2d(w_const, scale, precision):
     """n = 640: 639 = 10 x 62 + 19 columns, 39 x 16 + 15 rows.  1e-120 leaves the exponents'
-    range; h^2 W / 12 = 41 leaves the formats."""
+    range; h^2 W / 12 = 41 leaves the formats.  Mixed handles keep no omega / D."""
     op, gp = _pair(**{**KW2, "w_const": w_const}, coarse_cells=5, levels=8)
+    gp.precision = _fmg().FMG_FP64 if precision == "fp64" else _fmg().FMG_MIXED_FP32
     coarse = O.Level(_mesh(320), None, None, None, None, None, None)
     lev = O.build_level(op, 8, coarse)
     rng = np.random.default_rng(2100)
