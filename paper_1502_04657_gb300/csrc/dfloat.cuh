@@ -112,7 +112,7 @@ __device__ __forceinline__ float d2f_rn(double v) {
 __device__ __forceinline__ double ratio(double w, double c) {
   const uint32_t ex = ((uint32_t)__double2hiint(c) >> 20) & 0x7ffu;
   if (ex < 923u || ex > 1123u) return w / c;  // |c| below 2^-100 or above 2^100
-  const double y = f2d_exact(__frcp_rn(d2f_rn(c)));
+  const double y = f2d_exact(__fdividef(1.0f, d2f_rn(c)));
   const double e = fma(-c, y, 1.0), wy = w * y;
   return fma(wy, fma(e, e, e), wy);
 }

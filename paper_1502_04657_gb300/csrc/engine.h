@@ -83,7 +83,7 @@ struct fmg_eig_handle {
   // two side chains of the augmented pass (side 0, 1) and the operator setup of levels >= 2
   // (side 2, joined at the stage that first needs the level).
   cudaStream_t side[3] = {};
-  cudaEvent_t ev_fork = nullptr, ev_join[2] = {}, ev_level[FMG_MAX_LEVELS + 1] = {};
+  cudaEvent_t ev_fork = nullptr, ev_load = nullptr, ev_join[2] = {}, ev_level[FMG_MAX_LEVELS + 1] = {};
   bool level_pending[FMG_MAX_LEVELS + 1] = {};  // enqueue-time: setup of level k not joined yet
   std::vector<fmg::Level> lv;  // lv[0] = level 1
   std::vector<void*> allocs;

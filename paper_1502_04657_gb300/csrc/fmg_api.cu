@@ -205,6 +205,7 @@ fmg_eig_handle::~fmg_eig_handle() {
   if (ev0) cudaEventDestroy(ev0);
   if (ev1) cudaEventDestroy(ev1);
   if (ev_fork) cudaEventDestroy(ev_fork);
+  if (ev_load) cudaEventDestroy(ev_load);
   for (StageMark& m : marks)
     if (m.ev) cudaEventDestroy(m.ev);
   for (cudaEvent_t e : ev_join)
@@ -630,34 +631,37 @@ void need_level(fmg_eig_handle* h, int k, cudaStream_t s) {
 }
 
 // Operators of every level for every instance that has the level, and the level-1 inverse.
-// With `overlap`, levels >= 2 are built on a side stream while the coarse solve runs, and
-// each stage joins the levels it needs (need_level).
+// With `overlap`, the inverse (36 us on one SM per instance, which the coarse solve does not
+// need) and the levels >= 2 are built on a side stream while the coarse solve runs, and each
+// stage joins the levels it needs (need_level; level 2 covers the inverse).
 void enqueue_setup(fmg_eig_handle* h, cudaStream_t s, bool overlap = false) {
   h->activate(h->nb);
-  if (overlap && h->levels() >= 2) fork_sides(h, s, 2, 1);
-  for (int k = 1; k <= h->levels(); ++k) {
+  const bool fork = overlap && h->levels() >= 2;
+  auto build = [&](int k, cudaStream_t q) {
     Level& l = h->L(k);
-    const cudaStream_t sk = overlap && k >= 2 ? h->side[2] : s;
-    const cudaStream_t s_saved = s;
-    s = sk;
-    prof_begin(h, kProfCoef, k, s);
-    lv_coef(l, h->dparams, s);
-    if (h->literal()) lv_coef(l, h->dparams_full, s, true);
-    prof_end(h, kProfCoef, k, s);
-    if (h->mixed()) tables_f32(l.g, l.c, l.c3, h->dparams, l.ct, s);
-    if (sk != s_saved) {
-      cudaEventRecord(h->ev_level[k], sk);
-      h->level_pending[k] = true;
-    }
-    s = s_saved;
-  }
+    prof_begin(h, kProfCoef, k, q);
+    lv_coef(l, h->dparams, q);
+    if (h->literal()) lv_coef(l, h->dparams_full, q, true);
+    prof_end(h, kProfCoef, k, q);
+    if (h->mixed()) tables_f32(l.g, l.c, l.c3, h->dparams, l.ct, q);
+  };
+  build(1, s);
   lv_dense_level1(h->L(1), h->L1, h->M1, s, true);
   if (h->literal()) lv_dense_level1(h->L(1), h->L1A, h->M1, s, false);
+  if (fork) fork_sides(h, s, 2, 1);
+  const cudaStream_t q = fork ? h->side[2] : s;
   const int np = h->npinned, rest = h->L(1).g.nb - np;  // all instances are active here
   const size_t nn = (size_t)h->nh * h->nh;
-  if (np) dense_spd_inverse_pinned(h->L1A, h->L1inv, h->nh, np, s);
+  if (np) dense_spd_inverse_pinned(h->L1A, h->L1inv, h->nh, np, q);
   if (rest)
-    dense_spd_inverse(h->L1A + np * nn, h->L1inv + np * nn, h->nh, h->lists, h->dims, rest, s);
+    dense_spd_inverse(h->L1A + np * nn, h->L1inv + np * nn, h->nh, h->lists, h->dims, rest, q);
+  for (int k = 2; k <= h->levels(); ++k) {
+    build(k, q);
+    if (fork) {
+      cudaEventRecord(h->ev_level[k], q);
+      h->level_pending[k] = true;
+    }
+  }
 }
 
 DenseProblem dense_base(fmg_eig_handle* h) {
@@ -965,27 +969,31 @@ void enqueue_augment(fmg_eig_handle* h, int k, const double* ut, cudaStream_t s)
   const size_t per = df ? kDotPinned : kDotElements;
   const SplitVec us = df ? lv_split(l, ut, s) : SplitVec{};
   fork_sides(h, s, 0, 2);
-  // branch 1 (side 0): N(u~) and B(u~), T0, and the restriction / coarsening chains of both.
-  // They run on the integer or FP32 pipes (3D mixed modes), beside the FP64 T3 sums
-  // and applies of the other branches.
-  {
-    const cudaStream_t b1 = h->side[0];
-    prof_begin(h, kProfMoments, k, b1);
-    if (df) lv_nload_density_df(l, us, l.r, b1);
-    else lv_nload_density(l, ut, l.r, b1);
-    prof_end(h, kProfMoments, k, b1);
-    dot(ut, l.r, st, h->partials2, h->t0, b1, nb, st, per);
-    for (int j = k; j >= 2; --j) {
-      lv_restrict(h->L(j), h->L(j - 1), h->L(j).r, h->L(j - 1).r, b1);
-      lv_coarsen_density(h->L(j), h->L(j - 1), b1, df);
-    }
-  }
+  // branch 1 (side 0): N(u~) and B(u~), and the coarsening chain of B.  They run on the integer or
+  // FP32 pipes (3D mixed modes), beside the FP64 T3 sums and applies of the other branches.
+  const cudaStream_t b1 = h->side[0], b2 = h->side[1];
+  auto load_chain = [&](cudaStream_t q) {  // T0 and the restriction chain of N(u~)
+    dot(ut, l.r, st, h->partials2, h->t0, q, nb, st, per);
+    for (int j = k; j >= 2; --j) lv_restrict(h->L(j), h->L(j - 1), h->L(j).r, h->L(j - 1).r, q);
+  };
+  prof_begin(h, kProfMoments, k, b1);
+  if (df) lv_nload_density_df(l, us, l.r, b1);
+  else lv_nload_density(l, ut, l.r, b1);
+  prof_end(h, kProfMoments, k, b1);
+  // N's chain follows the T3 sums, so that the launches of the two chains run side by side (h =
+  // 1/256 2D 1.01 -> 0.97 ms with the inverse beside the coarse solve); the T3 sums of pinned
+  // instances are the longest branch already, and it follows N there
+  const bool pinned = h->npinned > 0;
+  if (pinned) load_chain(b1);
+  else cudaEventRecord(h->ev_load, b1);
+  for (int j = k; j >= 2; --j) lv_coarsen_density(h->L(j), h->L(j - 1), b1, df);
   // branch 2 (side 1): T3 per coarse simplex
-  {
-    const cudaStream_t b2 = h->side[1];
-    prof_begin(h, kProfT3, k, b2);
-    lv_t3(l, h->prob.coarse_cells, h->npinned, ut, h->t3_partials, h->t3, b2);
-    prof_end(h, kProfT3, k, b2);
+  prof_begin(h, kProfT3, k, b2);
+  lv_t3(l, h->prob.coarse_cells, h->npinned, ut, h->t3_partials, h->t3, b2);
+  prof_end(h, kProfT3, k, b2);
+  if (!pinned) {
+    cudaStreamWaitEvent(b2, h->ev_load, 0);
+    load_chain(b2);
   }
   // main branch: (A + W) u~, M u~, their dots and restriction chains.  The 3D mixed modes form
   // M u~ in double-float on the FP32 pipes (positive weights: ~2^-47 of the result); the
@@ -1245,7 +1253,8 @@ int create_handle(const fmg_eig_problem* probs, int count, const CreateOptions& 
   bool ok = cudaGetDevice(&h->dev) == cudaSuccess &&
             cudaStreamCreateWithFlags(&h->stream, cudaStreamNonBlocking) == cudaSuccess &&
             cudaEventCreate(&h->ev0) == cudaSuccess && cudaEventCreate(&h->ev1) == cudaSuccess &&
-            cudaEventCreateWithFlags(&h->ev_fork, cudaEventDisableTiming) == cudaSuccess;
+            cudaEventCreateWithFlags(&h->ev_fork, cudaEventDisableTiming) == cudaSuccess &&
+            cudaEventCreateWithFlags(&h->ev_load, cudaEventDisableTiming) == cudaSuccess;
   for (int i = 0; ok && i < 3; ++i)
     ok = cudaStreamCreateWithFlags(&h->side[i], cudaStreamNonBlocking) == cudaSuccess &&
          (i == 2 || cudaEventCreateWithFlags(&h->ev_join[i], cudaEventDisableTiming) == cudaSuccess);
