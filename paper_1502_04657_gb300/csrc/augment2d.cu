@@ -160,13 +160,7 @@ __device__ __forceinline__ void run_sums(const double (&v)[kRun], int e,
   long long i0 = 0, i1 = 0, i2 = 0, i3 = 0;
 #pragma unroll
   for (int q = 0; q < kRun; ++q) {
-    const int hi = __double2hiint(v[q]);
-    const unsigned long long m =
-        ((unsigned long long)(((uint32_t)hi & 0xfffffu) | 0x100000u) << 32 |
-         (uint32_t)__double2loint(v[q])) << 10;
-    const int sh = min(shift - ((hi >> 20) & 0x7ff), 63);
-    const long long t = (long long)(((m >> sh) + 1) >> 1), sg = hi >> 31;  // rounded
-    i0 += (t ^ sg) - sg;
+    i0 += fx_rounded(v[q], shift);
     i1 += i0;
     i2 += i1;
     i3 += i2;

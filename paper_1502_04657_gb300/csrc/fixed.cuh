@@ -97,6 +97,18 @@ __device__ __forceinline__ double to_double(fx<K> x, double scale) {
   return __ll2double_rn(x.v) * scale;
 }
 
+// v as an integer in units of 2^(e - B), |v| <= 2^e, rounded, on the integer pipes (a conversion
+// occupies the FP64 pipe like an FP64 operation); shift = e + 1084 - B
+__device__ __forceinline__ long long fx_rounded(double v, int shift) {
+  const int hi = __double2hiint(v);
+  const unsigned long long m =
+      ((unsigned long long)(((uint32_t)hi & 0xfffffu) | 0x100000u) << 32 |
+       (uint32_t)__double2loint(v)) << 10;
+  const int sh = min(shift - ((hi >> 20) & 0x7ff), 63);
+  const long long t = (long long)(((m >> sh) + 1) >> 1), sg = hi >> 31;
+  return (t ^ sg) - sg;
+}
+
 // u read in fixed point: scale = 2^(B1 - e)
 struct FxVec {
   const double* __restrict__ u;

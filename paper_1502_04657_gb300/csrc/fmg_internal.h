@@ -116,6 +116,10 @@ void residual2d(const Grid& g, const Coef2D& c, const double* f, const double* x
 void cheb2d(const Grid& g, const Coef2D& c, const double* f, const double* x, double* d,
             double* xo, double alpha, double beta, bool first, bool x_zero, cudaStream_t s);
 // rc = P^T rf; with rf2 given, also rc2 = P^T rf2 in the same launch
+// Levels whose restriction sums in integers: those above the V-cycle legs' (vcycle_legs.cu), to
+// whose FP64 sums the separate kernels are bit-identical.  (In 3D the same took a launch from 65
+// to 55 us and no time off a solve.)
+inline bool restrict_ints(const Grid& fine) { return fine.n >= 512; }
 void restrict2d(const Grid& fine, const Grid& coarse, const double* rf, double* rc,
                 cudaStream_t s, const double* rf2 = nullptr, double* rc2 = nullptr);
 // xf = (add ? xf : 0) + P ec (+ scale[b * scale_stride] * extra for instance b when extra is

@@ -120,6 +120,23 @@ def test_load_2d_not_finite():
     assert rel(out[ok], ref[ok]) <= 1e-13
 
 
+def test_restriction_2d_zeros_and_not_finite():
+    """r_c = P^T r_f (r = f for x = 0) with a zero quarter and an infinity, n = 640."""
+    op, gp = _pair(**KW2, coarse_cells=5, levels=8)
+    f = np.random.default_rng(2450).normal(size=(639, 639))
+    f[:, :160] = 0.0
+    f[333, 401] = np.inf
+    with _fmg().Solver(gp) as s:
+        rc = _empty(gp, 7)
+        s.residual_restrict(8, dev(f.ravel()), dev(np.zeros(f.size)), rc)
+    rc = host(rc)
+    ok = np.isfinite(rc)
+    f[333, 401] = 0.0
+    ref = O.prolongation(_mesh(320), _mesh(640)).T @ f.ravel()
+    assert 1 <= (~ok).sum() <= 4 and np.all(rc[ok & (ref == 0.0)] == 0.0)
+    assert np.abs((rc - ref)[ok]).max() <= 1e-13 * np.abs(ref).max()
+
+
 @pytest.mark.parametrize("sign", ["one", "mixed"])
 @pytest.mark.parametrize("kw,k", [(dict(KW2, coarse_cells=5, levels=7), 7),
                                   (dict(KW2, coarse_cells=7, levels=4), 4),
