@@ -75,58 +75,49 @@ WORKLOADS = {
 }
 FP64_FLOP_PER_CLK_SM = 4      # 2 DFMA per clock per SM (1.25 TFLOP/s nominal at 2070 MHz)
 N_SM = 152
-# Algorithmic FP64 flops and bytes per node of the finest-level launch:
-#   Jacobi 2D: the defect f - L x as 7 multiply-adds + the update x + (omega/D) r = 16 flop;
-#     24 B (x, f, x') + 40 B (4 couplings + omega/D)
-#   cubic load + density stencil 2D (closed forms over the 6 star triangles from per-edge
-#     numbers: 3 own edges x 5 + square 1 + 3 six-term sums 15 + cubic bracket 8 + diagonal 6
-#     + 3 off-diagonal entries x 8): 69 flop; 8 B read + 40 B written
-#   Jacobi 3D: 15 multiply-adds + update = 32 flop; 24 B + 72 B
-#   cubic load + density stencil 3D (symmetric sums of the 6 tetrahedra of a cube formed once,
-#     the power sums of the base vertices and the first middle vertex shared by two tetrahedra:
-#     90 flop with u^2, 2 u^3; star and edge sums 73; N, diagonal and 7 edge entries 86):
-#     249 flop; 8 B + 72 B
-# The third number counts FP64 instructions (DADD, DMUL and DFMA alike take one issue slot of
-# the FP64 pipe, 2 per SM per clock): the unit these kernels are bound by.  The Jacobi update
-# forms f - L x as one chain of fused multiply-adds from f, then x + (omega/D) r: 8 in 2D,
-# 16 in 3D.
+# The finest-level launches that compute in 64-bit fixed point (the level operator, and the cubic
+# load with the density stencil) are reported against the HBM copy rate, at the bytes per node
+# they cannot do without, with the FP64 flop of the closed forms they replace beside it:
+#   Jacobi: x, f, omega / D, x' = 32 B; FP64 flop of 7 (15) multiply-adds + update
+#   cubic load + density stencil: u in, N and 4 (8) entries out
 KERNELS = {
-    2: {"nload_density": (69.0, 48.0, 55.0), "jacobi": (16.0, 64.0, 8.0)},
-    3: {"nload_density": (249.0, 80.0, 198.0), "jacobi": (32.0, 96.0, 16.0)},
+    2: {"nload_density": (69.0, 48.0), "jacobi": (16.0, 32.0)},
+    3: {"nload_density": (249.0, 80.0), "jacobi": (32.0, 32.0)},
 }
-# Launches too small to fill the GPU as walks run node by node, each node forming the sums of
-# its own star: 2D 106 flop in 82 FP64 instructions (pair sums n_k + n_{k+1}), 3D 659 flop in
-# about 490 (sums over the link of the 24-tetrahedron star).
-NODE_KERNELS = {2: {"nload_density": (106.0, 48.0, 82.0)}, 3: {"nload_density": (659.0, 80.0, 490.0)}}
+# Small levels run these in FP64, node by node, against the FP64 multiply-add rate: flop, bytes
+# and FP64 instructions per node (DADD, DMUL and DFMA alike take one issue slot of the FP64
+# pipe, 2 per SM per clock).  The Jacobi update forms f - L x as one chain of fused multiply-adds
+# from f, then x + (omega/D) r, and reads the stored couplings; the cubic load forms the sums of
+# its own star (2D pair sums n_k + n_{k+1}, 3D the link of the 24-tetrahedron star).
+NODE_KERNELS = {
+    2: {"nload_density": (106.0, 48.0, 82.0), "jacobi": (16.0, 64.0, 8.0)},
+    3: {"nload_density": (659.0, 80.0, 490.0), "jacobi": (32.0, 96.0, 16.0)},
+}
 
 
-def star_walks(dim: int, n: int, nb: int) -> bool:
-    """Whether the library runs a level of n cells per side (nb instances) as a column / plane
-    walk: when the walk's grid has at least two blocks per SM (30 x 64-node 2D blocks,
-    32 x 8 x 16-node 3D blocks)."""
-    m = n - 1
-    if dim == 2:
-        blocks = -(-m // 30) * -(-m // 64)
-    else:
-        blocks = -(-m // 32) * -(-m // 8) * -(-m // 16)
-    return blocks * nb >= 2 * N_SM
-# the kernel with the largest share of the solve in the ncu launch lists (2D FP64 solve:
-# k_jacobi2d 21 %; 3D FP64 solve: k_nload_density3d 35 %)
-DOMINANT = {2: "jacobi", 3: "nload_density"}
+def fixed_point(dim: int, n: int, name: str) -> bool:
+    """Whether an FP64 level of n cells per side runs the kernel in fixed point (and a 2D mixed
+    one its loads)."""
+    if name == "jacobi":
+        return n >= (512 if dim == 2 else 96)
+    return n >= (64 if dim == 2 else 32)
+
+
+# the kernel with the largest share of the solve in the ncu launch lists (2D FP64 solve: Jacobi
+# 24 %; 3D FP64 solve: Jacobi 24 %)
+DOMINANT = {2: "jacobi", 3: "jacobi"}
 # The single-precision V-cycle (mixed modes) is HBM-bound: a Jacobi sweep or residual reads x
 # and f and writes one vector, 3 x 4 bytes per node (3 x 2 with BF16 storage); the
 # coefficients are rebuilt from per-axis tables that stay in L1.
 MIXED_HBM_KERNELS = ("jacobi", "residual")
-# The mixed modes evaluate the cubic load + density stencil in double-float arithmetic on the
+# The 3D mixed modes evaluate the cubic load + density stencil in double-float arithmetic on the
 # FP32 pipes: the kernel is bound by instruction issue (4 warp instructions per SM per clock).
 # Thread instructions per node (smsp__inst_executed.sum x 32 / nodes) and DRAM bytes per node
-# from one ncu capture of each kernel: 2D the finest launch of the 10-level mixed solve
-# (node by node, 16,769,025 nodes); 3D the plane walk at h = 1/128 (2,048,383 nodes; the walk
-# runs every 3D level with n >= 128, so its per-node figures hold at h = 1/256).
+# from one ncu capture of the plane walk at h = 1/128 (2,048,383 nodes; the walk runs every 3D
+# level with n >= 128, so its per-node figures hold at h = 1/256).
 ISSUE_PER_CLK_SM = 4 * 32
-DF_INSTR_PER_NODE = {2: 618510721 * 32 / 16769025, 3: 200397029 * 32 / 2048383}
-DF_TRAFFIC_PER_NODE = {2: (136027392 + 609443328) / 16769025,
-                       3: (24750336 + 83417856) / 2048383}
+DF_INSTR_PER_NODE = 200397029 * 32 / 2048383
+DF_TRAFFIC_PER_NODE = (24750336 + 83417856) / 2048383
 
 
 def hbm_peak() -> tuple[float, str]:
@@ -135,14 +126,6 @@ def hbm_peak() -> tuple[float, str]:
             return float(json.load(f)["hbm_gbs"]), "of measured (STREAM-style copy)"
     except (OSError, KeyError, ValueError):
         return 6800.0, "of fallback"
-# DRAM bytes per node of a finest-level launch from one ncu capture of the current kernel
-# (dram__bytes_read.sum + dram__bytes_write.sum of the level-9 launch of the 9-level 2D
-# solve, 4,190,209 nodes), scaled by the nodes a launch processes.
-TRAFFIC_PER_NODE = {(2, "nload_density"): (34.109952e6 + 106.015232e6) / 4190209,
-                    # the first level-9 sweep of the 9-level 2D solve, 4,190,209 nodes
-                    (2, "jacobi"): (235144960 + 24157184) / 4190209,
-                    # 3D: the level-6 launch of the 6-level solve, 2,048,383 nodes
-                    (3, "nload_density"): (22.779648e6 + 83.184128e6) / 2048383}
 
 
 def rank_info():
@@ -759,51 +742,55 @@ def serve_cpu_baseline(count: int = 6, cap2: int = 6, cap3: int = 4) -> dict:
 
 
 def roofline(m: dict, clk: dict, fp64_peak: dict | None = None) -> tuple[dict, dict]:
-    """Roofline of the dominant kernel (and the others): FP64 kernels against the measured
-    FP64 multiply-add rate of this run's probe when given (fp64_peak), else the nominal rate
-    from unit counts and clock; the nominal fraction is kept beside the measured one."""
+    """Roofline of the dominant kernel (and the others): fixed-point and single-precision kernels
+    against the HBM copy rate, FP64 kernels (small levels) against the measured FP64 multiply-add
+    rate of this run's probe when given (fp64_peak), else the nominal rate from unit counts and
+    clock, the nominal fraction kept beside the measured one."""
     sm_max = (clk or {}).get("sm_max_mhz") or 2070
     nominal = FP64_FLOP_PER_CLK_SM * N_SM * sm_max * 1e6 / 1e12
     peak = fp64_peak["tflops"] if fp64_peak else nominal
+    hpeak, hsrc = hbm_peak()
     roof = {}
+    dim, n = m["dim"], m["n_finest"]
     nodes = m.get("dofs_finest_launch", m["dofs"])  # nodes one finest-level launch processes
     mixed = m.get("mixed")
-    if mixed:  # FP32 / BF16 V-cycle kernels against the HBM peak
-        bpn = 6.0 if mixed == "bf16" else 12.0
-        hpeak, hsrc = hbm_peak()
+
+    def hbm(ms, bpn, **more):
+        ach = bpn * nodes / (ms * 1e-3) / 1e9
+        return {"bound": "hbm", "achieved": ach, "peak": hpeak, "unit": "GB/s",
+                "frac": ach / hpeak, "traffic": None, "launch_ms": ms, "bytes_per_node": bpn,
+                "peak_source": hsrc, **more}
+
+    if mixed:  # FP32 / BF16 V-cycle kernels
         for name in MIXED_HBM_KERNELS:
             ms = m["profile"].get(name, -1.0)
             if ms and ms > 0:
-                ach = bpn * nodes / (ms * 1e-3) / 1e9
-                roof[name + "32"] = {"bound": "hbm", "achieved": ach, "peak": hpeak, "unit": "GB/s",
-                                     "frac": ach / hpeak, "traffic": None, "launch_ms": ms,
-                                     "bytes_per_node": bpn, "peak_source": hsrc}
-    ops_peak = peak / 2  # one FP64 instruction per multiply-add lane of the probe
-    table = dict(KERNELS[m["dim"]])
-    node_run = "n_finest" in m and not star_walks(m["dim"], m["n_finest"], m.get("nb_finest", 1))
-    if node_run:
-        table.update(NODE_KERNELS[m["dim"]])
-    for name, (flops, nbytes, ops) in table.items():
-        if mixed and name in MIXED_HBM_KERNELS:
-            continue
+                roof[name + "32"] = hbm(ms, 6.0 if mixed == "bf16" else 12.0)
+    for name in KERNELS[dim]:
         ms = m["profile"].get(name, -1.0)
-        if mixed and name == "nload_density" and ms and ms > 0:
+        if mixed and name in MIXED_HBM_KERNELS or not ms or ms <= 0:
+            continue
+        if mixed and dim == 3:
             ipeak = ISSUE_PER_CLK_SM * N_SM * sm_max * 1e6 / 1e12
-            ach = DF_INSTR_PER_NODE[m["dim"]] * nodes / (ms * 1e-3) / 1e12
+            ach = DF_INSTR_PER_NODE * nodes / (ms * 1e-3) / 1e12
             roof[name] = {"bound": "alu", "achieved": ach, "peak": ipeak, "unit": "Tinst/s",
-                          "frac": ach / ipeak, "traffic": DF_TRAFFIC_PER_NODE[m["dim"]] * nodes,
+                          "frac": ach / ipeak, "traffic": DF_TRAFFIC_PER_NODE * nodes,
                           "launch_ms": ms, "arithmetic": "double-float on the FP32 pipes",
                           "peak_source": ("instruction issue: 152 SMs x 4 schedulers x 32 lanes "
                                           "x sm_max_mhz (derived from unit counts and clock)")}
-            continue
-        if ms and ms > 0:
+        elif fixed_point(dim, n, name):
+            flops, nbytes = KERNELS[dim][name]
+            roof[name] = hbm(ms, nbytes, arithmetic="64-bit fixed point (integer pipes)",
+                             fp64_flop_equivalent={"per_node": flops, "peak": peak,
+                                                   "achieved": flops * nodes / (ms * 1e-3) / 1e12,
+                                                   "unit": "TFLOP/s"})
+        else:
+            flops, nbytes, ops = NODE_KERNELS[dim][name]
             ach = flops * nodes / (ms * 1e-3) / 1e12
-            # (the DRAM figures were captured on the walk kernels)
-            tpn = None if node_run and name in NODE_KERNELS[m["dim"]] else \
-                TRAFFIC_PER_NODE.get((m["dim"], name))
             ops_ach = ops * nodes / (ms * 1e-3) / 1e12
+            ops_peak = peak / 2  # one FP64 instruction per multiply-add lane of the probe
             roof[name] = {"bound": "alu", "achieved": ach, "peak": peak, "unit": "TFLOP/s",
-                          "frac": ach / peak, "traffic": tpn * nodes if tpn else None,
+                          "frac": ach / peak, "traffic": None,
                           "peak_nominal": nominal, "frac_nominal": ach / nominal,
                           "launch_ms": ms,
                           "hbm_gbs_algorithmic": nbytes * nodes / (ms * 1e-3) / 1e9,
@@ -811,7 +798,7 @@ def roofline(m: dict, clk: dict, fp64_peak: dict | None = None) -> tuple[dict, d
                                         "unit": "T FP64 instructions/s",
                                         "frac": ops_ach / ops_peak}}
     dom = DOMINANT[m["dim"]]
-    if dom not in roof:  # FP32 V-cycles (mixed modes): the FP64 nonlinear pass dominates
+    if dom not in roof:  # FP32 V-cycles (mixed modes): the nonlinear pass dominates
         dom = "nload_density"
     main = dict(roof.get(dom, {}))
     main["kernel"] = dom
