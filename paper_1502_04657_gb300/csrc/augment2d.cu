@@ -139,7 +139,8 @@ __global__ void k_nload_density2d_node(int n, int pitch, size_t st, double s60, 
 // (t < s) or T1 (t > s), so every column is the same length and every node is read once; the rows
 // are loaded 16 at a time (a row at a time, with the class of each node decided as it came,
 // waited out a memory latency per row: 532 us on 16.8M nodes) and summed in integers: 153 -> 107 us.
-// Only the 32 rows around a warp's diagonal need the comparison per lane.  Edges, diagonals and vertices (one block per cell) go apart.
+// Only the 32 rows around a warp's diagonal need the comparison per lane.  Edges, diagonals and
+// vertices (one block per cell) go apart.
 constexpr int kSums = 25;
 constexpr int kSumThreads = 128;
 constexpr int kSumRows = 128;

@@ -103,7 +103,6 @@ void mass2d(const Grid& g, const double* x, double* y, cudaStream_t s);
 // y = L x, z = M x
 void apply_mass2d(const Grid& g, const Coef2D& c, const double* x, double* y, double* z,
                   cudaStream_t s);
-// the same from the double-float split of x (mixed-precision modes)
 // f -= W u, W u = (A + W) u - A u from the coefficient sets cw (A + W) and ca (A)
 void sub_wmass2d(const Grid& g, const Coef2D& cw, const Coef2D& ca, const double* u, double* f,
                  cudaStream_t s);
@@ -133,7 +132,6 @@ void rhs2d(const Grid& g, const double* lam, const PotentialParams* p_dev, const
 // the same right-hand side evaluated in FP32 (mixed-precision iteration), stored in FP64
 void rhs2d_f32(const Grid& g, const double* lam, const PotentialParams* p_dev, const double* u,
                double* f, cudaStream_t s);
-// the same right-hand side in double-float arithmetic from the split u (mixed-precision modes)
 // Dense level-1 matrices L_1 and M_1 (n1-1)^2 square, row-major, interior numbering (one
 // pair per instance, back to back).
 void dense_level1_2d(const Grid& g, const Coef2D& c, double* L, double* M, cudaStream_t s);
@@ -201,7 +199,7 @@ void rhs3d_f32(const Grid& g, const double* lam, const PotentialParams* p_dev, c
                double* f, cudaStream_t s);
 void nload_density3d(const Grid& g, const double* u, double* nl, const Density3D& b,
                      cudaStream_t s);
-// double-float versions from the split u (mixed-precision modes)
+// double-float versions from the split u (3D mixed-precision modes)
 void rhs3d_df(const Grid& g, const double* lam, const PotentialParams* p_dev, SplitVec u,
               double* f, cudaStream_t s);
 // (the _df versions write the density stencil as double-float splits: see put_entry)

@@ -47,12 +47,6 @@ __device__ __forceinline__ double shfl_up1(double v) { return __shfl_up_sync(0xf
 __device__ __forceinline__ double shfl_down1(double v) {
   return __shfl_down_sync(0xffffffffu, v, 1);
 }
-__device__ __forceinline__ dfloat shfl_up1(dfloat v) {
-  return dfloat(__shfl_up_sync(0xffffffffu, v.hi, 1), __shfl_up_sync(0xffffffffu, v.lo, 1));
-}
-__device__ __forceinline__ dfloat shfl_down1(dfloat v) {
-  return dfloat(__shfl_down_sync(0xffffffffu, v.hi, 1), __shfl_down_sync(0xffffffffu, v.lo, 1));
-}
 template <typename T>
 __device__ __forceinline__ StarEdge<T> shfl_up1(const StarEdge<T>& e) {
   return {shfl_up1(e.s), shfl_up1(e.F), shfl_up1(e.E3)};
@@ -221,8 +215,8 @@ __device__ __forceinline__ void star2d_walk_fx(int n, int pitch, size_t st,
 }
 
 // Walks the rows of this thread's strip of instance blockIdx.z and calls out(k, star) for
-// every interior node it produces (k = the node's index in the batched arrays).  u is read
-// through get<T>: FP64 or the split double-float copy.  blockDim = (32, kStarWarps).
+// every interior node it produces (k = the node's index in the batched arrays).  blockDim = (32,
+// kStarWarps).
 template <typename T, int R, typename U, typename Out>
 __device__ __forceinline__ void star2d_walk(int n, int pitch, size_t st, const U& u, Out out) {
   const int lane = threadIdx.x;
