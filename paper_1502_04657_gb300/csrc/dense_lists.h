@@ -28,6 +28,9 @@ struct DenseLists {
   __host__ __device__ int tripptr(int nh) const { return x3(nh) + nx; }  // end of the staged part
   __host__ __device__ int trip(int nh) const { return tripptr(nh) + nq + 1; }
   __host__ __device__ int total(int nh) const { return trip(nh) + ntrip; }
+  // entries kept on the device, whose kernels copy 16 bytes at a time: none for a mesh whose lists
+  // could not be built (it is refused)
+  int stored(int nh) const { return npat ? (total(nh) + 7) / 8 * 8 : 0; }
 };
 
 // Fill `out` (capacity kDenseMaxLists) for the ntri simplices tri[t * nv + v] (coarse interior

@@ -529,18 +529,20 @@ void build_coarse(fmg_eig_handle* h) {
   for (int k = 1; dim == 3 && h->mixed() && k <= h->levels() && !h->npinned; ++k)
     if (tma_sweep_applies(h->L(k).g)) h->npinned = h->cnt[k];
   if (h->npinned) build_pinned_tables(h, tri);
-  // (a mesh beyond the lists' capacities is beyond dense_smem_bytes' limit too, and refused)
+  // (a mesh beyond the lists' capacities is beyond dense_smem_bytes' limit too, and refused; it
+  // has no lists)
   std::vector<uint16_t> lists(kDenseMaxLists);
   if (!build_dense_lists(h->nh, h->ntri, h->nvert, tri.data(), lists.data(), &h->dims))
     h->dims = DenseLists{};
-  const size_t nl = (h->dims.total(h->nh) + 7) / 8 * 8;  // the kernel copies 16 bytes at a time
+  const size_t nl = h->dims.stored(h->nh);
   h->tri = h->alloc<int>(tri.size());
-  h->lists = h->alloc<uint16_t>(nl);
+  if (nl) h->lists = h->alloc<uint16_t>(nl);
   if (!h->dry) {
     cudaMemcpyAsync(h->tri, tri.data(), tri.size() * sizeof(int), cudaMemcpyHostToDevice,
                     h->stream);
-    cudaMemcpyAsync(h->lists, lists.data(), nl * sizeof(uint16_t), cudaMemcpyHostToDevice,
-                    h->stream);
+    if (nl)
+      cudaMemcpyAsync(h->lists, lists.data(), nl * sizeof(uint16_t), cudaMemcpyHostToDevice,
+                      h->stream);
   }
   const size_t nn = (size_t)h->nh * h->nh;
   h->L1 = h->alloc<double>(nn * nb);
