@@ -23,6 +23,11 @@ struct Level {
   Coef3D c3{};
   Coef2D cw{};  // A + W (the same arrays as c unless the form is paper-literal)
   Coef3D cw3{};
+  // Every array allocated for c, c3 and for cw, cw3 of the paper-literal form; c .. cw3 point to
+  // those that the instances' present forms use (form_operator), nfx and nfxw of them fixed point.
+  Coef2D all{}, allw{};
+  Coef3D all3{}, allw3{};
+  int nfx = 0, nfxw = 0;
   double *x = nullptr, *xt = nullptr, *f = nullptr, *r = nullptr, *u = nullptr,
          *y = nullptr, *z = nullptr;
   Density2D b{};          // density stencil of u~ (augmented pass), 2D
@@ -121,6 +126,8 @@ struct fmg_eig_handle {
   bool literal() const { return prob.operator_form == FMG_PAPER_LITERAL; }
   bool mixed() const { return prob.precision != FMG_FP64; }
   bool bf16() const { return prob.precision == FMG_MIXED_BF16; }
+  // every level keeps its couplings, which Chebyshev steps and W u of the literal form read
+  bool stores_couplings() const { return prob.smoother == FMG_SMOOTH_CHEBYSHEV || literal(); }
   // the nonlinear kernels compute in double-float arithmetic (3D mixed modes)
   bool dfloat_loads() const { return mixed() && prob.dim == 3; }
   // profiling: event pairs around the first finest-level launch of each profiled step
@@ -171,6 +178,8 @@ namespace fmg {
 
 int validate(const fmg_eig_problem* p);
 bool same_shared_settings(const fmg_eig_problem& a, const fmg_eig_problem& b);
+// the levels (bit k) on which p's operator takes the fixed-point form
+uint32_t fx_levels(const fmg_eig_problem& p);
 int create_handle(const fmg_eig_problem* probs, int count, const CreateOptions& opt,
                   fmg_eig_handle** out);
 // Device bytes create_handle will allocate for these instances (an upper bound).

@@ -17,6 +17,7 @@
 #include <new>
 #include <numeric>
 #include <tuple>
+#include <type_traits>
 #include <vector>
 
 #include "engine.h"
@@ -51,11 +52,13 @@ Level view(const Level& l, int first, int count) {
     if (c->fxt) {
       c->fxt += (size_t)first * 4 * (l.g.n + 1);
       c->fxh += first;
+      if (c->fits) c->fits += first;
     }
   for (Coef3D* c : {&v.c3, &v.cw3})
     if (c->fxt) {
       c->fxt += (size_t)first * 6 * (l.g.n + 1);
       c->fxh += first;
+      if (c->fits) c->fits += first;
     }
   v.ct = CoefT{};
   v.g.nb = count;
@@ -67,9 +70,12 @@ Level view(const Level& l, int first, int count) {
 namespace {
 
 // ---- dimension dispatch of the level kernels -----------------------------------------------
-void lv_coef(Level& l, const PotentialParams* p, cudaStream_t s, bool full = false) {
-  if (l.g.dim == 2) coef2d_setup(l.g, p, full ? l.cw : l.c, s);
-  else coef3d_setup(l.g, p, full ? l.cw3 : l.c3, s);
+// stored_whatever: the level keeps couplings for all its instances, whatever their form
+void lv_coef(Level& l, const PotentialParams* p, bool stored_whatever, cudaStream_t s,
+             bool full = false) {
+  const bool ratio_fx = !stored_whatever;
+  if (l.g.dim == 2) coef2d_setup(l.g, p, full ? l.cw : l.c, ratio_fx, s);
+  else coef3d_setup(l.g, p, full ? l.cw3 : l.c3, ratio_fx, s);
 }
 void lv_apply(Level& l, const double* x, double* y, cudaStream_t s) {
   if (l.g.dim == 2) apply2d(l.g, l.c, x, y, s);
@@ -308,6 +314,91 @@ cudaError_t fmg::upload_params(fmg_eig_handle* h, cudaStream_t s) {
 
 namespace fmg {
 
+// ---- forms of the level operators ----------------------------------------------------------
+// Per instance and level (full: of A + W in the paper-literal form): fixed point, where it
+// applies and its formats hold the potential, or FP64 with stored couplings.
+bool fx_form(const Grid& g, const fmg_eig_problem& p, bool full) {
+  if (!(g.dim == 2 ? fxop2d_applies(g) : fxop3d_applies(g) && p.precision == FMG_FP64)) return false;
+  PotentialParams q = potential(p);
+  if (full) q.operator_form = FMG_W_LEFT;
+  return (g.dim == 2 ? fxop2d_scale(g.n, g.h, q) : fxop3d_scale(g.n, g.h, q)).holds;
+}
+
+int count_fx(const fmg_eig_handle* h, const Level& l, bool full) {
+  int m = 0;
+  for (int b = 0; b < l.cap; ++b) m += fx_form(l.g, h->probs[b], full);
+  return m;
+}
+
+uint32_t fx_levels(const fmg_eig_problem& p) {
+  uint32_t m = 0;
+  Grid g;
+  g.dim = p.dim;
+  g.n = p.coarse_cells;
+  for (int k = 1; k <= FMG_MAX_LEVELS && g.n <= 32768; ++k, g.n *= 2) {
+    g.h = p.box_len / g.n;
+    if (fx_form(g, p, true)) m |= 1u << k;
+  }
+  return m;
+}
+
+// The arrays of one level operator that its instances' forms use, from those allocated so far
+// (all), which grow as needed: tables always, couplings where an instance is FP64 (or the
+// smoother or W u of the literal form reads them), omega / D but for mixed fixed-point levels.
+double** coupling(Coef2D& c, int q) {
+  double** const p[4] = {&c.cC, &c.cE, &c.cN, &c.cNE};
+  return p[q];
+}
+double** coupling(Coef3D& c, int q) { return &c.a[q]; }
+
+template <typename Coef>
+void form_operator(fmg_eig_handle* h, const Level& l, Coef& all, Coef& c, int nfx, bool full) {
+  const bool d2 = l.g.dim == 2;
+  const int entries = d2 ? 4 : 8, tables = d2 ? 8 : 15, fxtables = d2 ? 4 : 6;
+  const size_t s = l.g.stride * l.cap, line = (size_t)(l.g.n + 1) * l.cap;
+  const bool stored = nfx < l.cap || h->stores_couplings();
+  const bool dinv = stored || !h->mixed(), both = nfx > 0 && nfx < l.cap;
+  if (!all.tab) all.tab = h->alloc<double>(tables * line);
+  for (int q = 0; stored && q < entries; ++q)
+    if (!*coupling(all, q)) *coupling(all, q) = h->alloc<double>(s);
+  if (dinv && !all.dinv) all.dinv = h->alloc<double>(s);
+  if (nfx && !all.fxt) {
+    all.fxt = h->alloc<long long>(fxtables * line);
+    all.fxh = h->alloc<std::remove_pointer_t<decltype(all.fxh)>>(l.cap);
+  }
+  if (both && !all.fits) {  // (batches only, whose potentials stay)
+    int* fits = h->alloc<int>(l.cap);
+    std::vector<int> host(l.cap);
+    for (int b = 0; b < l.cap; ++b) host[b] = fx_form(l.g, h->probs[b], full);
+    if (!h->dry)
+      cudaMemcpyAsync(fits, host.data(), sizeof(int) * l.cap, cudaMemcpyHostToDevice, h->stream);
+    all.fits = fits;
+  }
+  c = all;
+  for (int q = 0; !stored && q < entries; ++q) *coupling(c, q) = nullptr;
+  if (!dinv) c.dinv = nullptr;
+  if (!nfx) {
+    c.fxt = nullptr;
+    c.fxh = nullptr;
+  }
+  if (!both) c.fits = nullptr;
+}
+
+// Both operators of a level.
+void form_level(fmg_eig_handle* h, Level& l) {
+  l.nfx = count_fx(h, l, false);
+  l.nfxw = h->literal() ? count_fx(h, l, true) : l.nfx;
+  if (l.g.dim == 2) {
+    form_operator(h, l, l.all, l.c, l.nfx, false);
+    if (h->literal()) form_operator(h, l, l.allw, l.cw, l.nfxw, true);
+    else l.cw = l.c;
+  } else {
+    form_operator(h, l, l.all3, l.c3, l.nfx, false);
+    if (h->literal()) form_operator(h, l, l.allw3, l.cw3, l.nfxw, true);
+    else l.cw3 = l.c3;
+  }
+}
+
 void build_levels(fmg_eig_handle* h) {
   const fmg_eig_problem& p = h->prob;
   const int dim = p.dim;
@@ -324,61 +415,15 @@ void build_levels(fmg_eig_handle* h) {
     l.g.nb = l.cap;
     l.g.walk_all = (p.flags & FMG_FLAG_STAR_WALKS) != 0;
     const size_t s = l.g.stride * l.cap;
-    // the fixed-point form (fx) reads no couplings; Chebyshev steps and W u of the literal form do
-    const bool fx = dim == 2 ? fxop2d_applies(l.g) : fxop3d_applies(l.g) && !h->mixed();
-    const bool stored = !fx || p.smoother == FMG_SMOOTH_CHEBYSHEV || h->literal();
-    const bool dinv = stored || !h->mixed();
     if (dim == 2) {
-      if (stored) {
-        l.c.cC = h->alloc<double>(s);
-        l.c.cE = h->alloc<double>(s);
-        l.c.cN = h->alloc<double>(s);
-        l.c.cNE = h->alloc<double>(s);
-      }
-      if (dinv) l.c.dinv = h->alloc<double>(s);
-      l.c.tab = h->alloc<double>(8 * (size_t)(l.g.n + 1) * l.cap);
       l.b.C = h->alloc<double>(s);
       l.b.E = h->alloc<double>(s);
       l.b.N = h->alloc<double>(s);
       l.b.NE = h->alloc<double>(s);
-      if (fx) {
-        l.c.fxt = h->alloc<long long>(4 * (size_t)(l.g.n + 1) * l.cap);
-        l.c.fxh = h->alloc<FxHead2D>(l.cap);
-      }
-      l.cw = l.c;
-      if (h->literal()) {
-        if (fx) {
-          l.cw.fxt = h->alloc<long long>(4 * (size_t)(l.g.n + 1) * l.cap);
-          l.cw.fxh = h->alloc<FxHead2D>(l.cap);
-        }
-        l.cw.cC = h->alloc<double>(s);
-        l.cw.cE = h->alloc<double>(s);
-        l.cw.cN = h->alloc<double>(s);
-        l.cw.cNE = h->alloc<double>(s);
-        l.cw.dinv = h->alloc<double>(s);
-        l.cw.tab = h->alloc<double>(8 * (size_t)(l.g.n + 1) * l.cap);
-      }
     } else {
-      if (stored)
-        for (int q = 0; q < 8; ++q) l.c3.a[q] = h->alloc<double>(s);
-      if (dinv) l.c3.dinv = h->alloc<double>(s);
-      l.c3.tab = h->alloc<double>(15 * (size_t)(l.g.n + 1) * l.cap);
       for (int q = 0; q < 8; ++q) l.b3.a[q] = h->alloc<double>(s);
-      if (fx) {
-        l.c3.fxt = h->alloc<long long>(6 * (size_t)(l.g.n + 1) * l.cap);
-        l.c3.fxh = h->alloc<FxHead3D>(l.cap);
-      }
-      l.cw3 = l.c3;
-      if (h->literal()) {
-        if (fx) {
-          l.cw3.fxt = h->alloc<long long>(6 * (size_t)(l.g.n + 1) * l.cap);
-          l.cw3.fxh = h->alloc<FxHead3D>(l.cap);
-        }
-        for (int q = 0; q < 8; ++q) l.cw3.a[q] = h->alloc<double>(s);
-        l.cw3.dinv = h->alloc<double>(s);
-        l.cw3.tab = h->alloc<double>(15 * (size_t)(l.g.n + 1) * l.cap);
-      }
     }
+    form_level(h, l);
     if (h->mixed()) {
       // single-precision V-cycle arrays: FP32, or bfloat16 storage (2 bytes) behind float*
       auto single = [&]() {
@@ -642,8 +687,8 @@ void enqueue_setup(fmg_eig_handle* h, cudaStream_t s, bool overlap = false) {
   auto build = [&](int k, cudaStream_t q) {
     Level& l = h->L(k);
     prof_begin(h, kProfCoef, k, q);
-    lv_coef(l, h->dparams, q);
-    if (h->literal()) lv_coef(l, h->dparams_full, q, true);
+    lv_coef(l, h->dparams, h->stores_couplings(), q);
+    if (h->literal()) lv_coef(l, h->dparams_full, h->stores_couplings(), q, true);
     prof_end(h, kProfCoef, k, q);
     if (h->mixed()) tables_f32(l.g, l.c, l.c3, h->dparams, l.ct, q);
   };
@@ -1240,6 +1285,49 @@ size_t estimate_bytes(const fmg_eig_problem* probs, int count) {
   return h.bytes;
 }
 
+// The whole solve as the handle's CUDA graph (replacing an earlier one).
+bool capture_solve(fmg_eig_handle* h) {
+  if (h->exec) cudaGraphExecDestroy(h->exec);
+  if (h->graph) cudaGraphDestroy(h->graph);
+  h->exec = nullptr;
+  h->graph = nullptr;
+  h->kernel_nodes = 0;
+  for (int i = 0; i < kProfCount; ++i) h->prof_armed[i] = true;
+  // stage marks: one event per stage that finishes instances
+  StageHook mark_hook = [h](int, int first, int count) {
+    fmg_eig_handle::StageMark m{nullptr, first, count};
+    if (cudaEventCreate(&m.ev) == cudaSuccess) {
+      cudaMemcpyAsync(h->opt.stage_lam + first, h->lam + first, sizeof(double) * count,
+                      cudaMemcpyDeviceToHost, h->stream);
+      cudaEventRecordWithFlags(m.ev, h->stream, cudaEventRecordExternal);
+    }
+    h->marks.push_back(m);
+  };
+  cudaError_t e = cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal);
+  if (e == cudaSuccess) {
+    enqueue_fmg(h, h->stream, h->opt.stage_lam ? &mark_hook : nullptr);
+    e = cudaStreamEndCapture(h->stream, &h->graph);
+  }
+  for (const auto& m : h->marks)
+    if (!m.ev && e == cudaSuccess) e = cudaErrorMemoryAllocation;
+  for (int i = 0; i < kProfCount; ++i) h->prof_armed[i] = false;
+  if (e == cudaSuccess) {
+    size_t n = 0;
+    e = cudaGraphGetNodes(h->graph, nullptr, &n);
+    std::vector<cudaGraphNode_t> nodes(n);
+    if (e == cudaSuccess && n) e = cudaGraphGetNodes(h->graph, nodes.data(), &n);
+    for (size_t i = 0; e == cudaSuccess && i < n; ++i) {
+      cudaGraphNodeType t;
+      e = cudaGraphNodeGetType(nodes[i], &t);
+      if (t == cudaGraphNodeTypeKernel) h->kernel_nodes++;
+    }
+  }
+  if (e == cudaSuccess) e = cudaGraphInstantiate(&h->exec, h->graph, 0);
+  h->activate(1);
+  if (e != cudaSuccess) cudaGetLastError();
+  return e == cudaSuccess;
+}
+
 int create_handle(const fmg_eig_problem* probs, int count, const CreateOptions& opt,
                   fmg_eig_handle** out) {
   if (!out || !probs || count < 1) return FMG_EINVAL;
@@ -1330,40 +1418,7 @@ int create_handle(const fmg_eig_problem* probs, int count, const CreateOptions& 
     *out = h;
     return FMG_OK;
   }
-  for (int i = 0; i < kProfCount; ++i) h->prof_armed[i] = true;
-  // stage marks: one event per stage that finishes instances
-  StageHook mark_hook = [h](int, int first, int count) {
-    fmg_eig_handle::StageMark m{nullptr, first, count};
-    if (cudaEventCreate(&m.ev) == cudaSuccess) {
-      cudaMemcpyAsync(h->opt.stage_lam + first, h->lam + first, sizeof(double) * count,
-                      cudaMemcpyDeviceToHost, h->stream);
-      cudaEventRecordWithFlags(m.ev, h->stream, cudaEventRecordExternal);
-    }
-    h->marks.push_back(m);
-  };
-  cudaError_t e = cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal);
-  if (e == cudaSuccess) {
-    enqueue_fmg(h, h->stream, opt.stage_lam ? &mark_hook : nullptr);
-    e = cudaStreamEndCapture(h->stream, &h->graph);
-  }
-  for (const auto& m : h->marks)
-    if (!m.ev && e == cudaSuccess) e = cudaErrorMemoryAllocation;
-  for (int i = 0; i < kProfCount; ++i) h->prof_armed[i] = false;
-  if (e == cudaSuccess) {
-    size_t n = 0;
-    e = cudaGraphGetNodes(h->graph, nullptr, &n);
-    std::vector<cudaGraphNode_t> nodes(n);
-    if (e == cudaSuccess && n) e = cudaGraphGetNodes(h->graph, nodes.data(), &n);
-    for (size_t i = 0; e == cudaSuccess && i < n; ++i) {
-      cudaGraphNodeType t;
-      e = cudaGraphNodeGetType(nodes[i], &t);
-      if (t == cudaGraphNodeTypeKernel) h->kernel_nodes++;
-    }
-  }
-  if (e == cudaSuccess) e = cudaGraphInstantiate(&h->exec, h->graph, 0);
-  h->activate(1);
-  if (e != cudaSuccess) {
-    cudaGetLastError();
+  if (!capture_solve(h)) {
     delete h;
     return FMG_ECUDA;
   }
@@ -1551,19 +1606,35 @@ int fmg_eig_set_params(fmg_eig_handle* h, const fmg_eig_problem* prob) {
   if (prob->levels != a.levels || shared_key(*prob) != shared_key(a)) return FMG_EINVAL;
   // the pinned staging copy is read by the next solve's upload, in stream order
   if (cudaStreamSynchronize(h->stream) != cudaSuccess) return FMG_ECUDA;
+  const fmg_eig_problem before = h->prob;
   h->prob.w_const = prob->w_const;
   for (int d = 0; d < 3; ++d) h->prob.w_quad[d] = prob->w_quad[d];
   h->prob.zeta = prob->zeta;
   h->prob.omega = prob->omega;
   h->probs[0] = h->prob;
   fill_params(h);
+  // the forms of the level operators follow the potential; a change of one needs another graph
+  bool reform = false;
+  for (const Level& l : h->lv)
+    reform = reform || count_fx(h, l, false) != l.nfx || (h->literal() && count_fx(h, l, true) != l.nfxw);
+  if (reform) {
+    if (cudaDeviceSynchronize() != cudaSuccess) return FMG_ECUDA;  // (solves on other streams)
+    try {
+      for (Level& l : h->lv) form_level(h, l);
+    } catch (const std::bad_alloc&) {
+      h->prob = h->probs[0] = before;
+      fill_params(h);
+      for (Level& l : h->lv) form_level(h, l);  // nothing more to allocate
+      return FMG_ENOMEM;
+    }
+  }
   if (upload_params(h, h->stream) != cudaSuccess ||
       cudaStreamSynchronize(h->stream) != cudaSuccess)
     return FMG_ECUDA;
   enqueue_setup(h, h->stream);  // keep the component entry points' operators current
   h->activate(1);
   if (cudaStreamSynchronize(h->stream) != cudaSuccess) return FMG_ECUDA;
-  return FMG_OK;
+  return !reform || capture_solve(h) ? FMG_OK : FMG_ECUDA;
 }
 
 int fmg_eig_kernel_count(const fmg_eig_handle* h) { return h ? h->kernel_nodes : 0; }

@@ -7,6 +7,7 @@
 #pragma once
 
 #include <cuda_runtime.h>
+#include <math.h>
 #include <stdint.h>
 
 #include "../../include/fmg_eig.h"
@@ -46,17 +47,26 @@ struct SplitVec {
   const float* lo;
 };
 
-// Fixed-point form of the 2D operator (fxop2d.cu), per instance: whether its formats hold the
-// potential, the shifts of the product sum and of the small terms, and their coefficients.
-struct PotentialParams;
+// Problem parameters that may change between solves of one handle.  They live in device
+// memory (uploaded at the start of every solve), so kernels take a device pointer to them.
+struct PotentialParams {
+  double w0, wx, wy, wz;
+  double zeta;
+  double omega;
+  int operator_form;
+  int pad;
+};
+
+// Fixed-point form of the 2D operator (fxop2d.cu), per instance: the shifts of the product sum
+// and of the small terms, and their coefficients.
 struct FxHead2D {
-  int ok, sa, sm, P, Q, R;
+  int sa, sm, P, Q, R;
   double omega;
 };
 
 // Stencil coefficients of L = A + W on one 2D level (see grid2d.cu for the closed forms).  The
-// levels of the fixed-point form keep the couplings only for the Chebyshev smoother and the
-// paper-literal form, and the mixed modes' no omega / cC either (null: their sweeps are single
+// instances of the fixed-point form need the couplings only for the Chebyshev smoother and the
+// paper-literal form, and in the mixed modes no omega / cC either (null: their sweeps are single
 // precision; a Jacobi sweep of the component call forms it from tab).
 struct Coef2D {
   double* cC;    // diagonal
@@ -65,15 +75,42 @@ struct Coef2D {
   double* cNE;   // coupling (i,j)-(i+1,j+1)
   double* dinv;  // omega / cC
   double* tab;   // 8 * (n + 1) separable parts of the coefficients per instance
-  // levels of the fixed-point form only: 4 (n + 1) table entries and a header per instance
+  // levels with instances of the fixed-point form: 4 (n + 1) table entries and a header per
+  // instance
   long long* fxt;
   FxHead2D* fxh;
+  // levels with instances of both forms: whether the instance takes the fixed-point one.  The
+  // kernels of each form leave the other's instances out.
+  const int* fits;
 };
 
 // Levels whose operator runs in fixed point (fxop2d.cu): from 512 cells per side on a sweep is
-// bound by the FP64 pipe (262k nodes: 3.3 us of it); below, by launch latency.  The choice
-// depends on n alone, so an instance of a batch takes the same form as alone.
+// bound by the FP64 pipe (262k nodes: 3.3 us of it); below, by launch latency.  The instances
+// whose potential the formats do not hold (fxop2d_scale) keep the stored couplings and the FP64
+// kernels.  The choice depends on n and the instance alone, so an instance of a batch takes the
+// same form as alone.
 inline bool fxop2d_applies(const Grid& g) { return g.dim == 2 && g.n >= 512; }
+// Scales of the fixed-point form: the potential's coefficients are below 2^-sa, the small ones
+// below 2^-ss.  holds: the formats hold them (see fxop2d.cu).
+struct FxScale {
+  int sa, ss;
+  bool holds;
+};
+__host__ __device__ inline FxScale fxop2d_scale(int n, double h, const PotentialParams& p) {
+  const double wl = p.operator_form == FMG_W_LEFT ? 1.0 : 0.0, h2 = h * h, L = n * h;
+  const double wsum = wl * (fabs(p.wx) + fabs(p.wy));
+  const double amax = h2 / 12.0 * (wl * fabs(p.w0) + wsum * (L * L + 0.3 * h2));
+  const double pmax = h2 * h2 * wsum;  // bounds the small coefficients
+  FxScale q;
+  q.sa = amax > 0.0 ? -(ilogb(amax) + 1) : 40;
+  q.sa = q.sa < 0 ? 0 : q.sa > 40 ? 40 : q.sa;
+  q.ss = pmax > 0.0 ? -(ilogb(pmax) + 1) : 90;
+  q.ss = q.ss < 0 ? 0 : q.ss > 90 ? 90 : q.ss;
+  // the small terms are 0.2 pmax of the maximum at most and lose 2^-26 of that: with pmax <=
+  // 2^-22 the loss is below 2^-50 (each rounding of the FP64 form at 4x: 2^-51)
+  q.holds = amax <= 1.0 / 64.0 && pmax <= 1.0 / 4194304.0 && q.ss - q.sa + 1 >= 0;
+  return q;
+}
 void fxop2d_tables(const Grid& g, const PotentialParams* p, const Coef2D& c, cudaStream_t s);
 void fxop2d_apply(const Grid& g, const Coef2D& c, const double* x, double* y, cudaStream_t s);
 void fxop2d_apply_mass(const Grid& g, const Coef2D& c, const double* x, double* y, double* mx,
@@ -86,18 +123,10 @@ void fxop2d_residual(const Grid& g, const Coef2D& c, const double* f, const doub
 void fxop2d_residual32(const Grid& g, const Coef2D& c, const double* f, const double* x, float* r,
                        bool bf, cudaStream_t s);
 
-// Problem parameters that may change between solves of one handle.  They live in device
-// memory (uploaded at the start of every solve), so kernels take a device pointer to them.
-struct PotentialParams {
-  double w0, wx, wy, wz;
-  double zeta;
-  double omega;
-  int operator_form;
-  int pad;
-};
-
 // ---- 2D level kernels (grid2d.cu) -------------------------------------------------------
-void coef2d_setup(const Grid& g, const PotentialParams* p_dev, const Coef2D& c, cudaStream_t s);
+// ratio_fx: omega / D of the fixed-point instances beside others as of such instances alone
+void coef2d_setup(const Grid& g, const PotentialParams* p_dev, const Coef2D& c, bool ratio_fx,
+                  cudaStream_t s);
 void apply2d(const Grid& g, const Coef2D& c, const double* x, double* y, cudaStream_t s);
 void mass2d(const Grid& g, const double* x, double* y, cudaStream_t s);
 // y = L x, z = M x
@@ -143,22 +172,40 @@ void start_vector(const Grid& g, double* c, int cstride, cudaStream_t s);
 // d = X, Y, Z, XY, XZ, YZ, XYZ (the coupling with p - d is a[1 + d] at p - d).
 // The levels of the fixed-point form keep a as Coef2D says.
 struct FxHead3D {  // as FxHead2D, for fxop3d.cu
-  int ok, sa, sm, P, A[3], F[3];
+  int sa, sm, P, A[3], F[3];
   double K[8];  // constant parts of the couplings (the others are in tab)
 };
 struct Coef3D {
   double* a[8];
   double* dinv;  // omega / diagonal
   double* tab;   // 15 * (n + 1) separable parts per instance
-  // FP64-mode levels of the fixed-point form only: 6 (n + 1) table entries and a header per
-  // instance
+  // FP64-mode levels with instances of the fixed-point form: 6 (n + 1) table entries and a
+  // header per instance
   long long* fxt;
   FxHead3D* fxh;
+  const int* fits;  // as Coef2D
 };
 // Levels whose operator runs in fixed point (fxop3d.cu), FP64 mode only: the mixed modes'
 // single-precision V-cycles amplify the rounding of the FP64 steps around them (see
 // dense_pinned.cu).  Below 96 cells per side the plane walk has too few blocks.
 inline bool fxop3d_applies(const Grid& g) { return g.dim == 3 && g.n >= 96; }
+// as fxop2d_scale
+__host__ __device__ inline FxScale fxop3d_scale(int n, double h, const PotentialParams& p) {
+  const double wl = p.operator_form == FMG_W_LEFT ? 1.0 : 0.0, h2 = h * h, L = n * h;
+  const double wsum = wl * (fabs(p.wx) + fabs(p.wy) + fabs(p.wz));
+  const double amax = h2 / 60.0 * (wl * fabs(p.w0) + wsum * (L * L + 0.31 * h2));
+  const double pmax = h2 * h2 * wsum;  // bounds the small coefficients (and their sum over a stencil)
+  FxScale q;
+  q.sa = amax > 0.0 ? -(ilogb(amax) + 1) : 40;
+  q.sa = q.sa < 0 ? 0 : q.sa > 40 ? 40 : q.sa;
+  q.ss = pmax > 0.0 ? -(ilogb(pmax) + 1) : 90;
+  q.ss = q.ss < 0 ? 0 : q.ss > 90 ? 90 : q.ss;
+  // the small terms are 0.06 pmax of the maximum at most; 30 bits of the pairs and of the
+  // coefficients (each below pmax / 89, hence 36 + ss) leave 2^-33 pmax of it: with pmax <=
+  // 2^-17, 2^-50 of the maximum against the 6 times the maximum that L / h reaches
+  q.holds = amax <= 1.0 / 64.0 && pmax <= 1.0 / 131072.0 && q.ss - q.sa + 11 >= 0;
+  return q;
+}
 void fxop3d_tables(const Grid& g, const PotentialParams* p, const Coef3D& c, cudaStream_t s);
 void fxop3d_apply(const Grid& g, const Coef3D& c, const double* x, double* y, cudaStream_t s);
 void fxop3d_apply_mass(const Grid& g, const Coef3D& c, const double* x, double* y, double* mx,
@@ -173,7 +220,8 @@ struct Density3D {
 struct Stencil15 {
   const double* a[8];
 };
-void coef3d_setup(const Grid& g, const PotentialParams* p_dev, const Coef3D& c, cudaStream_t s);
+void coef3d_setup(const Grid& g, const PotentialParams* p_dev, const Coef3D& c, bool ratio_fx,
+                  cudaStream_t s);
 void apply3d(const Grid& g, const Coef3D& c, const double* x, double* y, cudaStream_t s);
 void mass3d(const Grid& g, const double* x, double* y, cudaStream_t s);
 // y = L x, z = M x

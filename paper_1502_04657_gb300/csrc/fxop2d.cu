@@ -24,9 +24,11 @@
 // arithmetic: 4 rows a warp and 5 blocks per SM took 156 us (Jacobi) and 127 us (residual) on
 // 16.8M nodes, 8 rows and 4 blocks 180 and 142; the FP64 form took 225 and 198.
 //
-// Tiles with infinities, NaN, all zeros or an exponent outside +-kFxMaxExp, and instances
-// whose potential is too large for the fixed formats (h^2 |W| > 12/64 or h^4 (|wx| + |wy|) >
-// 2^-22), run the FP64 expressions of grid2d.cu.
+// Tiles with infinities, NaN, all zeros or an exponent outside +-kFxMaxExp run the FP64 expressions
+// of grid2d.cu.  Instances whose potential is too large for the fixed formats (fxop2d_scale: h^2 |W|
+// > 12/64 or h^4 (|wx| + |wy|) > 2^-22) take grid2d.cu's kernels and stored couplings: forming the
+// couplings from their 1D tables at every use, 15 FP64 operations per node where those kernels need
+// 8, took 2.00 ms for two V-cycles at h = 20/2048, the FP64 kernels 1.25.
 #include <cuda_bf16.h>
 
 #include "dfloat.cuh"
@@ -50,13 +52,10 @@ __global__ void k_fxop2d_tables(int n, double h, const PotentialParams* __restri
   const PotentialParams p = pp[blockIdx.y];
   tab += (size_t)blockIdx.y * 4 * (n + 1);
   const double wl = p.operator_form == FMG_W_LEFT ? 1.0 : 0.0;
-  const double h2 = h * h, h4 = h2 * h2, L = n * h;
+  const double h2 = h * h, h4 = h2 * h2;
   const double w0 = wl * p.w0, wx = wl * p.wx, wy = wl * p.wy;
-  const double amax = h2 / 12.0 * (fabs(w0) + (fabs(wx) + fabs(wy)) * (L * L + 0.3 * h2));
-  const double pmax = h4 * (fabs(wx) + fabs(wy));  // bounds the small coefficients
-  // amax < 2^-sa, pmax < 2^-ss
-  const int sa = amax > 0.0 ? max(0, min(40, -(ilogb(amax) + 1))) : 40;
-  const int ss = pmax > 0.0 ? max(0, min(90, -(ilogb(pmax) + 1))) : 90;
+  const FxScale fs = fxop2d_scale(n, h, p);
+  const int sa = fs.sa, ss = fs.ss;
   const double s = ldexp(1.0, 61 + sa), d = x;
   tab[x] = __double2ll_rn(s * (h2 * w0 / 12.0 + h4 * (wx + wy) / 40.0 + h4 * wx * d * d / 12.0));
   tab[(n + 1) + x] = __double2ll_rn(s * (h4 * wy * d * d / 12.0));
@@ -64,9 +63,6 @@ __global__ void k_fxop2d_tables(int n, double h, const PotentialParams* __restri
   tab[3 * (n + 1) + x] = __double2ll_rn(s * (h4 * wy * d / 12.0));
   if (x == 0) {
     FxHead2D q;
-    // the small terms are 0.2 pmax of the maximum at most and lose 2^-26 of that: with pmax <=
-    // 2^-22 the loss is below 2^-50, what the FP64 form's roundings at 4x leave
-    q.ok = amax <= 1.0 / 64.0 && pmax <= 1.0 / 4194304.0 && ss - sa + 1 >= 0;
     q.sa = sa - 3;       // shift of the products' sum
     q.sm = min(63, ss - sa + 1);  // shift of the small terms to the products' units
     const double t = ldexp(h4, 30 + ss);
@@ -116,7 +112,7 @@ __device__ __forceinline__ void store(__nv_bfloat16* o, size_t k, double v) {
 }
 
 // The tile in FP64, with the expressions of grid2d.cu / mixed.cu (the couplings, which these
-// levels don't store, from the same tables).
+// instances don't store, from the same tables).
 template <int MODE, typename S>
 __device__ __noinline__ void tile_fp64(int n, int pitch, size_t base, int ib, int i0, int j0,
                                        const Coef2D& c, const double* __restrict__ f,
@@ -200,7 +196,8 @@ __global__ void __launch_bounds__(32 * kWarps, kBlocks)
   }
   top = __reduce_max_sync(0xffffffffu, top);
   const int e = ((top + 1) >> 20) - 1022;
-  if (!hd.ok || e < -kFxMaxExp || e > kFxMaxExp) {
+  if (c.fits && !c.fits[ib]) return;  // an instance of the FP64 form
+  if (e < -kFxMaxExp || e > kFxMaxExp) {
     tile_fp64<MODE, S>(n, pitch, base, ib, i0, j0, c, f, x, out, mscale, mx);
     return;
   }

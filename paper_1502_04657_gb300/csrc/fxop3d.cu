@@ -29,8 +29,11 @@
 // The operator apply of the augmented pass also stores M x = h^3/60 S: the two applies took 195
 // and 573 us on 16.6M nodes, together 208 us.
 //
-// Tiles with infinities, NaN, all zeros or an exponent outside +-kFxMaxExp, and instances whose
-// potential is too large for the formats, run the FP64 expressions of grid3d.cu.
+// Tiles with infinities, NaN, all zeros or an exponent outside +-kFxMaxExp run the FP64 expressions
+// of grid3d.cu.  Instances whose potential is too large for the formats (fxop3d_scale: h^2 |W| >
+// 60/64 or h^4 s > 2^-17) take grid3d.cu's kernels and stored couplings: with the couplings formed
+// from their 1D tables at every use (46 FP64 operations per node and more, where those kernels need
+// 16) two V-cycles at h = 10/256 took 16.4 ms, the FP64 kernels 5.8.
 #include "dfloat.cuh"
 #include "fixed.cuh"
 #include "fmg_internal.h"
@@ -50,14 +53,11 @@ __global__ void k_fxop3d_tables(int n, double h, const PotentialParams* __restri
   const PotentialParams p = pp[blockIdx.y];
   tab += (size_t)blockIdx.y * 6 * (n + 1);
   const double wl = p.operator_form == FMG_W_LEFT ? 1.0 : 0.0;
-  const double h2 = h * h, h4 = h2 * h2, L = n * h;
+  const double h2 = h * h, h4 = h2 * h2;
   const double w[3] = {wl * p.wx, wl * p.wy, wl * p.wz}, w0 = wl * p.w0;
-  const double s = w[0] + w[1] + w[2], sabs = fabs(w[0]) + fabs(w[1]) + fabs(w[2]);
-  const double amax = h2 / 60.0 * (fabs(w0) + sabs * (L * L + 0.31 * h2));
-  const double pmax = h4 * sabs;  // bounds the small coefficients (and their sum over a stencil)
-  // amax < 2^-sa, pmax < 2^-ss
-  const int sa = amax > 0.0 ? max(0, min(40, -(ilogb(amax) + 1))) : 40;
-  const int ss = pmax > 0.0 ? max(0, min(90, -(ilogb(pmax) + 1))) : 90;
+  const double s = w[0] + w[1] + w[2];
+  const FxScale fs = fxop3d_scale(n, h, p);
+  const int sa = fs.sa, ss = fs.ss;
   const double sc = ldexp(1.0, 61 + sa), d = x;
   const double c0 = h2 * w0 / 60.0 + h4 * s / 504.0;
   for (int q = 0; q < 3; ++q) {
@@ -66,10 +66,6 @@ __global__ void k_fxop3d_tables(int n, double h, const PotentialParams* __restri
   }
   if (x == 0) {
     FxHead3D q;
-    // the small terms are 0.06 pmax of the maximum at most; 30 bits of the pairs and of the
-    // coefficients (each below pmax / 89, hence 36 + ss) leave 2^-33 pmax of it: with pmax <=
-    // 2^-17, 2^-50 of the maximum against the 6 times the maximum that L / h reaches
-    q.ok = amax <= 1.0 / 64.0 && pmax <= 1.0 / 131072.0 && ss - sa + 11 >= 0;
     q.sa = sa - 3;                 // shift of the products' sum
     q.sm = min(63, ss - sa + 11);  // shift of the small terms to the products' units
     const double t = ldexp(h4, 36 + ss);
@@ -117,7 +113,7 @@ __device__ __forceinline__ long dir(int d, int pitch, long plane) {
   return ox[d] + (long)oy[d] * pitch + oz[d] * plane;
 }
 
-// The block's nodes in FP64, with the expressions of grid3d.cu (the couplings, which these levels
+// The block's nodes in FP64, with the expressions of grid3d.cu (the couplings, which these instances
 // don't store, from k_coef3d's tables and constants).
 template <int MODE>
 __device__ __noinline__ void tile_fp64(int n, int pitch, size_t base, int ib, int x, int y, int z0,
@@ -211,7 +207,8 @@ __global__ void __launch_bounds__(kX * kY, 3)
   const int tf = top[1] == 0 ? 0 : min(top[1] + ((hexp - 3) << 20), 0x7ff00000);
   const int e = ((max(top[0], tf) + 1) >> 20) - 1022;
   const FxHead3D hd = c.fxh[ib];
-  if (!hd.ok || top[1] >= 0x7ff00000 || e < -kFxMaxExp || e > kFxMaxExp) {
+  if (c.fits && !c.fits[ib]) return;  // an instance of the FP64 form
+  if (top[1] >= 0x7ff00000 || e < -kFxMaxExp || e > kFxMaxExp) {
     tile_fp64<MODE>(n, pitch, base, ib, x, y, z0, z1, c, f, v, out, mscale, mv);
     return;
   }

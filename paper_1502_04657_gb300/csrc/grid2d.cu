@@ -15,7 +15,8 @@
 // FP64 on this part issues at ~1/64 of the FP32 rate, so the kernels here trade bandwidth for
 // FP64 instructions: the four coupling arrays and omega/D are materialised once per solve
 // (40 B/node extra traffic) and a sweep costs 8 FP64 instructions per node.  The levels from 512
-// cells per side on take the operator in fixed point instead, without the couplings (fxop2d.cu).
+// cells per side on take the operator in fixed point instead, without the couplings (fxop2d.cu),
+// for every potential that its formats hold.
 #include "fmg_internal.h"
 #include "dfloat.cuh"
 #include "star2d.cuh"
@@ -62,8 +63,10 @@ __device__ __forceinline__ double recip(double c) {
   return y;
 }
 
+// ratio_fx: the instances of the fixed-point form on a level of both take omega / C as k_dinv2d
+// forms it for them alone (levels that store their couplings for another reason don't).
 __global__ void k_coef2d(int n, int pitch, size_t st, const double* __restrict__ tab,
-                         const PotentialParams* __restrict__ pp, Coef2D c) {
+                         const PotentialParams* __restrict__ pp, Coef2D c, int ratio_fx) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   const int j = blockIdx.y * blockDim.y + threadIdx.y;
   if (i > n || j > n) return;
@@ -77,7 +80,7 @@ __global__ void k_coef2d(int n, int pitch, size_t st, const double* __restrict__
   c.cE[k] = tab[s + i] + tab[5 * s + j];
   c.cN[k] = tab[2 * s + i] + tab[6 * s + j];
   c.cNE[k] = tab[3 * s + i] + tab[7 * s + j];
-  c.dinv[k] = pp->omega * recip(cc);
+  c.dinv[k] = ratio_fx && c.fits && c.fits[ib] ? ratio(pp->omega, cc) : pp->omega * recip(cc);
 }
 
 // omega / D alone, for the levels that keep no couplings (the fixed-point operator's): five FP64
@@ -131,6 +134,7 @@ __device__ __forceinline__ double defect(const Coef2D& c, double f, const double
 __global__ void k_apply2d(int n, int pitch, size_t st, Coef2D c, const double* __restrict__ x,
                           double* __restrict__ y) {
   INTERIOR_2D
+  if (c.fits && c.fits[ib]) return;  // an instance of the fixed-point form
   y[k] = lop(c, x, k, pitch);
 }
 
@@ -156,6 +160,7 @@ __global__ void k_apply_mass2d(int n, int pitch, size_t st, double h2_12, Coef2D
                                const double* __restrict__ x, double* __restrict__ y,
                                double* __restrict__ z) {
   INTERIOR_2D
+  if (c.fits && c.fits[ib]) return;
   y[k] = lop(c, x, k, pitch);
   const double s = ((x[k + 1] + x[k - 1]) + (x[k + pitch] + x[k - pitch])) +
                    (x[k + pitch + 1] + x[k - pitch - 1]);
@@ -165,6 +170,7 @@ __global__ void k_apply_mass2d(int n, int pitch, size_t st, double h2_12, Coef2D
 __global__ void k_jacobi2d(int n, int pitch, size_t st, Coef2D c, const double* __restrict__ f,
                            const double* __restrict__ x, double* __restrict__ xo) {
   INTERIOR_2D
+  if (c.fits && c.fits[ib]) return;
   xo[k] = fma(c.dinv[k], defect(c, f[k], x, k, pitch), x[k]);
 }
 
@@ -191,6 +197,7 @@ __global__ void k_jacobi2d_zero(int n, int pitch, size_t st, Coef2D c, const dou
 __global__ void k_residual2d(int n, int pitch, size_t st, Coef2D c, const double* __restrict__ f,
                              const double* __restrict__ x, double* __restrict__ r) {
   INTERIOR_2D
+  if (c.fits && c.fits[ib]) return;
   r[k] = defect(c, f[k], x, k, pitch);
 }
 
@@ -477,10 +484,11 @@ dim3 block_of(const Grid& g) { return dim3(g.bx, g.by); }
 
 }  // namespace
 
-void coef2d_setup(const Grid& g, const PotentialParams* p, const Coef2D& c, cudaStream_t s) {
+void coef2d_setup(const Grid& g, const PotentialParams* p, const Coef2D& c, bool ratio_fx,
+                  cudaStream_t s) {
   k_coef1d<<<dim3((g.n + 1 + 127) / 128, g.nb), 128, 0, s>>>(g.n, g.h, p, c.tab);
   const dim3 grid = grid_of(g, g.n + 1, g.n + 1), block = block_of(g);
-  if (c.cC) k_coef2d<<<grid, block, 0, s>>>(g.n, g.pitch, g.stride, c.tab, p, c);
+  if (c.cC) k_coef2d<<<grid, block, 0, s>>>(g.n, g.pitch, g.stride, c.tab, p, c, ratio_fx);
   else if (c.dinv) k_dinv2d<<<grid, block, 0, s>>>(g.n, g.pitch, g.stride, c.tab, p, c.dinv);
   if (c.fxt) fxop2d_tables(g, p, c, s);
 }
@@ -488,7 +496,7 @@ void coef2d_setup(const Grid& g, const PotentialParams* p, const Coef2D& c, cuda
 void apply2d(const Grid& g, const Coef2D& c, const double* x, double* y, cudaStream_t s) {
   if (c.fxt) {
     fxop2d_apply(g, c, x, y, s);
-    return;
+    if (!c.fits) return;
   }
   k_apply2d<<<grid_of(g, g.n - 1, g.n - 1), block_of(g), 0, s>>>(g.n, g.pitch, g.stride, c, x,
                                                                   y);
@@ -498,7 +506,7 @@ void apply_mass2d(const Grid& g, const Coef2D& c, const double* x, double* y, do
                   cudaStream_t s) {
   if (c.fxt) {
     fxop2d_apply_mass(g, c, x, y, z, s);
-    return;
+    if (!c.fits) return;
   }
   k_apply_mass2d<<<grid_of(g, g.n - 1, g.n - 1), block_of(g), 0, s>>>(
       g.n, g.pitch, g.stride, g.h * g.h / 12.0, c, x, y, z);
@@ -519,7 +527,7 @@ void jacobi2d(const Grid& g, const Coef2D& c, const double* f, const double* x, 
               bool x_is_zero, cudaStream_t s) {
   if (c.fxt && !x_is_zero) {
     fxop2d_jacobi(g, c, f, x, xo, s);
-    return;
+    if (!c.fits) return;
   }
   if (x_is_zero)
     k_jacobi2d_zero<<<grid_of(g, g.n - 1, g.n - 1), block_of(g), 0, s>>>(g.n, g.pitch, g.stride,
@@ -539,7 +547,7 @@ void residual2d(const Grid& g, const Coef2D& c, const double* f, const double* x
                 cudaStream_t s) {
   if (c.fxt) {
     fxop2d_residual(g, c, f, x, r, s);
-    return;
+    if (!c.fits) return;
   }
   k_residual2d<<<grid_of(g, g.n - 1, g.n - 1), block_of(g), 0, s>>>(g.n, g.pitch, g.stride, c,
                                                                      f, x, r);

@@ -12,7 +12,7 @@
 // (Y, Z, XZ, YZ by permuting the axes; the coupling to p - d is the one of p - d to p).  The
 // mass stencil is h^3 (2/5 at C, 1/20 along axes and the body diagonal, 1/30 along face
 // diagonals).  As in 2D, the 8 coupling arrays and omega/D are materialised once per solve, but
-// for the FP64-mode levels whose operator runs in fixed point (fxop3d.cu).
+// for the FP64-mode instances and levels whose operator runs in fixed point (fxop3d.cu).
 
 #include "fmg_internal.h"
 #include "dfloat.cuh"
@@ -88,10 +88,11 @@ __device__ __forceinline__ double recip(double c) {
 // directions d (table 1 along d, 2 across), the face diagonals opposite axis e (table 3 on
 // the two axes of the face, 4 on e) and the body diagonal (table 1 on every axis).
 // STORED = false, for the levels that keep no couplings (the fixed-point operator's): omega / C
-// alone, five FP64 operations and one store per node.  16.6M nodes: 557 -> 280 us.
+// alone, five FP64 operations and one store per node.  16.6M nodes: 557 -> 280 us.  ratio_fx: as
+// k_coef2d.
 template <bool STORED>
 __global__ void k_coef3d(int n, int pitch, size_t st, double h, const double* __restrict__ tab,
-                         const PotentialParams* __restrict__ pp, Coef3D c) {
+                         const PotentialParams* __restrict__ pp, Coef3D c, int ratio_fx) {
   const int lane = threadIdx.x & 31;
   const int s = n + 1;
   const int row = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);  // j + (n + 1) l
@@ -108,6 +109,7 @@ __global__ void k_coef3d(int n, int pitch, size_t st, double h, const double* __
   const double axis = -h + w3 * (1.0 / 20.0), face = w3 * (1.0 / 30.0);
   const double K[8] = {6.0 * h + w3 * 0.4, axis, axis, axis, face, face, face, w3 * (1.0 / 20.0)};
   constexpr int kCount = STORED ? 8 : 1;
+  const bool quotient = !STORED || (ratio_fx && c.fits && c.fits[ib]);
   double R[kCount];
 #pragma unroll
   for (int q = 0; q < kCount; ++q)
@@ -122,7 +124,7 @@ __global__ void k_coef3d(int n, int pitch, size_t st, double h, const double* __
       if (STORED) c.a[q][k] = v;
       if (q == 0) cc = v;
     }
-    c.dinv[k] = STORED ? p.omega * recip(cc) : ratio(p.omega, cc);
+    c.dinv[k] = quotient ? ratio(p.omega, cc) : p.omega * recip(cc);
   }
 }
 
@@ -154,6 +156,7 @@ __device__ __forceinline__ double defect3(const Coef3D& c, double f, const doubl
 __global__ void k_apply3d(int n, int pitch, size_t st, Coef3D c, const double* __restrict__ x,
                           double* __restrict__ y) {
   INTERIOR_3D
+  if (c.fits && c.fits[ib]) return;  // an instance of the fixed-point form
   y[k] = lop3(c, x, k, pitch, plane);
 }
 
@@ -167,6 +170,7 @@ __global__ void k_sub_wmass3d(int n, int pitch, size_t st, Coef3D cw, Coef3D ca,
 __global__ void k_jacobi3d(int n, int pitch, size_t st, Coef3D c, const double* __restrict__ f,
                            const double* __restrict__ x, double* __restrict__ xo) {
   INTERIOR_3D
+  if (c.fits && c.fits[ib]) return;
   xo[k] = fma(c.dinv[k], defect3(c, f[k], x, k, pitch, plane), x[k]);
 }
 
@@ -192,6 +196,7 @@ __global__ void k_jacobi3d_zero(int n, int pitch, size_t st, Coef3D c, const dou
 __global__ void k_residual3d(int n, int pitch, size_t st, Coef3D c, const double* __restrict__ f,
                              const double* __restrict__ x, double* __restrict__ r) {
   INTERIOR_3D
+  if (c.fits && c.fits[ib]) return;
   r[k] = defect3(c, f[k], x, k, pitch, plane);
 }
 
@@ -220,6 +225,7 @@ __global__ void k_apply_mass3d(int n, int pitch, size_t st, double h3, Coef3D c,
                                const double* __restrict__ x, double* __restrict__ y,
                                double* __restrict__ z) {
   INTERIOR_3D
+  if (c.fits && c.fits[ib]) return;
   y[k] = lop3(c, x, k, pitch, plane);
   z[k] = h3 * mass_at(x, k, pitch, plane);
 }
@@ -824,12 +830,15 @@ dim3 block3(const Grid& g) { return dim3(g.bx, g.by); }
 
 }  // namespace
 
-void coef3d_setup(const Grid& g, const PotentialParams* p, const Coef3D& c, cudaStream_t s) {
+void coef3d_setup(const Grid& g, const PotentialParams* p, const Coef3D& c, bool ratio_fx,
+                  cudaStream_t s) {
   k_coef1d_3d<<<dim3((g.n + 1 + 127) / 128, g.nb), 128, 0, s>>>(g.n, g.h, p, c.tab);
   const int rows = (g.n + 1) * (g.n + 1);
   const dim3 grid((rows + 7) / 8, g.nb);
-  if (c.a[0]) k_coef3d<true><<<grid, 256, 0, s>>>(g.n, g.pitch, g.stride, g.h, c.tab, p, c);
-  else if (c.dinv) k_coef3d<false><<<grid, 256, 0, s>>>(g.n, g.pitch, g.stride, g.h, c.tab, p, c);
+  if (c.a[0])
+    k_coef3d<true><<<grid, 256, 0, s>>>(g.n, g.pitch, g.stride, g.h, c.tab, p, c, ratio_fx);
+  else if (c.dinv)
+    k_coef3d<false><<<grid, 256, 0, s>>>(g.n, g.pitch, g.stride, g.h, c.tab, p, c, ratio_fx);
   if (c.fxt) fxop3d_tables(g, p, c, s);
 }
 
@@ -838,7 +847,7 @@ void coef3d_setup(const Grid& g, const PotentialParams* p, const Coef3D& c, cuda
 void apply3d(const Grid& g, const Coef3D& c, const double* x, double* y, cudaStream_t s) {
   if (c.fxt) {
     fxop3d_apply(g, c, x, y, s);
-    return;
+    if (!c.fits) return;
   }
   k_apply3d<<<INTERIOR_LAUNCH(g)>>>(g.n, g.pitch, g.stride, c, x, y);
 }
@@ -847,7 +856,7 @@ void apply_mass3d(const Grid& g, const Coef3D& c, const double* x, double* y, do
                   cudaStream_t s) {
   if (c.fxt) {
     fxop3d_apply_mass(g, c, x, y, z, s);
-    return;
+    if (!c.fits) return;
   }
   k_apply_mass3d<<<INTERIOR_LAUNCH(g)>>>(g.n, g.pitch, g.stride, g.h * g.h * g.h, c, x, y, z);
 }
@@ -869,7 +878,7 @@ void jacobi3d(const Grid& g, const Coef3D& c, const double* f, const double* x, 
               bool x_is_zero, cudaStream_t s) {
   if (c.fxt && !x_is_zero) {
     fxop3d_jacobi(g, c, f, x, xo, s);
-    return;
+    if (!c.fits) return;
   }
   if (x_is_zero) k_jacobi3d_zero<<<INTERIOR_LAUNCH(g)>>>(g.n, g.pitch, g.stride, c, f, xo);
   else k_jacobi3d<<<INTERIOR_LAUNCH(g)>>>(g.n, g.pitch, g.stride, c, f, x, xo);
@@ -885,7 +894,7 @@ void residual3d(const Grid& g, const Coef3D& c, const double* f, const double* x
                 cudaStream_t s) {
   if (c.fxt) {
     fxop3d_residual(g, c, f, x, r, s);
-    return;
+    if (!c.fits) return;
   }
   k_residual3d<<<INTERIOR_LAUNCH(g)>>>(g.n, g.pitch, g.stride, c, f, x, r);
 }

@@ -105,6 +105,7 @@ __global__ void k_residual_mixed2d(int n, int pitch, size_t st_, Coef2D c,
                                    const double* __restrict__ f, const double* __restrict__ x,
                                    S* __restrict__ r) {
   INTERIOR_2D
+  if (c.fits && c.fits[ib]) return;  // an instance of the fixed-point form
   double v = fma(-c.cC[k], x[k], f[k]);  // f - L x as one chain from f
   v = fma(-c.cE[k], x[k + 1], v);
   v = fma(-c.cE[k - 1], x[k - 1], v);
@@ -611,9 +612,9 @@ void add_f32(const float* e, double* x, size_t n, cudaStream_t s, bool bf) {
 
 void residual_mixed(const Grid& g, const Coef2D& c2, const Coef3D& c3, const double* f,
                     const double* x, float* r, cudaStream_t s, bool bf) {
-  if (g.dim == 2 && c2.fxt) {
-    fxop2d_residual32(g, c2, f, x, r, bf, s);
-  } else if (g.dim == 2) {
+  if (g.dim == 2 && c2.fxt) fxop2d_residual32(g, c2, f, x, r, bf, s);
+  if (g.dim == 2) {
+    if (c2.fxt && !c2.fits) return;
     if (bf)
       k_residual_mixed2d<bf16><<<grid2(g, g.n - 1, g.n - 1), blk(g), 0, s>>>(g.n, g.pitch, g.stride, c2, f, x, sp<bf16>(r));
     else

@@ -164,7 +164,7 @@ extern "C" int fmg_eig_coarse_solve_noalloc(const fmg_eig_problem* prob, double*
     cudaGetLastError();
     return FMG_ECUDA;
   }
-  coef2d_setup(g, d.params, c, s);
+  coef2d_setup(g, d.params, c, false, s);
   dense_level1_2d(g, c, L1, M1, s);
   start_vector(g, cstart, nh + 1, s);
   dense_scf(d, 1, s);

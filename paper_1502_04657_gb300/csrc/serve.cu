@@ -61,9 +61,10 @@ double since(Clock::time_point t0) {
 // footprints (the per-level arrays scale with the instance count, shared tables are counted
 // once per instance instead of once per cohort).
 struct Footprints {
-  std::map<std::tuple<int, int, int, int, int>, size_t> cache;
+  std::map<std::tuple<int, int, int, int, int, uint32_t>, size_t> cache;
   size_t of(const fmg_eig_problem& p) {
-    const auto key = std::make_tuple(p.dim, p.coarse_cells, p.levels, p.precision, p.operator_form);
+    const auto key = std::make_tuple(p.dim, p.coarse_cells, p.levels, p.precision, p.operator_form,
+                                     fx_levels(p));
     auto it = cache.find(key);
     if (it != cache.end()) return it->second;
     const size_t b = estimate_bytes(&p, 1) + ((size_t)1 << 16);
@@ -93,7 +94,8 @@ struct PinnedSlots {
   void give(double* p, int n) { free_by_size[n].push_back(p); }
 };
 
-// the settings every instance of a cohort shares, and its sorted level counts
+// what every instance of a cohort shares (settings, forms of the level operators), and its sorted
+// level counts
 std::string cohort_key(const fmg_eig_problem& p, const std::vector<int>& levels_desc) {
   std::string k;
   auto put = [&k](const void* v, size_t n) { k.append(static_cast<const char*>(v), n); };
@@ -102,6 +104,8 @@ std::string cohort_key(const fmg_eig_problem& p, const std::vector<int>& levels_
   put(ints, sizeof(ints));
   put(&p.box_len, sizeof(double));
   put(&p.scf_tol, sizeof(double));
+  const uint32_t fx = fx_levels(p);
+  put(&fx, sizeof(fx));
   for (int l : levels_desc) put(&l, sizeof(int));
   return k;
 }
@@ -137,6 +141,8 @@ extern "C" int fmg_eig_serve(const fmg_eig_serve_config* cfg, const fmg_eig_requ
   }
   const double budget = cfg->hbm_budget_bytes > 0.0 ? cfg->hbm_budget_bytes : 0.8 * (double)free_b;
   Footprints fp;
+  std::vector<uint32_t> fx(n);
+  for (int i = 0; i < n; ++i) fx[i] = fx_levels(reqs[i].problem);
   for (int i = 0; i < n; ++i)
     if ((double)fp.of(reqs[i].problem) > budget) return FMG_EINVAL;  // could never be admitted
 
@@ -298,9 +304,14 @@ extern "C" int fmg_eig_serve(const fmg_eig_serve_config* cfg, const fmg_eig_requ
     // admissions
     while (!queue.empty() && (int)inflight.size() < cfg->max_inflight) {
       const fmg_eig_problem& front = reqs[queue.front()].problem;
+      // a cohort shares its settings and the forms of its level operators, which its pooled graph
+      // and memory are made for
+      auto joins = [&](int i) {
+        return fx[i] == fx[queue.front()] && same_shared_settings(reqs[i].problem, front);
+      };
       int same = 0;
       for (int i : queue)
-        if (same_shared_settings(reqs[i].problem, front)) ++same;
+        if (joins(i)) ++same;
       // a short window lets more requests of this kind join a cohort
       if (same < cfg->max_batch && next < n &&
           since(t0) - reqs[queue.front()].arrival_s < cfg->batch_window_s)
@@ -308,7 +319,7 @@ extern "C" int fmg_eig_serve(const fmg_eig_serve_config* cfg, const fmg_eig_requ
       std::vector<int> pick;
       for (int i : queue) {
         if ((int)pick.size() >= cfg->max_batch) break;
-        if (same_shared_settings(reqs[i].problem, front)) pick.push_back(i);
+        if (joins(i)) pick.push_back(i);
       }
       std::vector<int> sorted = pick;
       by_levels(sorted);
