@@ -61,10 +61,10 @@ double since(Clock::time_point t0) {
 // footprints (the per-level arrays scale with the instance count, shared tables are counted
 // once per instance instead of once per cohort).
 struct Footprints {
-  std::map<std::tuple<int, int, int, int, int, uint32_t>, size_t> cache;
+  std::map<std::tuple<int, int, int, int, int, int, uint32_t>, size_t> cache;
   size_t of(const fmg_eig_problem& p) {
     const auto key = std::make_tuple(p.dim, p.coarse_cells, p.levels, p.precision, p.operator_form,
-                                     fx_levels(p));
+                                     p.smoother, fx_levels(p));
     auto it = cache.find(key);
     if (it != cache.end()) return it->second;
     const size_t b = estimate_bytes(&p, 1) + ((size_t)1 << 16);
