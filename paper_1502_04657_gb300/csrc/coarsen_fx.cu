@@ -14,7 +14,8 @@
 // rest again).
 //
 // e comes from the diagonal entries of 2a and of the corners of its cell; a node with an entry
-// of 2^(e + 1) or more, a negative one, infinities or NaN, and zero tiles are summed in FP64.
+// of 2^(e + 1) or more, a negative one, infinities or NaN, and tiles of zeros or with e outside
+// +-kMaxExp are summed in FP64.
 #include <utility>
 
 #include "fixed.cuh"
@@ -24,6 +25,9 @@ namespace fmg {
 namespace {
 
 constexpr int kB = 55;  // entry = I 2^(e - kB); I < 2^(kB + 1), a sum < 2^(kB + 1) 146 < 2^64
+// From e = -965 on zeros and denormals are shifted out (by 63 or more), and the exponent field of
+// the smallest sum stays positive when e - kB - 2 is added to it.
+constexpr int kMaxExp = 900;
 
 template <int DIM>
 struct Mesh {
@@ -190,7 +194,7 @@ __global__ void __launch_bounds__(32 * kY, 4)
   top = __reduce_max_sync(0xffffffffu, top);
   const int e = ((top + 1) >> 20) - 1022;
   const size_t kc = ib * stc + ((size_t)L * (nc + 1) + J) * pc + I;
-  int bad = e < -4 * kFxMaxExp || e > 4 * kFxMaxExp - 100 ? -1 : 0;
+  int bad = e < -kMaxExp || e > kMaxExp ? -1 : 0;
   if (bad == 0) {
     unsigned long long acc[M::kEnt];
     start_targets<DIM>(acc, std::make_integer_sequence<int, M::kEnt>());
