@@ -56,39 +56,14 @@ __device__ __noinline__ void nload_density2d_fp64(int n, int pitch, size_t st, d
   });
 }
 
-template <int R>
-__global__ void __launch_bounds__(32 * kStarWarps, 4)
-    k_nload_density2d(int n, int pitch, size_t st, double s60, double s180,
-                      const double* __restrict__ u, double* __restrict__ nl,
-                      double* __restrict__ bC, double* __restrict__ bE,
-                      double* __restrict__ bN, double* __restrict__ bNE) {
-  const int e = star2d_exponent<R>(n, pitch, st, u);
-  if (e == kFxNone) {
-    nload_density2d_fp64<R>(n, pitch, st, s60, s180, u, nl, bC, bE, bN, bNE);
-    return;
-  }
-  const double a3 = fx_scale<kFx2>(s60, 3, e), a2 = fx_scale<kFx2>(s180, 2, e);
-  star2d_walk_fx<true, R>(n, pitch, st, u, e, [&](size_t k, const Star2DFx& p) {
-    nl[k] = to_double(star_cubic(p), a3);
-    bC[k] = to_double(madd<6>(p.u * madd<12>(p.u, p.M1), p.SF), a2);
-    bE[k] = to_double(madd<2>(fma(p.Hs, p.Hs + (p.uNE + p.uS), p.HF), p.qNE + p.qS), a2);
-    bN[k] = to_double(madd<2>(fma(p.Vs, p.Vs + (p.uNE + p.uW), p.VF), p.qNE + p.qW), a2);
-    bNE[k] = to_double(madd<2>(fma(p.Ds, p.Ds + (p.uE + p.uN), p.DF), p.qE + p.qN), a2);
-  });
-}
-
-// The same quantities node by node in FP64, for levels below n = 64: the cubic load through the
-// pair sums m_k = n_k + n_{k+1} (nload_at in grid2d.cu) and the density stencil from the two
-// triangle formulas above.  s60, s90, s180 = |K| / 60, / 90, / 180.
-__global__ void k_nload_density2d_node(int n, int pitch, size_t st, double s60, double s90,
-                                       double s180, const double* __restrict__ u,
-                                       double* __restrict__ nl, double* __restrict__ bC,
-                                       double* __restrict__ bE, double* __restrict__ bN,
-                                       double* __restrict__ bNE) {
-  const int i = 1 + blockIdx.x * blockDim.x + threadIdx.x;
-  const int j = 1 + blockIdx.y * blockDim.y + threadIdx.y;
-  if (i >= n || j >= n) return;
-  const size_t k = blockIdx.z * st + at(i, j, pitch);
+// N and the density stencil of one node in FP64: the cubic load through the pair sums m_k = n_k +
+// n_{k+1} (nload_at in grid2d.cu) and the density stencil from the two triangle formulas above.
+// s60, s90, s180 = |K| / 60, / 90, / 180.
+__device__ __forceinline__ void nload_density_at(size_t k, int pitch, double s60, double s90,
+                                                 double s180, const double* __restrict__ u,
+                                                 double* __restrict__ nl, double* __restrict__ bC,
+                                                 double* __restrict__ bE, double* __restrict__ bN,
+                                                 double* __restrict__ bNE) {
   const double up = u[k];
   const double nE = u[k + 1], nNE = u[k + pitch + 1], nN = u[k + pitch];
   const double nW = u[k - 1], nSW = u[k - pitch - 1], nS = u[k - pitch];
@@ -124,6 +99,59 @@ __global__ void k_nload_density2d_node(int n, int pitch, size_t st, double s60, 
                      u26 + fma(8.0 * up, nN, fma(2.0 * (up + nN), nNE + nW, qNE + qW)));
   bNE[k] = s180 * fma(6.0, qNE,
                       u26 + fma(8.0 * up, nNE, fma(2.0 * (up + nNE), nE + nN, qE + qN)));
+}
+
+// the same, called for the nodes that the fixed-point walk leaves short of bits
+__device__ __noinline__ void nload_density2d_redo(size_t k, int pitch, double s60, double s180,
+                                                  const double* __restrict__ u,
+                                                  double* __restrict__ nl, double* __restrict__ bC,
+                                                  double* __restrict__ bE, double* __restrict__ bN,
+                                                  double* __restrict__ bNE) {
+  nload_density_at(k, pitch, s60, 2.0 * s180, s180, u, nl, bC, bE, bN, bNE);
+}
+
+template <int R>
+__global__ void __launch_bounds__(32 * kStarWarps, 4)
+    k_nload_density2d(int n, int pitch, size_t st, double s60, double s180,
+                      const double* __restrict__ u, double* __restrict__ nl,
+                      double* __restrict__ bC, double* __restrict__ bE,
+                      double* __restrict__ bN, double* __restrict__ bNE) {
+  const int e = star2d_exponent<R>(n, pitch, st, u);
+  if (e == kFxNone) {
+    nload_density2d_fp64<R>(n, pitch, st, s60, s180, u, nl, bC, bE, bN, bNE);
+    return;
+  }
+  const double a3 = fx_scale<kFx2>(s60, 3, e), a2 = fx_scale<kFx2>(s180, 2, e);
+  unsigned redo = 0;
+  star2d_walk_fx<true, R>(n, pitch, st, u, e, [&](size_t k, const Star2DFx& p) {
+    const fx<kFx2> v = star_cubic(p);
+    bool lack = fx_short<kShortLoad2>(v);
+    auto put = [&](double* b, fx<kFx2> w) {
+      lack = lack || fx_short<kShortDensity2>(w);
+      b[k] = to_double(w, a2);
+    };
+    nl[k] = to_double(v, a3);
+    put(bC, madd<6>(p.u * madd<12>(p.u, p.M1), p.SF));
+    put(bE, madd<2>(fma(p.Hs, p.Hs + (p.uNE + p.uS), p.HF), p.qNE + p.qS));
+    put(bN, madd<2>(fma(p.Vs, p.Vs + (p.uNE + p.uW), p.VF), p.qNE + p.qW));
+    put(bNE, madd<2>(fma(p.Ds, p.Ds + (p.uE + p.uN), p.DF), p.qE + p.qN));
+    redo = redo << 1 | (unsigned)lack;
+  });
+  star2d_redo<R>(n, pitch, st, redo, [&](size_t k) {
+    nload_density2d_redo(k, pitch, s60, s180, u, nl, bC, bE, bN, bNE);
+  });
+}
+
+// The same quantities node by node, for levels below n = 64
+__global__ void k_nload_density2d_node(int n, int pitch, size_t st, double s60, double s90,
+                                       double s180, const double* __restrict__ u,
+                                       double* __restrict__ nl, double* __restrict__ bC,
+                                       double* __restrict__ bE, double* __restrict__ bN,
+                                       double* __restrict__ bNE) {
+  const int i = 1 + blockIdx.x * blockDim.x + threadIdx.x;
+  const int j = 1 + blockIdx.y * blockDim.y + threadIdx.y;
+  if (i >= n || j >= n) return;
+  nload_density_at(blockIdx.z * st + at(i, j, pitch), pitch, s60, s90, s180, u, nl, bC, bE, bN, bNE);
 }
 
 // ---- T3 class sums -----------------------------------------------------------------------

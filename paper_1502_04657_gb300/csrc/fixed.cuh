@@ -11,12 +11,17 @@
 // tile's maximum, squares 2^-56 and cubes 2^-53 of their maxima; 3D, whose sums of 24
 // tetrahedra need the headroom, K = 59.  The results are converted to FP64 and scaled once.
 //
-// The error is relative to the tile's maximum, FP64's to each node's own terms, so the tile has
+// The error is relative to the tile's maximum, FP64's to each node's own terms.  So the tile has
 // to have one sign (no cancellation; the ground state's iterates do): a tile whose values of
-// the rarer sign exceed 2^-12 of the others, with nonzero values below 2^-50 of its largest,
+// the rarer sign exceed 2^-12 of the others, with nonzero values below 2^-32 of its largest,
 // whose exponent lies outside +-kFxMaxExp (infinities and NaN included), or of zeros, is
 // computed in FP64 by the same walk (a called
-// function: inlined, its register pressure spilled the fixed-point path).  Measured
+// function: inlined, its register pressure spilled the fixed-point path).  And a node whose
+// results are short of bits, because its star lies far below the tile's largest value (next to a
+// corner of the box, or on a steep slope), is evaluated again in FP64: a cubic load below 2^36 (2D)
+// or 2^40 (3D) units, a density entry below 2^44.  The roundings add up to at most 20 (2D) or 400
+// (3D) units of a cubic load and 20 or 150 of a density entry, so every load keeps 4e-10 and every
+// density entry 1e-11 of itself in the worst case.  Measured
 // against 113-bit arithmetic on ground-state-like inputs, relative 2-norm of the cubic load,
 // fixed point and FP64: 2D sine mode 6.6e-17 and 9.1e-17, 3D sine mode 1.56e-16 and 1.70e-16,
 // 3D steep trap 1.64e-16 both.
@@ -109,6 +114,12 @@ __device__ __forceinline__ long long fx_rounded(double v, int shift) {
   return (t ^ sg) - sg;
 }
 
+// |x| < 2^T (T > 32): too few bits for the result of a single node
+template <int T, int K>
+__device__ __forceinline__ bool fx_short(fx<K> x) {
+  return (unsigned)((int)(x.v >> 32) + (1 << (T - 32))) < (2u << (T - 32));
+}
+
 // u read in fixed point: scale = 2^(B1 - e)
 struct FxVec {
   const double* __restrict__ u;
@@ -120,7 +131,7 @@ __device__ __forceinline__ T get(const FxVec& u, size_t k) {
 }
 
 constexpr int kFxMaxExp = 250;
-constexpr int kFxRange = 50;      // values below 2^-50 of a tile's largest would vanish
+constexpr int kFxRange = 32;      // a tile with values below 2^-32 of its largest is left to FP64
 constexpr int kFxNone = -100000;  // no fixed-point exponent: compute the tile in FP64
 // The largest high words (without sign) of a tile's positive and negative values, and its
 // smallest nonzero one (less 1).

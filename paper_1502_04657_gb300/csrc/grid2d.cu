@@ -388,6 +388,19 @@ __device__ __noinline__ void rhs2d_fp64(int n, int pitch, size_t st, double h2_2
   });
 }
 
+// The FP64 evaluation of the nodes that the fixed-point walks leave short of bits (called: the
+// walks' registers don't grow by it)
+__device__ __noinline__ void nload2d_at(size_t k, int pitch, double scale,
+                                        const double* __restrict__ u, double* __restrict__ out) {
+  out[k] = scale * nload_at<double>(u, k, pitch);
+}
+__device__ __noinline__ void rhs2d_at(size_t k, int pitch, double h2_24, double nscale, double l,
+                                      const double* __restrict__ u, double* __restrict__ f) {
+  double m1;
+  const double nl = nload_at<double>(u, k, pitch, &m1);
+  f[k] = fma(l, h2_24 * fma(12.0, u[k], m1), -nscale * nl);
+}
+
 template <int R>
 __global__ void __launch_bounds__(32 * kStarWarps, 4)
     k_nload2d(int n, int pitch, size_t st, double scale, const double* __restrict__ u,
@@ -398,9 +411,13 @@ __global__ void __launch_bounds__(32 * kStarWarps, 4)
     return;
   }
   const double s = fx_scale<kFx2>(scale, 3, e);
+  unsigned redo = 0;
   star2d_walk_fx<false, R>(n, pitch, st, u, e, [&](size_t k, const Star2DFx& p) {
-    out[k] = to_double(star_cubic(p), s);
+    const fx<kFx2> v = star_cubic(p);
+    redo = redo << 1 | (unsigned)fx_short<kShortLoad2>(v);
+    out[k] = to_double(v, s);
   });
+  star2d_redo<R>(n, pitch, st, redo, [&](size_t k) { nload2d_at(k, pitch, scale, u, out); });
 }
 
 // f = lambda M u - N(u); the mass stencil h^2/12 (6 u_p + neighbour sum) reuses the cubic
@@ -417,9 +434,14 @@ __global__ void __launch_bounds__(32 * kStarWarps, 4)
     return;
   }
   const double s1 = l * fx_scale<kFx2>(h2_24, 1, e), s3 = fx_scale<kFx2>(nscale, 3, e);
+  unsigned redo = 0;
   star2d_walk_fx<false, R>(n, pitch, st, u, e, [&](size_t k, const Star2DFx& p) {
-    f[k] = fma(s1, __ll2double_rn(madd<12>(p.u, p.M1).v), -to_double(star_cubic(p), s3));
+    const fx<kFx2> v = star_cubic(p);
+    redo = redo << 1 | (unsigned)fx_short<kShortLoad2>(v);
+    f[k] = fma(s1, __ll2double_rn(madd<12>(p.u, p.M1).v), -to_double(v, s3));
   });
+  star2d_redo<R>(n, pitch, st, redo,
+                 [&](size_t k) { rhs2d_at(k, pitch, h2_24, nscale, l, u, f); });
 }
 
 // FP32 auxiliary right-hand side of the mixed-precision iteration (same closed forms in

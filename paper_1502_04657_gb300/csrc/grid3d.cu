@@ -547,6 +547,31 @@ __device__ __noinline__ void nload_density3d_fp64(int n, int pitch, size_t st, d
   });
 }
 
+// the nodes that the walks in fixed point leave short of bits, through the link sums of star3
+__device__ __noinline__ void nload3d_at(size_t k, int pitch, long plane, double scale,
+                                        const double* __restrict__ u, double* __restrict__ out) {
+  double nl;
+  star3<double, false>(u, k, pitch, plane, nl, nullptr);
+  out[k] = scale * nl;
+}
+__device__ __noinline__ void rhs3d_at(size_t k, int pitch, long plane, double h3, double zn, double l,
+                                      const double* __restrict__ u, double* __restrict__ f) {
+  double nl;
+  star3<double, false>(u, k, pitch, plane, nl, nullptr);
+  f[k] = fma(l, h3 * mass_at(u, k, pitch, plane), -zn * nl);
+}
+__device__ __noinline__ void nload_density3d_at(size_t k, int pitch, long plane, double s140,
+                                                double s210, double s420,
+                                                const double* __restrict__ u,
+                                                double* __restrict__ nl, const Density3D& b) {
+  double v, e[8];
+  star3<double, true>(u, k, pitch, plane, v, e);
+  nl[k] = s140 * v;
+  b.a[0][k] = s210 * e[0];
+#pragma unroll
+  for (int d = 0; d < 7; ++d) b.a[1 + d][k] = s420 * e[1 + d];
+}
+
 template <int P>
 __global__ void __launch_bounds__(kS3X * kS3Y, 3)
     k_nload3d(int n, int pitch, size_t st, double scale6, const double* __restrict__ u,
@@ -554,9 +579,16 @@ __global__ void __launch_bounds__(kS3X * kS3Y, 3)
   const int e = star3_exponent<P>(n, pitch, st, u);
   if (e != kFxNone) {
     const double s = fx_scale<kFx3>(scale6, 3, e);
-    star3_walk<false, P, fx<kFx3>>(
-        n, pitch, st, FxVec{u, fx_pow2(fx<kFx3>::B1 - e)},
-        [&](size_t k, const Star3T<fx<kFx3>>& p) { out[k] = to_double(star3_cubic6(p), s); });
+    unsigned redo = 0;
+    star3_walk<false, P, fx<kFx3>>(n, pitch, st, FxVec{u, fx_pow2(fx<kFx3>::B1 - e)},
+                                [&](size_t k, const Star3T<fx<kFx3>>& p) {
+      const fx<kFx3> v = star3_cubic6(p);
+      redo = redo << 1 | (unsigned)fx_short<kShortLoad3>(v);
+      out[k] = to_double(v, s);
+    });
+    star3_redo<P>(n, pitch, st, redo, [&](size_t k) {
+      nload3d_at(k, pitch, (long)(n + 1) * pitch, 6.0 * scale6, u, out);
+    });
     return;
   }
   nload3d_fp64<P>(n, pitch, st, scale6, u, out);
@@ -573,9 +605,15 @@ __global__ void __launch_bounds__(kS3X * kS3Y, 3)
   const int e = star3_exponent<P>(n, pitch, st, u);
   if (e != kFxNone) {
     const double s1 = l * fx_scale<kFx3>(h3_120, 1, e), s3 = fx_scale<kFx3>(zn, 3, e);
+    unsigned redo = 0;
     star3_walk<false, P, fx<kFx3>>(n, pitch, st, FxVec{u, fx_pow2(fx<kFx3>::B1 - e)},
                                 [&](size_t k, const Star3T<fx<kFx3>>& p) {
-      f[k] = fma(s1, __ll2double_rn(madd<24>(p.u, p.S1).v), -to_double(star3_cubic6(p), s3));
+      const fx<kFx3> v = star3_cubic6(p);
+      redo = redo << 1 | (unsigned)fx_short<kShortLoad3>(v);
+      f[k] = fma(s1, __ll2double_rn(madd<24>(p.u, p.S1).v), -to_double(v, s3));
+    });
+    star3_redo<P>(n, pitch, st, redo, [&](size_t k) {
+      rhs3d_at(k, pitch, (long)(n + 1) * pitch, 120.0 * h3_120, 6.0 * zn, l, u, f);
     });
     return;
   }
@@ -595,17 +633,27 @@ __global__ void __launch_bounds__(kS3X * kS3Y, 3)
     using T = fx<kFx3>;
     const double a3 = fx_scale<kFx3>(s140_6, 3, e), a2 = fx_scale<kFx3>(s210_2, 2, e),
                  c2 = fx_scale<kFx3>(s420_2, 2, e);
+    unsigned redo = 0;
     star3_walk<true, P, T>(n, pitch, st, FxVec{u, fx_pow2(T::B1 - e)},
                         [&](size_t k, const Star3T<T>& p) {
-      nl[k] = to_double(star3_cubic6(p), a3);
-      b.a[0][k] = to_double(madd<4>(madd<36>(p.q, p.u * p.S1), p.S2), a2);
+      const T v = star3_cubic6(p), c = madd<4>(madd<36>(p.q, p.u * p.S1), p.S2);
+      bool lack = fx_short<kShortLoad3>(v) || fx_short<kShortDensity3>(c);
+      nl[k] = to_double(v, a3);
+      b.a[0][k] = to_double(c, a2);
       const T u2 = twice(p.u);
 #pragma unroll
       for (int d = 0; d < 7; ++d) {
         const T t = fma(p.u, p.un[d], p.q + p.qn[d]);  // u_p^2 + u_q^2 + u_p u_q
         const T g = fma(madd<2>(p.un[d], u2), p.E1[d], p.E2[d]);
-        b.a[1 + d][k] = to_double((d >= 3 && d < 6) ? madd<8>(t, g) : madd<12>(t, g), c2);
+        const T w = (d >= 3 && d < 6) ? madd<8>(t, g) : madd<12>(t, g);
+        lack = lack || fx_short<kShortDensity3>(w);
+        b.a[1 + d][k] = to_double(w, c2);
       }
+      redo = redo << 1 | (unsigned)lack;
+    });
+    star3_redo<P>(n, pitch, st, redo, [&](size_t k) {
+      nload_density3d_at(k, pitch, (long)(n + 1) * pitch, 6.0 * s140_6, 2.0 * s210_2, 2.0 * s420_2,
+                         u, nl, b);
     });
     return;
   }

@@ -27,6 +27,7 @@
 namespace fmg {
 
 constexpr int kFx2 = 61;  // fixed-point format of the walk (fixed.cuh)
+constexpr int kShortLoad2 = 36, kShortDensity2 = 44;  // results that a node takes in FP64
 
 template <typename T>
 struct StarEdge {
@@ -212,6 +213,26 @@ __device__ __forceinline__ void star2d_walk_fx(int n, int pitch, size_t st,
     u0 = u1; q0 = q1;
     u0R = u1R; q0R = q1R;
   }
+}
+
+// node(k) for the nodes that a fixed-point walk of this warp left short of bits.  redo: one bit per
+// row that the lane produced, the latest lowest.  The nodes are spread over the lanes: an FP64
+// instruction takes a warp the same time for one node as for 32.
+template <int R, typename Node>
+__device__ __forceinline__ void star2d_redo(int n, int pitch, size_t st, unsigned redo, Node node) {
+  __shared__ unsigned short list[kStarWarps][32 * R];
+  __shared__ int count[kStarWarps];
+  if (!__any_sync(0xffffffffu, redo)) return;
+  const int lane = threadIdx.x, w = threadIdx.y;
+  const int j0 = 1 + R * (blockIdx.y * blockDim.y + w), last = min(j0 + R, n) - 1;
+  if (lane == 0) count[w] = 0;
+  __syncwarp();
+  for (; redo; redo &= redo - 1)
+    list[w][atomicAdd(&count[w], 1)] = (unsigned short)(lane * R + (last - (__ffs(redo) - 1) - j0));
+  __syncwarp();
+  for (int q = lane; q < count[w]; q += 32)
+    node(blockIdx.z * st + (size_t)(j0 + list[w][q] % R) * pitch + kStarCols * blockIdx.x +
+         list[w][q] / R);
 }
 
 // Walks the rows of this thread's strip of instance blockIdx.z and calls out(k, star) for

@@ -20,7 +20,7 @@
 // T5 (Z, YZ).  A corner of the cube lies in all six (v, W) or in two: X in T0 + T1, Y in
 // T2 + T3, Z in T4 + T5, XY in T0 + T2, XZ in T1 + T4, YZ in T3 + T5.
 //
-// Layout of the work: a block covers a 32 x 8 tile of columns and walks 16 planes upwards.
+// Layout of the work: a block covers a 32 x 8 tile of columns and walks 16 (or 4) planes upwards.
 // For each plane z it stages u, u^2, u^3 of plane z + 1 (tile and halo) in shared memory,
 // forms the 6 tetrahedra of every cube of layer z (corners in planes z and z + 1) into
 // shared memory, and then each thread finishes its node of plane z (the four cubes of layer z
@@ -36,6 +36,7 @@
 namespace fmg {
 
 constexpr int kFx3 = 59;  // fixed-point format of the walk (fixed.cuh)
+constexpr int kShortLoad3 = 40, kShortDensity3 = 44;  // results that a node takes in FP64
 
 constexpr int kS3X = 32, kS3Y = 8;               // tile of columns (= threads)
 constexpr int kS3Z = 16;                         // planes per block of a double-float walk
@@ -131,6 +132,32 @@ __device__ __forceinline__ int star3_exponent(int n, int pitch, size_t st, const
   m.neg = top[1];
   m.low = low;
   return m.exponent();
+}
+
+// node(k) for the nodes that a fixed-point walk of this block left short of bits.  redo: one bit per
+// plane that the thread produced, the latest lowest.  The nodes are spread over the threads (in the
+// shared memory that the walk has left): an FP64 instruction takes a warp the same time for one
+// node as for 32.
+template <int P, typename Node>
+__device__ __forceinline__ void star3_redo(int n, int pitch, size_t st, unsigned redo, Node node) {
+  extern __shared__ double s3sm[];
+  int* const count = reinterpret_cast<int*>(s3sm);
+  unsigned short* const list = reinterpret_cast<unsigned short*>(count + 1);
+  if (!__syncthreads_or(redo != 0)) return;
+  const int tid = threadIdx.y * kS3X + threadIdx.x;
+  const int nzc = star3_zchunks(n, P), ib = blockIdx.z / nzc;
+  const int z0 = 1 + (int)(blockIdx.z - ib * nzc) * P, last = min(z0 + P, n) - 1;
+  if (tid == 0) *count = 0;
+  __syncthreads();
+  for (; redo; redo &= redo - 1)
+    list[atomicAdd(count, 1)] = (unsigned short)((last - (__ffs(redo) - 1) - z0) * kS3X * kS3Y + tid);
+  __syncthreads();
+  const int total = *count;
+  for (int q = tid; q < total; q += kS3X * kS3Y) {
+    const int c = list[q], x = 1 + blockIdx.x * kS3X + c % kS3X,
+              y = 1 + blockIdx.y * kS3Y + c / kS3X % kS3Y, z = z0 + c / (kS3X * kS3Y);
+    node(ib * st + ((size_t)z * (n + 1) + y) * pitch + x);
+  }
 }
 
 // blockDim = (kS3X, kS3Y), kS3Smem bytes of dynamic shared memory; instance
