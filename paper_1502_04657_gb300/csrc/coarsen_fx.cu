@@ -5,17 +5,17 @@
 // A coarse node takes its 4 (8) entries from 30 (138) stored fine ones in 64 (290) weighted
 // sums, which in FP64 (2 lanes per clock) cost more than reading the 16 (64) entries per coarse
 // node that memory has to deliver.  The entries int u^2 phi phi are non-negative for a u of one
-// sign, so a warp (32 coarse nodes of a row) takes one exponent e, reads each entry once as an
-// integer in units of 2^(e - 55) and adds multiples 1, 2 or 4 of it (the weights in quarters)
-// to the sums of all its targets; each target is converted once.  Only the truncation to 55
-// bits of the largest entry rounds (its mean, half a unit each, is added back), where the FP64
-// form rounds every sum.  Measured: 16.6M 3D nodes 931 -> 245 us, 16.8M 2D nodes 370 -> 137 us
+// sign, so a thread takes one exponent e for its coarse node, reads each entry as an integer in
+// units of 2^(e - 55) and adds multiples 1, 2 or 4 of it (the weights in quarters) to the sums of
+// all its targets; each target is converted once.  Only the truncation to 55 bits of the largest
+// entry around the node rounds (its mean, half a unit each, is added back), where the FP64 form
+// rounds every sum.  Measured: 16.6M 3D nodes 931 -> 245 us, 16.8M 2D nodes 370 -> 137 us
 // (in 3D 623 us with one load per entry: half of each sector was used, and L2 had to deliver the
 // rest again).
 //
-// e comes from the diagonal entries of 2a and of the corners of its cell; a node with an entry
-// of 2^(e + 1) or more, a negative one, infinities or NaN, and tiles of zeros or with e outside
-// +-kMaxExp are summed in FP64.
+// e comes from the diagonal entries of 2a and of the corners of its cell.  Nodes with an entry of
+// 2^(e + 1) or more, a negative one, infinities or NaN, a sum below 2^-9 of the largest entry (one
+// that is exactly zero, or kept too few bits), zeros only or e outside +-kMaxExp are summed in FP64.
 #include <utility>
 
 #include "fixed.cuh"
@@ -28,6 +28,7 @@ constexpr int kB = 55;  // entry = I 2^(e - kB); I < 2^(kB + 1), a sum < 2^(kB +
 // From e = -965 on zeros and denormals are shifted out (by 63 or more), and the exponent field of
 // the smallest sum stays positive when e - kB - 2 is added to it.
 constexpr int kMaxExp = 900;
+constexpr int kLeast = 46;  // bits a sum has at least (73 units, at most, are lost to truncation)
 
 template <int DIM>
 struct Mesh {
@@ -134,11 +135,22 @@ __device__ __forceinline__ unsigned long long entry_fixed(double e, int shift, i
   return m >> min((unsigned)sh, 63u);
 }
 
+// Integers of the lane before in this lane's units: 2^k larger ones lose k bits (at most
+// kMaxStep; nodes whose left neighbour's exponent is further above theirs are summed in FP64).
+constexpr int kMaxStep = 12;
+struct Left {
+  int up, down;
+  __device__ __forceinline__ unsigned long long units(unsigned long long i, int& bad) const {
+    bad |= (1 << (kB + 1 - 32 - up)) - 1 - (int)(i >> 32);  // an entry from 2^(e + 1) on
+    return i >> down << up;
+  }
+};
+
 // The entries D of one row of the cell (fine nodes 2a - 1, 2a, 2a + 1 in x): a thread loads the
 // pair from 2a on and takes 2a - 1 from the lane before it.
 template <int DIM, int D, int R>
 __device__ __forceinline__ void add_row(const Entries<DIM>& f, size_t kf, int pitch, long plane,
-                                        int shift, int& bad,
+                                        int shift, const Left& left, int& bad,
                                         unsigned long long (&acc)[1 << DIM]) {
   constexpr bool l = Tab<DIM>::k.used(D, 3 * R), m = Tab<DIM>::k.used(D, 3 * R + 1),
                  r = Tab<DIM>::k.used(D, 3 * R + 2);
@@ -153,6 +165,7 @@ __device__ __forceinline__ void add_row(const Entries<DIM>& f, size_t kf, int pi
       if constexpr (l) {
         unsigned long long j = __shfl_up_sync(0xffffffffu, i, 1);
         if (threadIdx.x == 0) j = entry_fixed(__ldg(p - 1), shift, bad);
+        else j = left.units(j, bad);
         add_targets<DIM, D, 3 * R>(j, acc, targets);
       }
     }
@@ -161,14 +174,15 @@ __device__ __forceinline__ void add_row(const Entries<DIM>& f, size_t kf, int pi
 
 template <int DIM, int... Q>
 __device__ __forceinline__ void add_entries(const Entries<DIM>& f, size_t kf, int pitch,
-                                            long plane, int shift, int& bad,
+                                            long plane, int shift, const Left& left, int& bad,
                                             unsigned long long (&acc)[1 << DIM],
                                             std::integer_sequence<int, Q...>) {
   constexpr int E = 1 << DIM;
-  (add_row<DIM, Q % E, Q / E>(f, kf, pitch, plane, shift, bad, acc), ...);
+  (add_row<DIM, Q % E, Q / E>(f, kf, pitch, plane, shift, left, bad, acc), ...);
 }
 
-// blockDim (32, kY): a warp per coarse row piece; planes and instances share blockIdx.z.
+// blockDim (32, kY): a warp per coarse row piece (the lanes pass on the entry left of their
+// pair); planes and instances share blockIdx.z.
 // Entries towards coarse boundary nodes are formed as well (from interior fine entries only);
 // nothing but the next coarsening reads them, for its own boundary entries.
 constexpr int kY = 4;
@@ -191,20 +205,32 @@ __global__ void __launch_bounds__(32 * kY, 4)
     if (v == M::kPos / 2 || corner)
       top = max(top, __double2hiint(__ldg(f.a[0] + kf + offset<DIM>(v, pf, planef))));
   }
-  top = __reduce_max_sync(0xffffffffu, top);
-  const int e = ((top + 1) >> 20) - 1022;
+  const int e0 = ((top + 1) >> 20) - 1022;
   const size_t kc = ib * stc + ((size_t)L * (nc + 1) + J) * pc + I;
-  int bad = e < -kMaxExp || e > kMaxExp ? -1 : 0;
-  if (bad == 0) {
+  int bad = e0 < -kMaxExp || e0 > kMaxExp ? -1 : 0;
+  if (__any_sync(0xffffffffu, bad == 0)) {
+    const int e = bad == 0 ? e0 : 0;
+    const int before = __shfl_up_sync(0xffffffffu, bad == 0 ? e0 : 4096, 1);
+    const int step = threadIdx.x == 0 ? 0 : before - e;
+    if (step > kMaxStep) bad = -1;
+    const Left left{min(max(step, 0), kMaxStep), min(max(-step, 0), 63)};
     unsigned long long acc[M::kEnt];
     start_targets<DIM>(acc, std::make_integer_sequence<int, M::kEnt>());
-    add_entries<DIM>(f, kf, pf, planef, e + 1085 - kB, bad, acc,
+    add_entries<DIM>(f, kf, pf, planef, e + 1085 - kB, left, bad, acc,
                      std::make_integer_sequence<int, M::kEnt * M::kPos / 3>());
-    bad = __any_sync(0xffffffffu, bad < 0) ? -1 : 0;
-    if (bad == 0 && I < nc) {
+    // an entry that the lane before could not take in (and passed on)
+    const int passed = __shfl_up_sync(0xffffffffu, bad, 1);
+    if (threadIdx.x && passed < 0) bad = -1;
+#pragma unroll
+    for (int T = 0; T < M::kEnt; ++T) {
+      const bool inner = (!M::dx(T) || I + 1 < nc) && (!M::dy(T) || J + 1 < nc) &&
+                         (!M::dz(T) || L + 1 < nc);
+      if (inner && (acc[T] >> kLeast) == 0) bad = -1;
+    }
+    if (bad >= 0 && I < nc) {
 #pragma unroll
       for (int T = 0; T < M::kEnt; ++T) {
-        const double d = __ull2double_rn(acc[T]);  // at least 1
+        const double d = __ull2double_rn(acc[T]);
         c.a[T][kc] = __hiloint2double(__double2hiint(d) + (e - kB - 2) * (1 << 20),
                                       __double2loint(d));
       }
