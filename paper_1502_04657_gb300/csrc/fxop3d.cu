@@ -204,8 +204,9 @@ __global__ void __launch_bounds__(kX * kY, 3)
     }
   }
   __syncthreads();
-  const int tf = top[1] == 0 ? 0 : min(top[1] + ((hexp - 3) << 20), 0x7ff00000);
-  const int e = ((max(top[0], tf) + 1) >> 20) - 1022;
+  // f / h counts an eighth (exponents are added as such: the sum of high words may wrap)
+  const int ex = ((top[0] + 1) >> 20) - 1022, ef = ((top[1] + 1) >> 20) - 1022 + hexp - 3;
+  const int e = top[1] == 0 ? ex : max(ex, ef);
   const FxHead3D hd = c.fxh[ib];
   if (c.fits && !c.fits[ib]) return;  // an instance of the FP64 form
   if (top[1] >= 0x7ff00000 || e < -kFxMaxExp || e > kFxMaxExp) {
