@@ -14,9 +14,13 @@
 //       small = -h^4 [ 17/180 (wx + wy) x + 7/360 wy (E + W) + 7/360 wx (N + S) ],
 //     with a = ax[i] + ay[j], bx[i], by[j] from 1D tables, scaled by 2^(61 + sa) so that they
 //     fill the integers, and the small terms (h^2 below the others) from the high words.
-// Only the products, x and f round, at 2^-58 of the tile's maximum or below (FP64 rounds each
-// of its operations at 2^-53, and each stored coupling -1 + O(h^2) at 2^-53: a relative
-// perturbation of W by 2^-53 / h^2, 4e-9 at h = 1/4096, that this form does not have).
+// Only the products, x and f round, at 2^-58 of the tile's maximum, and the small terms at 2^-50 of
+// it or below (2^-26 of h^4 (wx + wy)).  FP64 rounds each of its operations at 2^-53, and each
+// stored coupling -1 + O(h^2) at 2^-53: a relative perturbation of W by 2^-53 / h^2, 4e-9 at h =
+// 1/4096, that this form does not have.  FP64's rounding is relative to each node's own stencil, so
+// a tile where some lane's values (of its and the neighbouring lanes' columns) lie 2^-7 or more
+// below the largest takes an exponent per lane, which costs a second conversion of each neighbour's
+// value (16.8M nodes, every tile so: Jacobi 15 us more, apply 23).
 // The operator apply of the augmented pass also stores M x = h^2/12 (6x + sum of the six), whose
 // sum is at hand: the two applies took 117 and 227 us on 16.8M nodes, together 152 us.
 // The update x + (omega / D) r is one FP64 operation as before.  What is left is the instruction
@@ -43,6 +47,7 @@ constexpr int kRows = 4;       // rows a warp produces
 constexpr int kWarps = 4;      // warps of a block, stacked in y
 constexpr int kCols = 62;      // columns a warp produces
 constexpr int kBlocks = 5;     // resident blocks per SM
+constexpr int kLaneRange = 7;  // lanes of a tile of one exponent: within 2^-7 of its largest
 
 // Tables ax, ay, bx, by (n + 1 entries each) and the header of each instance.
 __global__ void k_fxop2d_tables(int n, double h, const PotentialParams* __restrict__ pp,
@@ -158,49 +163,22 @@ __device__ __noinline__ void tile_fp64(int n, int pitch, size_t base, int ib, in
     }
 }
 
-template <int MODE, typename S>
-__global__ void __launch_bounds__(32 * kWarps, kBlocks)
-    k_fxop2d(int n, int pitch, size_t st, const __grid_constant__ Coef2D c,
-             const double* __restrict__ f, const double* __restrict__ x, S* __restrict__ out,
-             double mscale, double* __restrict__ mx) {
-  const int lane = threadIdx.x, ib = blockIdx.z;
-  const int i0 = kCols * blockIdx.x + 2 * lane;  // this lane's columns i0, i0 + 1
-  const int j0 = 1 + kRows * (blockIdx.y * kWarps + threadIdx.y);
-  if (j0 >= n) return;  // uniform over the warp
-  const size_t base = ib * st;
-  const bool in = i0 <= n;  // (i0 + 1 <= n + 1 < pitch then)
+// The tile of a warp, rows j0 - 1 .. j0 + kRows of x in xv (this lane's columns i0, i0 + 1), in units
+// of 2^(e - kB).  LANES: e is the lane's own; lanes with fp64 set pass their values on and are
+// evaluated in FP64 at the end.
+template <int MODE, typename S, bool LANES>
+__device__ __forceinline__ void tile_fixed(int n, int pitch, size_t base, int ib, int i0, int j0,
+                                           const Coef2D& c, const double* __restrict__ f,
+                                           const double* __restrict__ x, S* __restrict__ out,
+                                           double mscale, double* __restrict__ mx,
+                                           const double2 (&xv)[kRows + 2], int e, bool fp64) {
+  const int lane = threadIdx.x;
+  const bool in = i0 <= n;
   const double2 zero = make_double2(0.0, 0.0);
-  double2 xv[kRows + 2];
-#pragma unroll
-  for (int t = 0; t < kRows + 2; ++t) {
-    const int r = j0 - 1 + t;
-    xv[t] = in && r <= n ? *reinterpret_cast<const double2*>(x + base + (size_t)r * pitch + i0) : zero;
-  }
-  // f is read here for the exponent and again, from L1, when its row is due
   auto f_row = [&](int r) {
     return in && r < n ? *reinterpret_cast<const double2*>(f + base + (size_t)r * pitch + i0) : zero;
   };
   const FxHead2D hd = c.fxh[ib];
-  // the tile's exponent: f counts an eighth (|f| <= 8 2^e fits beside the stencil of x)
-  int top = 0, topf = 0;
-#pragma unroll
-  for (int t = 0; t < kRows + 2; ++t)
-    top = max(top, max(__double2hiint(xv[t].x) & 0x7fffffff, __double2hiint(xv[t].y) & 0x7fffffff));
-  if (!applies(MODE)) {
-#pragma unroll
-    for (int t = 0; t < kRows; ++t) {
-      const double2 v = f_row(j0 + t);
-      topf = max(topf, max(__double2hiint(v.x) & 0x7fffffff, __double2hiint(v.y) & 0x7fffffff));
-    }
-    top = max(top, topf - (3 << 20));
-  }
-  top = __reduce_max_sync(0xffffffffu, top);
-  const int e = ((top + 1) >> 20) - 1022;
-  if (c.fits && !c.fits[ib]) return;  // an instance of the FP64 form
-  if (e < -kFxMaxExp || e > kFxMaxExp) {
-    tile_fp64<MODE, S>(n, pitch, base, ib, i0, j0, c, f, x, out, mscale, mx);
-    return;
-  }
   const int shift = e + 1022 + 5;
   const double back = fx_pow2(e - kB), mback = mscale * back;
   const long long* tab = c.fxt + (size_t)ib * 4 * (n + 1);
@@ -216,8 +194,13 @@ __global__ void __launch_bounds__(32 * kWarps, kBlocks)
     Row q;
     q.a = to_fixed(v.x, shift);
     q.b = to_fixed(v.y, shift);
-    q.l = __shfl_up_sync(0xffffffffu, q.b, 1);
-    q.r = __shfl_down_sync(0xffffffffu, q.a, 1);
+    if (LANES) {  // the lanes beside have their own units
+      q.l = to_fixed(__shfl_up_sync(0xffffffffu, v.y, 1), shift);
+      q.r = to_fixed(__shfl_down_sync(0xffffffffu, v.x, 1), shift);
+    } else {
+      q.l = __shfl_up_sync(0xffffffffu, q.b, 1);
+      q.r = __shfl_down_sync(0xffffffffu, q.a, 1);
+    }
     return q;
   };
   // one node: (A + W) x in units of 2^(e - kB)
@@ -249,7 +232,8 @@ __global__ void __launch_bounds__(32 * kWarps, kBlocks)
         rb = to_fixed(v.y, shift) - rb;
       }
       const size_t k = base + (size_t)j * pitch + i0;
-      const bool oka = lane > 0 && i0 <= n - 1, okb = lane < 31 && i0 + 1 <= n - 1;
+      const bool oka = lane > 0 && i0 <= n - 1 && !(LANES && fp64),
+                 okb = lane < 31 && i0 + 1 <= n - 1 && !(LANES && fp64);
       double va = __ll2double_rn(ra), vb = __ll2double_rn(rb);
       if (jacobi(MODE)) {
         double2 di;
@@ -285,6 +269,77 @@ __global__ void __launch_bounds__(32 * kWarps, kBlocks)
     s = m;
     m = p;
   }
+  if (LANES && fp64) tile_fp64<MODE, S>(n, pitch, base, ib, i0, j0, c, f, x, out, mscale, mx);
+}
+
+__device__ __forceinline__ int high(double v) { return __double2hiint(v) & 0x7fffffff; }
+
+// The same with an exponent per lane, for the tiles whose lanes differ (called, and x read again: the
+// common path keeps its registers).
+template <int MODE, typename S>
+__device__ __noinline__ void tile_lanes(int n, int pitch, size_t base, int ib, int i0, int j0,
+                                        const Coef2D& c, const double* __restrict__ f,
+                                        const double* __restrict__ x, S* __restrict__ out,
+                                        double mscale, double* __restrict__ mx, int top) {
+  double2 xv[kRows + 2];
+#pragma unroll
+  for (int t = 0; t < kRows + 2; ++t) {
+    const int r = j0 - 1 + t;
+    xv[t] = i0 <= n && r <= n ? *reinterpret_cast<const double2*>(x + base + (size_t)r * pitch + i0)
+                              : make_double2(0.0, 0.0);
+  }
+  const int e = ((top + 1) >> 20) - 1022;
+  const bool fp64 = e < -kFxMaxExp || e > kFxMaxExp;
+  tile_fixed<MODE, S, true>(n, pitch, base, ib, i0, j0, c, f, x, out, mscale, mx, xv, fp64 ? 0 : e,
+                            fp64);
+}
+
+template <int MODE, typename S>
+__global__ void __launch_bounds__(32 * kWarps, kBlocks)
+    k_fxop2d(int n, int pitch, size_t st, const __grid_constant__ Coef2D c,
+             const double* __restrict__ f, const double* __restrict__ x, S* __restrict__ out,
+             double mscale, double* __restrict__ mx) {
+  const int lane = threadIdx.x, ib = blockIdx.z;
+  const int i0 = kCols * blockIdx.x + 2 * lane;  // this lane's columns i0, i0 + 1
+  const int j0 = 1 + kRows * (blockIdx.y * kWarps + threadIdx.y);
+  if (j0 >= n) return;  // uniform over the warp
+  const size_t base = ib * st;
+  const bool in = i0 <= n;  // (i0 + 1 <= n + 1 < pitch then)
+  double2 xv[kRows + 2];
+#pragma unroll
+  for (int t = 0; t < kRows + 2; ++t) {
+    const int r = j0 - 1 + t;
+    xv[t] = in && r <= n ? *reinterpret_cast<const double2*>(x + base + (size_t)r * pitch + i0)
+                         : make_double2(0.0, 0.0);
+  }
+  // the largest of the lane's x and its neighbours', and of its f, which counts an eighth (|f| <=
+  // 8 2^e fits beside the stencil of x).  f is read here and again, from L1, when its row is due.
+  int top = 0;
+#pragma unroll
+  for (int t = 0; t < kRows + 2; ++t) top = max(top, max(high(xv[t].x), high(xv[t].y)));
+  top = max(top, max(__shfl_up_sync(0xffffffffu, top, 1), __shfl_down_sync(0xffffffffu, top, 1)));
+  if (!applies(MODE)) {
+    int topf = 0;
+#pragma unroll
+    for (int t = 0; t < kRows; ++t)
+      if (in && j0 + t < n) {
+        const double2 v =
+            *reinterpret_cast<const double2*>(f + base + (size_t)(j0 + t) * pitch + i0);
+        topf = max(topf, max(high(v.x), high(v.y)));
+      }
+    top = max(top, topf - (3 << 20));
+  }
+  if (c.fits && !c.fits[ib]) return;  // an instance of the FP64 form
+  // the tile's exponent, and its least lane's (lanes of zeros: none)
+  const int most = __reduce_max_sync(0xffffffffu, top);
+  const unsigned least = __reduce_min_sync(0xffffffffu, (unsigned)top - 1u);
+  const int e = ((most + 1) >> 20) - 1022;
+  if (e < -kFxMaxExp || e > kFxMaxExp)
+    tile_fp64<MODE, S>(n, pitch, base, ib, i0, j0, c, f, x, out, mscale, mx);
+  else if ((int)(least >> 20) - 1022 + kLaneRange < e)
+    tile_lanes<MODE, S>(n, pitch, base, ib, i0, j0, c, f, x, out, mscale, mx, top);
+  else
+    tile_fixed<MODE, S, false>(n, pitch, base, ib, i0, j0, c, f, x, out, mscale, mx, xv, e, false);
 }
 
 template <int MODE, typename S>

@@ -31,3 +31,57 @@ def test_right_hand_side_near_the_largest_number_3d():
             out.append(host(y))
     assert np.isfinite(out[1]).all()
     assert (np.abs(out[0] / out[1] - 1.0) <= 1e-13).all()
+
+
+def _fields(n, dim):
+    """Values of one sign and of both that fall by 2^-40 across 32 nodes of one axis, a wide
+    Gaussian, and such a slope beside a patch of zeros."""
+    rng = np.random.default_rng(3300)
+    shape = (n - 1,) * dim
+    x = np.arange(1, n, dtype=np.float64)
+    out = {}
+    for axis in range(dim):
+        line = [1] * dim
+        line[dim - 1 - axis] = n - 1
+        decay = np.exp2(-1.25 * x).reshape(line)
+        out[f"decay{axis}"] = decay * rng.uniform(0.5, 1.0, size=shape)
+        out[f"mixed{axis}"] = decay * rng.normal(size=shape)
+    r2 = sum(np.meshgrid(*[(x / n - 0.4) ** 2] * dim, indexing="ij"))
+    out["gauss"] = np.exp(-150.0 * r2)
+    patch = out["decay0"].copy()
+    patch[n // 3:n // 2] = 0.0
+    out["zeros"] = patch
+    return out
+
+
+def _star_max(v):
+    """The largest magnitude of each node's stencil (its 3^dim box: the stencil and corners)."""
+    from scipy.ndimage import maximum_filter
+
+    return maximum_filter(np.abs(v), size=3, mode="constant")
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+def test_every_node_2d(precision):
+    """n = 640.  Rounding of at most 16 units of 2^-58 of the largest of 6 x 6 nodes, which lies at
+    most 2^6.25 above a node's own stencil here: 2^-47 of it; 1e-13, as for values of one size."""
+    from oracle import fmg_oracle as O
+
+    fmg = _fmg()
+    op = O.Problem(dim=2, coarse_cells=5, levels=8, w_const=0.3, w_quad=(1.0, 2.5, 0.0), zeta=7.0)
+    p = fmg.Problem(dim=2, coarse_cells=5, levels=8, w_const=0.3, w_quad=(1.0, 2.5, 0.0), zeta=7.0,
+                    precision=fmg.FMG_FP64 if precision == "fp64" else fmg.FMG_MIXED_FP32)
+    coarse = O.Level(O.Mesh(2, 320, 1.0), None, None, None, None, None, None)
+    lev = O.build_level(op, 8, coarse)
+    n = 640
+    y = torch.empty(p.size(8), dtype=torch.float64, device="cuda")
+    fields = _fields(n, 2)
+    with fmg.Solver(p) as s:
+        for name, x in fields.items():
+            f = fields["mixed0" if name != "mixed0" else "decay1"]
+            top = np.maximum(8 * _star_max(x), np.abs(f))
+            s.apply_operator(8, dev(x.ravel()), y)
+            assert (np.abs(host(y) - lev.L @ x.ravel()) <= 1e-13 * 8 * _star_max(x).ravel()).all(), name
+            s.jacobi(8, dev(f.ravel()), dev(x.ravel()), y)
+            ref = O.jacobi(lev, f.ravel(), x.ravel(), op.omega)
+            assert (np.abs(host(y) - ref) <= 1e-13 * top.ravel()).all(), name
