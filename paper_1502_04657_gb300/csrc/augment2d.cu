@@ -139,7 +139,7 @@ __global__ void __launch_bounds__(32 * kStarWarps, 4)
   });
   star2d_redo<R>(n, pitch, st, redo, [&](size_t k) {
     nload_density2d_redo(k, pitch, s60, s180, u, nl, bC, bE, bN, bNE);
-  });
+  }, [&] { nload_density2d_fp64<R>(n, pitch, st, s60, s180, u, nl, bC, bE, bN, bNE); });
 }
 
 // The same quantities node by node, for levels below n = 64

@@ -19,7 +19,8 @@
 // function: inlined, its register pressure spilled the fixed-point path).  And a node whose
 // results are short of bits, because its star lies far below the tile's largest value (next to a
 // corner of the box, or on a steep slope), is evaluated again in FP64: a cubic load below 2^36 (2D)
-// or 2^40 (3D) units, a density entry below 2^44.  The roundings add up to at most 20 (2D) or 400
+// or 2^40 (3D) units, a density entry below 2^44 (the whole tile where these are half of its nodes,
+// or half of its columns lie 2^-7 below its largest value).  The roundings add up to at most 20 (2D) or 400
 // (3D) units of a cubic load and 20 or 150 of a density entry, so every load keeps 4e-10 and every
 // density entry 1e-11 of itself in the worst case.  Measured
 // against 113-bit arithmetic on ground-state-like inputs, relative 2-norm of the cubic load,
@@ -132,6 +133,7 @@ __device__ __forceinline__ T get(const FxVec& u, size_t k) {
 
 constexpr int kFxMaxExp = 250;
 constexpr int kFxRange = 32;      // a tile with values below 2^-32 of its largest is left to FP64
+constexpr int kFxLow = 7;         // a column 2^-7 below the largest is short of bits all over
 constexpr int kFxNone = -100000;  // no fixed-point exponent: compute the tile in FP64
 // The largest high words (without sign) of a tile's positive and negative values, and its
 // smallest nonzero one (less 1).
@@ -148,6 +150,11 @@ struct FxTop {
     pos = __reduce_max_sync(0xffffffffu, pos);
     neg = __reduce_max_sync(0xffffffffu, neg);
     low = __reduce_min_sync(0xffffffffu, low);
+  }
+  // whether these values, not all zero (or outside the mesh), are below 2^(e - kFxLow)
+  __device__ __forceinline__ bool far_below(int e) const {
+    const int top = max(pos, neg);
+    return top > 0 && ((top + 1) >> 20) - 1022 + kFxLow < e;
   }
   // e with |u| <= 2^e (1 - 2^-20) (the margin keeps the signed splits of products in range),
   // or kFxNone

@@ -417,7 +417,8 @@ __global__ void __launch_bounds__(32 * kStarWarps, 4)
     redo = redo << 1 | (unsigned)fx_short<kShortLoad2>(v);
     out[k] = to_double(v, s);
   });
-  star2d_redo<R>(n, pitch, st, redo, [&](size_t k) { nload2d_at(k, pitch, scale, u, out); });
+  star2d_redo<R>(n, pitch, st, redo, [&](size_t k) { nload2d_at(k, pitch, scale, u, out); },
+                 [&] { nload2d_fp64<R>(n, pitch, st, scale, u, out); });
 }
 
 // f = lambda M u - N(u); the mass stencil h^2/12 (6 u_p + neighbour sum) reuses the cubic
@@ -441,7 +442,8 @@ __global__ void __launch_bounds__(32 * kStarWarps, 4)
     f[k] = fma(s1, __ll2double_rn(madd<12>(p.u, p.M1).v), -to_double(v, s3));
   });
   star2d_redo<R>(n, pitch, st, redo,
-                 [&](size_t k) { rhs2d_at(k, pitch, h2_24, nscale, l, u, f); });
+                 [&](size_t k) { rhs2d_at(k, pitch, h2_24, nscale, l, u, f); },
+                 [&] { rhs2d_fp64<R>(n, pitch, st, h2_24, nscale, l, u, f); });
 }
 
 // FP32 auxiliary right-hand side of the mixed-precision iteration (same closed forms in

@@ -588,7 +588,7 @@ __global__ void __launch_bounds__(kS3X * kS3Y, 3)
     });
     star3_redo<P>(n, pitch, st, redo, [&](size_t k) {
       nload3d_at(k, pitch, (long)(n + 1) * pitch, 6.0 * scale6, u, out);
-    });
+    }, [&] { nload3d_fp64<P>(n, pitch, st, scale6, u, out); });
     return;
   }
   nload3d_fp64<P>(n, pitch, st, scale6, u, out);
@@ -614,7 +614,7 @@ __global__ void __launch_bounds__(kS3X * kS3Y, 3)
     });
     star3_redo<P>(n, pitch, st, redo, [&](size_t k) {
       rhs3d_at(k, pitch, (long)(n + 1) * pitch, 120.0 * h3_120, 6.0 * zn, l, u, f);
-    });
+    }, [&] { rhs3d_fp64<P>(n, pitch, st, h3_120, zn, l, u, f); });
     return;
   }
   rhs3d_fp64<P>(n, pitch, st, h3_120, zn, l, u, f);
@@ -654,7 +654,7 @@ __global__ void __launch_bounds__(kS3X * kS3Y, 3)
     star3_redo<P>(n, pitch, st, redo, [&](size_t k) {
       nload_density3d_at(k, pitch, (long)(n + 1) * pitch, 6.0 * s140_6, 2.0 * s210_2, 2.0 * s420_2,
                          u, nl, b);
-    });
+    }, [&] { nload_density3d_fp64<P>(n, pitch, st, s140_6, s210_2, s420_2, u, nl, b); });
     return;
   }
   nload_density3d_fp64<P>(n, pitch, st, s140_6, s210_2, s420_2, u, nl, b);

@@ -112,8 +112,10 @@ __device__ __forceinline__ int star2d_exponent(int n, int pitch, size_t st, cons
     const int r = j0 - 1 + t;
     if (i <= n && r <= n) m.add(p[(size_t)r * pitch]);
   }
+  const FxTop column = m;
   m.warp_max();
-  return m.exponent();
+  const int e = m.exponent();
+  return 2 * __popc(__ballot_sync(0xffffffffu, column.far_below(e))) > 32 ? kFxNone : e;
 }
 
 // The walk in fixed point.  Sums of fixed-point values are exact, so the three opposite edges a
@@ -215,14 +217,19 @@ __device__ __forceinline__ void star2d_walk_fx(int n, int pitch, size_t st,
   }
 }
 
-// node(k) for the nodes that a fixed-point walk of this warp left short of bits.  redo: one bit per
-// row that the lane produced, the latest lowest.  The nodes are spread over the lanes: an FP64
-// instruction takes a warp the same time for one node as for 32.
-template <int R, typename Node>
-__device__ __forceinline__ void star2d_redo(int n, int pitch, size_t st, unsigned redo, Node node) {
+// node(k) for the nodes that a fixed-point walk of this warp left short of bits, or tile() for half
+// of its nodes and more.  redo: one bit per row that the lane produced, the latest lowest.  The nodes
+// are spread over the lanes: an FP64 instruction takes a warp the same time for one node as for 32.
+template <int R, typename Node, typename Tile>
+__device__ __forceinline__ void star2d_redo(int n, int pitch, size_t st, unsigned redo, Node node,
+                                            Tile tile) {
   __shared__ unsigned short list[kStarWarps][32 * R];
   __shared__ int count[kStarWarps];
   if (!__any_sync(0xffffffffu, redo)) return;
+  if (__reduce_add_sync(0xffffffffu, __popc(redo)) > kStarCols * R / 2) {
+    tile();
+    return;
+  }
   const int lane = threadIdx.x, w = threadIdx.y;
   const int j0 = 1 + R * (blockIdx.y * blockDim.y + w), last = min(j0 + R, n) - 1;
   if (lane == 0) count[w] = 0;

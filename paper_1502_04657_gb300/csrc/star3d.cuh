@@ -120,6 +120,7 @@ __device__ __forceinline__ int star3_exponent(int n, int pitch, size_t st, const
 #pragma unroll 6
     for (int z = z0 - 1; z <= z1; ++z) m.add(p[z * plane]);
   }
+  const FxTop columns = m;
   m.warp_max();
   __syncthreads();
   if ((tid & 31) == 0) {
@@ -131,15 +132,17 @@ __device__ __forceinline__ int star3_exponent(int n, int pitch, size_t st, const
   m.pos = top[0];
   m.neg = top[1];
   m.low = low;
-  return m.exponent();
+  const int e = m.exponent();
+  return 2 * __syncthreads_count(columns.far_below(e)) > kS3X * kS3Y ? kFxNone : e;
 }
 
-// node(k) for the nodes that a fixed-point walk of this block left short of bits.  redo: one bit per
-// plane that the thread produced, the latest lowest.  The nodes are spread over the threads (in the
-// shared memory that the walk has left): an FP64 instruction takes a warp the same time for one
-// node as for 32.
-template <int P, typename Node>
-__device__ __forceinline__ void star3_redo(int n, int pitch, size_t st, unsigned redo, Node node) {
+// node(k) for the nodes that a fixed-point walk of this block left short of bits, or tile() for half
+// of its nodes and more.  redo: one bit per plane that the thread produced, the latest lowest.  The
+// nodes are spread over the threads (in the shared memory that the walk has left): an FP64
+// instruction takes a warp the same time for one node as for 32.
+template <int P, typename Node, typename Tile>
+__device__ __forceinline__ void star3_redo(int n, int pitch, size_t st, unsigned redo, Node node,
+                                           Tile tile) {
   extern __shared__ double s3sm[];
   int* const count = reinterpret_cast<int*>(s3sm);
   unsigned short* const list = reinterpret_cast<unsigned short*>(count + 1);
@@ -153,6 +156,11 @@ __device__ __forceinline__ void star3_redo(int n, int pitch, size_t st, unsigned
     list[atomicAdd(count, 1)] = (unsigned short)((last - (__ffs(redo) - 1) - z0) * kS3X * kS3Y + tid);
   __syncthreads();
   const int total = *count;
+  if (total > kS3X * kS3Y * P / 2) {
+    __syncthreads();  // the walk takes the shared memory
+    tile();
+    return;
+  }
   for (int q = tid; q < total; q += kS3X * kS3Y) {
     const int c = list[q], x = 1 + blockIdx.x * kS3X + c % kS3X,
               y = 1 + blockIdx.y * kS3Y + c / kS3X % kS3Y, z = z0 + c / (kS3X * kS3Y);
