@@ -18,8 +18,11 @@
 //                     + sum_faces (s / 168 - w_o / 120) p_face ],  o the axis across the face;
 //       al = ax[i] + ay[j] + az[l] and be_d come from 1D tables scaled to fill the integers, the
 //       small terms (h^2 below the others) take the upper 30 bits of the pairs.
-// Only the products, x and f round, at 2^-57 of the tile's maximum (FP64 rounds each of its 15
-// operations and every stored coupling at 2^-53).  f is scaled by 1 / h in FP64.
+// Only the products, x and f round, at 2^-57 of the tile's maximum, and the small terms at 2^-50 of
+// it or below (2^-33 of h^4 s); f / h, up to 8 times the maximum, is rounded by FP64.  FP64 rounds each
+// of its 15 operations and every stored coupling at 2^-53, relative to the node's own stencil: a
+// block where three nodes in a column lie 2^-20 or more below its largest value (or, for x = 0,
+// where f does) is left to FP64, so that every node keeps 2^-30 of its own stencil.
 //
 // Measured on 16.6M nodes: Jacobi 438 -> 270 us, residual 413 -> 223 us.  The instruction rate
 // bounds it (some 400 integer instructions per node, half of the issue slots used), then the
@@ -29,8 +32,8 @@
 // The operator apply of the augmented pass also stores M x = h^3/60 S: the two applies took 195
 // and 573 us on 16.6M nodes, together 208 us.
 //
-// Tiles with infinities, NaN, all zeros or an exponent outside +-kFxMaxExp run the FP64 expressions
-// of grid3d.cu.  Instances whose potential is too large for the formats (fxop3d_scale: h^2 |W| >
+// Blocks with infinities, NaN, all zeros or an exponent outside +-kFxMaxExp run the FP64 expressions
+// of grid3d.cu, too.  Instances whose potential is too large for the formats (fxop3d_scale: h^2 |W| >
 // 60/64 or h^4 s > 2^-17) take grid3d.cu's kernels and stored couplings: with the couplings formed
 // from their 1D tables at every use (46 FP64 operations per node and more, where those kernels need
 // 16) two V-cycles at h = 10/256 took 16.4 ms, the FP64 kernels 5.8.
@@ -43,6 +46,7 @@ namespace {
 
 constexpr int kB = 57;                       // x = I 2^(e - kB); |S| <= 60 2^kB
 constexpr int kX = 32, kY = 8, kZ = 8;       // tile of columns (= threads), planes per block
+constexpr int kRange = 20;                   // range of a block, in bits
 constexpr int kNX = kX + 2, kNodes = (kX + 2) * (kY + 2);
 
 // Tables ax, ay, az, bx, by, bz (n + 1 entries each) and the header of each instance.
@@ -104,6 +108,8 @@ __device__ __forceinline__ long long to_fixed(double v, int shift) {
   return (t ^ sg) - sg;
 }
 
+__device__ __forceinline__ int high(double v) { return __double2hiint(v) & 0x7fffffff; }
+
 enum Mode { kJacobiMode, kResidualMode, kApplyMode, kApplyMassMode };
 constexpr bool applies(int mode) { return mode == kApplyMode || mode == kApplyMassMode; }
 
@@ -159,6 +165,7 @@ __global__ void __launch_bounds__(kX * kY, 3)
              double* __restrict__ mv) {
   __shared__ long long su[kZ + 2][kNodes];  // planes z0 - 1 .. z0 + kZ
   __shared__ int top[2];
+  __shared__ unsigned low[2];
   const int nzc = (n - 1 + kZ - 1) / kZ, ib = blockIdx.z / nzc;
   const int z0 = 1 + (int)(blockIdx.z - ib * nzc) * kZ, z1 = min(z0 + kZ, n);
   const int x0 = 1 + blockIdx.x * kX, y0 = 1 + blockIdx.y * kY;
@@ -175,13 +182,17 @@ __global__ void __launch_bounds__(kX * kY, 3)
   const double* pa = v + base + (long)ya * pitch + xa;
   const double* pb = v + base + (long)yb * pitch + xb;
   const double* pf = f + base + (long)y * pitch + x;
-  if (tid < 2) top[tid] = 0;
+  if (tid < 2) {
+    top[tid] = 0;
+    low[tid] = 0xffffffffu;
+  }
   __syncthreads();
   // the whole tile is loaded first (a block's loads in flight at once), its exponent taken, and
   // its integers stored to shared memory, so that the planes below need no barrier
   double va[kZ + 2], vb[kZ + 2];
   {
     int m = 0, mf = 0;
+    unsigned lx = 0xffffffffu, lf = 0xffffffffu;  // least nonzero values, less 1
 #pragma unroll
     for (int t = 0; t < kZ + 2; ++t) {
       const int z = z0 - 1 + t;
@@ -191,16 +202,30 @@ __global__ void __launch_bounds__(kX * kY, 3)
     if (!applies(MODE) && active) {
 #pragma unroll
       for (int t = 0; t < kZ; ++t)
-        if (z0 + t < z1) mf = max(mf, __double2hiint(pf[(z0 + t) * plane]) & 0x7fffffff);
+        if (z0 + t < z1) {
+          const int v = high(pf[(z0 + t) * plane]);
+          mf = max(mf, v);
+          lf = min(lf, (unsigned)v - 1u);
+        }
     }
 #pragma unroll
-    for (int t = 0; t < kZ + 2; ++t)
-      m = max(m, max(__double2hiint(va[t]) & 0x7fffffff, __double2hiint(vb[t]) & 0x7fffffff));
+    for (int t = 1; t <= kZ; ++t) {
+      const int a = max(max(high(va[t - 1]), high(va[t])), high(va[t + 1])),
+                b = max(max(high(vb[t - 1]), high(vb[t])), high(vb[t + 1]));
+      m = max(m, max(a, b));
+      lx = min(lx, min((unsigned)a - 1u, (unsigned)b - 1u));
+    }
     m = __reduce_max_sync(0xffffffffu, m);
-    mf = __reduce_max_sync(0xffffffffu, mf);
+    lx = __reduce_min_sync(0xffffffffu, lx);
+    if (!applies(MODE)) {
+      mf = __reduce_max_sync(0xffffffffu, mf);
+      lf = __reduce_min_sync(0xffffffffu, lf);
+    }
     if ((tid & 31) == 0) {
       atomicMax(&top[0], m);
       atomicMax(&top[1], mf);
+      atomicMin(&low[0], lx);
+      atomicMin(&low[1], lf);
     }
   }
   __syncthreads();
@@ -209,7 +234,8 @@ __global__ void __launch_bounds__(kX * kY, 3)
   const int e = top[1] == 0 ? ex : max(ex, ef);
   const FxHead3D hd = c.fxh[ib];
   if (c.fits && !c.fits[ib]) return;  // an instance of the FP64 form
-  if (top[1] >= 0x7ff00000 || e < -kFxMaxExp || e > kFxMaxExp) {
+  const int least = top[0] ? (int)(low[0] >> 20) - 1022 : (int)(low[1] >> 20) - 1022 + hexp - 3;
+  if (top[1] >= 0x7ff00000 || e < -kFxMaxExp || e > kFxMaxExp || least + kRange < e) {
     tile_fp64<MODE>(n, pitch, base, ib, x, y, z0, z1, c, f, v, out, mscale, mv);
     return;
   }

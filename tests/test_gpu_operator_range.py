@@ -85,3 +85,47 @@ def test_every_node_2d(precision):
             s.jacobi(8, dev(f.ravel()), dev(x.ravel()), y)
             ref = O.jacobi(lev, f.ravel(), x.ravel(), op.omega)
             assert (np.abs(host(y) - ref) <= 1e-13 * top.ravel()).all(), name
+
+
+def test_every_node_3d():
+    """n = 96.  Blocks whose columns hold a stencil below 2^-20 of the block's largest value are
+    evaluated in FP64; in the others 12 units of 2^-57 (and 2^-50 times h^4 |W''| of the formats'
+    limit) leave 2^-32 of a node's own stencil; 1e-9."""
+    kw = dict(dim=3, coarse_cells=3, levels=6, w_const=0.3, w_quad=(1.0, 2.0, 1.5))
+    n = 96
+    fields = _fields(n, 3)
+    got = []
+    for s in _mixed_and_fp64(**kw):
+        with s:
+            y = torch.empty(s.level_size(6), dtype=torch.float64, device="cuda")
+            rows = []
+            for name, x in fields.items():
+                f = fields["mixed0" if name != "mixed0" else "decay1"] / n
+                s.apply_operator(6, dev(x.ravel()), y)
+                rows.append(host(y).copy())
+                s.jacobi(6, dev(f.ravel()), dev(x.ravel()), y)
+                rows.append(host(y).copy())
+            got.append(rows)
+    for i, (name, x) in enumerate(fields.items()):
+        f = fields["mixed0" if name != "mixed0" else "decay1"] / n
+        star = _star_max(x).ravel()
+        a, b = got[0][2 * i], got[1][2 * i]
+        assert (np.abs(a - b) <= 1e-9 * 12.0 / n * star).all(), name
+        # Jacobi: omega / D is below n / 9
+        top = np.maximum(12.0 / n * star, np.abs(f.ravel())) * n / 9
+        a, b = got[0][2 * i + 1], got[1][2 * i + 1]
+        assert (np.abs(a - b) <= 1e-9 * top).all(), name
+
+
+def test_right_hand_side_of_wide_range_from_zero_3d():
+    """x = 0: the residual is f at every node, whatever the range of f (n = 96), to rounding in its
+    restriction."""
+    kw = dict(dim=3, coarse_cells=3, levels=6, w_const=0.3, w_quad=(1.0, 2.0, 1.5))
+    got = []
+    for s in _mixed_and_fp64(**kw):
+        with s:
+            rc = torch.empty(s.level_size(5), dtype=torch.float64, device="cuda")
+            f = _fields(96, 3)["decay0"]
+            s.residual_restrict(6, dev(f.ravel()), dev(np.zeros(f.size)), rc)
+            got.append(host(rc))
+    assert (np.abs(got[0] / got[1] - 1.0) <= 1e-9).all()
