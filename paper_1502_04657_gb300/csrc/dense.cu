@@ -912,13 +912,17 @@ __device__ __noinline__ bool inverse_fp64(const double* L, double* A, double* Y,
 }
 
 constexpr int kInverseRounds = 2;
+// Largest entry of I - L X0 for which two rounds reach FP64 rounding (each about multiplies the
+// residual by that much): 1e-7 for the operators of any resolved potential, above it from condition
+// numbers of some 1e3 on (an A + W that a negative potential brings near singularity).
+constexpr float kInverseStart = 3.8e-6f;
 
 // L^{-1} of the SPD level-1 operator, one CTA per instance: the single-precision inverse of
 // the sweep operator (~1e-6), then X <- X + Y (I - L X) with Y that inverse: the residual in
 // FP64 over the nonzeros of L (15 or 7 per row, so the FP64 work is n^2 x that, not n^3), the
 // product in single precision on a residual that shrinks by ~1e6 a round; two rounds leave the
-// rounding of I - L X.  An L whose single-precision elimination meets a non-positive pivot
-// takes the FP64 LDL^T.
+// rounding of I - L X.  An L whose single-precision elimination meets a non-positive pivot, or
+// leaves a residual above kInverseStart, takes the FP64 LDL^T.
 __global__ void __launch_bounds__(kThreads) k_spd_inverse(const double* __restrict__ L,
                                                           double* __restrict__ Linv, int n,
                                                           const uint16_t* __restrict__ lists,
@@ -935,9 +939,12 @@ __global__ void __launch_bounds__(kThreads) k_spd_inverse(const double* __restri
   double* dinv = X + n * n;
   for (int e = tid; e < n * n; e += kThreads) R[(e / n) * ns + e % n] = (float)L[e];
   __syncthreads();
-  if (!sweep_inverse(R, Y, ns, 0.0f, nullptr, piv, n, &pivots_ok)) {
+  auto in_fp64 = [&] {
     const bool ok = inverse_fp64(L, reinterpret_cast<double*>(R), X, dinv, n);
     for (int e = tid; e < n * n; e += kThreads) Linv[e] = ok ? X[e] : nan("");
+  };
+  if (!sweep_inverse(R, Y, ns, 0.0f, nullptr, piv, n, &pivots_ok)) {
+    in_fp64();
     return;
   }
   for (int e = tid; e < n * n; e += kThreads) X[e] = -(double)Y[(e / n) * ns + e % n];
@@ -945,6 +952,7 @@ __global__ void __launch_bounds__(kThreads) k_spd_inverse(const double* __restri
   const int nq = (n + 3) / 4;
   for (int round = 0; round < kInverseRounds; ++round) {
     __syncthreads();
+    bool large = false;
     for (int e = tid; e < n * n; e += kThreads) {
       const int i = e / n, j = e - i * n;
       double r = i == j ? 1.0 : 0.0;
@@ -953,8 +961,12 @@ __global__ void __launch_bounds__(kThreads) k_spd_inverse(const double* __restri
         r = fma(-L[i * n + k], X[k * n + j], r);
       }
       R[i * ns + j] = (float)r;
+      large = large || !(fabsf((float)r) <= kInverseStart);
     }
-    __syncthreads();
+    if (__syncthreads_or(round == 0 && large)) {
+      in_fp64();
+      return;
+    }
     for (int e = tid; e < n * nq; e += kThreads) {
       const int i = e / nq, j = 4 * (e - i * nq);
       float4 a = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
