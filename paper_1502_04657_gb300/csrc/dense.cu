@@ -55,8 +55,10 @@ constexpr int kWarps = kThreads / 32;
 // Relative residual below which Newton takes over (where its matrix is positive definite).  Over
 // coarse meshes of 3 to 9 (2D) and 3, 4 (3D) cells, zeta 1 to 5000 and traps 1 to 1000, 0.1
 // needed 3 to 22 steps where 1e-2 needed 3 to 47, never more, for the same ground state; 0.3
-// sometimes needed more (33 against 22).
-constexpr double kSwitch = 0.1;
+// sometimes needed more (33 against 22).  Beyond (zeta to 1e5, large negative or positive w_const,
+// under-resolved meshes) Newton from so far can wander to the cap: the problem then starts again
+// with 1e-2.
+constexpr float kSwitch = 0.1f, kSwitchAgain = 1e-2f;
 constexpr int kMaxChord = 2;      // steps with an inverse of an earlier iterate, per inverse
 constexpr int kMaxN = kDenseMaxNh + 1;
 constexpr int kTile = 4;          // elements per side of a thread's tile in the FP32 sweep
@@ -713,7 +715,8 @@ __device__ __noinline__ bool solve_fp64(const DenseProblem& p, Smem<NV>& s, doub
 // One CTA of 256 threads per problem, a batch of problems one CTA each (two resident per SM:
 // at most 128 registers and half of the shared memory).  The iteration count is bounded by
 // max_iter (chord steps, at most kMaxChord per inverse, are not counted: they replace the
-// refinement of the Newton correction); hitting it sets status 1.
+// refinement of the Newton correction); hitting it a second time, after a fresh start with
+// kSwitchAgain, sets status 1.
 // ASSEMBLE: only assemble K0, M and G(c_init) into K_out, M_out, G_out.
 template <int NV, bool ASSEMBLE>
 __global__ void __launch_bounds__(kThreads, 2) k_dense_scf(const __grid_constant__ DenseProblem p) {
@@ -735,7 +738,8 @@ __global__ void __launch_bounds__(kThreads, 2) k_dense_scf(const __grid_constant
     const int v = p.tri[e];
     s.tri[e] = (uint16_t)(v < 0 ? nh : v);
   }
-  if (tid <= nh) {
+  auto start = [&] {
+    if (tid > nh) return;
     double c = 0.0;
     if (p.c_init) c = tid < n ? p.c_init[ib * (nh + 1) + tid] : 0.0;
     else if (tid == nh) c = 1.0;
@@ -746,11 +750,12 @@ __global__ void __launch_bounds__(kThreads, 2) k_dense_scf(const __grid_constant
     s.w[tid] = c;
     s.w2[tid] = c * c;
     s.w3[tid] = 2.0 * (c * c * c);
-    if (p.aug && tid < nh) {
-      s.gA[tid] = p.gA[ib * nh + tid];
-      s.gM[tid] = p.gM[ib * nh + tid];
-      s.t1[tid] = p.t1[ib * nh + tid];
-    }
+  };
+  start();
+  if (p.aug && tid < nh) {
+    s.gA[tid] = p.gA[ib * nh + tid];
+    s.gM[tid] = p.gM[ib * nh + tid];
+    s.t1[tid] = p.t1[ib * nh + tid];
   }
   if (tid == kThreads - 1) {
     s.auu = p.aug ? p.auu[ib] : 0.0;
@@ -816,7 +821,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_dense_scf(const __grid_constant
   bool zero = p.aug && !p.c_init;              // the start c = u~
   bool newton = false;
   bool failed = false;  // the Newton matrix of this iterate had a non-positive pivot
-  float rn = 0.0f;
+  float rn = 0.0f, reach = kSwitch;
   for (;;) {
     bool converged = false, chord = false;
     if (!failed) {
@@ -830,8 +835,17 @@ __global__ void __launch_bounds__(kThreads, 2) k_dense_scf(const __grid_constant
       chord = chords < kMaxChord && rn < 0.05f * last &&
               (converged || 4.0f * rn * rn <= last * (float)p.tol);
       if (converged) status = 0;
+      if (!chord && it >= p.max_iter && !converged && reach == kSwitch) {
+        start();
+        reach = kSwitchAgain;
+        zero = p.aug && !p.c_init;
+        it = 0;
+        chords = kMaxChord;
+        __syncthreads();
+        continue;
+      }
       if (!chord && (converged || it >= p.max_iter)) break;
-      if (!chord) newton = rn <= (float)kSwitch;
+      if (!chord) newton = rn <= reach;
     } else {
       newton = false;
     }
