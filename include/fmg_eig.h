@@ -115,7 +115,8 @@ typedef struct fmg_eig_problem {
   int32_t smoother;     /* FMG_SMOOTH_JACOBI | FMG_SMOOTH_CHEBYSHEV | FMG_SMOOTH_CG        */
   int32_t precision;    /* FMG_FP64 | FMG_MIXED_FP32 | FMG_MIXED_BF16                      */
   int32_t operator_form;/* FMG_W_LEFT | FMG_PAPER_LITERAL                                  */
-  int32_t scf_max_iter; /* cap on nonlinear iterations per small solve (e.g. 100)          */
+  int32_t scf_max_iter; /* cap on nonlinear iterations per small solve (e.g. 100); one that  */
+                        /* hits it starts again once, more cautiously                       */
   int32_t flags;        /* FMG_FLAG_* bits (0 = defaults)                                  */
   double box_len;       /* L > 0                                                           */
   double w_const;       /* W(x) = w_const + sum_d w_quad[d] x_d^2                          */
@@ -166,7 +167,10 @@ void fmg_eig_destroy(fmg_eig_handle* h);
 /* Change the potential (w_const, w_quad), zeta and omega of an existing handle: the PDE of
  * Example 4.1 with new coefficients on the same mesh hierarchy.  Every other field of *prob
  * must equal the handle's (FMG_EINVAL otherwise).  Synchronises the handle's stream; the
- * next solve uses the new values (they are uploaded from pinned host memory per solve).   */
+ * next solve uses the new values (they are uploaded from pinned host memory per solve).
+ * Where the new potential changes the arithmetic of a level's operator (see the accuracy of the
+ * component entry points), the solve graph is recorded again, and the first such change may
+ * allocate: FMG_ENOMEM leaves the handle with its old values.                               */
 int fmg_eig_set_params(fmg_eig_handle* h, const fmg_eig_problem* prob);
 
 /* Instrumentation (no counterpart in the paper).  fmg_eig_kernel_count: kernel launches
@@ -301,6 +305,20 @@ int fmg_eig_level_tile(const fmg_eig_handle* h, int32_t level, int32_t* bx, int3
  * Component entry points: the steps of the hot path, one call each, on device vectors in the
  * interior layout above.  Each call is asynchronous on `stream` (NULL = handle's stream) and
  * uses the handle's level buffers as scratch, so calls on one handle must not overlap.
+ *
+ * Accuracy.  Where a level's kernels compute in FP64, every node is rounded relative to the
+ * terms of its own stencil.  Others compute in 64-bit fixed point with an exponent for a tile
+ * of nodes and round at 2^-50 of the tile's largest value or below; what they keep of a single
+ * node, however far below that value it lies (further ones are evaluated in FP64):
+ *   operator, residual, Jacobi step (2D from 512 cells per side, 3D FP64 mode from 96, where
+ *     h^2 |W| is below 3/16 or 15/16): 2^-42 of the largest |x| of the 6 x 6 nodes around it in
+ *     2D, 2^-30 of the largest |x| of its own stencil in 3D;
+ *   cubic load and right-hand side (2D from 64 cells, 3D FP64 mode from 32; tiles of one sign):
+ *     4e-10 of the load itself;
+ *   density stencil and its coarsening (augmented matrices): 1e-11 of each entry per level;
+ *   restriction (2D from 512 cells): 2^-53 of the largest of the 15 residuals around a pair of
+ *     coarse nodes.
+ * Infinities and NaN reach the nodes whose stencil they lie in.
  * ---------------------------------------------------------------------------------------- */
 
 /* y = L_k x with L = A + W (FMG_W_LEFT) or A (FMG_PAPER_LITERAL): the operator of the

@@ -113,16 +113,6 @@ __device__ __forceinline__ T half_sums(T a, T b) {
   return v;
 }
 
-// 1 / d by Newton's iteration from the hardware's approximate reciprocal (about 2^-20 relative
-// error; two steps reach FP64 rounding).
-__device__ __forceinline__ double recip(double d) {
-  double y;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(d));
-  y = fma(y, fma(-d, y, 1.0), y);
-  y = fma(y, fma(-d, y, 1.0), y);
-  return y;
-}
-
 // The exponent of v, and 2^e as a float (clamped to its range)
 __device__ __forceinline__ int exponent_of(double v) {
   return ((__double2hiint(v) >> 20) & 0x7ff) - 1023;

@@ -22,6 +22,7 @@
 #include <math.h>
 #include <stdint.h>
 
+#include "dfloat.cuh"
 #include "fmg_internal.h"
 
 namespace fmg {
@@ -68,16 +69,6 @@ __device__ double block_sum(double v, double* red) {
   t = warp_sum(t);
   __syncthreads();  // red may be reused right away
   return t;
-}
-
-// 1 / d by Newton's iteration from the hardware's approximate reciprocal (about 2^-20 relative
-// error; two steps reach FP64 rounding).
-__device__ __forceinline__ double recip(double d) {
-  double y;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(d));
-  y = fma(y, fma(-d, y, 1.0), y);
-  y = fma(y, fma(-d, y, 1.0), y);
-  return y;
 }
 
 // Two block-wide sums at once, each in block_sum's order (so each result is bit-identical to

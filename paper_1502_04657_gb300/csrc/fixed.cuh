@@ -121,6 +121,28 @@ __device__ __forceinline__ bool fx_short(fx<K> x) {
   return (unsigned)((int)(x.v >> 32) + (1 << (T - 32))) < (2u << (T - 32));
 }
 
+// the same, truncated; shift = e + 1085 - B
+__device__ __forceinline__ long long fx_truncated(double v, int shift) {
+  const int hi = __double2hiint(v);
+  const unsigned long long m =
+      ((unsigned long long)(((uint32_t)hi & 0xfffffu) | 0x100000u) << 32 |
+       (uint32_t)__double2loint(v)) << 10;
+  const int sh = min(shift - ((hi >> 20) & 0x7ff), 63);
+  const long long t = (long long)(m >> sh), sg = hi >> 31;
+  return (t ^ sg) - sg;
+}
+
+// high word of a 64 x 64 product (|a|, |b| < 2^63 - 2^31), within a unit and a half
+__device__ __forceinline__ long long fx_mul_hi(long long a, long long b) {
+  const int al = (int)a, bl = (int)b;
+  const int ah = (int)(a >> 32) + (int)((uint32_t)al >> 31);
+  const int bh = (int)(b >> 32) + (int)((uint32_t)bl >> 31);
+  return (long long)ah * bh + (((long long)al * bh + (long long)ah * bl) >> 32);
+}
+
+// high word of |v|
+__device__ __forceinline__ int fx_high(double v) { return __double2hiint(v) & 0x7fffffff; }
+
 // u read in fixed point: scale = 2^(B1 - e)
 struct FxVec {
   const double* __restrict__ u;

@@ -79,27 +79,6 @@ __global__ void k_fxop2d_tables(int n, double h, const PotentialParams* __restri
   }
 }
 
-// high word of a 64 x 64 product (|a|, |b| < 2^62), within a unit and a half
-__device__ __forceinline__ long long mul_hi(long long a, long long b) {
-  const int al = (int)a, bl = (int)b;
-  const int ah = (int)(a >> 32) + (int)((uint32_t)al >> 31);
-  const int bh = (int)(b >> 32) + (int)((uint32_t)bl >> 31);
-  return (long long)ah * bh + (((long long)al * bh + (long long)ah * bl) >> 32);
-}
-
-// v 2^(kB - e) as an integer (truncated), |v| <= 2^e, on the integer pipes (a conversion
-// occupies the FP64 pipe like an FP64 operation)
-__device__ __forceinline__ long long to_fixed(double v, int shift) {  // shift = e + 1022 + 5
-  const int hi = __double2hiint(v);
-  const int ex = (hi >> 20) & 0x7ff;
-  const unsigned long long m =
-      ((unsigned long long)(((uint32_t)hi & 0xfffffu) | 0x100000u) << 32 |
-       (uint32_t)__double2loint(v)) << 10;
-  const int sh = min(shift - ex, 63);
-  const long long t = (long long)(m >> sh), sg = hi >> 31;
-  return (t ^ sg) - sg;
-}
-
 // v 2^e by the exponent field: v normal and nonzero, the result in the normal range
 __device__ __forceinline__ double times_pow2(double v, int e) {
   return __hiloint2double(__double2hiint(v) + e * (1 << 20), __double2loint(v));
@@ -179,7 +158,7 @@ __device__ __forceinline__ void tile_fixed(int n, int pitch, size_t base, int ib
     return in && r < n ? *reinterpret_cast<const double2*>(f + base + (size_t)r * pitch + i0) : zero;
   };
   const FxHead2D hd = c.fxh[ib];
-  const int shift = e + 1022 + 5;
+  const int shift = e + 1085 - kB;
   const double back = fx_pow2(e - kB), mback = mscale * back;
   const long long* tab = c.fxt + (size_t)ib * 4 * (n + 1);
   const int ia = min(i0, n), ic = min(i0 + 1, n);
@@ -192,11 +171,11 @@ __device__ __forceinline__ void tile_fixed(int n, int pitch, size_t base, int ib
   };
   auto row = [&](const double2& v) {
     Row q;
-    q.a = to_fixed(v.x, shift);
-    q.b = to_fixed(v.y, shift);
+    q.a = fx_truncated(v.x, shift);
+    q.b = fx_truncated(v.y, shift);
     if (LANES) {  // the lanes beside have their own units
-      q.l = to_fixed(__shfl_up_sync(0xffffffffu, v.y, 1), shift);
-      q.r = to_fixed(__shfl_down_sync(0xffffffffu, v.x, 1), shift);
+      q.l = fx_truncated(__shfl_up_sync(0xffffffffu, v.y, 1), shift);
+      q.r = fx_truncated(__shfl_down_sync(0xffffffffu, v.x, 1), shift);
     } else {
       q.l = __shfl_up_sync(0xffffffffu, q.b, 1);
       q.r = __shfl_down_sync(0xffffffffu, q.a, 1);
@@ -212,7 +191,7 @@ __device__ __forceinline__ void tile_fixed(int n, int pitch, size_t base, int ib
     s6 = 6 * x0 + t + d;
     long long sm = (long long)hd.P * (int)(x0 >> 32) + (long long)hd.Q * (int)(ew >> 32) +
                    (long long)hd.R * (int)(ns >> 32);
-    long long w = mul_hi(a, s6) + mul_hi(bx, (xe - xw) + g) + mul_hi(by, (xn - xs) + g);
+    long long w = fx_mul_hi(a, s6) + fx_mul_hi(bx, (xe - xw) + g) + fx_mul_hi(by, (xn - xs) + g);
     w += (sm >> hd.sm) + half;
     return 4 * x0 - t + (w >> hd.sa);
   };
@@ -228,8 +207,8 @@ __device__ __forceinline__ void tile_fixed(int n, int pitch, size_t base, int ib
       long long rb = node(m.b, m.r, m.a, p.b, s.b, p.r, s.a, axb + ay, bxb, by, mb);
       if (!applies(MODE)) {
         const double2 v = f_row(j);
-        ra = to_fixed(v.x, shift) - ra;
-        rb = to_fixed(v.y, shift) - rb;
+        ra = fx_truncated(v.x, shift) - ra;
+        rb = fx_truncated(v.y, shift) - rb;
       }
       const size_t k = base + (size_t)j * pitch + i0;
       const bool oka = lane > 0 && i0 <= n - 1 && !(LANES && fp64),
@@ -271,8 +250,6 @@ __device__ __forceinline__ void tile_fixed(int n, int pitch, size_t base, int ib
   }
   if (LANES && fp64) tile_fp64<MODE, S>(n, pitch, base, ib, i0, j0, c, f, x, out, mscale, mx);
 }
-
-__device__ __forceinline__ int high(double v) { return __double2hiint(v) & 0x7fffffff; }
 
 // The same with an exponent per lane, for the tiles whose lanes differ (called, and x read again: the
 // common path keeps its registers).
@@ -316,7 +293,7 @@ __global__ void __launch_bounds__(32 * kWarps, kBlocks)
   // 8 2^e fits beside the stencil of x).  f is read here and again, from L1, when its row is due.
   int top = 0;
 #pragma unroll
-  for (int t = 0; t < kRows + 2; ++t) top = max(top, max(high(xv[t].x), high(xv[t].y)));
+  for (int t = 0; t < kRows + 2; ++t) top = max(top, max(fx_high(xv[t].x), fx_high(xv[t].y)));
   top = max(top, max(__shfl_up_sync(0xffffffffu, top, 1), __shfl_down_sync(0xffffffffu, top, 1)));
   if (!applies(MODE)) {
     int topf = 0;
@@ -325,7 +302,7 @@ __global__ void __launch_bounds__(32 * kWarps, kBlocks)
       if (in && j0 + t < n) {
         const double2 v =
             *reinterpret_cast<const double2*>(f + base + (size_t)(j0 + t) * pitch + i0);
-        topf = max(topf, max(high(v.x), high(v.y)));
+        topf = max(topf, max(fx_high(v.x), fx_high(v.y)));
       }
     top = max(top, topf - (3 << 20));
   }

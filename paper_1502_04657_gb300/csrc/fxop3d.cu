@@ -88,28 +88,6 @@ __global__ void k_fxop3d_tables(int n, double h, const PotentialParams* __restri
   }
 }
 
-// high word of a 64 x 64 product (|a|, |b| < 2^63 - 2^31), within a unit and a half
-__device__ __forceinline__ long long mul_hi(long long a, long long b) {
-  const int al = (int)a, bl = (int)b;
-  const int ah = (int)(a >> 32) + (int)((uint32_t)al >> 31);
-  const int bh = (int)(b >> 32) + (int)((uint32_t)bl >> 31);
-  return (long long)ah * bh + (((long long)al * bh + (long long)ah * bl) >> 32);
-}
-
-// v 2^(kB - e) as an integer (truncated), |v| <= 2^e; shift = e + 1085 - kB
-__device__ __forceinline__ long long to_fixed(double v, int shift) {
-  const int hi = __double2hiint(v);
-  const int ex = (hi >> 20) & 0x7ff;
-  const unsigned long long m =
-      ((unsigned long long)(((uint32_t)hi & 0xfffffu) | 0x100000u) << 32 |
-       (uint32_t)__double2loint(v)) << 10;
-  const int sh = min(shift - ex, 63);
-  const long long t = (long long)(m >> sh), sg = hi >> 31;
-  return (t ^ sg) - sg;
-}
-
-__device__ __forceinline__ int high(double v) { return __double2hiint(v) & 0x7fffffff; }
-
 enum Mode { kJacobiMode, kResidualMode, kApplyMode, kApplyMassMode };
 constexpr bool applies(int mode) { return mode == kApplyMode || mode == kApplyMassMode; }
 
@@ -203,15 +181,15 @@ __global__ void __launch_bounds__(kX * kY, 3)
 #pragma unroll
       for (int t = 0; t < kZ; ++t)
         if (z0 + t < z1) {
-          const int v = high(pf[(z0 + t) * plane]);
+          const int v = fx_high(pf[(z0 + t) * plane]);
           mf = max(mf, v);
           lf = min(lf, (unsigned)v - 1u);
         }
     }
 #pragma unroll
     for (int t = 1; t <= kZ; ++t) {
-      const int a = max(max(high(va[t - 1]), high(va[t])), high(va[t + 1])),
-                b = max(max(high(vb[t - 1]), high(vb[t])), high(vb[t + 1]));
+      const int a = max(max(fx_high(va[t - 1]), fx_high(va[t])), fx_high(va[t + 1])),
+                b = max(max(fx_high(vb[t - 1]), fx_high(vb[t])), fx_high(vb[t + 1]));
       m = max(m, max(a, b));
       lx = min(lx, min((unsigned)a - 1u, (unsigned)b - 1u));
     }
@@ -252,8 +230,8 @@ __global__ void __launch_bounds__(kX * kY, 3)
                         hd.F[2]) / 2;
 #pragma unroll
   for (int t = 0; t < kZ + 2; ++t) {
-    su[t][tid] = to_fixed(va[t], shift);
-    if (e1 < kNodes) su[t][e1] = to_fixed(vb[t], shift);
+    su[t][tid] = fx_truncated(va[t], shift);
+    if (e1 < kNodes) su[t][e1] = fx_truncated(vb[t], shift);
   }
   __syncthreads();
   if (!active) return;
@@ -323,8 +301,8 @@ __global__ void __launch_bounds__(kX * kY, 3)
         q += (long long)hd.F[2] * (int)(p >> 28);
       }
       const long long t = 8 * u + pa2, S = 2 * (t + pf2) + t;
-      long long w = mul_hi(axy + tab[2 * (n + 1) + z], S) + mul_hi(bx, 2 * ex + dx) +
-                    mul_hi(by, 2 * ey + dy) + mul_hi(tab[5 * (n + 1) + z], 2 * ez + dz);
+      long long w = fx_mul_hi(axy + tab[2 * (n + 1) + z], S) + fx_mul_hi(bx, 2 * ex + dx) +
+                    fx_mul_hi(by, 2 * ey + dy) + fx_mul_hi(tab[5 * (n + 1) + z], 2 * ez + dz);
       w += (q >> hd.sm) + half;
       long long r = r6 + (w >> hd.sa);
       if (!applies(MODE)) r = __double2ll_rn(fv * fs) - r;

@@ -52,17 +52,6 @@ __global__ void k_coef1d(int n, double h, const PotentialParams* __restrict__ pp
   tab[7 * s + x] = wl * h4 * p.wy * ad;
 }
 
-// 1 / c by Newton's iteration y <- y (2 - c y) from the hardware's approximate reciprocal
-// (rcp.approx.ftz.f64, measured 2^-20 relative error on this part): two steps take it below FP64
-// rounding (4 DFMA, no conversions on the FP64 pipe, instead of a full division).
-__device__ __forceinline__ double recip(double c) {
-  double y;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(c));
-  y = fma(y, fma(-c, y, 1.0), y);
-  y = fma(y, fma(-c, y, 1.0), y);
-  return y;
-}
-
 // ratio_fx: the instances of the fixed-point form on a level of both take omega / C as k_dinv2d
 // forms it for them alone (levels that store their couplings for another reason don't).
 __global__ void k_coef2d(int n, int pitch, size_t st, const double* __restrict__ tab,
@@ -229,8 +218,9 @@ __global__ void k_restrict2d(int nc, int pc, int pf, size_t stc, size_t stf, Res
     }
   // coarse node 2P + d: fine centre column 4P + 2d is v[.][2 + 2d].  INTS: in integers, in
   // units of 2^(e - 57) with e the exponent of this thread's values (seven FP64 operations per
-  // coarse node bound the kernel otherwise: 16.8M nodes 53 -> 43 us); infinities, NaN and zeros in
-  // FP64.
+  // coarse node bound the kernel otherwise: 16.8M nodes 53 -> 43 us), so each node rounds at 2^-55 of
+  // the largest of the pair's 15 values, where FP64 rounds six sums at 2^-53 of its own; infinities,
+  // NaN and zeros in FP64.
   double out[2];
   int top = 0;
   if (INTS) {

@@ -65,13 +65,15 @@ FIELDS = ["sine", "steep", "decay0", "decay1"]
 
 
 @pytest.mark.parametrize("kind", FIELDS)
-@pytest.mark.parametrize("size", sorted(SIZES))
-def test_every_node_keeps_its_digits(size, kind):
+@pytest.mark.parametrize("size,walks", [(s, False) for s in sorted(SIZES)] +
+                         [("2d_n48", True), ("3d_n24", True)])
+def test_every_node_keeps_its_digits(size, walks, kind):
+    """walks: forced below the levels that take them by default (n = 64 in 2D, 32 in 3D)."""
     dim, cells, levels = SIZES[size]
     fmg = _fmg()
     zeta, lam = 50.0, 17.0
     p = fmg.Problem(dim=dim, coarse_cells=cells, levels=levels, w_quad=(1.0, 1.0, 1.0), zeta=zeta,
-                    flags=fmg.FMG_FLAG_NO_AUTOTUNE)
+                    flags=fmg.FMG_FLAG_NO_AUTOTUNE | (fmg.FMG_FLAG_STAR_WALKS if walks else 0))
     n = p.cells(levels)
     u = _field(kind, dim, n)
     for sign in (1.0, -1.0):
