@@ -313,8 +313,9 @@ int fmg_eig_level_tile(const fmg_eig_handle* h, int32_t level, int32_t* bx, int3
  *   operator, residual, Jacobi step (2D from 512 cells per side, 3D FP64 mode from 96, where
  *     h^2 |W| is below 3/16 or 15/16): 2^-42 of the largest |x| of the 6 x 6 nodes around it in
  *     2D, 2^-30 of the largest |x| of its own stencil in 3D;
- *   cubic load and right-hand side (2D from 64 cells, 3D FP64 mode from 32; tiles of one sign):
- *     4e-10 of the load itself;
+ *   cubic load (2D from 64 cells, 3D FP64 mode from 32; tiles of one sign): 4e-10 of itself;
+ *   right-hand side (the same levels): 2^-32 of |lambda| M |u| + zeta N(|u|), for a lambda of
+ *     the size of zeta u^2 or above;
  *   density stencil and its coarsening (augmented matrices): 1e-11 of each entry per level;
  *   restriction (2D from 512 cells): 2^-53 of the largest of the 15 residuals around a pair of
  *     coarse nodes.

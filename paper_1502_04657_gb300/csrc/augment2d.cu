@@ -116,7 +116,7 @@ __global__ void __launch_bounds__(32 * kStarWarps, 4)
                       const double* __restrict__ u, double* __restrict__ nl,
                       double* __restrict__ bC, double* __restrict__ bE,
                       double* __restrict__ bN, double* __restrict__ bNE) {
-  const int e = star2d_exponent<R>(n, pitch, st, u);
+  const int e = star2d_exponent<R, true>(n, pitch, st, u);
   if (e == kFxNone) {
     nload_density2d_fp64<R>(n, pitch, st, s60, s180, u, nl, bC, bE, bN, bNE);
     return;

@@ -395,7 +395,7 @@ template <int R>
 __global__ void __launch_bounds__(32 * kStarWarps, 4)
     k_nload2d(int n, int pitch, size_t st, double scale, const double* __restrict__ u,
               double* __restrict__ out) {
-  const int e = star2d_exponent<R>(n, pitch, st, u);
+  const int e = star2d_exponent<R, true>(n, pitch, st, u);
   if (e == kFxNone) {
     nload2d_fp64<R>(n, pitch, st, scale, u, out);
     return;
@@ -419,7 +419,7 @@ __global__ void __launch_bounds__(32 * kStarWarps, 4)
             const double* __restrict__ lam, const PotentialParams* __restrict__ pp,
             const double* __restrict__ u, double* __restrict__ f) {
   const double nscale = pp[blockIdx.z].zeta * h2_120, l = lam[blockIdx.z];
-  const int e = star2d_exponent<R>(n, pitch, st, u);
+  const int e = star2d_exponent<R, false>(n, pitch, st, u);
   if (e == kFxNone) {
     rhs2d_fp64<R>(n, pitch, st, h2_24, nscale, l, u, f);
     return;
@@ -427,9 +427,9 @@ __global__ void __launch_bounds__(32 * kStarWarps, 4)
   const double s1 = l * fx_scale<kFx2>(h2_24, 1, e), s3 = fx_scale<kFx2>(nscale, 3, e);
   unsigned redo = 0;
   star2d_walk_fx<false, R>(n, pitch, st, u, e, [&](size_t k, const Star2DFx& p) {
-    const fx<kFx2> v = star_cubic(p);
-    redo = redo << 1 | (unsigned)fx_short<kShortLoad2>(v);
-    f[k] = fma(s1, __ll2double_rn(madd<12>(p.u, p.M1).v), -to_double(v, s3));
+    const fx<kFx2> m = madd<12>(p.u, p.M1);
+    redo = redo << 1 | (unsigned)fx_short<kShortMass2>(m);
+    f[k] = fma(s1, __ll2double_rn(m.v), -to_double(star_cubic(p), s3));
   });
   star2d_redo<R>(n, pitch, st, redo,
                  [&](size_t k) { rhs2d_at(k, pitch, h2_24, nscale, l, u, f); },

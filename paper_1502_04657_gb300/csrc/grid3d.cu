@@ -565,7 +565,7 @@ template <int P>
 __global__ void __launch_bounds__(kS3X * kS3Y, 3)
     k_nload3d(int n, int pitch, size_t st, double scale6, const double* __restrict__ u,
               double* __restrict__ out) {
-  const int e = star3_exponent<P>(n, pitch, st, u);
+  const int e = star3_exponent<P, true>(n, pitch, st, u);
   if (e != kFxNone) {
     const double s = fx_scale<kFx3>(scale6, 3, e);
     unsigned redo = 0;
@@ -591,15 +591,15 @@ __global__ void __launch_bounds__(kS3X * kS3Y, 3)
             const double* __restrict__ u, double* __restrict__ f) {
   const int ib = blockIdx.z / star3_zchunks(n, P);
   const double l = lam[ib], zn = pp[ib].zeta * nscale6;
-  const int e = star3_exponent<P>(n, pitch, st, u);
+  const int e = star3_exponent<P, false>(n, pitch, st, u);
   if (e != kFxNone) {
     const double s1 = l * fx_scale<kFx3>(h3_120, 1, e), s3 = fx_scale<kFx3>(zn, 3, e);
     unsigned redo = 0;
     star3_walk<false, P, fx<kFx3>>(n, pitch, st, FxVec{u, fx_pow2(fx<kFx3>::B1 - e)},
                                 [&](size_t k, const Star3T<fx<kFx3>>& p) {
-      const fx<kFx3> v = star3_cubic6(p);
-      redo = redo << 1 | (unsigned)fx_short<kShortLoad3>(v);
-      f[k] = fma(s1, __ll2double_rn(madd<24>(p.u, p.S1).v), -to_double(v, s3));
+      const fx<kFx3> m = madd<24>(p.u, p.S1);
+      redo = redo << 1 | (unsigned)fx_short<kShortMass3>(m);
+      f[k] = fma(s1, __ll2double_rn(m.v), -to_double(star3_cubic6(p), s3));
     });
     star3_redo<P>(n, pitch, st, redo, [&](size_t k) {
       rhs3d_at(k, pitch, (long)(n + 1) * pitch, 120.0 * h3_120, 6.0 * zn, l, u, f);
@@ -617,7 +617,7 @@ __global__ void __launch_bounds__(kS3X * kS3Y, 3)
     k_nload_density3d(int n, int pitch, size_t st, double s140_6, double s210_2,
                       double s420_2, const double* __restrict__ u, double* __restrict__ nl,
                       Density3D b) {
-  const int e = star3_exponent<P>(n, pitch, st, u);
+  const int e = star3_exponent<P, true>(n, pitch, st, u);
   if (e != kFxNone) {
     using T = fx<kFx3>;
     const double a3 = fx_scale<kFx3>(s140_6, 3, e), a2 = fx_scale<kFx3>(s210_2, 2, e),

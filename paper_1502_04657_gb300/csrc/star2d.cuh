@@ -28,6 +28,7 @@ namespace fmg {
 
 constexpr int kFx2 = 61;  // fixed-point format of the walk (fixed.cuh)
 constexpr int kShortLoad2 = 36, kShortDensity2 = 44;  // results that a node takes in FP64
+constexpr int kShortMass2 = 41;  // 12 u + M1 of the right-hand side
 
 template <typename T>
 struct StarEdge {
@@ -100,8 +101,9 @@ void star2d_dispatch(const Grid& lv, F f) {
 }
 
 // The fixed-point exponent of this warp's tile (its 32 columns, R rows and the row before and
-// after them), or kFxNone; uniform over the warp.  The walk reads the tile again from L1.
-template <int R>
+// after them), or kFxNone; uniform over the warp.  The walk reads the tile again from L1.  LOAD: half of the
+// columns far below the largest value leave the tile to FP64.
+template <int R, bool LOAD>
 __device__ __forceinline__ int star2d_exponent(int n, int pitch, size_t st, const double* u) {
   const int i = kStarCols * blockIdx.x + threadIdx.x;
   const int j0 = 1 + R * (blockIdx.y * blockDim.y + threadIdx.y);
@@ -115,7 +117,7 @@ __device__ __forceinline__ int star2d_exponent(int n, int pitch, size_t st, cons
   const FxTop column = m;
   m.warp_max();
   const int e = m.exponent();
-  return 2 * __popc(__ballot_sync(0xffffffffu, column.far_below(e))) > 32 ? kFxNone : e;
+  return LOAD && 2 * __popc(__ballot_sync(0xffffffffu, column.far_below(e))) > 32 ? kFxNone : e;
 }
 
 // The walk in fixed point.  Sums of fixed-point values are exact, so the three opposite edges a

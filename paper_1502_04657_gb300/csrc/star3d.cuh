@@ -37,6 +37,7 @@ namespace fmg {
 
 constexpr int kFx3 = 59;  // fixed-point format of the walk (fixed.cuh)
 constexpr int kShortLoad3 = 40, kShortDensity3 = 44;  // results that a node takes in FP64
+constexpr int kShortMass3 = 42;  // 24 u + S1 of the right-hand side
 
 constexpr int kS3X = 32, kS3Y = 8;               // tile of columns (= threads)
 constexpr int kS3Z = 16;                         // planes per block of a double-float walk
@@ -99,8 +100,9 @@ void star3_dispatch(const Grid& lv, F f) {
 }
 
 // The fixed-point exponent of this block's tile (its P planes and the halo of the walk), or
-// kFxNone.  Reads the tile once; the walk reads it again from L2.
-template <int P>
+// kFxNone.  Reads the tile once; the walk reads it again from L2.  LOAD: half of the columns far below
+// the largest value leave the tile to FP64.
+template <int P, bool LOAD>
 __device__ __forceinline__ int star3_exponent(int n, int pitch, size_t st, const double* u) {
   __shared__ int top[2];
   const int tid = threadIdx.y * kS3X + threadIdx.x;
@@ -133,7 +135,7 @@ __device__ __forceinline__ int star3_exponent(int n, int pitch, size_t st, const
   m.neg = top[1];
   m.low = low;
   const int e = m.exponent();
-  return 2 * __syncthreads_count(columns.far_below(e)) > kS3X * kS3Y ? kFxNone : e;
+  return LOAD && 2 * __syncthreads_count(columns.far_below(e)) > kS3X * kS3Y ? kFxNone : e;
 }
 
 // node(k) for the nodes that a fixed-point walk of this block left short of bits, or tile() for half
