@@ -129,3 +129,50 @@ def test_right_hand_side_of_wide_range_from_zero_3d():
             s.residual_restrict(6, dev(f.ravel()), dev(np.zeros(f.size)), rc)
             got.append(host(rc))
     assert (np.abs(got[0] / got[1] - 1.0) <= 1e-9).all()
+
+
+@pytest.mark.parametrize("box", [0.01, 5.0, 30.0])
+def test_box_length_2d(box):
+    """n = 640 on boxes of other lengths (0.01, 5: fixed point; 30: FP64 with stored couplings), to
+    1e-13 of the largest value, as test_gpu_fixed_point has it on the unit box."""
+    from oracle import fmg_oracle as O
+
+    fmg = _fmg()
+    kw = dict(dim=2, coarse_cells=5, levels=8, w_const=0.3, w_quad=(1.0, 4.0, 0.0), zeta=7.0,
+              box_len=box)
+    op, p = O.Problem(**kw), fmg.Problem(**kw)
+    inside = fmg.Problem(**{**kw, "w_quad": (0.0, 0.0, 0.0)})
+    stores = fmg.estimate_bytes([p]) > fmg.estimate_bytes([inside]) + 4 * 8 * 640 ** 2
+    assert stores == (box == 30.0)
+    lev = O.build_level(op, 8, O.Level(O.Mesh(2, 320, box), None, None, None, None, None, None))
+    rng = np.random.default_rng(3500)
+    x, f = rng.normal(size=(2, p.size(8)))
+    y = torch.empty(p.size(8), dtype=torch.float64, device="cuda")
+    rc = torch.empty(p.size(7), dtype=torch.float64, device="cuda")
+    with fmg.Solver(p) as s:
+        s.apply_operator(8, dev(x), y)
+        ref = lev.L @ x
+        assert np.abs(host(y) - ref).max() <= 1e-13 * np.abs(ref).max()
+        s.jacobi(8, dev(f), dev(x), y)
+        ref = O.jacobi(lev, f, x, op.omega)
+        assert np.abs(host(y) - ref).max() <= 1e-13 * np.abs(ref).max()
+        s.residual_restrict(8, dev(f), dev(x), rc)
+        ref = lev.P.T @ (f - lev.L @ x)
+        assert np.abs(host(rc) - ref).max() <= 1e-13 * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("box", [0.01, 3.0])
+def test_box_length_3d(box):
+    """n = 96: fixed point against FP64 with stored couplings, 1e-13 of the largest value."""
+    kw = dict(dim=3, coarse_cells=3, levels=6, w_const=0.3, w_quad=(1.0, 2.0, 1.5), box_len=box)
+    rng = np.random.default_rng(3600)
+    x, f = rng.normal(size=(2, 95 ** 3))
+    got = []
+    for s in _mixed_and_fp64(**kw):
+        with s:
+            y, z = (torch.empty(x.size, dtype=torch.float64, device="cuda") for _ in range(2))
+            s.apply_operator(6, dev(x), y)
+            s.jacobi(6, dev(f * box / 96), dev(x), z)
+            got.append((host(y), host(z)))
+    for a, b in zip(*got):
+        assert np.abs(a - b).max() <= 1e-13 * np.abs(b).max()
