@@ -169,8 +169,9 @@ void fmg_eig_destroy(fmg_eig_handle* h);
  * must equal the handle's (FMG_EINVAL otherwise).  Synchronises the handle's stream; the
  * next solve uses the new values (they are uploaded from pinned host memory per solve).
  * Where the new potential changes the arithmetic of a level's operator (see the accuracy of the
- * component entry points), the solve graph is recorded again, and the first such change may
- * allocate: FMG_ENOMEM leaves the handle with its old values.                               */
+ * component entry points), the solve graph is recorded again, and so must be the caller's own
+ * graphs of component calls; the first such change may allocate (FMG_ENOMEM leaves the handle
+ * with its old values).                                                                     */
 int fmg_eig_set_params(fmg_eig_handle* h, const fmg_eig_problem* prob);
 
 /* Instrumentation (no counterpart in the paper).  fmg_eig_kernel_count: kernel launches

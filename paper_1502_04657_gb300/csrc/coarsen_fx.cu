@@ -9,9 +9,11 @@
 // units of 2^(e - 55) and adds multiples 1, 2 or 4 of it (the weights in quarters) to the sums of
 // all its targets; each target is converted once.  Only the truncation to 55 bits of the largest
 // entry around the node rounds (its mean, half a unit each, is added back), where the FP64 form
-// rounds every sum.  Measured: 16.6M 3D nodes 931 -> 245 us, 16.8M 2D nodes 370 -> 137 us
+// rounds every sum.  Measured: 16.6M 3D nodes 931 -> 280 us, 16.8M 2D nodes 370 -> 145 us
 // (in 3D 623 us with one load per entry: half of each sector was used, and L2 had to deliver the
-// rest again).
+// rest again; 245 and 137 us with one exponent per warp, which lost the entries far below its
+// largest; an exponent per thread with the neighbour's value shuffled, not its integer, spilled 1.3 KB
+// per thread in 3D).
 //
 // e comes from the diagonal entries of 2a and of the corners of its cell.  Nodes with an entry of
 // 2^(e + 1) or more, a negative one, infinities or NaN, a sum below 2^-9 of the largest entry (one

